@@ -28,8 +28,37 @@ WsLayout cc_ws_layout(int64_t N, int g, int K) {
     L.tensor = take(Kpad * (size_t)(64 + 1) * 4);
     L.tstate = take((size_t)N * 8);
     L.idx_prev = take((size_t)N * 2);
+    const bool pr = cc_prune_applies(N, K);
+    auto take_if = [&](size_t bytes) { size_t o = off; if (pr) off += cc_align_up(bytes, 256); return o; };
+    const size_t n_chunks = cc_align_up((size_t)(K + 63) / 64, 8), groups = (size_t)((N + 511) / 512);
+    const size_t Kp = (size_t)cc_tree_positions(K);
+    L.xs = take_if((size_t)N * g * 2);
+    L.pos = take_if((size_t)N * 4);
+    L.idx_s = take_if((size_t)N * 2);
+    L.ub = take_if((size_t)N * 4);
+    L.rise = take_if(groups * 16 * 4);
+    L.gap = take_if(cc_prune_gap_words(N, K) * 4);
+    L.list = take_if(groups * 4 * n_chunks * 2);
+    L.list_n = take_if(groups * 4 * 4);
+    L.order = take_if(Kp * 4);
+    L.tree = take_if(Kp * 4);
+    L.first = take_if(Kp * 4);
+    L.cs = take_if((size_t)K * g * 4);
+    L.c_prev = take_if((size_t)K * g * 4);
+    L.boxes = take_if(4 * n_chunks * g * 4);
+    L.moved = take_if(n_chunks * 4);
     L.total = off;
     return L;
+}
+
+// Pruned E-step: worth its preparation (tree, sort, lists) from this many distances on.
+bool cc_prune_applies(int64_t N, int K) { return N >= 32768 && K >= 2048 && N * (int64_t)K >= (int64_t)1 << 33; }
+
+// Words of the per (row block, chunk) gaps kept between the iterations of a fit; none where they would take
+// more than 4 GB (few chunks near a point there: the bounding boxes alone rule nearly all out).
+size_t cc_prune_gap_words(int64_t N, int K) {
+    const size_t w = (size_t)((N + 511) / 512) * 16 * cc_align_up((size_t)(K + 63) / 64, 8);
+    return w <= ((size_t)1 << 30) ? w : 0;
 }
 
 namespace {
@@ -112,12 +141,101 @@ bool use_tensor_path(const cc_ctx* ctx, int g, int K) {
     return true;   // AUTO and TENSOR: the tensor-core kernels win wherever they apply
 }
 
+PruneBuffers prune_buffers(const cc_ctx* ctx, const WsLayout& L, int64_t N, int g, int K) {
+    char* ws = static_cast<char*>(ctx->ws);
+    PruneBuffers b;
+    b.N = N; b.K = K; b.ld = (int)cc_align_up((size_t)(K + 63) / 64, 8);
+    b.Xs = reinterpret_cast<uint16_t*>(ws + L.xs);
+    b.pos = reinterpret_cast<unsigned*>(ws + L.pos);
+    b.idx_s = reinterpret_cast<uint16_t*>(ws + L.idx_s);
+    b.dist_s = reinterpret_cast<float*>(ws + L.dist_tmp);
+    b.ub = reinterpret_cast<float*>(ws + L.ub);
+    b.rise = reinterpret_cast<float*>(ws + L.rise);
+    b.gap = cc_prune_gap_words(N, K) ? reinterpret_cast<float*>(ws + L.gap) : nullptr;
+    b.list = reinterpret_cast<uint16_t*>(ws + L.list);
+    b.list_n = reinterpret_cast<unsigned*>(ws + L.list_n);
+    b.order = reinterpret_cast<unsigned*>(ws + L.order);
+    b.tree = reinterpret_cast<unsigned*>(ws + L.tree);
+    b.first = reinterpret_cast<unsigned*>(ws + L.first);
+    b.Cs = reinterpret_cast<float*>(ws + L.cs);
+    b.C_prev = reinterpret_cast<float*>(ws + L.c_prev);
+    b.box_t = reinterpret_cast<float*>(ws + L.boxes);
+    b.box_c = b.box_t + (size_t)2 * g * b.ld;
+    b.moved = reinterpret_cast<float*>(ws + L.moved);
+    // operand image (at most 96 bytes per position) and FP32 table where the exhaustive scan keeps its own
+    b.gB = reinterpret_cast<unsigned char*>(ws + L.tensor);
+    b.rescan = reinterpret_cast<float*>(ws + L.tensor + cc_align_up((size_t)K, 256) * 96);
+    b.tstate = reinterpret_cast<float2*>(ws + L.tstate);
+    b.status = reinterpret_cast<unsigned*>(ws + L.status);
+    b.flagged = reinterpret_cast<unsigned*>(ws + L.flagged);
+    b.acc = reinterpret_cast<long long*>(ws + L.status) + 24;  // words 48..53
+    return b;
+}
+
+// Tree over the centroids; with X, also the points in the order of its leaves.
+cudaError_t prune_order(cc_ctx* ctx, const PruneBuffers& b, const uint16_t* X, int g, const float* C, cudaStream_t st) {
+    cudaError_t e = cc_launch_tree(ctx, C, b.K, g, b.order, b.first, b.tree, st);
+    if (e != cudaSuccess || !X) return e;
+    int levels = 0;
+    while ((1 << levels) < cc_tree_positions(b.K)) ++levels;
+    return cc_launch_sort_points(ctx, X, b.N, g, b.tree, levels, reinterpret_cast<uint16_t*>(b.tstate), b.pos, b.first, b.Xs, st);
+}
+
+// Up to this sub-vector length the bounding boxes alone leave well under all chunks to a first E-step.
+constexpr int PRUNE_COLD_G = 6;
+
+bool use_pruned(const cc_ctx* ctx, int64_t N, int g, int K, int e_steps) {
+    return ctx->path == CC_PATH_AUTO && cc_prune_applies(N, K) && (g <= PRUNE_COLD_G || (g <= 8 && e_steps >= 4));
+}
+
 cudaError_t assign_any(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, int g, const float* C, int K,
                        uint16_t* idx, float* dist, double* objective, int64_t* n_resolved, cudaStream_t st) {
+    if (use_pruned(ctx, N, g, K, 1)) {
+        const PruneBuffers b = prune_buffers(ctx, L, N, g, K);
+        cudaError_t e = prune_order(ctx, b, X, g, C, st);
+        if (e == cudaSuccess) e = cc_launch_assign_pruned(ctx, b, g, C, CC_PRUNE_COLD, st);
+        if (e == cudaSuccess && (objective || n_resolved)) e = cc_launch_sum_exact(ctx, b, true, objective, n_resolved, st);
+        if (e == cudaSuccess)
+            e = cc_launch_unsort(ctx, b.pos, N, b.idx_s, b.dist_s, idx, dist, reinterpret_cast<unsigned*>(b.tstate), b.status, b.flagged, st);
+        return e;
+    }
     if (!dist) dist = reinterpret_cast<float*>(static_cast<char*>(ctx->ws) + L.dist_tmp);
     if (use_tensor_path(ctx, g, K))
         return cc_launch_assign_tensor(ctx, L, X, N, g, C, K, idx, dist, objective, n_resolved, st);
     return cc_launch_assign_ffma(ctx, L, X, N, g, C, K, idx, dist, objective, n_resolved, st);
+}
+
+// The Lloyd loop on points in spatial order: sorted once, codes and distances put back at the end.
+cudaError_t fit_pruned(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, int g, int K, int iters, float* C,
+                       uint16_t* idx, float* dist, int32_t* counts, double* objective_trace, cudaStream_t st) {
+    const PruneBuffers b = prune_buffers(ctx, L, N, g, K);
+    uint16_t* idx_prev = reinterpret_cast<uint16_t*>(static_cast<char*>(ctx->ws) + L.idx_prev);
+    cudaError_t e = prune_order(ctx, b, X, g, C, st);
+    for (int it = 0; it < iters && e == cudaSuccess; ++it) {
+        bool have_max = true;
+        if (it == 0 && g > PRUNE_COLD_G) {
+            e = cc_launch_assign_tensor(ctx, L, b.Xs, N, g, C, K, b.idx_s, b.dist_s, nullptr, nullptr, st);
+            have_max = false;
+        } else {
+            // the chunks are redrawn once the centroids have left their starting points, and in every
+            // iteration where no gaps depend on them
+            const bool redraw = it == 1 || (it > 1 && !b.gap);
+            if (redraw) e = prune_order(ctx, b, nullptr, g, C, st);
+            if (e == cudaSuccess)
+                e = cc_launch_assign_pruned(ctx, b, g, C, it == 0 ? CC_PRUNE_COLD : redraw ? CC_PRUNE_RESTART : CC_PRUNE_NEXT, st);
+        }
+        if (e == cudaSuccess && objective_trace) e = cc_launch_sum_exact(ctx, b, have_max, objective_trace + it, nullptr, st);
+        if (e != cudaSuccess) break;
+        if (it == 0) {
+            e = cc_launch_update(ctx, L, b.Xs, N, g, b.idx_s, K, C, counts, st);
+            if (e == cudaSuccess && iters > 1)
+                e = cudaMemcpyAsync(idx_prev, b.idx_s, sizeof(uint16_t) * (size_t)N, cudaMemcpyDeviceToDevice, st);
+        } else {
+            e = cc_launch_update_delta(ctx, L, b.Xs, N, g, b.idx_s, idx_prev, K, C, counts, st);
+        }
+    }
+    if (e == cudaSuccess) e = cc_launch_unsort(ctx, b.pos, N, b.idx_s, b.dist_s, idx, dist, nullptr, b.status, b.flagged, st);
+    return e;
 }
 
 }  // namespace
@@ -382,6 +500,8 @@ cc_status cc_fit(cc_ctx* ctx, const uint16_t* X, int64_t N, int g, int K, int it
     if (cudaSetDevice(ctx->device) != cudaSuccess) return CC_ERR_CUDA;
     const WsLayout L = cc_ws_layout(N, g, K);
     cudaStream_t st = (cudaStream_t)stream;
+    if (iters > 0 && use_pruned(ctx, N, g, K, iters))
+        return from_cuda(fit_pruned(ctx, L, X, N, g, K, iters, C, idx, dist, counts, objective_trace, st));
     for (int it = 0; it < iters; ++it) {
         cudaError_t e = assign_any(ctx, L, X, N, g, C, K, idx, dist, objective_trace ? objective_trace + it : nullptr,
                                    nullptr, st);

@@ -62,7 +62,8 @@ constexpr int CC_ARRIVAL_WORD = 64, CC_ARRIVAL_COUNTERS = 960;
 // Carving of the workspace for a problem (N, g, K).  All offsets 256-byte aligned.
 struct WsLayout {
     size_t status;     // CC_STATUS_BYTES: 1024 x u32: [0] status bits, [2..3] flagged counter (u64), [8] last-block counter of the objective
-                       // sum, [32..35] tensor-path parameters, [36] codebook quantiser's maximum, [64..1023] arrival
+                       // sum, [32..35] tensor-path parameters, [36] codebook quantiser's maximum, [40] largest distance, [41] a counter,
+                       // [48..53] exact objective sum (zero between calls), [64..1023] arrival
                        // counters of the layer forward's split reduction (zero between calls)
     size_t cprep;      // staged codebook for the FFMA E-step
     size_t flagged;    // u32 list of points sent to the exact stage
@@ -76,8 +77,38 @@ struct WsLayout {
     size_t tensor;     // staging of the tensor-core E-step (split codebook operand)
     size_t tstate;     // float2 N: (second-best chunk minimum, best chunk id) from the tensor-core scan
     size_t idx_prev;   // u16 N: codes of the previous M-step inside cc_fit
+    // pruned E-step (nothing where it does not apply, see cc_prune_applies)
+    size_t xs;         // u16 N x g: points in spatial order
+    size_t pos;        // u32 N: point -> position
+    size_t idx_s;      // u16 N: codes by position
+    size_t ub;         // float N: upper bounds of the last E-step
+    size_t rise;       // float per row block of 32 points
+    size_t gap;        // float row blocks x chunks (only where it is used, see cc_prune_gap_words)
+    size_t list;       // u16 tiles of 128 points x chunks
+    size_t list_n;     // u32 tiles
+    size_t order;      // u32 Kp: position -> centroid
+    size_t tree;       // u32 Kp: nodes of the k-d tree
+    size_t first;      // u32 Kp: leaf -> position of its first point; scratch of the tree
+    size_t cs;         // float K x g: codebook by position
+    size_t c_prev;     // float K x g: codebook of the last E-step
+    size_t boxes;      // float 2 x chunks x 2 g
+    size_t moved;      // float chunks
     size_t total;
 };
+
+// Buffers of the pruned E-step (cc_assign_pruned.cu), carved from the workspace.
+struct PruneBuffers {
+    int64_t N;
+    int K, ld;
+    uint16_t* Xs; unsigned* pos; uint16_t* idx_s; float* dist_s;
+    float* ub; float* rise; float* gap;
+    uint16_t* list; unsigned* list_n; unsigned* order; unsigned* tree; unsigned* first;
+    float* Cs; float* C_prev; float* box_t; float* box_c; float* moved;
+    unsigned char* gB; float* rescan; float2* tstate; unsigned* status; unsigned* flagged; long long* acc;
+};
+enum { CC_PRUNE_COLD = 0,      // first E-step: bounds from the tree leaf each point falls into
+       CC_PRUNE_RESTART = 1,   // bounds from the previous codes; the chunks may have been redrawn, kept gaps start anew
+       CC_PRUNE_NEXT = 2 };    // same chunks as in the previous E-step
 
 constexpr int CC_KPAD = 1024;          // staged codebook is padded to a multiple of this
 constexpr int CC_OBJ_BLOCKS = 1024;    // partial sums of the objective reduction
@@ -125,6 +156,18 @@ cudaError_t cc_launch_tensor_finish_only(cc_ctx*, const WsLayout&, const uint16_
 cudaError_t cc_launch_assign_tail(cc_ctx*, const WsLayout&, const uint16_t* X, int64_t N, int g, const float* C,
                                   int K, uint16_t* idx, float* dist, double* objective, int64_t* n_resolved,
                                   cudaStream_t);
+
+// Spatial order and pruned E-step.
+bool cc_prune_applies(int64_t N, int K);
+size_t cc_prune_gap_words(int64_t N, int K);
+int cc_tree_positions(int K);
+cudaError_t cc_launch_tree(cc_ctx*, const float* C, int K, int g, unsigned* order, unsigned* scratch, unsigned* tree, cudaStream_t);
+cudaError_t cc_launch_sort_points(cc_ctx*, const uint16_t* X, int64_t N, int g, const unsigned* tree, int levels, uint16_t* leaf,
+                                  unsigned* pos, unsigned* first, uint16_t* Xs, cudaStream_t);
+cudaError_t cc_launch_unsort(cc_ctx*, const unsigned* pos, int64_t N, const uint16_t* idx_s, const float* dist_s, uint16_t* idx,
+                             float* dist, unsigned* marks, unsigned* status, unsigned* flagged, cudaStream_t);
+cudaError_t cc_launch_assign_pruned(cc_ctx*, const PruneBuffers&, int g, const float* C, int mode, cudaStream_t);
+cudaError_t cc_launch_sum_exact(cc_ctx*, const PruneBuffers&, bool have_max, double* objective, int64_t* n_resolved, cudaStream_t);
 
 // Compressed linear layer: y = x . decode(C16, idx)^T (+ bias), the decoded weight never stored.
 size_t cc_linear_scratch_bytes(int64_t M, int64_t d_out, int64_t d_in, int sm_count);

@@ -43,6 +43,11 @@ __device__ __forceinline__ bool elect_one() {
     return e != 0u;
 }
 
+// One arrival for a converged warp.
+__device__ __forceinline__ void mbar_arrive_warp(uint32_t bar) {
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar) : "memory");
+}
+
 // Bounded wait.  Returns false when the CTA is aborting (this or another waiter timed out).
 // Every lane of a warp waits on the same barrier word with the same parity, so the branches are
 // uniform across the warp and say so (bra.uni): the compiler then needs no convergence barriers
