@@ -143,8 +143,12 @@ chunk_bounds_kernel(const float* __restrict__ C, int K, const unsigned* __restri
 }
 
 // ---------------------------------------------------------------------------------------------
-// A list entry is 16 bits: the chunk (10 bits) and the row blocks of the tile that need it (4 bits above).
+// A list entry is 16 bits: the chunk (10 bits), the row blocks of the tile that need it (4 bits above), and
+// in the first entry of a pair whether every warp has to look at that pair (see the scan).  A list is padded to
+// whole pairs with an entry that nobody needs.
 constexpr int PR_MASK_SHIFT = 10;
+constexpr unsigned PR_CHUNK_MASK = (1u << PR_MASK_SHIFT) - 1u, PR_LOOK = 1u << 14;
+constexpr int PR_LOOK_EVERY = 4;         // pairs
 
 struct ListArgs {
     const uint16_t* Xs; int64_t N;
@@ -359,6 +363,7 @@ pruned_list_kernel(const ListArgs a) {
     int inc = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
+    const int total = __shfl_sync(0xffffffffu, inc, 31);
     const int64_t out_tile = (int64_t)blockIdx.x * PR_TILES + tile;
     uint16_t* out = a.list + out_tile * a.ld;
     for (int j = part; j < n_words; j += 4) {
@@ -367,9 +372,14 @@ pruned_list_kernel(const ListArgs a) {
         unsigned m = 0u;
 #pragma unroll
         for (int q = 0; q < 4; ++q) m |= ((need[tile * 4 + q][j] >> lane) & 1u) << q;
-        if (m) out[at] = (uint16_t)((m << PR_MASK_SHIFT) | (unsigned)(j * 32 + lane));
+        const int pair = at >> 1;
+        const bool look = !(at & 1) && ((pair % PR_LOOK_EVERY) == PR_LOOK_EVERY - 1 || at + 2 >= total);
+        if (m) out[at] = (uint16_t)((look ? PR_LOOK : 0u) | (m << PR_MASK_SHIFT) | (unsigned)(j * 32 + lane));
     }
-    if (part == 0 && lane == 31) a.list_n[out_tile] = (unsigned)inc;
+    if (part == 0 && lane == 0) {
+        if (total & 1) out[total] = 0;
+        a.list_n[out_tile] = (unsigned)total;
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -378,14 +388,14 @@ pruned_list_kernel(const ListArgs a) {
 //   warps 0..3  epilogue: warp w owns row block w = TMEM lanes 32 w.., and writes that block's rows of the A
 //               operand, one tile ahead (loads two tiles ahead)
 //   warp 4      copies lists and chunks (one thread)
-//   warp 5      issues the MMAs (one thread): 128 points x 64 centroids into one of two accumulators
-// An entry whose mask leaves a row block out costs that warp nothing: the MMA thread releases the accumulator in
-// its stead, and entries are announced on a ring of eight barriers, so that a warp has to look at (wait for and
-// release) every eighth entry only, which keeps it within one phase of every barrier, and at a tile's last
-// entry, after which the tile's A rows are free.
+//   warp 5      issues the MMAs (one thread): 128 points x two chunks of the list at a time
+// A pair of chunks whose masks leave a row block out costs that warp nothing: the MMA thread releases the
+// accumulator in its stead.  Pairs are announced on a ring of eight barriers, and every warp looks at (waits for
+// and releases) at least every fourth pair, which keeps it within one phase of every barrier, and a tile's last
+// pair, after which the tile's A rows are free.
 // Measured on the way here: a successful wait on an mbarrier costs an issuing thread about 110 cycles right behind
-// an MMA, a further one 45, the MMA and its commit together 48 (N = 64): one issuer for four tiles left the
-// epilogue waiting (335 cycles per 128 x 64 block and SM; one issuer per tile 222).
+// an MMA, a further one 45, the MMA and its commit together 48 (N = 64).  Per 128 x 64 block and SM: one issuer
+// for four tiles 335 cycles, one issuer per tile 222, one block per tile with a handshake per chunk 217.
 constexpr int PS_THREADS = 6 * 32;
 constexpr int PS_BLOCKS = 4;             // resident per SM
 constexpr int PS_LISTS = 3;
@@ -482,7 +492,7 @@ assign_pruned_kernel(const ScanArgs a) {
     uint16_t* sL = reinterpret_cast<uint16_t*>(sB + STAGES * 2 * CH);    // PS_LISTS lists
     uint64_t* bars = reinterpret_cast<uint64_t*>(sL + PS_LISTS * PR_MAX_CHUNKS);
     uint64_t* b_full = bars, *b_empty = bars + STAGES, *t_full = bars + 2 * STAGES, *t_empty = t_full + PS_RING;
-    uint64_t* a_full = t_empty + 2, *l_full = a_full + 2, *l_empty = l_full + PS_LISTS;
+    uint64_t* a_full = t_empty + 1, *l_full = a_full + 2, *l_empty = l_full + PS_LISTS;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(l_empty + PS_LISTS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* sN = reinterpret_cast<volatile int*>(tmem_slot + 2);   // PS_LISTS list lengths
@@ -494,7 +504,8 @@ assign_pruned_kernel(const ScanArgs a) {
         auto init = [&](uint64_t* b, int n) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(n)); };
         for (int s = 0; s < STAGES; ++s) { init(b_full + s, 1); init(b_empty + s, 1); }
         for (int s = 0; s < PS_RING; ++s) init(t_full + s, 1);
-        for (int s = 0; s < 2; ++s) { init(t_empty + s, 4); init(a_full + s, TM); }
+        init(t_empty, 4);
+        for (int s = 0; s < 2; ++s) init(a_full + s, TM);
         for (int s = 0; s < PS_LISTS; ++s) { init(l_full + s, 1); init(l_empty + s, 5); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -520,8 +531,8 @@ assign_pruned_kernel(const ScanArgs a) {
                 const int buf = lists % PS_LISTS;
                 if (lists >= PS_LISTS && !mbar_wait(smem_u32(l_empty + buf), ((lists / PS_LISTS) & 1) ^ 1, abort_flag)) return false;
                 sN[buf] = n_next;
-                const uint32_t bytes = (uint32_t)(n_next * 2 + 15) & ~15u, bar = smem_u32(l_full + buf);
-                if (bytes) {
+                const uint32_t bytes = (uint32_t)((n_next + 1) / 2 * 4 + 15) & ~15u, bar = smem_u32(l_full + buf);
+                if (n_next) {
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                                  ::"r"(smem_u32(sL + buf * PR_MAX_CHUNKS)),
@@ -542,17 +553,14 @@ assign_pruned_kernel(const ScanArgs a) {
                 const int n = sN[buf];
                 const uint16_t* L = sL + buf * PR_MAX_CHUNKS;
                 for (int e = 0; e < n; e += 2) {
-                    constexpr unsigned cm = (1u << PR_MASK_SHIFT) - 1u;
                     const unsigned two = *reinterpret_cast<const unsigned*>(L + e);
-                    const unsigned c0 = two & cm, c1 = (two >> 16) & cm;
                     if (!mbar_wait(smem_u32(b_empty + st), ph ^ 1, abort_flag)) { ok = false; break; }
                     const uint32_t bar = smem_u32(b_full + st), dst = smem_u32(sB + st * 2 * CH);
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(e + 1 < n ? 2 * CH : CH) : "memory");
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(2 * CH) : "memory");
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                 ::"r"(dst), "l"(a.gB + (int64_t)c0 * CH), "r"(CH), "r"(bar) : "memory");
-                    if (e + 1 < n)
-                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                     ::"r"(dst + CH), "l"(a.gB + (int64_t)c1 * CH), "r"(CH), "r"(bar) : "memory");
+                                 ::"r"(dst), "l"(a.gB + (two & PR_CHUNK_MASK) * CH), "r"(CH), "r"(bar) : "memory");
+                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"(dst + CH), "l"(a.gB + ((two >> 16) & PR_CHUNK_MASK) * CH), "r"(CH), "r"(bar) : "memory");
                     ++total;
                     if (++st == STAGES) { st = 0; ph ^= 1; }
                 }
@@ -572,12 +580,12 @@ assign_pruned_kernel(const ScanArgs a) {
     } else if (warp == 5) {
         // ------------------------------------------------------------ MMA: one thread issues
         if (elect_one()) {
-            const uint32_t idesc = (1u << 4) | ((uint32_t)(PR_CHUNK >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+            const uint32_t idesc = (1u << 4) | ((uint32_t)(2 * PR_CHUNK >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
             const uint64_t descA0 = make_desc(smem_u32(sA), TM * 16, 128);
             const uint64_t descB0 = make_desc(smem_u32(sB), 128, KD * 16);
             bool ok = true;
             int st = 0;
-            uint32_t ph = 0, seq = 0u;                       // seq: entries so far
+            uint32_t ph = 0, seq = 0u;                       // seq: pairs so far
             for (int it = 0; it < n_iter && ok; ++it) {
                 const int buf = it % PS_LISTS, ab = it & 1;
                 ok = mbar_wait(smem_u32(l_full + buf), (it / PS_LISTS) & 1, abort_flag) &&
@@ -586,37 +594,28 @@ assign_pruned_kernel(const ScanArgs a) {
                 const int n = sN[buf];
                 const uint16_t* L = sL + buf * PR_MAX_CHUNKS;
                 const uint64_t descA = descA0 + (uint64_t)((ab * A_TILE) >> 4);
-                for (int e = 0; e < n && ok; e += 2) {
+                for (int e = 0; e < n && ok; e += 2, ++seq) {
                     const unsigned two = *reinterpret_cast<const unsigned*>(L + e);
-                    ok = mbar_wait(smem_u32(b_full + st), ph, abort_flag);
+                    const unsigned m = ((two >> PR_MASK_SHIFT) | (two >> (16 + PR_MASK_SHIFT))) & 15u;
+                    const unsigned left_out = (two & PR_LOOK) ? 0u : 4u - (unsigned)__popc(m);
+                    ok = mbar_wait(smem_u32(b_full + st), ph, abort_flag) && mbar_wait(smem_u32(t_empty), (seq & 1u) ^ 1u, abort_flag);
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    if (left_out) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(t_empty)), "r"(left_out) : "memory");
+                    const uint64_t descB = descB0 + (uint64_t)((st * 2 * CH) >> 4);
 #pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        if (e + q >= n || !ok) continue;
-                        const bool look = (seq % PS_RING) == PS_RING - 1 || e + q + 1 == n;
-                        const unsigned left_out = look ? 0u : 4u - (unsigned)__popc((two >> (16 * q + PR_MASK_SHIFT)) & 15u);
-                        const uint32_t slot = seq & 1u, te = smem_u32(t_empty + slot);
-                        ok = mbar_wait(te, ((seq >> 1) & 1u) ^ 1u, abort_flag);
-                        if (!ok) break;
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        if (left_out) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(te), "r"(left_out) : "memory");
-                        const uint64_t descB = descB0 + (uint64_t)(((st * 2 + q) * CH) >> 4);
-#pragma unroll
-                        for (int s = 0; s < KD / 16; ++s) {
-                            const uint64_t da = descA + (uint64_t)((s * 2 * (TM * 16)) >> 4);
-                            const uint64_t db = descB + (uint64_t)((s * 2 * 128) >> 4);
-                            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                                         ::"r"(tmem + slot * PR_CHUNK), "l"(da), "l"(db), "r"(idesc), "r"(s > 0 ? 1u : 0u) : "memory");
-                        }
-                        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                                     ::"r"(smem_u32(t_full + (seq % PS_RING))) : "memory");
-                        ++seq;
+                    for (int s = 0; s < KD / 16; ++s) {
+                        const uint64_t da = descA + (uint64_t)((s * 2 * (TM * 16)) >> 4);
+                        const uint64_t db = descB + (uint64_t)((s * 2 * 128) >> 4);
+                        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                                     ::"r"(tmem), "l"(da), "l"(db), "r"(idesc), "r"(s > 0 ? 1u : 0u) : "memory");
                     }
-                    if (ok)   // the pair may be overwritten once these MMAs have read it
-                        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                                     ::"r"(smem_u32(b_empty + st)) : "memory");
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                                 ::"r"(smem_u32(t_full + (seq % PS_RING))) : "memory");
+                    // the pair may be overwritten once these MMAs have read it
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                                 ::"r"(smem_u32(b_empty + st)) : "memory");
                     if (++st == STAGES) { st = 0; ph ^= 1; }
                 }
                 if (ok) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(l_empty + buf)) : "memory");
@@ -632,11 +631,15 @@ assign_pruned_kernel(const ScanArgs a) {
         constexpr float u = (float)Cfg::ERR_UNITS * 5.9604644775390625e-8f;
         auto point = [&](int it) { return ((int64_t)blockIdx.x + (int64_t)it * gridDim.x) * TM + r; };
         auto point_or_none = [&](int it) { return it < n_iter ? point(it) : a.N; };
-        // ||x||^2 less everything that a computed score may be too large by, for gap's lower bound on a distance
+        // For gap: base + invS_dn * score is a lower bound on the squared distance, rounding of the square root and
+        // of the subtractions included: ||x||^2 less everything that a computed score may be too large by, the whole
+        // scaled down a little.
+        constexpr float dn = 1.0f - 4.0f * u - 4e-6f;
+        const float invS_dn = prm.invS * dn;
         auto base_of = [&](const unsigned* w) {
             const float A = word_norm<G>(w);
-            return A * (1.0f - 5.0f * u - 1e-6f) - prm.invS * (1e-4f * sqrtf(A * (float)G) + norm_abs_loss<G>(prm)) -
-                   (float)G * 5.0f * u * 3.73e-9f;           // coordinates below 2^-14 count as 2^-14
+            return dn * (A * (1.0f - 5.0f * u - 1e-6f) - prm.invS * (1e-4f * sqrtf(A * (float)G) + norm_abs_loss<G>(prm)) -
+                         (float)G * 5.0f * u * 3.73e-9f);    // coordinates below 2^-14 count as 2^-14
         };
         constexpr int W = (G + 1) / 2;
         unsigned xw[W];
@@ -647,7 +650,9 @@ assign_pruned_kernel(const ScanArgs a) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(a_full)) : "memory");
         load_words<G>(a.Xs, point_or_none(1), a.N, xw);
-        uint32_t okw = 1u, seq = 0u;
+        const uint32_t tf = smem_u32(t_full), te = smem_u32(t_empty);
+        const unsigned interest = (0x10001u << (PR_MASK_SHIFT + warp)) | PR_LOOK;
+        uint32_t okw = 1u, seq = 0u;                         // seq: pairs so far
         for (int it = 0; it < n_iter && okw; ++it) {
             const int buf = it % PS_LISTS;
             base_now = base_next;
@@ -674,37 +679,48 @@ assign_pruned_kernel(const ScanArgs a) {
             const uint16_t* L = sL + buf * PR_MAX_CHUNKS;
             float b1 = INFINITY, b2 = INFINITY;
             int bc = 0;
-            for (int e = 0; e < n; ++e, ++seq) {
-                const unsigned ent = L[e];
-                const bool mine = (ent >> (PR_MASK_SHIFT + warp)) & 1u;
-                if (!mine && (seq % PS_RING) != PS_RING - 1 && e + 1 < n) continue;
-                const unsigned chunk = ent & ((1u << PR_MASK_SHIFT) - 1u);
+            auto take = [&](unsigned chunk, uint32_t taddr, bool last) {
                 float mv = 0.f;
                 if constexpr (GAP) mv = __ldg(a.moved + chunk);
-                mbar_wait_acc(smem_u32(t_full + (seq % PS_RING)), (seq / PS_RING) & 1u, abort_flag, okw);
-                if (!okw) break;
-                const uint32_t slot = seq & 1u;
-                if (!mine) { mbar_arrive_warp(smem_u32(t_empty + slot)); continue; }
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 uint32_t v0[32], v1[32];
-                TMEM_LD32(v0, tbase + slot * PR_CHUNK);
-                TMEM_LD32(v1, tbase + slot * PR_CHUNK + 32);
+                TMEM_LD32(v0, taddr);
+                TMEM_LD32(v1, taddr + 32);
                 TMEM_WAIT64(v0, v1);
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                mbar_arrive_warp(smem_u32(t_empty + slot));
+                if (last) {                                  // this warp's last look at the accumulator
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    mbar_arrive_warp(te);
+                }
                 const float mn = chunk_min64(v0, v1);
                 const bool better = mn < b1;
                 b2 = better ? b1 : fminf(b2, mn);
                 bc = better ? (int)chunk : bc;
                 b1 = better ? mn : b1;
                 if constexpr (GAP) {
-                    // distance to the chunk, rounded down, less ub; smallest over the row block
-                    const float d2 = fmaxf(fmaf(mn, prm.invS, base_now) * (1.0f - 4.0f * u - 1e-6f), 0.f);
+                    // distance to the chunk less ub, smallest over the row block, with the totals of both sides at this
+                    // time added so that later ones can be taken off
                     float s;
-                    asm("sqrt.approx.f32 %0, %1;" : "=f"(s) : "f"(d2));
-                    s = redux_min(fmaf(s, 1.0f - 1e-6f, -ub));
+                    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(fmaxf(fmaf(mn, invS_dn, base_now), 0.f)));
+                    s = redux_min(s - ub);
                     if (lane == 0) gap_row[chunk] = __fadd_rd(__fadd_rd(s, mv), rise);
                 }
+            };
+            // A wait that gives up is only acted upon after the tile: once the abort flag is up the remaining waits
+            // return at their next look at it, and reading an accumulator that was never written or releasing it once
+            // more harms nothing.
+            const unsigned* pairs = reinterpret_cast<const unsigned*>(L);
+            unsigned two = n > 0 ? pairs[0] : 0u;
+            for (int e = 0; e < n; e += 2) {
+                const unsigned now = two;
+                two = pairs[(e >> 1) + 1];                   // at most one word past the list, inside the ring place or the next
+                const uint32_t bar = tf + (seq & (PS_RING - 1)) * 8, par = (seq / PS_RING) & 1u;
+                ++seq;
+                if (!(now & interest)) continue;
+                mbar_wait_acc(bar, par, abort_flag, okw);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const bool m0 = now & (1u << (PR_MASK_SHIFT + warp)), m1 = now & (1u << (16 + PR_MASK_SHIFT + warp));
+                if (m0) take(now & PR_CHUNK_MASK, tbase, !m1);
+                if (m1) take((now >> 16) & PR_CHUNK_MASK, tbase + PR_CHUNK, true);
+                if (!m0 && !m1) mbar_arrive_warp(te);
             }
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(l_empty + buf)) : "memory");
@@ -856,7 +872,7 @@ pruned_resolve_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __
             const unsigned ent = __ldg(L + e);
             if (!((ent >> bit) & 1u)) continue;
             if ((turn++ & 1) != half) continue;
-            const int p = (int)(ent & ((1u << PR_MASK_SHIFT) - 1u)) * PR_CHUNK + q;
+            const int p = (int)(ent & PR_CHUNK_MASK) * PR_CHUNK + q;
             if (p >= K) continue;
             float c[G], dq = 0.f;
 #pragma unroll
