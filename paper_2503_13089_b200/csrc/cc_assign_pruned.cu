@@ -387,8 +387,8 @@ pruned_list_kernel(const ListArgs a) {
 // share an SM and its tensor memory, so that the waits of one are covered by the others.
 //   warps 0..3  epilogue: warp w owns row block w = TMEM lanes 32 w.., and writes that block's rows of the A
 //               operand, one tile ahead (loads two tiles ahead)
-//   warp 4      copies lists and chunks (one thread)
-//   warp 5      issues the MMAs (one thread): 128 points x two chunks of the list at a time
+//   warp 4      copies lists and chunks and issues the MMAs (one thread): 128 points x two chunks of the list at
+//               a time
 // A pair of chunks whose masks leave a row block out costs that warp nothing: the MMA thread releases the
 // accumulator in its stead.  Pairs are announced on a ring of eight barriers, and every warp looks at (waits for
 // and releases) at least every fourth pair, which keeps it within one phase of every barrier, and a tile's last
@@ -396,7 +396,7 @@ pruned_list_kernel(const ListArgs a) {
 // Measured on the way here: a successful wait on an mbarrier costs an issuing thread about 110 cycles right behind
 // an MMA, a further one 45, the MMA and its commit together 48 (N = 64).  Per 128 x 64 block and SM: one issuer
 // for four tiles 335 cycles, one issuer per tile 222, one block per tile with a handshake per chunk 217.
-constexpr int PS_THREADS = 6 * 32;
+constexpr int PS_THREADS = 5 * 32;
 constexpr int PS_BLOCKS = 4;             // resident per SM
 constexpr int PS_LISTS = 3;
 constexpr int PS_RING = 8;
@@ -491,7 +491,7 @@ assign_pruned_kernel(const ScanArgs a) {
     unsigned char* sB = sA + 2 * A_TILE;                                 // STAGES pairs of chunks
     uint16_t* sL = reinterpret_cast<uint16_t*>(sB + STAGES * 2 * CH);    // PS_LISTS lists
     uint64_t* bars = reinterpret_cast<uint64_t*>(sL + PS_LISTS * PR_MAX_CHUNKS);
-    uint64_t* b_full = bars, *b_empty = bars + STAGES, *t_full = bars + 2 * STAGES, *t_empty = t_full + PS_RING;
+    uint64_t* b_full = bars, *t_full = bars + STAGES, *t_empty = t_full + PS_RING;
     uint64_t* a_full = t_empty + 1, *l_full = a_full + 2, *l_empty = l_full + PS_LISTS;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(l_empty + PS_LISTS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -502,11 +502,11 @@ assign_pruned_kernel(const ScanArgs a) {
 
     if (tid == 0) {
         auto init = [&](uint64_t* b, int n) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(n)); };
-        for (int s = 0; s < STAGES; ++s) { init(b_full + s, 1); init(b_empty + s, 1); }
+        for (int s = 0; s < STAGES; ++s) init(b_full + s, 1);
         for (int s = 0; s < PS_RING; ++s) init(t_full + s, 1);
         init(t_empty, 4);
         for (int s = 0; s < 2; ++s) init(a_full + s, TM);
-        for (int s = 0; s < PS_LISTS; ++s) { init(l_full + s, 1); init(l_empty + s, 5); }
+        for (int s = 0; s < PS_LISTS; ++s) { init(l_full + s, 1); init(l_empty + s, 4); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -520,16 +520,20 @@ assign_pruned_kernel(const ScanArgs a) {
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 4) {
-        // ------------------------------------------------------------ copies: lists (two tiles ahead), chunks
+        // ------------------------------------------------------------ copies and MMAs: one thread
         if (elect_one()) {
-            int st = 0, total = 0, lists = 0;
-            uint32_t ph = 0;
+            const uint32_t idesc = (1u << 4) | ((uint32_t)(2 * PR_CHUNK >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+            const uint64_t descA0 = make_desc(smem_u32(sA), TM * 16, 128);
+            const uint64_t descB0 = make_desc(smem_u32(sB), 128, KD * 16);
+            const uint32_t te = smem_u32(t_empty), tf = smem_u32(t_full), bf = smem_u32(b_full), sb = smem_u32(sB);
             bool ok = true;
+            // lists: sent two tiles ahead
+            int lists = 0;
             auto length = [&](int it) { return it < n_iter ? (int)__ldg(a.list_n + blockIdx.x + (int64_t)it * gridDim.x) : 0; };
             int n_next = length(0), n_after = length(1);
-            auto send_list = [&]() {                         // the next list into its ring place
+            auto send_list = [&]() {
                 const int buf = lists % PS_LISTS;
-                if (lists >= PS_LISTS && !mbar_wait(smem_u32(l_empty + buf), ((lists / PS_LISTS) & 1) ^ 1, abort_flag)) return false;
+                if (lists >= PS_LISTS && !mbar_wait(smem_u32(l_empty + buf), ((lists / PS_LISTS) & 1) ^ 1, abort_flag)) { ok = false; return; }
                 sN[buf] = n_next;
                 const uint32_t bytes = (uint32_t)((n_next + 1) / 2 * 4 + 15) & ~15u, bar = smem_u32(l_full + buf);
                 if (n_next) {
@@ -543,82 +547,87 @@ assign_pruned_kernel(const ScanArgs a) {
                 ++lists;
                 n_next = n_after;
                 n_after = length(lists + 1);
-                return true;
             };
-            while (lists < 2 && lists < n_iter && ok) ok = send_list();
-            for (int it = 0; it < n_iter && ok; ++it) {
-                const int buf = it % PS_LISTS;
-                ok = mbar_wait(smem_u32(l_full + buf), (it / PS_LISTS) & 1, abort_flag);
-                if (!ok) break;
-                const int n = sN[buf];
-                const uint16_t* L = sL + buf * PR_MAX_CHUNKS;
-                for (int e = 0; e < n; e += 2) {
-                    const unsigned two = *reinterpret_cast<const unsigned*>(L + e);
-                    if (!mbar_wait(smem_u32(b_empty + st), ph ^ 1, abort_flag)) { ok = false; break; }
-                    const uint32_t bar = smem_u32(b_full + st), dst = smem_u32(sB + st * 2 * CH);
+            // chunks: a cursor walks the lists that have been sent, as far ahead as there are free stages
+            int c_it = -1, c_left = 0, c_st = 0, copied = 0;
+            const unsigned* c_at = nullptr;
+            auto fill = [&](int limit) {
+                while (copied < limit) {
+                    while (c_left == 0) {
+                        if (c_it + 1 >= lists) return;
+                        ++c_it;
+                        const int buf = c_it % PS_LISTS;
+                        if (!mbar_wait(smem_u32(l_full + buf), (c_it / PS_LISTS) & 1, abort_flag)) { ok = false; return; }
+                        c_left = (sN[buf] + 1) / 2;
+                        c_at = reinterpret_cast<const unsigned*>(sL + buf * PR_MAX_CHUNKS);
+                    }
+                    const unsigned two = *c_at++;
+                    --c_left;
+                    const uint32_t bar = bf + c_st * 8, dst = sb + c_st * 2 * CH;
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(2 * CH) : "memory");
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                                  ::"r"(dst), "l"(a.gB + (two & PR_CHUNK_MASK) * CH), "r"(CH), "r"(bar) : "memory");
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                                  ::"r"(dst + CH), "l"(a.gB + ((two >> 16) & PR_CHUNK_MASK) * CH), "r"(CH), "r"(bar) : "memory");
-                    ++total;
-                    if (++st == STAGES) { st = 0; ph ^= 1; }
+                    ++copied;
+                    if (++c_st == STAGES) c_st = 0;
                 }
-                if (ok && lists < n_iter) ok = send_list();  // the list after the next
-            }
-            if (*abort_flag) {   // let the copies in flight land before the CTA exits (bounded)
-                for (int c = total > STAGES ? total - STAGES : 0; c < total; ++c) {
-                    const long long t0 = clock64();
-                    while (!mbar_try(smem_u32(b_full + c % STAGES), (c / STAGES) & 1) && clock64() - t0 < WAIT_LIMIT) {}
-                }
-                for (int c = lists > PS_LISTS ? lists - PS_LISTS : 0; c < lists; ++c) {
-                    const long long t0 = clock64();
-                    while (!mbar_try(smem_u32(l_full + c % PS_LISTS), (c / PS_LISTS) & 1) && clock64() - t0 < WAIT_LIMIT) {}
-                }
-            }
-        }
-    } else if (warp == 5) {
-        // ------------------------------------------------------------ MMA: one thread issues
-        if (elect_one()) {
-            const uint32_t idesc = (1u << 4) | ((uint32_t)(2 * PR_CHUNK >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
-            const uint64_t descA0 = make_desc(smem_u32(sA), TM * 16, 128);
-            const uint64_t descB0 = make_desc(smem_u32(sB), 128, KD * 16);
-            bool ok = true;
-            int st = 0;
-            uint32_t ph = 0, seq = 0u;                       // seq: pairs so far
+            };
+            send_list();
+            if (n_iter > 1) send_list();
+            int st = 0, done = 0;                            // done: pairs multiplied so far
+            uint32_t ph = 0, par = 0u, ring = 0u;            // phase of the stage, of the accumulator; place on the ring
             for (int it = 0; it < n_iter && ok; ++it) {
                 const int buf = it % PS_LISTS, ab = it & 1;
                 ok = mbar_wait(smem_u32(l_full + buf), (it / PS_LISTS) & 1, abort_flag) &&
                      mbar_wait(smem_u32(a_full + ab), (it >> 1) & 1, abort_flag);
                 if (!ok) break;
                 const int n = sN[buf];
-                const uint16_t* L = sL + buf * PR_MAX_CHUNKS;
+                const unsigned* L = reinterpret_cast<const unsigned*>(sL + buf * PR_MAX_CHUNKS);
                 const uint64_t descA = descA0 + (uint64_t)((ab * A_TILE) >> 4);
-                for (int e = 0; e < n && ok; e += 2, ++seq) {
-                    const unsigned two = *reinterpret_cast<const unsigned*>(L + e);
-                    const unsigned m = ((two >> PR_MASK_SHIFT) | (two >> (16 + PR_MASK_SHIFT))) & 15u;
-                    const unsigned left_out = (two & PR_LOOK) ? 0u : 4u - (unsigned)__popc(m);
-                    ok = mbar_wait(smem_u32(b_full + st), ph, abort_flag) && mbar_wait(smem_u32(t_empty), (seq & 1u) ^ 1u, abort_flag);
-                    if (!ok) break;
+                if (copied < done + STAGES) fill(done + STAGES - (done ? 1 : 0));
+                for (int e = 0; e < n; e += 2, ++L) {
+                    const unsigned two = *L;
+                    uint32_t good = 1u;
+                    mbar_wait_acc(bf + st * 8, ph, abort_flag, good);
+                    mbar_wait_acc(te, par ^ 1u, abort_flag, good);       // the accumulator is free, so the previous MMAs are through
+                    if (!good || !ok) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    if (left_out) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(t_empty)), "r"(left_out) : "memory");
+                    const unsigned left_out = __popc(~(two | (two >> 16)) & (15u << PR_MASK_SHIFT));
+                    if (left_out && !(two & PR_LOOK)) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(te), "r"(left_out) : "memory");
                     const uint64_t descB = descB0 + (uint64_t)((st * 2 * CH) >> 4);
 #pragma unroll
                     for (int s = 0; s < KD / 16; ++s) {
                         const uint64_t da = descA + (uint64_t)((s * 2 * (TM * 16)) >> 4);
                         const uint64_t db = descB + (uint64_t)((s * 2 * 128) >> 4);
-                        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                                     ::"r"(tmem), "l"(da), "l"(db), "r"(idesc), "r"(s > 0 ? 1u : 0u) : "memory");
+                        if (s == 0)
+                            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, 0, 0;\n\t"
+                                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                                         ::"r"(tmem), "l"(da), "l"(db), "r"(idesc) : "memory");
+                        else
+                            asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.b32 p, 0, 0;\n\t"
+                                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                                         ::"r"(tmem), "l"(da), "l"(db), "r"(idesc) : "memory");
                     }
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                                 ::"r"(smem_u32(t_full + (seq % PS_RING))) : "memory");
-                    // the pair may be overwritten once these MMAs have read it
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                                 ::"r"(smem_u32(b_empty + st)) : "memory");
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tf + ring * 8) : "memory");
+                    par ^= 1u;
+                    ring = (ring + 1) & (PS_RING - 1);
                     if (++st == STAGES) { st = 0; ph ^= 1; }
+                    fill(done + STAGES);                     // pairs 0 .. done - 1 are through
+                    ++done;
+                    if (lists == it + 2 && lists < n_iter && (e >= 4 || e + 2 >= n)) send_list();   // the list after the next
                 }
-                if (ok) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(l_empty + buf)) : "memory");
+                if (ok && lists == it + 2 && lists < n_iter) send_list();
+            }
+            if (*abort_flag) {   // let the copies in flight land before the CTA exits (bounded)
+                for (int c = copied > STAGES ? copied - STAGES : 0; c < copied; ++c) {
+                    const long long t0 = clock64();
+                    while (!mbar_try(bf + (c % STAGES) * 8, (c / STAGES) & 1) && clock64() - t0 < WAIT_LIMIT) {}
+                }
+                for (int c = lists > PS_LISTS ? lists - PS_LISTS : 0; c < lists; ++c) {
+                    const long long t0 = clock64();
+                    while (!mbar_try(smem_u32(l_full + c % PS_LISTS), (c / PS_LISTS) & 1) && clock64() - t0 < WAIT_LIMIT) {}
+                }
             }
         }
     } else {
@@ -701,7 +710,9 @@ assign_pruned_kernel(const ScanArgs a) {
                     float s;
                     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(fmaxf(fmaf(mn, invS_dn, base_now), 0.f)));
                     s = redux_min(s - ub);
-                    if (lane == 0) gap_row[chunk] = __fadd_rd(__fadd_rd(s, mv), rise);
+                    s = __fadd_rd(__fadd_rd(s, mv), rise);
+                    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %2, 0;\n\t@p st.global.f32 [%0], %1;\n\t}"
+                                 ::"l"(gap_row + chunk), "f"(s), "r"(lane) : "memory");
                 }
             };
             // A wait that gives up is only acted upon after the tile: once the abort flag is up the remaining waits
