@@ -67,8 +67,22 @@ __device__ __forceinline__ void mbar_wait_acc(uint32_t bar, uint32_t parity, vol
         "MBW_LOOP:\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "@p bra.uni MBW_DONE;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra.uni MBW_DONE;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra.uni MBW_DONE;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra.uni MBW_DONE;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra.uni MBW_DONE;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra.uni MBW_DONE;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra.uni MBW_DONE;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra.uni MBW_DONE;\n\t"
         "add.u32 n, n, 1;\n\t"
-        "and.b32 f, n, 15;\n\t"                    // a failed try has already slept in hardware: look up every 16
+        "and.b32 f, n, 1;\n\t"                     // look up every 16 tries
         "setp.ne.u32 q, f, 0;\n\t"
         "@q bra.uni MBW_LOOP;\n\t"
         "ld.volatile.shared.u32 f, [%3];\n\t"
