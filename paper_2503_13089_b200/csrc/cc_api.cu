@@ -45,7 +45,7 @@ WsLayout cc_ws_layout(int64_t N, int g, int K) {
     L.first = take_if(Kp * 4);
     L.cs = take_if((size_t)K * g * 4);
     L.c_prev = take_if((size_t)K * g * 4);
-    L.boxes = take_if(4 * n_chunks * g * 4);
+    L.boxes = take_if(n_chunks * (4 * g + 3) * 4);
     L.moved = take_if(n_chunks * 4);
     L.total = off;
     return L;

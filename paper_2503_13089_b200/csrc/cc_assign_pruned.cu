@@ -7,7 +7,9 @@
 //     centroid it had in the previous iteration, or (first E-step) the best of the chunks around the tree leaf
 //     it falls into.  A list kernel finds for each row block the chunks that may hold a centroid within ub of one
 //     of its points, by two lower bounds:
-//       - the distance to the chunk's bounding box, of the row block's own box or of each of its points,
+//       - the distance to the chunk's bounding box, of the row block's own box and, where no gaps are kept, of each
+//         of its points (where they are, a chunk that only the points could rule out is scored once instead: its gap
+//         is then the true one, and a box's gap would be used up by the next iteration's moves),
 //       - inside a fit, the gap kept from the last look at the chunk: min over the block's points of (distance to
 //         the chunk, or to its box, - ub).  Since then that difference has shrunk by at most the sum of the
 //         chunk's largest centroid moves plus the sum of the block's largest increases of ub.  Both sums are
@@ -90,8 +92,11 @@ pruned_prep_kernel(const float* __restrict__ C, int K, int n_pos, const unsigned
     *reinterpret_cast<uint4*>(dst) = w;
 }
 
-// One warp per chunk: bounding box (by coordinate for one lane per chunk: box_t[t][chunk], lower then upper;
-// and by chunk for one chunk per warp: box_c[chunk][2 G]) and, with C_prev, the largest move of a member since
+// Stride of box_c in floats: centre and half width of each coordinate, padded to whole 16-byte words.
+template <int G> struct BoxRow { static constexpr int STRIDE = (2 * G + 3) / 4 * 4; };
+
+// One warp per chunk: bounding box (by coordinate for one lane per chunk: box_t[t][chunk], lower then upper ends;
+// and by chunk for one chunk per warp: box_c, centres and half widths, these a little too wide) and, with C_prev, the largest move of a member since
 // the last E-step, added to the chunk's total.  C_prev is brought up to date.
 template <int G>
 __global__ void __launch_bounds__(256)
@@ -131,8 +136,10 @@ chunk_bounds_kernel(const float* __restrict__ C, int K, const unsigned* __restri
         if (lane == 0) {
             box_t[t * n_chunks + c] = a;
             box_t[(G + t) * n_chunks + c] = b;
-            box_c[(int64_t)c * 2 * G + t] = a;
-            box_c[(int64_t)c * 2 * G + G + t] = b;
+            // |x - centre| rounds by 2^-24 of itself, which near the box is its half width: widened by 2^-22 of that
+            const float m = odd ? 0.f : 0.5f * a + 0.5f * b;
+            box_c[c * BoxRow<G>::STRIDE + t] = m;
+            box_c[c * BoxRow<G>::STRIDE + G + t] = __fmul_ru(fmaxf(__fsub_ru(b, m), __fsub_ru(m, a)), 1.0f + 2.3841858e-7f);
         }
     }
     if (lane == 0) {
@@ -160,7 +167,6 @@ struct ListArgs {
     const TcParams* params;
     float* ub; float* rise;              // N; per row block, the sum of the largest increases of ub
     float* gap;                          // row blocks x ld: what the last look at the chunk left
-    int point_test;
     uint16_t* list; unsigned* list_n; unsigned* status;
 };
 
@@ -305,9 +311,14 @@ pruned_list_kernel(const ListArgs a) {
     // row block against chunk
     const float ubmax2 = ubmax * ubmax * 1.000001f;
     float* gap = GAP ? a.gap + row * a.ld : nullptr;
-    for (int j = 0; j < n_words; ++j) {
+    unsigned words = ubmax >= 0.f ? 0xffffffffu >> (32 - n_words) : 0u;
+    if constexpr (!GAP) words &= __ballot_sync(0xffffffffu, lane < n_words && in_group[lane] != 0u);
+    unsigned mine_w = 0u;                                        // lane j: chunks 32 j .. of this row block
+    while (words) {
+        const int j = __ffs(words) - 1;
+        words &= words - 1;
         const int c = j * 32 + lane;
-        bool nd = c < a.n_chunks && ubmax >= 0.f;
+        bool nd = c < a.n_chunks;
         if constexpr (!GAP) nd = nd && ((in_group[j] >> lane) & 1u);
         float mv = 0.f;
         if constexpr (MODE == PL_NEXT) {
@@ -319,41 +330,39 @@ pruned_list_kernel(const ListArgs a) {
             }
         }
         unsigned todo = __ballot_sync(0xffffffffu, nd);
-        if (todo) {
-            if (nd) {
-                const float lb = box_distance2(c, lo, hi);
-                nd = !(lb > ubmax2);
-                // what the box says is kept like a scored distance, with the totals of both sides at this time
-                // added so that later ones can be taken off
-                if (GAP && !nd) gap[c] = __fadd_rd(__fadd_rd(__fsub_rd(__fsqrt_rd(lb), ubmax), mv), rise);
-            }
-            todo = __ballot_sync(0xffffffffu, nd);
-            if (a.point_test) {                              // box against each of the 32 points
-                unsigned left = todo;
-                while (left) {
-                    const int b = __ffs(left) - 1;
-                    left &= left - 1;
-                    const float* box = a.box_c + (int64_t)(j * 32 + b) * 2 * G;
-                    float lb = 0.f;
+        if (!todo) continue;
+        if (nd) {
+            const float lb = box_distance2(c, lo, hi);
+            nd = !(lb > ubmax2);
+            // what the box says is kept like a scored distance, with the totals of both sides at this time
+            // added so that later ones can be taken off
+            if (GAP && !nd) gap[c] = __fadd_rd(__fadd_rd(__fsub_rd(__fsqrt_rd(lb), ubmax), mv), rise);
+        }
+        todo = __ballot_sync(0xffffffffu, nd);
+        if constexpr (!GAP) {                                    // box against each of the 32 points
+            unsigned left = todo;
+            while (left) {
+                const int b = __ffs(left) - 1;
+                left &= left - 1;
+                const float4* box = reinterpret_cast<const float4*>(a.box_c + (j * 32 + b) * BoxRow<G>::STRIDE);
+                float v[BoxRow<G>::STRIDE];
 #pragma unroll
-                    for (int t = 0; t < G; ++t) {
-                        const float q = fmaxf(fmaxf(__ldg(box + t) - x[t], x[t] - __ldg(box + G + t)), 0.f);
-                        lb = fmaf(q, q, lb);
-                    }
-                    lb *= shrink;
-                    if (!__any_sync(0xffffffffu, !(lb > ue2))) {
-                        todo &= ~(1u << b);
-                        if constexpr (GAP) {
-                            const float s = redux_min(live ? __fsub_rd(__fsqrt_rd(lb), ue) : INFINITY);
-                            const float m = __shfl_sync(0xffffffffu, mv, b);
-                            if (lane == 0) gap[j * 32 + b] = __fadd_rd(__fadd_rd(s, m), rise);
-                        }
-                    }
+                for (int k = 0; k < BoxRow<G>::STRIDE / 4; ++k) {
+                    const float4 f = __ldg(box + k);
+                    v[4 * k] = f.x; v[4 * k + 1] = f.y; v[4 * k + 2] = f.z; v[4 * k + 3] = f.w;
                 }
+                float lb = 0.f;
+#pragma unroll
+                for (int t = 0; t < G; ++t) {
+                    const float q = fmaxf(fabsf(x[t] - v[t]) - v[G + t], 0.f);
+                    lb = fmaf(q, q, lb);
+                }
+                if (!__any_sync(0xffffffffu, !(lb * shrink > ue2))) todo &= ~(1u << b);
             }
         }
-        if (lane == 0) need[w][j] = todo;
+        if (lane == j) mine_w = todo;
     }
+    need[w][lane] = mine_w;
     __syncthreads();
     // one list per tile, chunks in ascending order: a tile's four warps share its words
     const int tile = w >> 2, part = w & 3;
@@ -366,7 +375,11 @@ pruned_list_kernel(const ListArgs a) {
     const int total = __shfl_sync(0xffffffffu, inc, 31);
     const int64_t out_tile = (int64_t)blockIdx.x * PR_TILES + tile;
     uint16_t* out = a.list + out_tile * a.ld;
-    for (int j = part; j < n_words; j += 4) {
+    unsigned full = __ballot_sync(0xffffffffu, any != 0u);
+    for (int turn = 0; full; ++turn) {
+        const int j = __ffs(full) - 1;
+        full &= full - 1;
+        if ((turn & 3) != part) continue;
         const unsigned word = __shfl_sync(0xffffffffu, any, j);
         const int at = __shfl_sync(0xffffffffu, inc - mine, j) + __popc(word & ((1u << lane) - 1u));
         unsigned m = 0u;
@@ -383,29 +396,33 @@ pruned_list_kernel(const ListArgs a) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Scan.  A thread block is one pipeline for one tile at a time (tiles blockIdx.x, + gridDim.x, ..); four blocks
-// share an SM and its tensor memory, so that the waits of one are covered by the others.
-//   warps 0..3  epilogue: warp w owns row block w = TMEM lanes 32 w.., and writes that block's rows of the A
-//               operand, one tile ahead (loads two tiles ahead)
-//   warp 4      copies lists and chunks and issues the MMAs (one thread): 128 points x two chunks of the list at
-//               a time
-// A pair of chunks whose masks leave a row block out costs that warp nothing: the MMA thread releases the
-// accumulator in its stead.  Pairs are announced on a ring of eight barriers, and every warp looks at (waits for
-// and releases) at least every fourth pair, which keeps it within one phase of every barrier, and a tile's last
-// pair, after which the tile's A rows are free.
+// Scan.  A thread block is one pipeline for one tile at a time (tiles blockIdx.x, + gridDim.x, ..); two blocks share
+// an SM and its tensor memory, so that the waits of one are covered by the other.
+//   warps 0..7  epilogue: warp w owns row block w % 4 = TMEM lanes 32 (w % 4).. and takes the first (w < 4) or the
+//               second chunk of each pair of list entries; warps 0..3 also write their rows of the A operand, one
+//               tile ahead (loads two tiles ahead)
+//   warp 8      copies lists and chunks (one thread)
+//   warp 9      issues the MMAs (one thread): 128 points x two chunks into one of two accumulators
+// A pair costs nothing to a warp that needs neither of it: the MMA thread releases the accumulator in its stead.
+// Pairs are announced on a ring of eight barriers, and every warp looks at (waits for and releases) at least every
+// fourth pair, which keeps it within one phase of every barrier, and a tile's last pair, after which the tile's
+// A rows are free.
 // Measured on the way here: a successful wait on an mbarrier costs an issuing thread about 110 cycles right behind
-// an MMA, a further one 45, the MMA and its commit together 48 (N = 64).  Per 128 x 64 block and SM: one issuer
-// for four tiles 335 cycles, one issuer per tile 222, one block per tile with a handshake per chunk 217.
-constexpr int PS_THREADS = 5 * 32;
-constexpr int PS_BLOCKS = 4;             // resident per SM
+// an MMA, a further one 45, the MMA and its commit together 48 (N = 64); a waiting warp is back at work about 90
+// cycles after the arrival.  What counts is therefore the chain of a pair: announcement, load of the accumulator, its
+// release, next MMA.  Per 128 x 64 block and SM: one issuer for four tiles 335 cycles, one issuer per tile 222; a
+// pipeline per tile with a handshake per chunk 217, per pair 167 with one accumulator and both chunks by the same warp.
+constexpr int PS_EPI = 8;
+constexpr int PS_THREADS = (PS_EPI + 2) * 32;
+constexpr int PS_BLOCKS = 2;             // resident per SM
 constexpr int PS_LISTS = 3;
 constexpr int PS_RING = 8;
 
 template <int G> struct PrCfg {
     using Cfg = TcCfg<G>;
     static constexpr int CH_BYTES = PR_CHUNK * Cfg::KD * 2;
-    static constexpr int STAGES = Cfg::KD == 16 ? 6 : Cfg::KD == 32 ? 3 : 2;   // pairs of chunks: 24 KB
-    static constexpr int SMEM = 2 * Cfg::A_TILE + STAGES * 2 * CH_BYTES + PS_LISTS * PR_MAX_CHUNKS * 2 + 512;
+    static constexpr int STAGES = Cfg::KD == 16 ? 10 : Cfg::KD == 32 ? 6 : 4;   // pairs of chunks
+    static constexpr int SMEM = 2 * Cfg::A_TILE + STAGES * 2 * CH_BYTES + PS_LISTS * PR_MAX_CHUNKS * 2 + 2 * 3 * TM * 4 + 512;
 };
 
 struct ScanArgs {
@@ -490,9 +507,10 @@ assign_pruned_kernel(const ScanArgs a) {
     unsigned char* sA = smem_raw;                                        // 2 tiles
     unsigned char* sB = sA + 2 * A_TILE;                                 // STAGES pairs of chunks
     uint16_t* sL = reinterpret_cast<uint16_t*>(sB + STAGES * 2 * CH);    // PS_LISTS lists
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sL + PS_LISTS * PR_MAX_CHUNKS);
-    uint64_t* b_full = bars, *t_full = bars + STAGES, *t_empty = t_full + PS_RING;
-    uint64_t* a_full = t_empty + 1, *l_full = a_full + 2, *l_empty = l_full + PS_LISTS;
+    float* merge = reinterpret_cast<float*>(sL + PS_LISTS * PR_MAX_CHUNKS);   // [2][best, second, chunk][TM]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(merge + 2 * 3 * TM);
+    uint64_t* b_full = bars, *b_empty = bars + STAGES, *t_full = bars + 2 * STAGES, *t_empty = t_full + PS_RING;
+    uint64_t* a_full = t_empty + 2, *l_full = a_full + 2, *l_empty = l_full + PS_LISTS;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(l_empty + PS_LISTS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* sN = reinterpret_cast<volatile int*>(tmem_slot + 2);   // PS_LISTS list lengths
@@ -502,16 +520,15 @@ assign_pruned_kernel(const ScanArgs a) {
 
     if (tid == 0) {
         auto init = [&](uint64_t* b, int n) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(n)); };
-        for (int s = 0; s < STAGES; ++s) init(b_full + s, 1);
+        for (int s = 0; s < STAGES; ++s) { init(b_full + s, 1); init(b_empty + s, 1); }
         for (int s = 0; s < PS_RING; ++s) init(t_full + s, 1);
-        init(t_empty, 4);
-        for (int s = 0; s < 2; ++s) init(a_full + s, TM);
-        for (int s = 0; s < PS_LISTS; ++s) { init(l_full + s, 1); init(l_empty + s, 4); }
+        for (int s = 0; s < 2; ++s) { init(t_empty + s, PS_EPI); init(a_full + s, TM); }
+        for (int s = 0; s < PS_LISTS; ++s) { init(l_full + s, 1); init(l_empty + s, PS_EPI + 1); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(2 * PR_CHUNK));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(4 * PR_CHUNK));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -519,21 +536,18 @@ assign_pruned_kernel(const ScanArgs a) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
 
-    if (warp == 4) {
-        // ------------------------------------------------------------ copies and MMAs: one thread
+    if (warp == PS_EPI) {
+        // ------------------------------------------------------------ copies: lists (two tiles ahead), chunks
         if (elect_one()) {
-            const uint32_t idesc = (1u << 4) | ((uint32_t)(2 * PR_CHUNK >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
-            const uint64_t descA0 = make_desc(smem_u32(sA), TM * 16, 128);
-            const uint64_t descB0 = make_desc(smem_u32(sB), 128, KD * 16);
-            const uint32_t te = smem_u32(t_empty), tf = smem_u32(t_full), bf = smem_u32(b_full), sb = smem_u32(sB);
-            bool ok = true;
-            // lists: sent two tiles ahead
-            int lists = 0;
+            const uint32_t bf = smem_u32(b_full), sb = smem_u32(sB);
+            int st = 0, total = 0, lists = 0;
+            uint32_t ph = 0, good = 1u;
             auto length = [&](int it) { return it < n_iter ? (int)__ldg(a.list_n + blockIdx.x + (int64_t)it * gridDim.x) : 0; };
             int n_next = length(0), n_after = length(1);
-            auto send_list = [&]() {
+            auto send_list = [&]() {                         // the next list into its ring place
                 const int buf = lists % PS_LISTS;
-                if (lists >= PS_LISTS && !mbar_wait(smem_u32(l_empty + buf), ((lists / PS_LISTS) & 1) ^ 1, abort_flag)) { ok = false; return; }
+                if (lists >= PS_LISTS) mbar_wait_acc(smem_u32(l_empty + buf), ((lists / PS_LISTS) & 1) ^ 1, abort_flag, good);
+                if (!good) return;
                 sN[buf] = n_next;
                 const uint32_t bytes = (uint32_t)((n_next + 1) / 2 * 4 + 15) & ~15u, bar = smem_u32(l_full + buf);
                 if (n_next) {
@@ -548,79 +562,33 @@ assign_pruned_kernel(const ScanArgs a) {
                 n_next = n_after;
                 n_after = length(lists + 1);
             };
-            // chunks: a cursor walks the lists that have been sent, as far ahead as there are free stages
-            int c_it = -1, c_left = 0, c_st = 0, copied = 0;
-            const unsigned* c_at = nullptr;
-            auto fill = [&](int limit) {
-                while (copied < limit) {
-                    while (c_left == 0) {
-                        if (c_it + 1 >= lists) return;
-                        ++c_it;
-                        const int buf = c_it % PS_LISTS;
-                        if (!mbar_wait(smem_u32(l_full + buf), (c_it / PS_LISTS) & 1, abort_flag)) { ok = false; return; }
-                        c_left = (sN[buf] + 1) / 2;
-                        c_at = reinterpret_cast<const unsigned*>(sL + buf * PR_MAX_CHUNKS);
-                    }
-                    const unsigned two = *c_at++;
-                    --c_left;
-                    const uint32_t bar = bf + c_st * 8, dst = sb + c_st * 2 * CH;
+            send_list();
+            if (n_iter > 1) send_list();
+            for (int it = 0; it < n_iter && good; ++it) {
+                const int buf = it % PS_LISTS;
+                mbar_wait_acc(smem_u32(l_full + buf), (it / PS_LISTS) & 1, abort_flag, good);
+                if (!good) break;
+                const int n = sN[buf];
+                const unsigned* L = reinterpret_cast<const unsigned*>(sL + buf * PR_MAX_CHUNKS);
+                unsigned next = n > 0 ? *L : 0u;
+                for (int e = 0; e < n; e += 2) {
+                    const unsigned two = next;
+                    next = *++L;                             // at most one word past the list, inside the ring place or what follows
+                    const uint32_t bar = bf + st * 8, dst = sb + st * 2 * CH;
+                    mbar_wait_acc(bar + STAGES * 8, ph ^ 1, abort_flag, good);           // b_empty
+                    if (!good) break;
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(2 * CH) : "memory");
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                                  ::"r"(dst), "l"(a.gB + (two & PR_CHUNK_MASK) * CH), "r"(CH), "r"(bar) : "memory");
                     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                                  ::"r"(dst + CH), "l"(a.gB + ((two >> 16) & PR_CHUNK_MASK) * CH), "r"(CH), "r"(bar) : "memory");
-                    ++copied;
-                    if (++c_st == STAGES) c_st = 0;
-                }
-            };
-            send_list();
-            if (n_iter > 1) send_list();
-            int st = 0, done = 0;                            // done: pairs multiplied so far
-            uint32_t ph = 0, par = 0u, ring = 0u;            // phase of the stage, of the accumulator; place on the ring
-            for (int it = 0; it < n_iter && ok; ++it) {
-                const int buf = it % PS_LISTS, ab = it & 1;
-                ok = mbar_wait(smem_u32(l_full + buf), (it / PS_LISTS) & 1, abort_flag) &&
-                     mbar_wait(smem_u32(a_full + ab), (it >> 1) & 1, abort_flag);
-                if (!ok) break;
-                const int n = sN[buf];
-                const unsigned* L = reinterpret_cast<const unsigned*>(sL + buf * PR_MAX_CHUNKS);
-                const uint64_t descA = descA0 + (uint64_t)((ab * A_TILE) >> 4);
-                if (copied < done + STAGES) fill(done + STAGES - (done ? 1 : 0));
-                for (int e = 0; e < n; e += 2, ++L) {
-                    const unsigned two = *L;
-                    uint32_t good = 1u;
-                    mbar_wait_acc(bf + st * 8, ph, abort_flag, good);
-                    mbar_wait_acc(te, par ^ 1u, abort_flag, good);       // the accumulator is free, so the previous MMAs are through
-                    if (!good || !ok) { ok = false; break; }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const unsigned left_out = __popc(~(two | (two >> 16)) & (15u << PR_MASK_SHIFT));
-                    if (left_out && !(two & PR_LOOK)) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(te), "r"(left_out) : "memory");
-                    const uint64_t descB = descB0 + (uint64_t)((st * 2 * CH) >> 4);
-#pragma unroll
-                    for (int s = 0; s < KD / 16; ++s) {
-                        const uint64_t da = descA + (uint64_t)((s * 2 * (TM * 16)) >> 4);
-                        const uint64_t db = descB + (uint64_t)((s * 2 * 128) >> 4);
-                        if (s == 0)
-                            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, 0, 0;\n\t"
-                                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                                         ::"r"(tmem), "l"(da), "l"(db), "r"(idesc) : "memory");
-                        else
-                            asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.b32 p, 0, 0;\n\t"
-                                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                                         ::"r"(tmem), "l"(da), "l"(db), "r"(idesc) : "memory");
-                    }
-                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tf + ring * 8) : "memory");
-                    par ^= 1u;
-                    ring = (ring + 1) & (PS_RING - 1);
+                    ++total;
                     if (++st == STAGES) { st = 0; ph ^= 1; }
-                    fill(done + STAGES);                     // pairs 0 .. done - 1 are through
-                    ++done;
-                    if (lists == it + 2 && lists < n_iter && (e >= 4 || e + 2 >= n)) send_list();   // the list after the next
                 }
-                if (ok && lists == it + 2 && lists < n_iter) send_list();
+                if (good && lists < n_iter) send_list();     // the list after the next
             }
             if (*abort_flag) {   // let the copies in flight land before the CTA exits (bounded)
-                for (int c = copied > STAGES ? copied - STAGES : 0; c < copied; ++c) {
+                for (int c = total > STAGES ? total - STAGES : 0; c < total; ++c) {
                     const long long t0 = clock64();
                     while (!mbar_try(bf + (c % STAGES) * 8, (c / STAGES) & 1) && clock64() - t0 < WAIT_LIMIT) {}
                 }
@@ -630,10 +598,59 @@ assign_pruned_kernel(const ScanArgs a) {
                 }
             }
         }
+    } else if (warp == PS_EPI + 1) {
+        // ------------------------------------------------------------ MMA: one thread issues
+        if (elect_one()) {
+            const uint32_t idesc = (1u << 4) | ((uint32_t)(2 * PR_CHUNK >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+            const uint64_t descA0 = make_desc(smem_u32(sA), TM * 16, 128);
+            const uint64_t descB0 = make_desc(smem_u32(sB), 128, KD * 16);
+            const uint32_t te0 = smem_u32(t_empty), tf = smem_u32(t_full), bf = smem_u32(b_full);
+            int st = 0;
+            uint32_t ph = 0, ring = 0u, seq = 0u, good = 1u; // phase of the stage; place on the ring; pairs so far
+            for (int it = 0; it < n_iter && good; ++it) {
+                const int buf = it % PS_LISTS, ab = it & 1;
+                mbar_wait2_acc(smem_u32(l_full + buf), (it / PS_LISTS) & 1, smem_u32(a_full + ab), (it >> 1) & 1, abort_flag, good);
+                if (!good) break;
+                const int n = sN[buf];
+                const unsigned* L = reinterpret_cast<const unsigned*>(sL + buf * PR_MAX_CHUNKS);
+                const uint64_t descA = descA0 + (uint64_t)((ab * A_TILE) >> 4);
+                unsigned next = n > 0 ? *L : 0u;
+                for (int e = 0; e < n; e += 2, ++seq) {
+                    const unsigned two = next;
+                    next = *++L;
+                    const uint32_t slot = seq & 1u, te = te0 + slot * 8, bar = bf + st * 8;
+                    mbar_wait2_acc(bar, ph, te, ((seq >> 1) & 1u) ^ 1u, abort_flag, good);
+                    if (!good) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const unsigned left_out = __popc(~two & (0xf000fu << PR_MASK_SHIFT));
+                    if (left_out && !(two & PR_LOOK)) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(te), "r"(left_out) : "memory");
+                    const uint64_t descB = descB0 + (uint64_t)((st * 2 * CH) >> 4);
+#pragma unroll
+                    for (int s = 0; s < KD / 16; ++s) {
+                        const uint64_t da = descA + (uint64_t)((s * 2 * (TM * 16)) >> 4);
+                        const uint64_t db = descB + (uint64_t)((s * 2 * 128) >> 4);
+                        if (s == 0)
+                            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, 0, 0;\n\t"
+                                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                                         ::"r"(tmem + slot * (2 * PR_CHUNK)), "l"(da), "l"(db), "r"(idesc) : "memory");
+                        else
+                            asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.b32 p, 0, 0;\n\t"
+                                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                                         ::"r"(tmem + slot * (2 * PR_CHUNK)), "l"(da), "l"(db), "r"(idesc) : "memory");
+                    }
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tf + ring * 8) : "memory");
+                    // the pair may be overwritten once these MMAs have read it
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar + STAGES * 8) : "memory");
+                    ring = (ring + 1) & (PS_RING - 1);
+                    if (++st == STAGES) { st = 0; ph ^= 1; }
+                }
+                if (good) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(l_empty + buf)) : "memory");
+            }
+        }
     } else {
         // ------------------------------------------------------------ epilogue, and the A rows of the next tile
-        const int r = warp * 32 + lane;
-        const uint32_t tbase = __shfl_sync(0xffffffffu, tmem + ((uint32_t)(warp * 32) << 16), 0);
+        const int rb = warp & 3, half = warp >> 2, r = rb * 32 + lane;
+        const uint32_t tbase = __shfl_sync(0xffffffffu, tmem + ((uint32_t)(rb * 32) << 16) + half * PR_CHUNK, 0);
         const TcParams prm = *a.params;
         int ne = 0;
         if constexpr (Cfg::NQ == 2) ne = norm_exponent(prm.S, prm.qmax_bits);
@@ -655,30 +672,34 @@ assign_pruned_kernel(const ScanArgs a) {
         float base_now = 0.f, base_next = 0.f;
         load_words<G>(a.Xs, point_or_none(0), a.N, xw);
         if constexpr (GAP) base_next = base_of(xw);
-        write_a_row<G>(xw, ne, sA, r);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(a_full)) : "memory");
+        if (half == 0) {
+            write_a_row<G>(xw, ne, sA, r);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(a_full)) : "memory");
+        }
         load_words<G>(a.Xs, point_or_none(1), a.N, xw);
-        const uint32_t tf = smem_u32(t_full), te = smem_u32(t_empty);
-        const unsigned interest = (0x10001u << (PR_MASK_SHIFT + warp)) | PR_LOOK;
+        const uint32_t tf = smem_u32(t_full), te0 = smem_u32(t_empty);
+        const unsigned mine = 1u << (16 * half + PR_MASK_SHIFT + rb), interest = mine | PR_LOOK;
         uint32_t okw = 1u, seq = 0u;                         // seq: pairs so far
-        for (int it = 0; it < n_iter && okw; ++it) {
+        for (int it = 0; it < n_iter; ++it) {                // to the end also after giving up: the halves meet once a tile
             const int buf = it % PS_LISTS;
             base_now = base_next;
             if (it + 1 < n_iter) {
                 // the place was last read for tile it - 1, whose last entry this warp has seen
                 const int nb = (it + 1) & 1;
                 if constexpr (GAP) base_next = base_of(xw);
-                write_a_row<G>(xw, ne, sA + nb * A_TILE, r);
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(a_full + nb)) : "memory");
+                if (half == 0) {
+                    write_a_row<G>(xw, ne, sA + nb * A_TILE, r);
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(a_full + nb)) : "memory");
+                }
                 load_words<G>(a.Xs, point_or_none(it + 2), a.N, xw);
             }
             const int64_t i = point(it);
             float ub = 0.f, rise = 0.f;
             float* gap_row = nullptr;
             if constexpr (GAP) {
-                const int64_t row = ((int64_t)blockIdx.x + (int64_t)it * gridDim.x) * 4 + warp;
+                const int64_t row = ((int64_t)blockIdx.x + (int64_t)it * gridDim.x) * 4 + rb;
                 ub = i < a.N ? __ldg(a.ub + i) : -INFINITY;
                 rise = __ldg(a.rise + row);
                 gap_row = a.gap + row * a.ld;
@@ -688,17 +709,30 @@ assign_pruned_kernel(const ScanArgs a) {
             const uint16_t* L = sL + buf * PR_MAX_CHUNKS;
             float b1 = INFINITY, b2 = INFINITY;
             int bc = 0;
-            auto take = [&](unsigned chunk, uint32_t taddr, bool last) {
+            // A wait that gives up is only acted upon after the tile: once the abort flag is up the remaining waits
+            // return at their next look at it, and reading an accumulator that was never written or releasing it once
+            // more harms nothing.
+            const unsigned* pairs = reinterpret_cast<const unsigned*>(L);
+            unsigned two = n > 0 ? pairs[0] : 0u;
+            for (int e = 0; e < n; e += 2) {
+                const unsigned now = two;
+                two = pairs[(e >> 1) + 1];                   // at most one word past the list, inside the ring place or the next
+                const uint32_t bar = tf + (seq & (PS_RING - 1)) * 8, par = (seq / PS_RING) & 1u;
+                ++seq;
+                if (!(now & interest)) continue;
+                mbar_wait_acc(bar, par, abort_flag, okw);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t slot = (seq - 1) & 1u, te = te0 + slot * 8;
+                if (!(now & mine)) { mbar_arrive_warp(te); continue; }
+                const unsigned chunk = (now >> (16 * half)) & PR_CHUNK_MASK;
                 float mv = 0.f;
                 if constexpr (GAP) mv = __ldg(a.moved + chunk);
                 uint32_t v0[32], v1[32];
-                TMEM_LD32(v0, taddr);
-                TMEM_LD32(v1, taddr + 32);
+                TMEM_LD32(v0, tbase + slot * (2 * PR_CHUNK));
+                TMEM_LD32(v1, tbase + slot * (2 * PR_CHUNK) + 32);
                 TMEM_WAIT64(v0, v1);
-                if (last) {                                  // this warp's last look at the accumulator
-                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                    mbar_arrive_warp(te);
-                }
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                mbar_arrive_warp(te);
                 const float mn = chunk_min64(v0, v1);
                 const bool better = mn < b1;
                 b2 = better ? b1 : fminf(b2, mn);
@@ -714,34 +748,25 @@ assign_pruned_kernel(const ScanArgs a) {
                     asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %2, 0;\n\t@p st.global.f32 [%0], %1;\n\t}"
                                  ::"l"(gap_row + chunk), "f"(s), "r"(lane) : "memory");
                 }
-            };
-            // A wait that gives up is only acted upon after the tile: once the abort flag is up the remaining waits
-            // return at their next look at it, and reading an accumulator that was never written or releasing it once
-            // more harms nothing.
-            const unsigned* pairs = reinterpret_cast<const unsigned*>(L);
-            unsigned two = n > 0 ? pairs[0] : 0u;
-            for (int e = 0; e < n; e += 2) {
-                const unsigned now = two;
-                two = pairs[(e >> 1) + 1];                   // at most one word past the list, inside the ring place or the next
-                const uint32_t bar = tf + (seq & (PS_RING - 1)) * 8, par = (seq / PS_RING) & 1u;
-                ++seq;
-                if (!(now & interest)) continue;
-                mbar_wait_acc(bar, par, abort_flag, okw);
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const bool m0 = now & (1u << (PR_MASK_SHIFT + warp)), m1 = now & (1u << (16 + PR_MASK_SHIFT + warp));
-                if (m0) take(now & PR_CHUNK_MASK, tbase, !m1);
-                if (m1) take((now >> 16) & PR_CHUNK_MASK, tbase + PR_CHUNK, true);
-                if (!m0 && !m1) mbar_arrive_warp(te);
             }
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(l_empty + buf)) : "memory");
-            if (okw && i < a.N) a.tstate[i] = make_float2(b2, __int_as_float(bc));
+            // the two halves of a row block meet; the place of this tile is written again two tiles on
+            float* place = merge + (it & 1) * (3 * TM) + r;
+            if (half == 1) { place[0] = b1; place[TM] = b2; place[2 * TM] = __int_as_float(bc); }
+            asm volatile("bar.sync %0, 64;" ::"r"(1 + rb) : "memory");
+            if (half == 0 && okw && i < a.N) {
+                const float o1 = place[0], o2 = place[TM];
+                if (o1 < b1) { b2 = fminf(b1, o2); bc = __float_as_int(place[2 * TM]); }   // equal minima: the gap is 0 and
+                else b2 = fminf(b2, o1);                                                   // the point goes to the exact stage
+                a.tstate[i] = make_float2(b2, __int_as_float(bc));
+            }
         }
     }
     if (*abort_flag && lane == 0) atomicOr(a.status, CC_DEV_TIMEOUT);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * PR_CHUNK));
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(4 * PR_CHUNK));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -991,7 +1016,7 @@ cudaError_t run_pruned(cc_ctx* ctx, const PruneBuffers& b, const float* C, int m
     const int K = b.K, n_chunks = (K + PR_CHUNK - 1) / PR_CHUNK;
     const int64_t n_groups = (b.N + PR_GROUP - 1) / PR_GROUP;
     TcParams* params = reinterpret_cast<TcParams*>(reinterpret_cast<char*>(b.status) + 128);
-    const bool cold = mode == CC_PRUNE_COLD, restart = mode != CC_PRUNE_NEXT;
+    const bool cold = mode == CC_PRUNE_COLD, restart = cold || mode == CC_PRUNE_RESTART;
     cudaError_t e;
     static bool attr_dev[64] = {};
     bool& have = attr_dev[ctx->device & 63];
@@ -1021,7 +1046,6 @@ cudaError_t run_pruned(cc_ctx* ctx, const PruneBuffers& b, const float* C, int m
         a.first = b.first; a.home_chunks = G <= 4 ? 1 : 4; a.codes = b.idx_s;
         a.box_t = b.box_t; a.box_c = b.box_c; a.moved = b.moved; a.params = params;
         a.ub = b.ub; a.rise = b.rise; a.gap = b.gap;
-        a.point_test = mode != CC_PRUNE_NEXT && G <= 8;
         a.list = b.list; a.list_n = b.list_n; a.status = b.status;
         ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
         const unsigned blocks = (unsigned)n_groups;

@@ -91,7 +91,7 @@ struct WsLayout {
     size_t first;      // u32 Kp: leaf -> position of its first point; scratch of the tree
     size_t cs;         // float K x g: codebook by position
     size_t c_prev;     // float K x g: codebook of the last E-step
-    size_t boxes;      // float 2 x chunks x 2 g
+    size_t boxes;      // float chunks x (2 g + 2 g + 3)
     size_t moved;      // float chunks
     size_t total;
 };
