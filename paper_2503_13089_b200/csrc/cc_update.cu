@@ -37,14 +37,16 @@ __device__ __forceinline__ void add_coord(uint16_t h, ull* lo, ull* hi) {
 // sectors instead of 32.  With few clusters the same words are hit by many points at once and the
 // reductions queue up in L2; the sums are then kept in R copies (copy = block % R, one after the
 // other, `copy_elems` words apart; the counts likewise, K apart) which the finish kernel adds up.
-template <int G>
+// COUNT: the gradient with respect to the codebook needs no counts, and a point's count is a request of its own beside
+// the one or two of its sums.
+template <int G, bool COUNT>
 __global__ void __launch_bounds__(256)
 update_accumulate_kernel(const uint16_t* __restrict__ X, int64_t N, const uint16_t* __restrict__ idx, int K,
                          ull* __restrict__ sum_lo, ull* __restrict__ sum_hi, int* __restrict__ counts, int R) {
     const int copy = (int)(blockIdx.x % (unsigned)R);
     sum_lo += (int64_t)copy * K * G;
     sum_hi += (int64_t)copy * K * G;
-    counts += (int64_t)copy * K;
+    if constexpr (COUNT) counts += (int64_t)copy * K;
     const int64_t total = N * G;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     constexpr int EB = 4;                            // elements per thread and round: their loads are issued together
@@ -63,7 +65,7 @@ update_accumulate_kernel(const uint16_t* __restrict__ X, int64_t N, const uint16
             const int j = jj[p];
             if (j >= K) continue;
             const int t = (int)(e % G);
-            if (t == 0) atomicAdd(counts + j, 1);
+            if constexpr (COUNT) { if (t == 0) atomicAdd(counts + j, 1); }
             add_coord(hh[p], sum_lo + (int64_t)j * G + t, sum_hi + (int64_t)j * G + t);
         }
     }
@@ -239,7 +241,8 @@ cudaError_t launch_accumulate(int sm_count, const uint16_t* X, int64_t N, const 
     int64_t blocks = (N * G + 255) / 256;
     const int64_t cap = (int64_t)sm_count * 16;
     if (blocks > cap) blocks = cap;
-    update_accumulate_kernel<G><<<(unsigned)blocks, 256, 0, st>>>(X, N, idx, K, sum_lo, sum_hi, counts, R);
+    if (counts) update_accumulate_kernel<G, true><<<(unsigned)blocks, 256, 0, st>>>(X, N, idx, K, sum_lo, sum_hi, counts, R);
+    else update_accumulate_kernel<G, false><<<(unsigned)blocks, 256, 0, st>>>(X, N, idx, K, sum_lo, sum_hi, nullptr, R);
     return cudaGetLastError();
 }
 
@@ -269,7 +272,7 @@ cudaError_t launch_private(cc_ctx* ctx, const uint16_t* X, int64_t N, const uint
 // shared-memory kernel ran: it keeps a single copy).  *count_copies is where the (copies of the)
 // counts were accumulated: the caller's array when R = 1.
 cudaError_t accumulate_all(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, int g, const uint16_t* idx,
-                           int K, int32_t* counts, int& R, int32_t** count_copies, cudaStream_t st) {
+                           int K, int32_t* counts, int& R, int32_t** count_copies, bool want_counts, cudaStream_t st) {
     char* ws = static_cast<char*>(ctx->ws);
     ull* sum_lo = reinterpret_cast<ull*>(ws + L.sum_lo);
     ull* sum_hi = reinterpret_cast<ull*>(ws + L.sum_hi);
@@ -294,7 +297,8 @@ cudaError_t accumulate_all(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, in
     cudaError_t e;
     if ((e = cudaMemsetAsync(sum_lo, 0, used, st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(sum_hi, 0, used, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(cc, 0, sizeof(int32_t) * (size_t)K * R, st)) != cudaSuccess) return e;
+    if (!want_counts) cc = nullptr;
+    else if ((e = cudaMemsetAsync(cc, 0, sizeof(int32_t) * (size_t)K * R, st)) != cudaSuccess) return e;
     if (N > 0) {
         ProfScope ps(ctx, CC_K_UPDATE_ACCUM, st);
 #define CALL(G) e = launch_accumulate<G>(ctx->sm_count, X, N, idx, K, sum_lo, sum_hi, cc, R, st)
@@ -311,7 +315,7 @@ cudaError_t cc_launch_update(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, 
     char* ws = static_cast<char*>(ctx->ws);
     int R = cc_sum_copies(K, g);
     int32_t* count_copies = nullptr;
-    const cudaError_t e = accumulate_all(ctx, L, X, N, g, idx, K, counts, R, &count_copies, st);
+    const cudaError_t e = accumulate_all(ctx, L, X, N, g, idx, K, counts, R, &count_copies, true, st);
     if (e != cudaSuccess) return e;
     {
         ProfScope ps(ctx, CC_K_UPDATE_FINISH, st);
@@ -331,7 +335,7 @@ cudaError_t cc_launch_codebook_grad(cc_ctx* ctx, const WsLayout& L, const uint16
     int32_t* counts = reinterpret_cast<int32_t*>(ws + L.positions);
     int R = cc_sum_copies(K, g);
     int32_t* count_copies = nullptr;
-    const cudaError_t e = accumulate_all(ctx, L, dX, N, g, idx, K, counts, R, &count_copies, st);
+    const cudaError_t e = accumulate_all(ctx, L, dX, N, g, idx, K, counts, R, &count_copies, false, st);
     if (e != cudaSuccess) return e;
     ProfScope ps(ctx, CC_K_UPDATE_FINISH, st);
     grad_finish_kernel<<<(K * g + 255) / 256, 256, 0, st>>>(reinterpret_cast<long long*>(ws + L.sum_lo),
