@@ -169,9 +169,18 @@ cudaError_t cc_launch_unsort(cc_ctx*, const unsigned* pos, int64_t N, const uint
 cudaError_t cc_launch_assign_pruned(cc_ctx*, const PruneBuffers&, int g, const float* C, int mode, cudaStream_t);
 cudaError_t cc_launch_sum_exact(cc_ctx*, const PruneBuffers&, bool have_max, double* objective, int64_t* n_resolved, cudaStream_t);
 
+// Scratch of the layer forward in the workspace: the status block, a copy of the codebook with padded rows, the rest.
+constexpr size_t CC_LINEAR_SCRATCH_FROM = CC_STATUS_BYTES + (size_t)65536 * 32;
+
 // Compressed linear layer: y = x . decode(C16, idx)^T (+ bias), the decoded weight never stored.
 size_t cc_linear_scratch_bytes(int64_t M, int64_t d_out, int64_t d_in, int sm_count);
 int cc_linear_q_table_max(void);
+// The same for many tokens (cc_linear_wide.cu): the weight is decoded once into tiles in the workspace.
+bool cc_linear_wide_applies(int64_t M, int64_t d_out, int64_t d_in, int splits, int sm_count);
+size_t cc_linear_wide_bytes(int64_t M, int64_t d_out, int64_t d_in);
+cudaError_t cc_launch_linear_wide(cc_ctx*, const uint16_t* x, int64_t M, const uint16_t* C16, bool padded, const unsigned char* qtab,
+                                  const float* qscale, int K, int g, const uint16_t* idx, int64_t d_out, int64_t d_in,
+                                  const float* bias, float* y, int splits, cudaStream_t);
 cudaError_t cc_launch_linear_forward(cc_ctx*, const uint16_t* x, int64_t M, const uint16_t* C16, const unsigned char* qtab,
                                      const float* qscale, int K, int g, const uint16_t* idx, int64_t d_out, int64_t d_in,
                                      const float* bias, float* y, cudaStream_t);

@@ -25,6 +25,7 @@
 
 #include "cc_common.cuh"
 #include "cc_tcgen05.cuh"
+#include "cc_linear_rows.cuh"
 
 namespace {
 
@@ -52,61 +53,8 @@ __host__ __device__ constexpr int b_lbo(int nt) { return nt * 16 + 16; }
 __host__ __device__ constexpr int b_stage_bytes(int nt) { return (LKB / 8) * b_lbo(nt); }
 __device__ __forceinline__ int tile_off(int r, int kc, int lbo, int sbo) { return kc * lbo + (r >> 3) * sbo + (r & 7) * 16; }
 
-// Row of G halves of the codebook as raw bit patterns.
-template <int G>
-__device__ __forceinline__ void load_code_row(const uint16_t* __restrict__ C16, int code, uint16_t* h) {
-    const uint16_t* row = C16 + (int64_t)code * G;
-    if constexpr (G % 8 == 0) {
-#pragma unroll
-        for (int v = 0; v < G / 8; ++v) {
-            const uint4 u = __ldg(reinterpret_cast<const uint4*>(row) + v);
-            const unsigned w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) { h[v * 8 + 2 * k] = w[k] & 0xffffu; h[v * 8 + 2 * k + 1] = w[k] >> 16; }
-        }
-    } else if constexpr (G % 4 == 0) {
-#pragma unroll
-        for (int v = 0; v < G / 4; ++v) {
-            const uint2 u = __ldg(reinterpret_cast<const uint2*>(row) + v);
-            h[v * 4] = u.x & 0xffffu; h[v * 4 + 1] = u.x >> 16; h[v * 4 + 2] = u.y & 0xffffu; h[v * 4 + 3] = u.y >> 16;
-        }
-    } else if constexpr (G % 2 == 0) {
-#pragma unroll
-        for (int v = 0; v < G / 2; ++v) {
-            const unsigned u = __ldg(reinterpret_cast<const unsigned*>(row) + v);
-            h[v * 2] = u & 0xffffu; h[v * 2 + 1] = u >> 16;
-        }
-    } else {
-#pragma unroll
-        for (int t = 0; t < G; ++t) h[t] = __ldg(row + t);
-    }
-}
-
-// The same row as G / 2 32-bit words (even G).
-template <int G>
-__device__ __forceinline__ void load_code_row_words(const uint16_t* __restrict__ C16, int code, uint32_t* w) {
-    const uint16_t* row = C16 + (int64_t)code * G;
-    if constexpr (G % 8 == 0) {
-#pragma unroll
-        for (int v = 0; v < G / 8; ++v) {
-            const uint4 u = __ldg(reinterpret_cast<const uint4*>(row) + v);
-            w[4 * v] = u.x; w[4 * v + 1] = u.y; w[4 * v + 2] = u.z; w[4 * v + 3] = u.w;
-        }
-    } else if constexpr (G % 4 == 0) {
-#pragma unroll
-        for (int v = 0; v < G / 4; ++v) {
-            const uint2 u = __ldg(reinterpret_cast<const uint2*>(row) + v);
-            w[2 * v] = u.x; w[2 * v + 1] = u.y;
-        }
-    } else {
-#pragma unroll
-        for (int v = 0; v < G / 2; ++v) w[v] = __ldg(reinterpret_cast<const unsigned*>(row) + v);
-    }
-}
-
 // Quantised codebook (4 bits per value, two values per byte, low nibble first; Section 5.3): the whole
-// table sits in shared memory, and a 256-entry table turns a byte into its two dequantised FP16 values
-// (value = round-to-nearest-even FP16 of nibble * scale, the nibble a two's-complement number).
+// table sits in shared memory, and a 256-entry table turns a byte into its two dequantised FP16 values.
 constexpr int LQ_TABLE_MAX = 128 * 1024;   // bytes of packed codebook that fit beside the stages
 constexpr int LQ_BULK_PIECE = 32 * 1024;   // bytes per bulk copy of the table
 constexpr int LQ_WIDE_FROM = 256;
@@ -124,7 +72,8 @@ __device__ __forceinline__ void load_code_row_words_q(const unsigned char* __res
 // in_features (chunks_per_split stages each).  out: y itself (splits == 1) or this split's slab of
 // partial sums, both M x d_out FP32 row-major.
 // QUANT: the codebook is the packed 4-bit table `qtab` (K G / 2 bytes) with its scale instead of C16.
-template <int G, bool QUANT, int STAGES>
+// PADDED: the rows of C16 are row_pad(G) values apart.
+template <int G, bool QUANT, bool PADDED, int STAGES>
 __global__ void __launch_bounds__(LTHREADS, 1)
 linear_forward_kernel(const uint16_t* __restrict__ x, int M, const uint16_t* __restrict__ C16,
                       const unsigned char* __restrict__ qtab, const float* __restrict__ qscale, int K,
@@ -188,12 +137,7 @@ linear_forward_kernel(const uint16_t* __restrict__ x, int M, const uint16_t* __r
     if constexpr (QUANT) {
         // the packed codebook and the byte -> two FP16 values table, once per CTA
         const float s = __ldg(qscale);
-        if (tid < 256) {
-            const int lo = ((tid & 15) ^ 8) - 8, hi = ((tid >> 4) ^ 8) - 8;     // sign-extended nibbles
-            const unsigned a = __half_as_ushort(__float2half_rn(__fmul_rn((float)lo, s)));
-            const unsigned b = __half_as_ushort(__float2half_rn(__fmul_rn((float)hi, s)));
-            lut2[tid] = a | (b << 16);
-        }
+        if (tid < 256) lut2[tid] = q4_pair(tid, s);
         const int bytes = K * (G / 2);
         for (int v = (bytes / 16) * 16 + tid; v < bytes; v += LTHREADS) qt[v] = __ldg(qtab + v);
     }
@@ -223,82 +167,46 @@ linear_forward_kernel(const uint16_t* __restrict__ x, int M, const uint16_t* __r
             // ---- A: gather, transpose, store.  item = (block of 8 in_features, code group)
             // IPT items per thread and pass: all their codes are requested first, then all their rows, so that a
             // pass costs two trips to L2 whatever IPT is (the rows of IPT items must fit the registers)
-            constexpr int IPT = (G % 2 == 0 && G <= 8) ? 2 : 1;
+            constexpr int IPT = (G <= 8 && (PADDED || G % 2 == 0)) ? 2 : 1, W = (G + 1) / 2;
             for (int item0 = ptid; item0 < (LKB / 8) * n_grp; item0 += IPT * stage_threads) {
-                if constexpr (G % 2 == 0) {
-                    // rows kept as 32-bit words (two out_features each): half the registers of a 16-bit copy
-                    uint32_t v[IPT][8][G / 2];
-                    int code[IPT][8];
-                    int ibs[IPT], grps[IPT];
+                // rows kept as 32-bit words (two out_features each)
+                uint32_t v[IPT][8][W];
+                int code[IPT][8];
+                int ibs[IPT], grps[IPT];
 #pragma unroll
-                    for (int q = 0; q < IPT; ++q) {
-                        const int item = item0 + q * stage_threads;
-                        const bool live = item < (LKB / 8) * n_grp;
-                        ibs[q] = live ? item / n_grp : 0;
-                        grps[q] = live ? grp_lo + (item - ibs[q] * n_grp) : -1;
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            const int i = i0 + ibs[q] * 8 + u;
-                            code[q][u] = (live && i < d_in) ? (int)__ldg(idx + (int64_t)i * out_groups + grps[q]) : -1;
-                        }
-                    }
-#pragma unroll
-                    for (int q = 0; q < IPT; ++q) {
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            if (code[q][u] >= 0) {
-                                if constexpr (QUANT) load_code_row_words_q<G>(qt, lut2, code[q][u], v[q][u]);
-                                else load_code_row_words<G>(C16, code[q][u], v[q][u]);
-                            } else {
-#pragma unroll
-                                for (int t = 0; t < G / 2; ++t) v[q][u][t] = 0u;
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int q = 0; q < IPT; ++q) {
-                        if (grps[q] < 0) continue;
-#pragma unroll
-                        for (int t = 0; t < G; ++t) {
-                            const int r = grps[q] * G + t - o0;     // row of the tile = out_feature - o0
-                            if (r < 0 || r >= LM) continue;
-                            const unsigned sel = (t & 1) ? 0x7632u : 0x5410u;   // high or low halves of two words
-                            uint4 w;
-                            w.x = __byte_perm(v[q][0][t / 2], v[q][1][t / 2], sel);
-                            w.y = __byte_perm(v[q][2][t / 2], v[q][3][t / 2], sel);
-                            w.z = __byte_perm(v[q][4][t / 2], v[q][5][t / 2], sel);
-                            w.w = __byte_perm(v[q][6][t / 2], v[q][7][t / 2], sel);
-                            *reinterpret_cast<uint4*>(tA + tile_off(r, ibs[q], A_LBO, A_SBO)) = w;
-                        }
-                    }
-                } else {
-                    const int ib = item0 / n_grp, grp = grp_lo + (item0 - (item0 / n_grp) * n_grp);
-                    uint16_t v[8][G];
-                    int code[8];
+                for (int q = 0; q < IPT; ++q) {
+                    const int item = item0 + q * stage_threads;
+                    const bool live = item < (LKB / 8) * n_grp;
+                    ibs[q] = live ? item / n_grp : 0;
+                    grps[q] = live ? grp_lo + (item - ibs[q] * n_grp) : -1;
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
-                        const int i = i0 + ib * 8 + u;
-                        code[u] = (i < d_in) ? (int)__ldg(idx + (int64_t)i * out_groups + grp) : -1;
+                        const int i = i0 + ibs[q] * 8 + u;
+                        code[q][u] = (live && i < d_in) ? (int)__ldg(idx + (int64_t)i * out_groups + grps[q]) : -1;
                     }
+                }
+#pragma unroll
+                for (int q = 0; q < IPT; ++q) {
 #pragma unroll
                     for (int u = 0; u < 8; ++u) {
-                        if (code[u] >= 0) {
-                            load_code_row<G>(C16, code[u], v[u]);
+                        if (code[q][u] >= 0) {
+                            if constexpr (QUANT) load_code_row_words_q<G>(qt, lut2, code[q][u], v[q][u]);
+                            else if constexpr (PADDED) load_row_padded<G>(C16, (unsigned)code[q][u], v[q][u]);
+                            else load_row<G>(C16, (unsigned)code[q][u], (unsigned)K - 1u, v[q][u]);
                         } else {
 #pragma unroll
-                            for (int t = 0; t < G; ++t) v[u][t] = 0;
+                            for (int t = 0; t < W; ++t) v[q][u][t] = 0u;
                         }
                     }
+                }
+#pragma unroll
+                for (int q = 0; q < IPT; ++q) {
+                    if (grps[q] < 0) continue;
 #pragma unroll
                     for (int t = 0; t < G; ++t) {
-                        const int r = grp * G + t - o0;
+                        const int r = grps[q] * G + t - o0;         // row of the tile = out_feature - o0
                         if (r < 0 || r >= LM) continue;
-                        uint4 w;
-                        w.x = (unsigned)v[0][t] | ((unsigned)v[1][t] << 16);
-                        w.y = (unsigned)v[2][t] | ((unsigned)v[3][t] << 16);
-                        w.z = (unsigned)v[4][t] | ((unsigned)v[5][t] << 16);
-                        w.w = (unsigned)v[6][t] | ((unsigned)v[7][t] << 16);
-                        *reinterpret_cast<uint4*>(tA + tile_off(r, ib, A_LBO, A_SBO)) = w;
+                        *reinterpret_cast<uint4*>(tA + tile_off(r, ibs[q], A_LBO, A_SBO)) = transpose_piece<W>(v[q], t);
                     }
                 }
             }
@@ -362,7 +270,7 @@ linear_forward_kernel(const uint16_t* __restrict__ x, int M, const uint16_t* __r
         }
     } else {
         // ------------------------------------------------------------ MMA warp: one thread issues
-        if (lane == 0) {
+        if (elect_one()) {
             // kind::f16: D = F32 (bits 4-5 = 1), A = B = F16 (0), both K-major, N >> 3 at bit 17, M >> 4 at bit 24
             const int mma_n = NT < LNT_MAX ? NT : LNT_MAX;          // 512 tokens per CTA are two MMAs of 256 columns
             const uint32_t idesc = (1u << 4) | ((uint32_t)(mma_n >> 3) << 17) | ((uint32_t)(LM >> 4) << 24);
@@ -637,6 +545,25 @@ linear_gemv_q4_kernel(const uint16_t* __restrict__ x, int M, const unsigned char
     }
 }
 
+// Copy of the codebook with rows of `pad` values, a power of two, so that a gather is one load (load_row_padded).
+__global__ void __launch_bounds__(256)
+linear_pad_rows_kernel(const uint16_t* __restrict__ C16, int K, int g, int pad, uint16_t* __restrict__ table) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= K) return;
+    const uint16_t* src = C16 + (int64_t)j * g;
+    uint2* dst = reinterpret_cast<uint2*>(table + (int64_t)j * pad);
+    for (int t = 0; t < pad; t += 4) {
+        unsigned h[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) h[u] = t + u < g ? (unsigned)__ldg(src + t + u) : 0u;
+        dst[t / 4] = make_uint2(h[0] | h[1] << 16, h[2] | h[3] << 16);
+    }
+}
+
+// Codes from which the copy pays: as a launch it takes about 4 us, and it saves some 12 us a million codes at g = 6
+// (33 tokens, g = 6, K = 1024: 512 x 512 17.4 us without, 21.5 with it).
+constexpr int64_t LINEAR_PAD_FROM = 400000;
+
 struct GemvPlan { int o_blocks, splits, rows_per_split; };
 
 GemvPlan gemv_plan(int64_t d_in, int out_groups, int sm_count) {
@@ -659,7 +586,15 @@ size_t gemv_smem(int g, int K, int rows, int mt) {
     return 128 + ((size_t)rows * mt * 4 + 15) / 16 * 16 + (tail + 15) / 16 * 16;
 }
 
-struct LinearPlan { int NT, a_pad, stages, tmem_cols, o_tiles, tok_blocks, splits, chunks_per_split; size_t smem; };
+// Tokens from which decoding the weight once and multiplying it afterwards (cc_linear_wide.cu) is the faster way
+// (4096 x 4096, g = 4, K = 65536: 128 tokens 42 against 46 us, 192 tokens 52 against 46, 512 tokens 85 against 52), earlier
+// where the tiles of this kernel fill the SMs by themselves, so that its waves are the coarser (11008 x 4096, g = 8,
+// 128 tokens: 95 against 67 us; g = 6, 33 tokens: 83 against about 80).
+constexpr int LINEAR_WIDE_FROM = 192, LINEAR_WIDE_FEWEST = 96;
+
+constexpr int LINEAR_SPLITS_MORE = 8;   // splits beyond those that fill the SMs once are tried up to this many
+
+struct LinearPlan { int NT, a_pad, stages, tmem_cols, o_tiles, tok_blocks, splits, chunks_per_split, fill; size_t smem; };   // fill: splits that fill the SMs once
 
 // nt_max: tokens per CTA (256, or 64 with a quantised codebook in shared memory); table_bytes: that codebook.
 LinearPlan linear_plan(int64_t M, int64_t d_out, int64_t d_in, int sm_count, int nt_max = LNT_MAX, size_t table_bytes = 0,
@@ -681,8 +616,19 @@ LinearPlan linear_plan(int64_t M, int64_t d_out, int64_t d_in, int sm_count, int
     int splits = sm_count / (p.o_tiles * p.tok_blocks);             // fill the SMs when there are few tiles
     if (splits > chunks / 4) splits = chunks / 4;                   // at least four stages of work per CTA
     if (splits < 1) splits = 1;
-    p.chunks_per_split = (chunks + splits - 1) / splits;
-    p.splits = (chunks + p.chunks_per_split - 1) / p.chunks_per_split;
+    p.fill = splits;
+    // More splits where the last wave would leave most SMs idle (86 tiles on 148 SMs: five splits make 2.9 waves of a
+    // fifth each; 33 tokens, 11008 x 4096, g = 6: 80 -> 62 us): clocks of a wave count as its stages, two stages' worth of
+    // setting up, and the slabs' traffic.  A stage is 8192 / g gathers at 0.73 a clock.
+    const double stage_clk = 8192.0 / g / 0.73 + 4.0 * p.NT, slab_clk = (double)M * (double)d_out * 8.0 / 2000.0;
+    double least = 0.0;
+    const int most = chunks / 4 < LINEAR_SPLITS_MORE ? chunks / 4 : LINEAR_SPLITS_MORE;
+    for (int cand = splits; cand <= most || cand == splits; ++cand) {
+        const int cps = (chunks + cand - 1) / cand, real = (chunks + cps - 1) / cps;
+        const int64_t ctas = (int64_t)p.o_tiles * p.tok_blocks * real;
+        const double t = (double)((ctas + sm_count - 1) / sm_count) * (cps + 2) * stage_clk + (real > 1 ? 4000.0 + real * slab_clk : 0.0);
+        if (cand == splits || t < 0.95 * least) { least = t; p.splits = real; p.chunks_per_split = cps; }
+    }
     p.a_pad = (table_bytes == 0 && p.NT <= 64) ? 1 : 0;
     p.stages = (wide || (table_bytes != 0 && p.NT > LQ_NT_MAX)) ? 2 : LSTAGES;
     p.smem = (size_t)p.stages * (a_stage(p.a_pad) + (size_t)b_stage_bytes(p.NT)) + 256;
@@ -696,7 +642,10 @@ size_t cc_linear_scratch_bytes(int64_t M, int64_t d_out, int64_t d_in, int sm_co
     // enough for either form of the codebook: the quantised one takes narrower token blocks and may split more
     const LinearPlan p = linear_plan(M, d_out, d_in, sm_count);     // g <= 4: the shape with the fewest CTAs, hence the most splits
     const LinearPlan q = linear_plan(M, d_out, d_in, sm_count, LQ_NT_MAX, 16);
-    int splits = p.splits > q.splits ? p.splits : q.splits;
+    int splits = p.fill > q.fill ? p.fill : q.fill;
+    if (splits < LINEAR_SPLITS_MORE) splits = LINEAR_SPLITS_MORE;
+    const int chunks = (int)((d_in + LKB - 1) / LKB);
+    if (splits > chunks / 4) splits = chunks / 4;
     if (splits < 2) splits = 0;    // a single CTA per tile writes y itself
     if (M <= LG_M_MAX) {
         // the few-token kernel of the quantised codebook always goes through its slabs; the most slices come
@@ -704,7 +653,9 @@ size_t cc_linear_scratch_bytes(int64_t M, int64_t d_out, int64_t d_in, int sm_co
         const GemvPlan v = gemv_plan(d_in, (int)((d_out + 15) / 16), sm_count);
         if (v.splits > splits) splits = v.splits;
     }
-    return CC_STATUS_BYTES + (size_t)splits * (size_t)M * (size_t)d_out * 4;
+    const size_t own = CC_LINEAR_SCRATCH_FROM + (size_t)splits * (size_t)M * (size_t)d_out * 4;
+    const size_t wide = M >= LINEAR_WIDE_FEWEST ? cc_linear_wide_bytes(M, d_out, d_in) : 0;
+    return own > wide ? own : wide;
 }
 
 int cc_linear_q_table_max(void) { return LQ_TABLE_MAX; }
@@ -722,7 +673,7 @@ int cc_linear_q_table_max(void) { return LQ_TABLE_MAX; }
 
 namespace {
 
-template <int G, bool QUANT, int STAGES>
+template <int G, bool QUANT, bool PADDED, int STAGES>
 cudaError_t launch_linear_s(cc_ctx* ctx, const LinearPlan& p, const uint16_t* x, int M, const uint16_t* C16,
                             const unsigned char* qtab, const float* qscale, int K, const uint16_t* idx, int d_out, int d_in,
                             int out_groups, float* out, int64_t split_stride, const float* bias, unsigned* status,
@@ -736,13 +687,13 @@ cudaError_t launch_linear_s(cc_ctx* ctx, const LinearPlan& p, const uint16_t* x,
                                                   : (int)(LSTAGES * (a_stage(false) + b_stage_bytes(LQ_NT_MAX)) + 256 + 1024 + LQ_TABLE_MAX))
                                    : (STAGES == 2 ? (int)(2 * (a_stage(false) + b_stage_bytes(2 * LNT_MAX)) + 256)
                                                   : (int)(LSTAGES * (a_stage(true) + b_stage_bytes(LNT_MAX)) + 256));
-        const cudaError_t e = cudaFuncSetAttribute(linear_forward_kernel<G, QUANT, STAGES>,
+        const cudaError_t e = cudaFuncSetAttribute(linear_forward_kernel<G, QUANT, PADDED, STAGES>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
         if (e != cudaSuccess) return e;
         have = true;
     }
     const dim3 grid(p.o_tiles, p.tok_blocks, p.splits);
-    linear_forward_kernel<G, QUANT, STAGES><<<grid, LTHREADS, p.smem, st>>>(x, M, C16, qtab, qscale, K, idx, d_out, d_in,
+    linear_forward_kernel<G, QUANT, PADDED, STAGES><<<grid, LTHREADS, p.smem, st>>>(x, M, C16, qtab, qscale, K, idx, d_out, d_in,
                                                                             out_groups, p.NT, p.a_pad, p.tmem_cols,
                                                                             p.chunks_per_split, out, split_stride, bias, status, arrived,
                                                                             bias_final, y_final);
@@ -750,18 +701,18 @@ cudaError_t launch_linear_s(cc_ctx* ctx, const LinearPlan& p, const uint16_t* x,
 }
 
 // Two stages exist where the plan can ask for them: beside the 4-bit table, and for rows of at most 8 bytes.
-template <int G, bool QUANT>
+template <int G, bool QUANT, bool PADDED>
 cudaError_t launch_linear(cc_ctx* ctx, const LinearPlan& p, const uint16_t* x, int M, const uint16_t* C16,
                           const unsigned char* qtab, const float* qscale, int K, const uint16_t* idx, int d_out, int d_in,
                           int out_groups, float* out, int64_t split_stride, const float* bias, unsigned* status,
                           unsigned* arrived, const float* bias_final, float* y_final, cudaStream_t st) {
     if constexpr (QUANT || G <= 4) {
         if (p.stages == 2)
-            return launch_linear_s<G, QUANT, 2>(ctx, p, x, M, C16, qtab, qscale, K, idx, d_out, d_in, out_groups, out,
+            return launch_linear_s<G, QUANT, PADDED, 2>(ctx, p, x, M, C16, qtab, qscale, K, idx, d_out, d_in, out_groups, out,
                                                 split_stride, bias, status, arrived, bias_final, y_final, st);
     }
     if (p.stages != LSTAGES) return cudaErrorInvalidValue;
-    return launch_linear_s<G, QUANT, LSTAGES>(ctx, p, x, M, C16, qtab, qscale, K, idx, d_out, d_in, out_groups, out,
+    return launch_linear_s<G, QUANT, PADDED, LSTAGES>(ctx, p, x, M, C16, qtab, qscale, K, idx, d_out, d_in, out_groups, out,
                                               split_stride, bias, status, arrived, bias_final, y_final, st);
 }
 
@@ -815,11 +766,23 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
                                      const unsigned char* qtab, const float* qscale, int K, int g, const uint16_t* idx,
                                      int64_t d_out, int64_t d_in, const float* bias, float* y, cudaStream_t st) {
     // beside the table: token blocks of 64 with four stages, or, from LQ_WIDE_FROM tokens on, of 256 with two
-    const LinearPlan p = qtab ? linear_plan(M, d_out, d_in, ctx->sm_count, M >= LQ_WIDE_FROM ? LNT_MAX : LQ_NT_MAX, (size_t)K * (g / 2))
+    const LinearPlan p = qtab ? linear_plan(M, d_out, d_in, ctx->sm_count, M >= LQ_WIDE_FROM ? LNT_MAX : LQ_NT_MAX, (size_t)K * (g / 2), g)
                               : linear_plan(M, d_out, d_in, ctx->sm_count, LNT_MAX, 0, g);
+    const int64_t codes = (d_out + g - 1) / g * d_in;
+    // the codebook's own rows take one load (the widest wants them on 32-byte boundaries)
+    bool padded = row_pad(g) == g && (g < 16 || (reinterpret_cast<uintptr_t>(C16) & 31u) == 0);
+    if (!qtab && !padded && codes >= LINEAR_PAD_FROM && codes >= 4 * (int64_t)K) {
+        uint16_t* table = reinterpret_cast<uint16_t*>(static_cast<char*>(ctx->ws) + CC_STATUS_BYTES);
+        ProfScope ps(ctx, CC_K_OTHER, st);
+        linear_pad_rows_kernel<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(C16, K, g, row_pad(g), table);
+        C16 = table;
+        padded = true;
+    }
+    if (M >= (p.fill == 1 ? LINEAR_WIDE_FEWEST : LINEAR_WIDE_FROM) && cc_linear_wide_applies(M, d_out, d_in, p.fill, ctx->sm_count))
+        return cc_launch_linear_wide(ctx, x, M, C16, padded, qtab, qscale, K, g, idx, d_out, d_in, bias, y, p.fill, st);
     char* ws = static_cast<char*>(ctx->ws);
     unsigned* status = reinterpret_cast<unsigned*>(ws);
-    float* partial = reinterpret_cast<float*>(ws + CC_STATUS_BYTES);
+    float* partial = reinterpret_cast<float*>(ws + CC_LINEAR_SCRATCH_FROM);
     const int out_groups = (int)((d_out + g - 1) / g);
     const int64_t n = M * d_out;
     cudaError_t e = cudaSuccess;
@@ -861,7 +824,7 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
         fused = p.splits > 1 && M <= 16 && (int64_t)p.o_tiles * p.tok_blocks <= CC_ARRIVAL_COUNTERS;
         unsigned* arrived = fused ? status + CC_ARRIVAL_WORD : nullptr;
         if (qtab) {
-#define CALL(G) e = launch_linear<G, true>(ctx, p, x, (int)M, nullptr, qtab, qscale, K, idx, (int)d_out, (int)d_in, out_groups, out, n, b, status, arrived, bias, y, st)
+#define CALL(G) e = launch_linear<G, true, false>(ctx, p, x, (int)M, nullptr, qtab, qscale, K, idx, (int)d_out, (int)d_in, out_groups, out, n, b, status, arrived, bias, y, st)
             switch (g) {
                 case 2: CALL(2); break;   case 4: CALL(4); break;   case 6: CALL(6); break;   case 8: CALL(8); break;
                 case 10: CALL(10); break; case 12: CALL(12); break; case 14: CALL(14); break; case 16: CALL(16); break;
@@ -869,9 +832,11 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
             }
 #undef CALL
         } else {
-#define CALL(G) e = launch_linear<G, false>(ctx, p, x, (int)M, C16, nullptr, nullptr, K, idx, (int)d_out, (int)d_in, out_groups, out, n, b, status, arrived, bias, y, st)
+#define ROWS(G, PADDED) launch_linear<G, false, PADDED>(ctx, p, x, (int)M, C16, nullptr, nullptr, K, idx, (int)d_out, (int)d_in, out_groups, out, n, b, status, arrived, bias, y, st)
+#define CALL(G) if constexpr (row_pad(G) == G && G < 16) e = ROWS(G, true); else e = padded ? ROWS(G, true) : ROWS(G, false)
             CC_LINEAR_DISPATCH(g, CALL)
 #undef CALL
+#undef ROWS
         }
     }
     if (e != cudaSuccess) return e;
