@@ -362,18 +362,25 @@ linear_reduce_kernel(const float* __restrict__ partial, int splits, int64_t n, i
     }
 }
 
-// ---- A handful of tokens (M <= 4; M <= 2 for g > 8) on the 4-bit codebook: no tensor core.  With so few columns the MMA
-// idles and the tensor kernel's time is its producers' instructions; here a thread owns one code group (g
-// out_features), walks down the in_features of its CTA's slice, looks each code up in the packed table in
-// shared memory (one load of g / 2 bytes, then one load per 4-bit level from a 16-entry FP32 table, whose
-// entries lie in 16 different banks: no conflicts whatever the levels) and adds x times the g values
-// to M x g FP32 accumulators.  A product of two FP16 values is exact in FP32, so only the additions round.
-// CTA = 64 code groups x 16 interleaved sub-slices of the in_features; the sixteen partial sums meet in
-// shared memory in a fixed order, and the CTA writes its slab of partial sums (y itself when the layer
-// needs a single slice per block of code groups); the slabs are added in slice order by the CTA that
-// finishes last, or by linear_reduce_kernel: the same bits on every call.
-// blockIdx.x: block of 64 code groups; blockIdx.y: slice of rows_per_split in_features.
-constexpr int LG_THREADS = 1024, LG_GRPS = 64, LG_SUB = 16, LG_ROWS_MAX = 1024, LG_M_MAX = 4;
+// ---- A handful of tokens (M <= 4; M <= 2 for g > 8): no tensor core.  With so few columns the MMA idles and the tensor
+// kernel's time is its gathers; here a thread owns one code group (g out_features), walks down the in_features of its
+// CTA's range, looks each code up in shared memory and adds x times the g values to M x g FP32 accumulators.  A product
+// of two FP16 values is exact in FP32, so only the additions round.
+// 4-bit codebook (QUANT): the whole packed table is in shared memory; a code is one load of g / 2 bytes, then one load
+// per 4-bit level from a 16-entry FP32 table, whose entries lie in 16 different banks (no conflicts).
+// FP16 codebook: a table that does not fit is cut into slices, a CTA for each.  It reads all the codes of its range and
+// adds up those inside its slice; the others read a row of zeros behind it.  Reading every code once per slice is
+// cheap (coalesced, about 12 instructions each) beside a gather from L2, of which an SM gets 0.73 a clock through: one
+// token, 4096 x 4096, g = 4, K = 65536 (512 KB, three slices) 26.9 us as gathers, 17.2 so.
+// CTA = 64 threads' code groups x 16 interleaved sub-slices of the in_features; the sixteen partial sums meet in
+// shared memory in a fixed order, and the CTA writes its slab of partial sums (y itself when there is a single
+// slab); the slabs are added in order by the CTA that finishes last, or by linear_reduce_kernel: the same bits
+// on every call.
+// blockIdx.x: block of 64 code groups; y: range of rows_per_split in_features; z: slice of slice_rows codebook rows.
+constexpr int LG_THREADS = 1024, LG_GRPS = 64, LG_SUB = 16, LG_M_MAX = 4;
+constexpr int LG_X_MAX = 16 * 1024;                    // bytes of x (FP32) beside the table
+constexpr int LG_SMEM = 226 * 1024, LG_SLICE = LG_SMEM - 128 - LG_X_MAX - 64;   // bytes of a slice
+constexpr int LG_SLICES_MAX = 5;
 
 template <int G>
 __device__ __forceinline__ void gemv_levels(const unsigned char* row, unsigned (&lv)[G]) {
@@ -395,24 +402,69 @@ __device__ __forceinline__ void gemv_levels(const unsigned char* row, unsigned (
     }
 }
 
-template <int G, int MT>
+// Row of G halves from shared memory as FP32; rows of an odd number of values start in either half of a word.
+template <int G>
+__device__ __forceinline__ void gemv_row(const unsigned char* table, unsigned row, float (&c)[G]) {
+    constexpr int W = (G + 1) / 2;
+    uint32_t w[W];
+    if constexpr (G % 8 == 0) {
+        const uint4* p = reinterpret_cast<const uint4*>(table + (size_t)row * (2 * G));
+#pragma unroll
+        for (int v = 0; v < G / 8; ++v) { const uint4 u = p[v]; w[4 * v] = u.x; w[4 * v + 1] = u.y; w[4 * v + 2] = u.z; w[4 * v + 3] = u.w; }
+    } else if constexpr (G % 4 == 0) {
+        const uint2* p = reinterpret_cast<const uint2*>(table + (size_t)row * (2 * G));
+#pragma unroll
+        for (int v = 0; v < G / 4; ++v) { const uint2 u = p[v]; w[2 * v] = u.x; w[2 * v + 1] = u.y; }
+    } else if constexpr (G % 2 == 0) {
+        const uint32_t* p = reinterpret_cast<const uint32_t*>(table + (size_t)row * (2 * G));
+#pragma unroll
+        for (int v = 0; v < W; ++v) w[v] = p[v];
+    } else {
+        const uint32_t* p = reinterpret_cast<const uint32_t*>(table) + ((row * G) >> 1);
+        const bool shifted = row & 1u;
+        uint32_t u[W];
+#pragma unroll
+        for (int v = 0; v < W; ++v) u[v] = p[v];
+#pragma unroll
+        for (int v = 0; v < W; ++v) w[v] = shifted ? __funnelshift_r(u[v], v + 1 < W ? u[v + 1] : 0u, 16) : u[v];
+    }
+#pragma unroll
+    for (int t = 0; t < G; ++t) c[t] = __half2float(__ushort_as_half((unsigned short)((t & 1) ? w[t / 2] >> 16 : w[t / 2] & 0xffffu)));
+}
+
+// Rows of codes a thread requests together; the next ones are under way while these are used.
+__host__ __device__ constexpr int gemv_batch(int g, int mt) { return g * mt <= 8 ? 8 : 4; }
+// Neighbouring code groups per thread: two codes come in one word and share the loads of x.  For short rows of the FP16
+// codebook and layers of many codes: one token, g = 4, K = 65536, 11008 x 4096 39.8 -> 33.7 us, 4096 x 4096 18.7 -> 17.2;
+// with few codes the wider exchange at the end costs more (g = 3, 700 x 900 7.7 -> 9.3; g = 8, 4096 x 4096 16.2 -> 17.1).
+__host__ __device__ constexpr bool gemv_pair(int g, bool quant) { return g <= 4 && !quant; }
+constexpr int64_t LG_PAIR_FROM = 1 << 21;              // codes
+
+// PW: code groups per thread, 1 or 2 (2 wants an even number of groups and the codes on a word boundary).
+template <int G, int MT, bool QUANT, int PW>
 __global__ void __launch_bounds__(LG_THREADS, 1)
-linear_gemv_q4_kernel(const uint16_t* __restrict__ x, int M, const unsigned char* __restrict__ qtab,
-                      const float* __restrict__ qscale, int K, const uint16_t* __restrict__ idx, int d_out, int d_in,
-                      int out_groups, int rows_per_split, float* __restrict__ out, int64_t split_stride,
-                      unsigned* __restrict__ status, unsigned* __restrict__ arrived, const float* __restrict__ bias,
-                      float* __restrict__ y, int direct) {
+linear_gemv_kernel(const uint16_t* __restrict__ x, int M, const unsigned char* __restrict__ book,
+                   const float* __restrict__ qscale, int K, int slice_rows, const uint16_t* __restrict__ idx, int d_out, int d_in,
+                   int out_groups, int rows_per_split, float* __restrict__ out, int64_t split_stride,
+                   unsigned* __restrict__ status, unsigned* __restrict__ arrived, const float* __restrict__ bias,
+                   float* __restrict__ y, int direct) {
     extern __shared__ __align__(16) unsigned char gv_smem[];
+    constexpr int RB = gemv_batch(G, MT), STEP = RB * LG_SUB, GE = G * PW;       // out_features per thread
+    constexpr int ROWB = QUANT ? G / 2 : 2 * G;                                  // bytes of a codebook row
     uint64_t* qbar = reinterpret_cast<uint64_t*>(gv_smem);                       // the table has landed
     volatile int* abort_flag = reinterpret_cast<volatile int*>(gv_smem + 8);
-    float* lut16 = reinterpret_cast<float*>(gv_smem + 64);                       // level -> value
-    float* xs = reinterpret_cast<float*>(gv_smem + 128);                         // [row][MT]
-    unsigned char* qt = gv_smem + 128 + ((size_t)rows_per_split * MT * 4 + 15) / 16 * 16;   // packed table, later the exchange area
+    float* lut16 = reinterpret_cast<float*>(gv_smem + 64);                       // level -> value (QUANT)
+    float* xs = reinterpret_cast<float*>(gv_smem + 128);                         // [row][MT], zeros up to a whole step
+    const int rows_whole = (rows_per_split + STEP - 1) / STEP * STEP;
+    unsigned char* qt = gv_smem + 128 + (size_t)rows_whole * MT * 4;             // table, later the exchange area
     const int tid = threadIdx.x, gl = tid % LG_GRPS, sub = tid / LG_GRPS;
     const int i0 = blockIdx.y * rows_per_split;
     int rows = d_in - i0;
     rows = rows < rows_per_split ? rows : rows_per_split;
-    const int bytes = K * (G / 2);
+    const unsigned lo = (unsigned)blockIdx.z * (unsigned)slice_rows;
+    const unsigned n_rows = K - (int)lo < slice_rows ? K - lo : (unsigned)slice_rows;
+    const int bytes = (int)n_rows * ROWB;
+    const unsigned char* src_book = book + (size_t)lo * ROWB;
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(qbar)));
         *abort_flag = 0;
@@ -423,84 +475,106 @@ linear_gemv_q4_kernel(const uint16_t* __restrict__ x, int M, const unsigned char
             for (uint32_t off = 0; off < bulk; off += LQ_BULK_PIECE) {
                 const uint32_t n = bulk - off < (uint32_t)LQ_BULK_PIECE ? bulk - off : (uint32_t)LQ_BULK_PIECE;
                 asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                             ::"r"(smem_u32(qt + off)), "l"(qtab + off), "r"(n), "r"(bar) : "memory");
+                             ::"r"(smem_u32(qt + off)), "l"(src_book + off), "r"(n), "r"(bar) : "memory");
             }
         } else {
             asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
         }
     }
-    for (int v = (bytes / 16) * 16 + tid; v < bytes; v += LG_THREADS) qt[v] = __ldg(qtab + v);
-    if (tid < 16) {
-        const int level = (tid ^ 8) - 8;                                         // sign-extended
-        lut16[tid] = __half2float(__float2half_rn(__fmul_rn((float)level, __ldg(qscale))));   // the quantiser's own value
+    const int units = out_groups / PW, grp = blockIdx.x * LG_GRPS + gl;          // unit: the code groups of a thread
+    const bool live = grp < units;
+    const uint16_t* col = idx + (int64_t)i0 * out_groups + (live ? grp * PW : 0);
+    unsigned code[RB];
+    auto request = [&](int r0) {
+#pragma unroll
+        for (int u = 0; u < RB; ++u) {
+            const int r = r0 + u * LG_SUB;
+            const uint16_t* at = col + (int64_t)(r < rows ? r : 0) * out_groups;
+            if constexpr (PW == 2) code[u] = __ldg(reinterpret_cast<const unsigned*>(at));
+            else code[u] = __ldg(at);
+        }
+    };
+    request(sub);
+    for (int v = (bytes / 16) * 16 + tid; v < bytes; v += LG_THREADS) qt[v] = __ldg(src_book + v);
+    if constexpr (QUANT) {
+        if (tid < 16) {
+            const int level = (tid ^ 8) - 8;                                     // sign-extended
+            lut16[tid] = __half2float(__float2half_rn(__fmul_rn((float)level, __ldg(qscale))));   // the quantiser's own value
+        }
+    } else {
+        if (tid < ROWB + 4) qt[bytes + tid] = 0;                                 // the row of zeros
     }
-    for (int e = tid; e < rows * MT; e += LG_THREADS) {
+    for (int e = tid; e < rows_whole * MT; e += LG_THREADS) {
         const int r = e / MT, m = e - r * MT;
-        xs[e] = (m < M) ? __half2float(__ushort_as_half(__ldg(x + (int64_t)m * d_in + i0 + r))) : 0.f;
+        xs[e] = (m < M && r < rows) ? __half2float(__ushort_as_half(__ldg(x + (int64_t)m * d_in + i0 + r))) : 0.f;
     }
     __syncthreads();
-    bool ok = true, waited = false;                        // the first codes are requested before the wait for the table
+    const bool ok = mbar_wait(smem_u32(qbar), 0, abort_flag);                    // nobody goes on before the table has landed
 
-    const int grp = blockIdx.x * LG_GRPS + gl;
-    const bool live = grp < out_groups;
-    float acc[MT][G];
+    float acc[MT][GE];
 #pragma unroll
     for (int m = 0; m < MT; ++m)
 #pragma unroll
-        for (int t = 0; t < G; ++t) acc[m][t] = 0.f;
+        for (int t = 0; t < GE; ++t) acc[m][t] = 0.f;
     const unsigned kmax = (unsigned)K - 1u;
-    if (live) {
-        const uint16_t* col = idx + (int64_t)i0 * out_groups + grp;
-        constexpr int RB = 4;                                                    // rows whose codes are requested together
-        for (int r0 = sub; r0 < rows; r0 += RB * LG_SUB) {
-            unsigned code[RB];
+    if (live && ok) {
+        for (int r0 = sub; r0 < rows; r0 += STEP) {
+            unsigned now[RB];
+#pragma unroll
+            for (int u = 0; u < RB; ++u) now[u] = code[u];
+            request(r0 + STEP);
 #pragma unroll
             for (int u = 0; u < RB; ++u) {
                 const int r = r0 + u * LG_SUB;
-                code[u] = (r < rows) ? (unsigned)__ldg(col + (int64_t)r * out_groups) : 0u;
-            }
-            if (!waited) {
-                ok = mbar_wait(smem_u32(qbar), 0, abort_flag);
-                waited = true;
-                if (!ok) break;
-            }
-#pragma unroll
-            for (int u = 0; u < RB; ++u) {
-                const int r = r0 + u * LG_SUB;
-                if (r >= rows) break;
-                unsigned lv[G];
-                gemv_levels<G>(qt + (size_t)min(code[u], kmax) * (G / 2), lv);   // a code beyond the codebook must not leave it
+                if (QUANT && r >= rows) break;
                 float xv[MT];
+                if constexpr (MT == 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(xs + r * 4);
+                    xv[0] = v.x; xv[1] = v.y; xv[2] = v.z; xv[3] = v.w;
+                } else if constexpr (MT == 2) {
+                    const float2 v = *reinterpret_cast<const float2*>(xs + r * 2);
+                    xv[0] = v.x; xv[1] = v.y;
+                } else {
+                    xv[0] = xs[r];
+                }
 #pragma unroll
-                for (int m = 0; m < MT; ++m) xv[m] = xs[r * MT + m];
+                for (int p = 0; p < PW; ++p) {
+                    const unsigned one = PW == 1 ? now[u] : (p ? now[u] >> 16 : now[u] & 0xffffu);
+                    float c[G];
+                    if constexpr (QUANT) {
+                        unsigned lv[G];
+                        gemv_levels<G>(qt + (size_t)min(one, kmax) * ROWB, lv);  // a code beyond the codebook must not leave it
 #pragma unroll
-                for (int t = 0; t < G; ++t) {
-                    const float c = lut16[lv[t]];
+                        for (int t = 0; t < G; ++t) c[t] = lut16[lv[t]];
+                    } else {
+                        gemv_row<G>(qt, r < rows ? min(one - lo, n_rows) : n_rows, c);   // outside the slice, or past the last row: zeros
+                    }
 #pragma unroll
-                    for (int m = 0; m < MT; ++m) acc[m][t] = fmaf(xv[m], c, acc[m][t]);
+                    for (int m = 0; m < MT; ++m)
+#pragma unroll
+                        for (int t = 0; t < G; ++t) acc[m][p * G + t] = fmaf(xv[m], c[t], acc[m][p * G + t]);
                 }
             }
         }
     }
-    if (!waited) ok = mbar_wait(smem_u32(qbar), 0, abort_flag);   // nobody writes over the table's place before it has landed
     // ---- the sub-slices meet, one token at a time (the exchange area takes the table's place)
     __syncthreads();
-    float* red = reinterpret_cast<float*>(qt);                                   // [LG_SUB - 1][G][LG_GRPS]
-    float* dst = out + (int64_t)blockIdx.y * split_stride;
+    float* red = reinterpret_cast<float*>(qt);                                   // [LG_SUB - 1][GE][LG_GRPS]
+    float* dst = out + ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * split_stride;
 #pragma unroll
     for (int m = 0; m < MT; ++m) {
         if (sub > 0) {
 #pragma unroll
-            for (int t = 0; t < G; ++t) red[((sub - 1) * G + t) * LG_GRPS + gl] = acc[m][t];
+            for (int t = 0; t < GE; ++t) red[((sub - 1) * GE + t) * LG_GRPS + gl] = acc[m][t];
         }
         __syncthreads();
-        if (sub == 0 && m < M && grp < out_groups && !*abort_flag) {
+        if (sub == 0 && m < M && live && !*abort_flag) {
 #pragma unroll
-            for (int t = 0; t < G; ++t) {
+            for (int t = 0; t < GE; ++t) {
                 float s = acc[m][t];
 #pragma unroll
-                for (int q = 0; q < LG_SUB - 1; ++q) s += red[(q * G + t) * LG_GRPS + gl];
-                const int o = grp * G + t;
+                for (int q = 0; q < LG_SUB - 1; ++q) s += red[(q * GE + t) * LG_GRPS + gl];
+                const int o = grp * GE + t;
                 if (o < d_out) dst[(int64_t)m * d_out + o] = (direct && bias) ? s + __ldg(bias + o) : s;
             }
         }
@@ -511,33 +585,34 @@ linear_gemv_q4_kernel(const uint16_t* __restrict__ x, int M, const unsigned char
         const long long t0 = clock64();                                          // let the table's copies land (bounded)
         while (!mbar_try(smem_u32(qbar), 0) && clock64() - t0 < WAIT_LIMIT) {}
     }
-    // ---- the CTA that finishes last among the slices of this block of code groups adds the slabs, in slice
+    // ---- the CTA that finishes last among those of this block of code groups adds the slabs, in slab
     // order (the same bits whichever CTA that is), and the bias; it leaves the counter at zero for the next call.
     // Every CTA counts itself, also one that gave up, so that the counter always returns to zero.
     if (arrived) {
         __shared__ int last;
         __threadfence();                                                         // this thread's slab stores before the count
         __syncthreads();
-        if (tid == 0) last = atomicAdd(arrived + blockIdx.x, 1u) == gridDim.y - 1;
+        const unsigned slabs = gridDim.y * gridDim.z;
+        if (tid == 0) last = atomicAdd(arrived + blockIdx.x, 1u) == slabs - 1;
         __syncthreads();
         if (last) {
             __threadfence();
-            const int o_lo = blockIdx.x * LG_GRPS * G;
+            const int o_lo = blockIdx.x * LG_GRPS * GE;
             int width = d_out - o_lo;
-            width = width < LG_GRPS * G ? width : LG_GRPS * G;
+            width = width < LG_GRPS * GE ? width : LG_GRPS * GE;
             for (int e = tid; e < M * width; e += LG_THREADS) {
                 const int m = e / width, o = o_lo + (e - m * width);
                 const float* src = out + (int64_t)m * d_out + o;
                 float sum = bias ? __ldg(bias + o) : 0.f;
                 unsigned k = 0;
-                for (; k + 8 <= gridDim.y; k += 8) {                             // eight loads in flight, added in slice order
+                for (; k + 8 <= slabs; k += 8) {                             // eight loads in flight, added in slab order
                     float v[8];
 #pragma unroll
                     for (int u = 0; u < 8; ++u) v[u] = __ldcg(src + (int64_t)(k + u) * split_stride);
 #pragma unroll
                     for (int u = 0; u < 8; ++u) sum += v[u];
                 }
-                for (; k < gridDim.y; ++k) sum += __ldcg(src + (int64_t)k * split_stride);
+                for (; k < slabs; ++k) sum += __ldcg(src + (int64_t)k * split_stride);
                 y[(int64_t)m * d_out + o] = sum;
             }
             if (tid == 0) arrived[blockIdx.x] = 0u;
@@ -564,26 +639,38 @@ linear_pad_rows_kernel(const uint16_t* __restrict__ C16, int K, int g, int pad, 
 // (33 tokens, g = 6, K = 1024: 512 x 512 17.4 us without, 21.5 with it).
 constexpr int64_t LINEAR_PAD_FROM = 400000;
 
-struct GemvPlan { int o_blocks, splits, rows_per_split; };
+struct GemvPlan { int pw, o_blocks, slices, slice_rows, splits, rows_per_split; size_t smem; };
 
-GemvPlan gemv_plan(int64_t d_in, int out_groups, int sm_count) {
+// Slices of the codebook as its bytes ask for, splits of the in_features by a count of clocks: a CTA pays for its
+// table (about 40 bytes a clock), some 4000 for its beginning and end, and 10 a row of codes; CTAs come in waves of one per SM.
+GemvPlan gemv_plan(int64_t d_in, int out_groups, int sm_count, int K, int g, int mt, bool quant, bool words) {
     GemvPlan p;
-    p.o_blocks = (out_groups + LG_GRPS - 1) / LG_GRPS;
-    int splits = sm_count / p.o_blocks;                                          // one CTA per SM where the shape allows
-    if (splits < 1) splits = 1;
-    if ((int64_t)splits * 16 > d_in) splits = (int)((d_in + 15) / 16);           // at least 16 in_features per CTA
-    int64_t rows = (d_in + splits - 1) / splits;
-    if (rows > LG_ROWS_MAX) rows = LG_ROWS_MAX;
-    p.rows_per_split = (int)rows;
-    p.splits = (int)((d_in + rows - 1) / rows);
-    return p;
-}
-
-size_t gemv_smem(int g, int K, int rows, int mt) {
-    size_t tail = (size_t)K * (g / 2);
-    const size_t red = (size_t)(LG_SUB - 1) * g * LG_GRPS * 4;
+    p.pw = (words && out_groups % 2 == 0 && gemv_pair(g, quant) && out_groups * d_in >= LG_PAIR_FROM) ? 2 : 1;
+    p.o_blocks = (out_groups / p.pw + LG_GRPS - 1) / LG_GRPS;
+    const size_t row = quant ? (size_t)(g / 2) : (size_t)(2 * g);
+    p.slices = (int)(((size_t)K * row + LG_SLICE - 1) / LG_SLICE);
+    p.slice_rows = (K + p.slices - 1) / p.slices;
+    p.slice_rows = (p.slice_rows + 15) / 16 * 16;
+    p.slices = (K + p.slice_rows - 1) / p.slice_rows;
+    const int step = gemv_batch(g, mt) * LG_SUB, rows_max = LG_X_MAX / (4 * mt) / step * step;
+    const int ctas = p.o_blocks * p.slices;
+    int most = 3 * sm_count / ctas, least = (int)((d_in + rows_max - 1) / rows_max);
+    if ((int64_t)most * LG_SUB > d_in) most = (int)((d_in + LG_SUB - 1) / LG_SUB);   // at least 16 in_features per CTA
+    if (most < least) most = least;
+    double best = 0.0;
+    p.splits = 0;
+    for (int s = least; s <= most; ++s) {
+        const int64_t rows = (d_in + s - 1) / s;
+        const double t = (double)((ctas * s + sm_count - 1) / sm_count) * ((double)(p.slice_rows * row) / 40.0 + 4000.0 + 8.0 * p.pw * (double)rows);
+        if (p.splits == 0 || t < best) { best = t; p.splits = s; }
+    }
+    p.rows_per_split = (int)((d_in + p.splits - 1) / p.splits);
+    p.splits = (int)((d_in + p.rows_per_split - 1) / p.rows_per_split);
+    size_t tail = (size_t)p.slice_rows * row + (quant ? 0 : row + 4);
+    const size_t red = (size_t)(LG_SUB - 1) * g * p.pw * LG_GRPS * 4;
     if (tail < red) tail = red;
-    return 128 + ((size_t)rows * mt * 4 + 15) / 16 * 16 + (tail + 15) / 16 * 16;
+    p.smem = 128 + (size_t)((p.rows_per_split + step - 1) / step * step) * mt * 4 + (tail + 15) / 16 * 16;
+    return p;
 }
 
 // Tokens from which decoding the weight once and multiplying it afterwards (cc_linear_wide.cu) is the faster way
@@ -648,10 +735,12 @@ size_t cc_linear_scratch_bytes(int64_t M, int64_t d_out, int64_t d_in, int sm_co
     if (splits > chunks / 4) splits = chunks / 4;
     if (splits < 2) splits = 0;    // a single CTA per tile writes y itself
     if (M <= LG_M_MAX) {
-        // the few-token kernel of the quantised codebook always goes through its slabs; the most slices come
-        // with the fewest blocks of code groups, i.e. at g = 16
-        const GemvPlan v = gemv_plan(d_in, (int)((d_out + 15) / 16), sm_count);
-        if (v.splits > splits) splits = v.splits;
+        // the few-token kernel: three CTAs per SM at the most, or as many splits as x asks for (see gemv_plan); the most
+        // slabs come with the fewest blocks of code groups, i.e. at g = 16
+        const int o_blocks = (int)((d_out / 32 + LG_GRPS - 1) / LG_GRPS);
+        const int64_t least = LG_SLICES_MAX * ((d_in + 511) / 512);
+        const int64_t most = 3 * sm_count / (o_blocks < 1 ? 1 : o_blocks) + LG_SLICES_MAX;
+        if (splits < (most > least ? most : least)) splits = (int)(most > least ? most : least);
     }
     const size_t own = CC_LINEAR_SCRATCH_FROM + (size_t)splits * (size_t)M * (size_t)d_out * 4;
     const size_t wide = M >= LINEAR_WIDE_FEWEST ? cc_linear_wide_bytes(M, d_out, d_in) : 0;
@@ -720,41 +809,56 @@ cudaError_t launch_linear(cc_ctx* ctx, const LinearPlan& p, const uint16_t* x, i
 
 namespace {
 
-template <int G, int MT>
-cudaError_t launch_gemv(cc_ctx* ctx, const GemvPlan& p, const uint16_t* x, int M, const unsigned char* qtab,
+// Where the look-up kernel is the faster one.  M x g accumulators must fit the registers of 1024 threads per SM; the
+// FP16 codebook is read once per slice, which costs the less the fewer gathers it saves (4096 x 4096: g = 4, K = 65536
+// 26.9 -> 17.2 us at one token, 26.7 -> 25.7 at four; g = 6, K = 65500, four slices 30.8 -> 22.2 at one, on 11008 x 4096
+// 98 -> 94 at four, where the tensor kernel with padded rows takes 70; g = 16, K = 20000, three slices, two tokens 20.2
+// -> 24.4, not used).
+constexpr int gemv_tokens(int g) { return g <= 8 ? 4 : 2; }                  // 4-bit codebook
+bool gemv_fp16(int64_t M, int K, int g) {
+    return M <= (g <= 4 ? 4 : 2) && (size_t)K * (2 * g) <= (size_t)(g <= 8 ? 4 : 2) * LG_SLICE;
+}
+constexpr int gemv_pad(int64_t M) { return M <= 2 ? (int)M : 4; }
+
+template <int G, int MT, bool QUANT, int PW>
+cudaError_t launch_gemv_w(cc_ctx* ctx, const GemvPlan& p, const uint16_t* x, int M, const void* book,
                         const float* qscale, int K, const uint16_t* idx, int d_out, int d_in, int out_groups, float* out,
                         int64_t split_stride, unsigned* status, unsigned* arrived, const float* bias, float* y,
                         cudaStream_t st) {
     static bool attr_dev[64] = {};
     bool& have = attr_dev[ctx->device & 63];
     if (!have) {
-        const cudaError_t e = cudaFuncSetAttribute(linear_gemv_q4_kernel<G, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)gemv_smem(G, LQ_TABLE_MAX / (G / 2), LG_ROWS_MAX, MT));
+        const cudaError_t e = cudaFuncSetAttribute(linear_gemv_kernel<G, MT, QUANT, PW>, cudaFuncAttributeMaxDynamicSharedMemorySize, LG_SMEM);
         if (e != cudaSuccess) return e;
         have = true;
     }
-    const dim3 grid(p.o_blocks, p.splits);
-    linear_gemv_q4_kernel<G, MT><<<grid, LG_THREADS, gemv_smem(G, K, p.rows_per_split, MT), st>>>(
-        x, M, qtab, qscale, K, idx, d_out, d_in, out_groups, p.rows_per_split, out, split_stride, status, arrived, bias, y, p.splits == 1);
+    const dim3 grid(p.o_blocks, p.splits, p.slices);
+    linear_gemv_kernel<G, MT, QUANT, PW><<<grid, LG_THREADS, p.smem, st>>>(
+        x, M, static_cast<const unsigned char*>(book), qscale, K, p.slice_rows, idx, d_out, d_in, out_groups, p.rows_per_split, out,
+        split_stride, status, arrived, bias, y, p.splits * p.slices == 1);
     return cudaGetLastError();
 }
 
-// Tokens padded to 1, 2 or 4 (from 8 on the tensor kernel is as fast); M x g accumulators must fit the
-// registers of 1024 threads per SM.
-constexpr int gemv_tokens(int g) { return g <= 8 ? 4 : 2; }
+template <int G, int MT, bool QUANT>
+cudaError_t launch_gemv(cc_ctx* ctx, const GemvPlan& p, const uint16_t* x, int M, const void* book,
+                        const float* qscale, int K, const uint16_t* idx, int d_out, int d_in, int out_groups, float* out,
+                        int64_t split_stride, unsigned* status, unsigned* arrived, const float* bias, float* y,
+                        cudaStream_t st) {
+    if constexpr (gemv_pair(G, QUANT)) {
+        if (p.pw == 2) return launch_gemv_w<G, MT, QUANT, 2>(ctx, p, x, M, book, qscale, K, idx, d_out, d_in, out_groups, out, split_stride, status, arrived, bias, y, st);
+    }
+    return launch_gemv_w<G, MT, QUANT, 1>(ctx, p, x, M, book, qscale, K, idx, d_out, d_in, out_groups, out, split_stride, status, arrived, bias, y, st);
+}
 
-template <int G>
-cudaError_t launch_gemv_m(cc_ctx* ctx, const GemvPlan& p, const uint16_t* x, int M, const unsigned char* qtab,
+template <int G, bool QUANT>
+cudaError_t launch_gemv_m(cc_ctx* ctx, const GemvPlan& p, const uint16_t* x, int M, const void* book,
                           const float* qscale, int K, const uint16_t* idx, int d_out, int d_in, int out_groups, float* out,
                           int64_t split_stride, unsigned* status, unsigned* arrived, const float* bias, float* y,
                           cudaStream_t st) {
-    if (M == 1) return launch_gemv<G, 1>(ctx, p, x, M, qtab, qscale, K, idx, d_out, d_in, out_groups, out, split_stride, status, arrived, bias, y, st);
-    if (M == 2) return launch_gemv<G, 2>(ctx, p, x, M, qtab, qscale, K, idx, d_out, d_in, out_groups, out, split_stride, status, arrived, bias, y, st);
+    if (M == 1) return launch_gemv<G, 1, QUANT>(ctx, p, x, M, book, qscale, K, idx, d_out, d_in, out_groups, out, split_stride, status, arrived, bias, y, st);
+    if (M == 2) return launch_gemv<G, 2, QUANT>(ctx, p, x, M, book, qscale, K, idx, d_out, d_in, out_groups, out, split_stride, status, arrived, bias, y, st);
     if constexpr (gemv_tokens(G) >= 4) {
-        if (M <= 4) return launch_gemv<G, 4>(ctx, p, x, M, qtab, qscale, K, idx, d_out, d_in, out_groups, out, split_stride, status, arrived, bias, y, st);
-    }
-    if constexpr (gemv_tokens(G) >= 8) {
-        if (M <= 8) return launch_gemv<G, 8>(ctx, p, x, M, qtab, qscale, K, idx, d_out, d_in, out_groups, out, split_stride, status, arrived, bias, y, st);
+        if (M <= 4) return launch_gemv<G, 4, QUANT>(ctx, p, x, M, book, qscale, K, idx, d_out, d_in, out_groups, out, split_stride, status, arrived, bias, y, st);
     }
     return cudaErrorInvalidValue;
 }
@@ -765,6 +869,46 @@ cudaError_t launch_gemv_m(cc_ctx* ctx, const GemvPlan& p, const uint16_t* x, int
 cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, const uint16_t* C16,
                                      const unsigned char* qtab, const float* qscale, int K, int g, const uint16_t* idx,
                                      int64_t d_out, int64_t d_in, const float* bias, float* y, cudaStream_t st) {
+    char* ws = static_cast<char*>(ctx->ws);
+    unsigned* status = reinterpret_cast<unsigned*>(ws);
+    float* partial = reinterpret_cast<float*>(ws + CC_LINEAR_SCRATCH_FROM);
+    const int out_groups = (int)((d_out + g - 1) / g);
+    const int64_t n = M * d_out;
+    cudaError_t e = cudaSuccess;
+    if (qtab ? M <= gemv_tokens(g) : gemv_fp16(M, K, g)) {
+        // a handful of tokens: the shared-memory look-up kernel, then the same reduction (it also adds the bias)
+        const GemvPlan v = gemv_plan(d_in, out_groups, ctx->sm_count, K, g, gemv_pad(M), qtab != nullptr, (reinterpret_cast<uintptr_t>(idx) & 3u) == 0);
+        const int slabs_n = v.splits * v.slices;
+        unsigned* arrived = nullptr;
+        {
+            ProfScope ps(ctx, CC_K_LINEAR, st);
+            // counters of the finished slabs: the words of the status block kept for this (zero since
+            // cc_set_workspace, put back to zero by the kernel); with more blocks than counters the reduction
+            // is a kernel of its own
+            arrived = (slabs_n > 1 && v.o_blocks <= CC_ARRIVAL_COUNTERS) ? status + CC_ARRIVAL_WORD : nullptr;
+            float* slabs = slabs_n == 1 ? y : partial;           // a single slab is y (with the bias) itself
+            if (qtab) {
+#define CALL(G) e = launch_gemv_m<G, true>(ctx, v, x, (int)M, qtab, qscale, K, idx, (int)d_out, (int)d_in, out_groups, slabs, n, status, arrived, bias, y, st)
+                switch (g) {
+                    case 2: CALL(2); break;   case 4: CALL(4); break;   case 6: CALL(6); break;   case 8: CALL(8); break;
+                    case 10: CALL(10); break; case 12: CALL(12); break; case 14: CALL(14); break; case 16: CALL(16); break;
+                    default: return cudaErrorInvalidValue;
+                }
+#undef CALL
+            } else {
+#define CALL(G) e = launch_gemv_m<G, false>(ctx, v, x, (int)M, C16, nullptr, K, idx, (int)d_out, (int)d_in, out_groups, slabs, n, status, arrived, bias, y, st)
+                CC_LINEAR_DISPATCH(g, CALL)
+#undef CALL
+            }
+        }
+        if (e != cudaSuccess || arrived || slabs_n == 1) return e;
+        ProfScope ps(ctx, CC_K_LINEAR_REDUCE, st);
+        int64_t blocks = (n + 255) / 256;
+        const int64_t cap = (int64_t)ctx->sm_count * 8;
+        if (blocks > cap) blocks = cap;
+        linear_reduce_kernel<<<(unsigned)blocks, 256, 0, st>>>(partial, slabs_n, n, (int)d_out, bias, y);
+        return cudaGetLastError();
+    }
     // beside the table: token blocks of 64 with four stages, or, from LQ_WIDE_FROM tokens on, of 256 with two
     const LinearPlan p = qtab ? linear_plan(M, d_out, d_in, ctx->sm_count, M >= LQ_WIDE_FROM ? LNT_MAX : LQ_NT_MAX, (size_t)K * (g / 2), g)
                               : linear_plan(M, d_out, d_in, ctx->sm_count, LNT_MAX, 0, g);
@@ -772,7 +916,7 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
     // the codebook's own rows take one load (the widest wants them on 32-byte boundaries)
     bool padded = row_pad(g) == g && (g < 16 || (reinterpret_cast<uintptr_t>(C16) & 31u) == 0);
     if (!qtab && !padded && codes >= LINEAR_PAD_FROM && codes >= 4 * (int64_t)K) {
-        uint16_t* table = reinterpret_cast<uint16_t*>(static_cast<char*>(ctx->ws) + CC_STATUS_BYTES);
+        uint16_t* table = reinterpret_cast<uint16_t*>(ws + CC_STATUS_BYTES);
         ProfScope ps(ctx, CC_K_OTHER, st);
         linear_pad_rows_kernel<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(C16, K, g, row_pad(g), table);
         C16 = table;
@@ -780,39 +924,6 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
     }
     if (M >= (p.fill == 1 ? LINEAR_WIDE_FEWEST : LINEAR_WIDE_FROM) && cc_linear_wide_applies(M, d_out, d_in, p.fill, ctx->sm_count))
         return cc_launch_linear_wide(ctx, x, M, C16, padded, qtab, qscale, K, g, idx, d_out, d_in, bias, y, p.fill, st);
-    char* ws = static_cast<char*>(ctx->ws);
-    unsigned* status = reinterpret_cast<unsigned*>(ws);
-    float* partial = reinterpret_cast<float*>(ws + CC_LINEAR_SCRATCH_FROM);
-    const int out_groups = (int)((d_out + g - 1) / g);
-    const int64_t n = M * d_out;
-    cudaError_t e = cudaSuccess;
-    if (qtab && M <= gemv_tokens(g)) {
-        // a handful of tokens: the shared-memory look-up kernel, then the same reduction (it also adds the bias)
-        const GemvPlan v = gemv_plan(d_in, out_groups, ctx->sm_count);
-        unsigned* arrived = nullptr;
-        {
-            ProfScope ps(ctx, CC_K_LINEAR, st);
-            // counters of the finished slices: the words of the status block kept for this (zero since
-            // cc_set_workspace, put back to zero by the kernel); with more blocks than counters the reduction
-            // is a kernel of its own
-            arrived = (v.splits > 1 && v.o_blocks <= CC_ARRIVAL_COUNTERS) ? status + CC_ARRIVAL_WORD : nullptr;
-            float* slabs = v.splits == 1 ? y : partial;          // a single slice writes y (and the bias) itself
-#define CALL(G) e = launch_gemv_m<G>(ctx, v, x, (int)M, qtab, qscale, K, idx, (int)d_out, (int)d_in, out_groups, slabs, n, status, arrived, bias, y, st)
-            switch (g) {
-                case 2: CALL(2); break;   case 4: CALL(4); break;   case 6: CALL(6); break;   case 8: CALL(8); break;
-                case 10: CALL(10); break; case 12: CALL(12); break; case 14: CALL(14); break; case 16: CALL(16); break;
-                default: return cudaErrorInvalidValue;
-            }
-#undef CALL
-        }
-        if (e != cudaSuccess || arrived || v.splits == 1) return e;
-        ProfScope ps(ctx, CC_K_LINEAR_REDUCE, st);
-        int64_t blocks = (n + 255) / 256;
-        const int64_t cap = (int64_t)ctx->sm_count * 8;
-        if (blocks > cap) blocks = cap;
-        linear_reduce_kernel<<<(unsigned)blocks, 256, 0, st>>>(partial, v.splits, n, (int)d_out, bias, y);
-        return cudaGetLastError();
-    }
     bool fused = false;
     {
         ProfScope ps(ctx, CC_K_LINEAR, st);
