@@ -121,7 +121,7 @@ decode_transpose_vec_kernel(const uint16_t* __restrict__ C16, const uint16_t* __
     }
 }
 
-// PAPER_T decode of large matrices for g = 8 and 16: persistent CTAs walk over the tiles with the loads of the
+// PAPER_T decode of middling to large matrices for g = 8 and 16: persistent CTAs walk over the tiles with the loads of the
 // next tiles already in flight (the codes of tile k+2 and the codebook rows of tile k+1 are
 // requested before tile k goes through shared memory), because a tile's chain DRAM (codes) ->
 // gather -> transpose -> store is otherwise paid once per tile and four to eight resident CTAs do
@@ -282,6 +282,155 @@ cudaError_t launch_decode_pipe(int sm_count, const uint16_t* C16, const uint16_t
     return cudaGetLastError();
 }
 
+// PAPER_T decode of large matrices, g = 4 or 8, with the head of the codebook (all of it up to 190 KB) in shared memory.
+// What bounds a decode with a large codebook is the number of L2 sectors an SM can ask for (0.73 a clock), one for
+// each row that is not on the SM.  L1 keeps lines of four sectors of which a gather fills one, so it holds few rows:
+// 6 % hits at K = 65536, g = 4, where the same memory as a plain table holds 37 % of the rows.
+// Shared memory is taken from L1, and a gather under way needs a line there: with all of it taken, 160 lines or so
+// are left and the gathers from L2 wait for those (K = 65536: 338 us with 37 % of the rows on the SM, 281 without any,
+// 245 with 28 %).  So a codebook that does not fit keeps to the step of the carve-out below the last.
+// 8192 x 28672, g = 4, uniform codes: K = 65536 281 -> 245 us (262 -> 199 where codes of the head are the popular ones),
+// K = 30000 258 -> 178, K = 4096 156 -> 141; 11008 x 4096, g = 8: K = 20000 43 -> 39, K = 4096 35 -> 33, K = 65536
+// (14 % of the rows) 45 -> 45; g = 16: K = 65536 47 -> 52, K = 3000 43 -> 44, not used.
+// One CTA per SM, four groups of 256 threads, each with a tile and a barrier of its own; the codes of tile k + 2 and
+// the rows of tile k + 1 are under way while tile k is transposed and stored.
+constexpr int RES_GROUPS = 4, RES_THREADS = RES_GROUPS * 256;
+constexpr int RES_TILES = 24;                        // tiles per CTA from which filling the table is paid for
+constexpr int RES_SMEM = 226 * 1024, RES_TABLE = RES_SMEM - RES_GROUPS * kTileBytes;
+constexpr int RES_SMEM_PART = 194 * 1024, RES_TABLE_PART = RES_SMEM_PART - RES_GROUPS * kTileBytes;
+
+// Rows in shared memory, in whole 16-byte pieces (an even number at g = 4).
+int res_head(int K, int g) {
+    const int64_t all = (int64_t)K * g * 2;
+    if (all <= RES_TABLE) return g == 4 ? K / 2 * 2 : K;
+    const int most = RES_TABLE / (2 * g), part = RES_TABLE_PART / (2 * g);
+    return (4 * (int64_t)most >= 3 * (int64_t)K ? most : part) / 2 * 2;
+}
+
+bool res_applies(int K, int g) { return g == 4 || (g == 8 && 3 * (int64_t)res_head(K, g) >= K); }
+
+struct ResCodes { unsigned w[2]; unsigned live; };   // rows r0 and r0 + 32 of the tile; G = 4: two codes in a word
+
+template <int G>
+__device__ __forceinline__ void res_load_codes(const uint16_t* __restrict__ idx, DecodeTile p, int tiles_y, int r0, int c,
+                                               int64_t d_in, int64_t out_pad, int64_t opg, ResCodes& s) {
+    s.live = 0u;
+    if (p.by >= tiles_y) return;
+    const int64_t o = (int64_t)p.by * TD + 8 * c;
+    if (o >= out_pad) return;
+    const int64_t i = (int64_t)p.bx * TD + r0;
+    const uint16_t* src = idx + i * opg + (o / G);
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+        if (i + 32 * q < d_in) {
+            s.live |= 1u << q;
+            if constexpr (G == 4) s.w[q] = __ldg(reinterpret_cast<const unsigned*>(src + 32 * q * opg));
+            else s.w[q] = __ldg(src + 32 * q * opg);
+        }
+}
+
+// Row of a code: from the table where it lies below `head`, else from global memory.
+template <int BYTES>
+__device__ __forceinline__ void res_fetch(uint32_t table, const unsigned char* __restrict__ book, unsigned offset, unsigned head, uint32_t* v) {
+    if constexpr (BYTES == 8)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %4, %5;\n\t"
+                     "@p ld.shared.v2.b32 {%0, %1}, [%2];\n\t@!p ld.global.nc.v2.b32 {%0, %1}, [%3];\n\t}"
+                     : "=r"(v[0]), "=r"(v[1]) : "r"(table + offset), "l"(book + offset), "r"(offset), "r"(head));
+    else
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %6, %7;\n\t"
+                     "@p ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];\n\t@!p ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%5];\n\t}"
+                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(table + offset), "l"(book + offset), "r"(offset), "r"(head));
+}
+
+template <int G>
+__device__ __forceinline__ void res_gather(uint32_t table, const unsigned char* __restrict__ book, unsigned head, unsigned kmax,
+                                           const ResCodes& s, uint4 (&v)[2]) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        v[q] = make_uint4(0u, 0u, 0u, 0u);
+        if (!(s.live >> q & 1u)) continue;
+        // a code beyond the codebook must not leave it
+        if constexpr (G == 4) {
+            res_fetch<8>(table, book, min(s.w[q] & 0xffffu, kmax) * 8u, head, &v[q].x);
+            res_fetch<8>(table, book, min(s.w[q] >> 16, kmax) * 8u, head, &v[q].z);
+        } else {
+            res_fetch<16>(table, book, min(s.w[q], kmax) * 16u, head, &v[q].x);
+        }
+    }
+}
+
+template <int G>
+__global__ void __launch_bounds__(RES_THREADS, 1)
+decode_transpose_resident_kernel(const uint16_t* __restrict__ C16, const uint16_t* __restrict__ idx, int K, int head_rows,
+                                 int64_t d_out, int64_t d_in, int64_t out_pad, uint16_t* __restrict__ W_hat, int tiles_x, int tiles_y) {
+    extern __shared__ __align__(16) unsigned char decode_smem[];
+    const int group = threadIdx.x >> 8, tid = threadIdx.x & 255;
+    unsigned* tile = reinterpret_cast<unsigned*>(decode_smem + group * kTileBytes);
+    unsigned char* table = decode_smem + RES_GROUPS * kTileBytes;
+    const unsigned char* book = reinterpret_cast<const unsigned char*>(C16);
+    const unsigned head = (unsigned)head_rows * (2u * G), kmax = (unsigned)K - 1u;
+    const int c = tid & 7, r0 = tid >> 3;
+    const int64_t opg = out_pad / G;
+    const unsigned step = gridDim.x * RES_GROUPS, first = blockIdx.x * RES_GROUPS + group;
+    const int step_x = (int)(step % (unsigned)tiles_x), step_y = (int)(step / (unsigned)tiles_x);
+    DecodeTile t0 = {(int)(first % (unsigned)tiles_x), (int)(first / (unsigned)tiles_x)};
+    auto next = [&](DecodeTile p) { decode_next_tile(p, step_x, step_y, tiles_x); return p; };
+    auto emit = [&](DecodeTile p, const uint4 (&v)[2]) {
+        tile_put8(tile, r0, c, v[0]);
+        tile_put8(tile, r0 + 32, c, v[1]);
+        asm volatile("bar.sync %0, 256;" ::"r"(group + 1) : "memory");
+        uint4 even, odd;
+        tile_column8x2(tile, c, r0, even, odd);
+        const int64_t o = (int64_t)p.by * TD + 2 * r0, i = (int64_t)p.bx * TD + 8 * c;
+        if (i < d_in) {
+            uint16_t* dst = W_hat + o * d_in + i;
+            if (o < d_out) __stcs(reinterpret_cast<uint4*>(dst), even);
+            if (o + 1 < d_out) __stcs(reinterpret_cast<uint4*>(dst + d_in), odd);
+        }
+        asm volatile("bar.sync %0, 256;" ::"r"(group + 1) : "memory");   // the tile is free again
+    };
+    ResCodes sA, sB;
+    uint4 vA[2], vB[2];
+    DecodeTile t1 = next(t0);
+    res_load_codes<G>(idx, t0, tiles_y, r0, c, d_in, out_pad, opg, sA);
+    res_load_codes<G>(idx, t1, tiles_y, r0, c, d_in, out_pad, opg, sB);
+    for (unsigned v = threadIdx.x * 16; v < head; v += RES_THREADS * 16)
+        *reinterpret_cast<uint4*>(table + v) = __ldg(reinterpret_cast<const uint4*>(book + v));
+    __syncthreads();
+    const uint32_t tab = (uint32_t)__cvta_generic_to_shared(table);
+    res_gather<G>(tab, book, head, kmax, sA, vA);
+    // unrolled by two so that the register sets keep their roles: a register that waits for a load is never copied
+    while (t0.by < tiles_y) {
+        DecodeTile t2 = next(t1);
+        res_gather<G>(tab, book, head, kmax, sB, vB);                  // tile t1 (nothing live past the last one)
+        res_load_codes<G>(idx, t2, tiles_y, r0, c, d_in, out_pad, opg, sA);
+        emit(t0, vA);
+        if (t1.by >= tiles_y) break;
+        t0 = t2;
+        t2 = next(t2);
+        res_gather<G>(tab, book, head, kmax, sA, vA);
+        res_load_codes<G>(idx, t2, tiles_y, r0, c, d_in, out_pad, opg, sB);
+        emit(t1, vB);
+        t1 = t2;
+    }
+}
+
+template <int G>
+cudaError_t launch_decode_resident(cc_ctx* ctx, const uint16_t* C16, const uint16_t* idx, int K, int64_t d_out, int64_t d_in,
+                                   int64_t out_pad, uint16_t* W_hat, int tiles_x, int tiles_y, cudaStream_t st) {
+    static bool attr_dev[64] = {};
+    bool& have = attr_dev[ctx->device & 63];
+    if (!have) {
+        const cudaError_t e = cudaFuncSetAttribute(decode_transpose_resident_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM);
+        if (e != cudaSuccess) return e;
+        have = true;
+    }
+    const int head = res_head(K, G);
+    decode_transpose_resident_kernel<G><<<(unsigned)ctx->sm_count, RES_THREADS, RES_GROUPS * kTileBytes + head * 2 * G, st>>>(
+        C16, idx, K, head, d_out, d_in, out_pad, W_hat, tiles_x, tiles_y);
+    return cudaGetLastError();
+}
+
 // ROWS reshape: copy each row, padding it to in_pad elements.
 __global__ void __launch_bounds__(256)
 reshape_rows_kernel(const uint16_t* __restrict__ W, int64_t d_out, int64_t d_in, int64_t in_pad,
@@ -385,7 +534,11 @@ cudaError_t cc_launch_decode(cc_ctx* ctx, const uint16_t* C16, int K, int g, con
         // Enough tiles for persistent CTAs with loads in flight across tiles, and a codebook that
         // stays in L1: there the chain of latencies bounds a tile.  A larger codebook is bound by the
         // L2 sectors its gathers move, and more resident threads (the kernel below) serve it better.
-        // With g = 4 (8-byte rows, two gathers per 16 output bytes) the plain kernel measured faster.
+        // Many tiles: the codebook's head in shared memory (see the kernel above).
+        if (vec && n_tiles >= (int64_t)ctx->sm_count * RES_TILES && res_applies(K, g)) {
+            if (g == 4) return launch_decode_resident<4>(ctx, C16, idx, K, d_out, d_in, out_pad, W_hat, (int)grid.x, (int)grid.y, st);
+            return launch_decode_resident<8>(ctx, C16, idx, K, d_out, d_in, out_pad, W_hat, (int)grid.x, (int)grid.y, st);
+        }
         if (vec && (g == 8 || g == 16) && n_tiles >= (int64_t)ctx->sm_count * 8 &&
             (int64_t)K * g * 2 <= kPipeMaxTableBytes) {
             if (g == 8) return launch_decode_pipe<8>(ctx->sm_count, C16, idx, K, d_out, d_in, out_pad, W_hat, (int)grid.x, (int)grid.y, st);
