@@ -1,8 +1,8 @@
 // C ABI of the library: host-side validation, workspace carving, the Lloyd loop.
 // Every step of the path runs in the kernels of the other translation units; nothing here
 // computes on the host except the seeded choice of the K initial positions.
+#include <cstring>
 #include <new>
-#include <unordered_map>
 #include <vector>
 
 #include "cc_common.cuh"
@@ -77,6 +77,10 @@ cc_status check_common(const cc_ctx* ctx, int64_t N, int g, int K, bool need_ws)
     return CC_OK;
 }
 
+inline cc_status status_of(unsigned word) {
+    return word & CC_DEV_TIMEOUT ? CC_ERR_DEVICE_TIMEOUT : word & CC_DEV_NONFINITE ? CC_ERR_NONFINITE : CC_OK;
+}
+
 inline cc_status from_cuda(cudaError_t e) { return e == cudaSuccess ? CC_OK : CC_ERR_CUDA; }
 
 inline uint64_t splitmix64(uint64_t& s) {
@@ -84,6 +88,43 @@ inline uint64_t splitmix64(uint64_t& s) {
     z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
     return z ^ (z >> 31);
+}
+
+// Contents of the entries of an array 0, 1, 2, ... that a shuffle has touched: open addressing, at most half full.
+// (std::unordered_map took 16 ms for 65500 positions, this 3.)
+struct Touched {
+    std::vector<uint32_t> key, val;       // key + 1; 0: free
+    uint32_t mask;
+    explicit Touched(int64_t entries) {
+        uint32_t cap = 16;
+        while ((int64_t)cap < 4 * entries) cap *= 2;              // two touched entries a step
+        key.assign(cap, 0u);
+        val.resize(cap);
+        mask = cap - 1;
+    }
+    // The entry at position i, made (with its original content) if it is not there yet.
+    uint32_t& at(uint32_t i) {
+        uint32_t h = (i * 2654435769u) & mask;
+        while (key[h] != 0u && key[h] != i + 1u) h = (h + 1) & mask;
+        if (key[h] == 0u) { key[h] = i + 1u; val[h] = i; }
+        return val[h];
+    }
+};
+
+// Only the n touched entries of the shuffled array are kept.
+template <typename T>
+void sparse_shuffle(int64_t N, int64_t n, uint64_t seed, T* pos) {
+    Touched moved(n);
+    uint64_t s = seed;
+    for (int64_t i = 0; i < n; ++i) {
+        const int64_t j = i + (int64_t)(splitmix64(s) % (uint64_t)(N - i));
+        uint32_t& vi = moved.at((uint32_t)i);
+        uint32_t& vj = moved.at((uint32_t)j);
+        const uint32_t t = vj;
+        vj = vi;
+        vi = t;
+        pos[i] = (T)t;
+    }
 }
 
 // The same shuffle for any number n <= N of positions, written to 32-bit words: with many positions
@@ -103,36 +144,8 @@ bool partial_shuffle_u32(int64_t N, int64_t n, uint64_t seed, uint32_t* pos) {
         }
         return true;
     }
-    std::unordered_map<int64_t, int64_t> moved;
-    moved.reserve((size_t)n * 2);
-    for (int64_t i = 0; i < n; ++i) {
-        const int64_t j = i + (int64_t)(splitmix64(s) % (uint64_t)(N - i));
-        auto itj = moved.find(j);
-        const int64_t vj = (itj == moved.end()) ? j : itj->second;
-        auto iti = moved.find(i);
-        const int64_t vi = (iti == moved.end()) ? i : iti->second;
-        moved[j] = vi;
-        moved[i] = vj;
-        pos[i] = (uint32_t)vj;
-    }
+    try { sparse_shuffle(N, n, seed, pos); } catch (...) { return false; }
     return true;
-}
-
-// Only the K touched entries of the shuffled array are kept (a map from position to content).
-void partial_shuffle(int64_t N, int K, uint64_t seed, int64_t* pos) {
-    std::unordered_map<int64_t, int64_t> moved;
-    moved.reserve((size_t)K * 2);
-    uint64_t s = seed;
-    for (int64_t i = 0; i < K; ++i) {
-        const int64_t j = i + (int64_t)(splitmix64(s) % (uint64_t)(N - i));
-        auto itj = moved.find(j);
-        const int64_t vj = (itj == moved.end()) ? j : itj->second;
-        auto iti = moved.find(i);
-        const int64_t vi = (iti == moved.end()) ? i : iti->second;
-        moved[j] = vi;
-        moved[i] = vj;
-        pos[i] = vj;
-    }
 }
 
 bool use_tensor_path(const cc_ctx* ctx, int g, int K) {
@@ -190,6 +203,8 @@ bool use_pruned(const cc_ctx* ctx, int64_t N, int g, int K, int e_steps) {
 
 cudaError_t assign_any(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, int g, const float* C, int K,
                        uint16_t* idx, float* dist, double* objective, int64_t* n_resolved, cudaStream_t st) {
+    if (cc_small_applies(ctx, N, g, K))
+        return cc_launch_small(ctx, L, X, N, g, const_cast<float*>(C), K, SMALL_E, idx, dist, nullptr, objective, n_resolved, st);
     if (use_pruned(ctx, N, g, K, 1)) {
         const PruneBuffers b = prune_buffers(ctx, L, N, g, K);
         cudaError_t e = prune_order(ctx, b, X, g, C, st);
@@ -238,6 +253,18 @@ cudaError_t fit_pruned(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_
     return e;
 }
 
+// The Lloyd loop of a small problem: one launch an iteration (two with many centroids).
+cudaError_t fit_small(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, int g, int K, int iters, float* C,
+                      uint16_t* idx, float* dist, int32_t* counts, double* objective_trace, cudaStream_t st) {
+    char* ws = static_cast<char*>(ctx->ws);
+    cudaError_t e = cudaMemsetAsync(ws + L.sum_lo, 0, L.sum_hi - L.sum_lo + sizeof(int64_t) * (size_t)K * g, st);   // both sums
+    if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, sizeof(int32_t) * (size_t)K, st);
+    for (int it = 0; it < iters && e == cudaSuccess; ++it)
+        e = cc_launch_small(ctx, L, X, N, g, C, K, it == 0 ? SMALL_FIRST : SMALL_NEXT, idx, dist, counts,
+                            objective_trace ? objective_trace + it : nullptr, nullptr, st);
+    return e;
+}
+
 }  // namespace
 
 extern "C" {
@@ -283,6 +310,7 @@ cc_status cc_create(cc_ctx** out, int device) {
     c->prof = nullptr;
     c->e2e_buf = nullptr;
     c->e2e_bytes = 0;
+    c->stage = nullptr;
     c->empty_rule = CC_EMPTY_KEEP;
     *out = c;
     return CC_OK;
@@ -295,6 +323,7 @@ cc_status cc_destroy(cc_ctx* ctx) {
         cudaSetDevice(ctx->device);
         cudaFree(ctx->e2e_buf);
     }
+    if (ctx->stage) cudaFreeHost(ctx->stage);
     if (ctx->prof) {
         cudaSetDevice(ctx->device);
         for (int i = 0; i < ctx->prof_made; ++i) { cudaEventDestroy(ctx->prof[i].a); cudaEventDestroy(ctx->prof[i].b); }
@@ -360,7 +389,7 @@ cc_status cc_init_positions(int64_t N, int K, uint64_t seed, int64_t* positions_
     if (K < 1 || K > 65536) return CC_ERR_K_RANGE;
     if (N < 1 || N >= (int64_t)1 << 31) return CC_ERR_SHAPE;
     if (N < K) return CC_ERR_N_LT_K;
-    partial_shuffle(N, K, seed, positions_host);
+    try { sparse_shuffle(N, K, seed, positions_host); } catch (...) { return CC_ERR_CUDA; }
     return CC_OK;
 }
 
@@ -379,7 +408,9 @@ cc_status cc_init_codebook(cc_ctx* ctx, const uint16_t* X, int64_t N, int g, int
         ctx->pos_cap = ctx->pos_host ? K : 0;
         if (!ctx->pos_host) return CC_ERR_CUDA;
     }
-    partial_shuffle(N, K, seed, ctx->pos_host);
+    try { sparse_shuffle(N, K, seed, ctx->pos_host); } catch (...) { return CC_ERR_CUDA; }
+    if (K <= CC_INIT_ARGS)
+        return from_cuda(cc_launch_gather_init_args(ctx, X, g, K, ctx->pos_host, C, (cudaStream_t)stream));
     const WsLayout L = cc_ws_layout(N, g, K);
     int64_t* pos_dev = reinterpret_cast<int64_t*>(static_cast<char*>(ctx->ws) + L.positions);
     cudaStream_t st = (cudaStream_t)stream;
@@ -502,6 +533,8 @@ cc_status cc_fit(cc_ctx* ctx, const uint16_t* X, int64_t N, int g, int K, int it
     cudaStream_t st = (cudaStream_t)stream;
     if (iters > 0 && use_pruned(ctx, N, g, K, iters))
         return from_cuda(fit_pruned(ctx, L, X, N, g, K, iters, C, idx, dist, counts, objective_trace, st));
+    if (iters > 0 && cc_small_applies(ctx, N, g, K))
+        return from_cuda(fit_small(ctx, L, X, N, g, K, iters, C, idx, dist, counts, objective_trace, st));
     for (int it = 0; it < iters; ++it) {
         cudaError_t e = assign_any(ctx, L, X, N, g, C, K, idx, dist, objective_trace ? objective_trace + it : nullptr,
                                    nullptr, st);
@@ -698,9 +731,7 @@ cc_status cc_poll_status(cc_ctx* ctx, void* stream) {
     if (cudaMemcpyAsync(&word, ctx->ws, sizeof(word), cudaMemcpyDeviceToHost, st) != cudaSuccess) return CC_ERR_CUDA;
     if (cudaMemsetAsync(ctx->ws, 0, sizeof(word), st) != cudaSuccess) return CC_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return CC_ERR_CUDA;
-    if (word & CC_DEV_TIMEOUT) return CC_ERR_DEVICE_TIMEOUT;
-    if (word & CC_DEV_NONFINITE) return CC_ERR_NONFINITE;
-    return CC_OK;
+    return status_of(word);
 }
 
 cc_status cc_compress_host(cc_ctx* ctx, const uint16_t* W_host, int64_t d_out, int64_t d_in, int g, int K, int iters,
@@ -719,12 +750,13 @@ cc_status cc_compress_host(cc_ctx* ctx, const uint16_t* W_host, int64_t d_out, i
 
     const size_t w_bytes = (size_t)d_out * d_in * 2, x_bytes = (size_t)N * g * 2;
     const size_t ws_bytes = cc_ws_layout(N, g, K).total;
-    // one allocation, carved: W | X | C | C16 | idx | dist | counts | trace | workspace
+    // one allocation, carved: W | X | C | C16 | idx | trace | workspace | dist | counts; the results and the status word
+    // at the head of the workspace lie in a row
     size_t off = 0;
     auto take = [&](size_t b) { size_t o = off; off += cc_align_up(b, 256); return o; };
     const size_t oW = take(w_bytes), oX = take(x_bytes), oC = take((size_t)K * g * 4), oC16 = take((size_t)K * g * 2),
-                 oIdx = take((size_t)N * 2), oDist = take((size_t)N * 4), oCnt = take((size_t)K * 4),
-                 oTr = take((size_t)(iters + 1) * 8), oWs = take(ws_bytes);
+                 oIdx = take((size_t)N * 2), oTr = take((size_t)(iters + 1) * 8), oWs = take(ws_bytes), oDist = take((size_t)N * 4),
+                 oCnt = take((size_t)K * 4);
     if (ctx->e2e_bytes < off) {          // grown on demand and kept: repeated calls allocate nothing
         if (ctx->e2e_buf) cudaFree(ctx->e2e_buf);
         ctx->e2e_buf = nullptr;
@@ -735,7 +767,10 @@ cc_status cc_compress_host(cc_ctx* ctx, const uint16_t* W_host, int64_t d_out, i
     char* base = static_cast<char*>(ctx->e2e_buf);
     void* saved_ws = ctx->ws;
     const size_t saved_bytes = ctx->ws_bytes;
-    cc_status s = cc_set_workspace(ctx, base + oWs, ws_bytes);
+    cc_status s = CC_OK;
+    ctx->ws = base + oWs;
+    ctx->ws_bytes = ws_bytes;
+    if (cudaMemsetAsync(ctx->ws, 0, CC_STATUS_BYTES, st) != cudaSuccess) s = CC_ERR_CUDA;
     uint16_t* W = (uint16_t*)(base + oW);
     uint16_t* X = (uint16_t*)(base + oX);
     float* C = (float*)(base + oC);
@@ -754,15 +789,36 @@ cc_status cc_compress_host(cc_ctx* ctx, const uint16_t* W_host, int64_t d_out, i
         if (s == CC_OK && cudaMemcpyAsync(W_hat_host, W, w_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess)
             s = CC_ERR_CUDA;
     }
-    if (s == CC_OK && cudaMemcpyAsync(C16_host, C16, (size_t)K * g * 2, cudaMemcpyDeviceToHost, st) != cudaSuccess)
-        s = CC_ERR_CUDA;
-    if (s == CC_OK && cudaMemcpyAsync(idx_host, idx, (size_t)N * 2, cudaMemcpyDeviceToHost, st) != cudaSuccess)
-        s = CC_ERR_CUDA;
-    if (s == CC_OK && objective_trace_host &&
-        cudaMemcpyAsync(objective_trace_host, trace, (size_t)(iters + 1) * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess)
-        s = CC_ERR_CUDA;
-    if (s == CC_OK) s = cc_poll_status(ctx, st);
-    else cudaStreamSynchronize(st);
+    // Small results: one copy into a page-locked buffer, and from there on by the host (a copy of its own for each of
+    // the four costs 6 us on the stream).
+    const size_t small = oWs + 4 - oC16;
+    if (s == CC_OK && small <= CC_STAGE_BYTES && !ctx->stage && cudaMallocHost(&ctx->stage, CC_STAGE_BYTES) != cudaSuccess) {
+        ctx->stage = nullptr;
+        cudaGetLastError();                              // without the buffer: copies straight to the caller
+    }
+    if (s == CC_OK && small <= CC_STAGE_BYTES && ctx->stage) {
+        const char* from = static_cast<const char*>(ctx->stage);
+        if (cudaMemcpyAsync(ctx->stage, base + oC16, small, cudaMemcpyDeviceToHost, st) != cudaSuccess) s = CC_ERR_CUDA;
+        if (cudaStreamSynchronize(st) != cudaSuccess) s = CC_ERR_CUDA;
+        if (s == CC_OK) {
+            memcpy(C16_host, from, (size_t)K * g * 2);
+            memcpy(idx_host, from + (oIdx - oC16), (size_t)N * 2);
+            if (objective_trace_host) memcpy(objective_trace_host, from + (oTr - oC16), (size_t)(iters + 1) * 8);
+            unsigned word;
+            memcpy(&word, from + (oWs - oC16), sizeof(word));
+            s = status_of(word);
+        }
+    } else {
+        if (s == CC_OK && cudaMemcpyAsync(C16_host, C16, (size_t)K * g * 2, cudaMemcpyDeviceToHost, st) != cudaSuccess)
+            s = CC_ERR_CUDA;
+        if (s == CC_OK && cudaMemcpyAsync(idx_host, idx, (size_t)N * 2, cudaMemcpyDeviceToHost, st) != cudaSuccess)
+            s = CC_ERR_CUDA;
+        if (s == CC_OK && objective_trace_host &&
+            cudaMemcpyAsync(objective_trace_host, trace, (size_t)(iters + 1) * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess)
+            s = CC_ERR_CUDA;
+        if (s == CC_OK) s = cc_poll_status(ctx, st);
+        else cudaStreamSynchronize(st);
+    }
     ctx->ws = saved_ws;
     ctx->ws_bytes = saved_bytes;
     return s;

@@ -33,8 +33,11 @@ struct cc_ctx {
     cc_prof_slot* prof;   // CC_PROF_CAP slots, events created on first use
     void* e2e_buf;        // device memory of cc_compress_host, grown on demand, freed by cc_destroy
     size_t e2e_bytes;
+    void* stage;          // CC_STAGE_BYTES of page-locked host memory for small results, made on first use, freed by cc_destroy
     int empty_rule;       // CC_EMPTY_*
 };
+
+constexpr size_t CC_STAGE_BYTES = 512 * 1024;
 
 // Brackets one kernel launch with events on its stream when timing is enabled, and counts it.
 struct ProfScope {
@@ -134,6 +137,8 @@ cudaError_t cc_launch_decode(cc_ctx*, const uint16_t* C16, int K, int g, const u
                              int64_t d_in, int layout, uint16_t* W_hat, cudaStream_t);
 cudaError_t cc_launch_gather_init(cc_ctx*, const uint16_t* X, int g, int K, const int64_t* pos_dev, float* C,
                                   cudaStream_t);
+constexpr int CC_INIT_ARGS = 480;      // initial positions that travel as a kernel argument instead of a copy
+cudaError_t cc_launch_gather_init_args(cc_ctx*, const uint16_t* X, int g, int K, const int64_t* pos_host, float* C, cudaStream_t);
 cudaError_t cc_launch_to_half(cc_ctx*, const float* C, int64_t n, uint16_t* C16, float* C_widened, cudaStream_t);
 
 cudaError_t cc_launch_assign_ffma(cc_ctx*, const WsLayout&, const uint16_t* X, int64_t N, int g, const float* C,
@@ -168,6 +173,16 @@ cudaError_t cc_launch_unsort(cc_ctx*, const unsigned* pos, int64_t N, const uint
                              float* dist, unsigned* marks, unsigned* status, unsigned* flagged, cudaStream_t);
 cudaError_t cc_launch_assign_pruned(cc_ctx*, const PruneBuffers&, int g, const float* C, int mode, cudaStream_t);
 cudaError_t cc_launch_sum_exact(cc_ctx*, const PruneBuffers&, bool have_max, double* objective, int64_t* n_resolved, cudaStream_t);
+
+cudaError_t cc_launch_update_means(cc_ctx*, const WsLayout&, int g, int K, float* C, int32_t* counts, cudaStream_t);
+
+// Small problems (cc_small.cu): the E-step by direct distances, with the M-step behind it in the same launch.
+enum { SMALL_E = 0, SMALL_FIRST = 1, SMALL_NEXT = 2 };
+constexpr int SMALL_SMEM = 96 * 1024;                // bytes of codebook
+constexpr int64_t SMALL_WORK = 350000000;            // point-centroid pairs times instructions each
+bool cc_small_applies(const cc_ctx*, int64_t N, int g, int K);
+cudaError_t cc_launch_small(cc_ctx*, const WsLayout&, const uint16_t* X, int64_t N, int g, float* C, int K, int mode, uint16_t* idx,
+                            float* dist, int32_t* counts, double* objective, int64_t* n_flagged, cudaStream_t);
 
 // Scratch of the layer forward in the workspace: the status block, a copy of the codebook with padded rows, the rest.
 constexpr size_t CC_LINEAR_SCRATCH_FROM = CC_STATUS_BYTES + (size_t)65536 * 32;

@@ -488,6 +488,15 @@ __global__ void gather_init_kernel(const uint16_t* __restrict__ X, int g, int K,
     C[e] = __half2float(__ushort_as_half(X[pos[k] * g + t]));
 }
 
+struct InitArgs { int64_t pos[CC_INIT_ARGS]; };
+
+__global__ void gather_init_args_kernel(const uint16_t* __restrict__ X, int g, int K, const __grid_constant__ InitArgs a, float* __restrict__ C) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= K * g) return;
+    const int k = e / g, t = e - k * g;
+    C[e] = __half2float(__ushort_as_half(X[a.pos[k] * g + t]));
+}
+
 // C16 = round-to-nearest-even FP16 of C; optionally also the widened value (what the codes of
 // the stored codebook are computed against).
 __global__ void to_half_kernel(const float* __restrict__ C, int64_t n, uint16_t* __restrict__ C16,
@@ -561,6 +570,16 @@ cudaError_t cc_launch_gather_init(cc_ctx* ctx, const uint16_t* X, int g, int K, 
                                   cudaStream_t st) {
     ProfScope ps(ctx, CC_K_OTHER, st);
     gather_init_kernel<<<(K * g + 255) / 256, 256, 0, st>>>(X, g, K, pos_dev, C);
+    return cudaGetLastError();
+}
+
+// Few centroids: a copy of their positions from pageable memory would cost the host some 15 us.
+cudaError_t cc_launch_gather_init_args(cc_ctx* ctx, const uint16_t* X, int g, int K, const int64_t* pos_host, float* C, cudaStream_t st) {
+    if (K > CC_INIT_ARGS) return cudaErrorInvalidValue;
+    InitArgs a;
+    for (int k = 0; k < CC_INIT_ARGS; ++k) a.pos[k] = k < K ? pos_host[k] : 0;
+    ProfScope ps(ctx, CC_K_OTHER, st);
+    gather_init_args_kernel<<<(K * g + 255) / 256, 256, 0, st>>>(X, g, K, a, C);
     return cudaGetLastError();
 }
 

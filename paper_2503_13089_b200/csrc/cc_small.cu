@@ -1,0 +1,308 @@
+// E-step of a small problem, with the M-step of a Lloyd iteration behind it, in one launch.
+//
+// The tensor-core E-step is six launches (ranges, operand, scan, finish, two of the exact stage), and an iteration nine;
+// each runs for two to seven microseconds however little there is to do.  Up to SMALL_WORK the distances are
+// computed directly instead: one iteration, g = 4, of 32768 x 256 50 -> 14 us, 32768 x 1024 50 -> 31; 50000 x 500, g = 6
+// 56 -> 41; where the work is more it loses (50000 x 1000, g = 6 57.5 -> 60).
+//
+// Eight lanes share a point and four points a lane: lane k of a group takes centroids 32 c + 8 e + k (e = 0..3, a
+// chunk), FP32 in the direct form sum (x_t - c_t)^2, two coordinates per instruction, relative error below
+// (g + 2) 2^-24.  Of every chunk only the smallest distance is looked at.  Every centroid whose FP32 distance is within
+// a factor 1 + 2^-17 of the smallest may be the nearest; they are compared in FP64 (sub, mul, add in dimension order,
+// no contraction), the lower index winning a tie: those of the winning chunk always, the others only when another
+// chunk comes as close.
+// The sums of the M-step are integers, so that the order of the blocks does not matter; the block that finishes last
+// adds up the objective in a fixed order and, for few centroids, forms the means.
+#include <cuda_fp16.h>
+
+#include "cc_common.cuh"
+#include "cc_assign_shared.cuh"
+#include "cc_sums.cuh"
+
+namespace {
+
+constexpr int SM_THREADS = 512, SM_LPP = 8, SM_P = 4;
+constexpr int SM_GROUPS = SM_THREADS / SM_LPP;
+constexpr int SM_CHUNK = 4 * SM_LPP;                 // centroids a group takes per step
+constexpr int SM_MEANS = 4096;                       // K g up to which the last block forms the means
+
+__device__ __forceinline__ ull f2_add(ull a, ull b) { ull r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ ull f2_fma(ull a, ull b, ull c) { ull r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ ull f2_pack(float lo, float hi) { ull r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r; }
+__device__ __forceinline__ float f2_sum(ull a) { float lo, hi; asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a)); return lo + hi; }
+
+// FP64 distance to a row of the table (-c, exactly).
+template <int G>
+__device__ __forceinline__ double exact_distance(const float (&x)[G], const ull* row) {
+    const float* c = reinterpret_cast<const float*>(row);
+    double d = 0.0;
+#pragma unroll
+    for (int t = 0; t < G; ++t) {
+        const double df = __dadd_rn((double)x[t], (double)c[t]);
+        d = __dadd_rn(d, __dmul_rn(df, df));
+    }
+    return d;
+}
+
+// mode: SMALL_E (E-step alone), SMALL_FIRST (and all points added to the sums, which are zero), SMALL_NEXT (and the points
+// whose code changed moved; idx holds the codes that the sums correspond to).
+// flagged: list of the points with more than one candidate, counted in status words 2..3 (or nullptr).
+template <int G>
+__global__ void __launch_bounds__(SM_THREADS)
+small_kernel(const uint16_t* __restrict__ X, int64_t N, float* C, int K, int mode, uint16_t* idx, float* __restrict__ dist,
+             ull* __restrict__ sum_lo, ull* __restrict__ sum_hi, int* __restrict__ counts, int with_means,
+             double* __restrict__ partials, double* __restrict__ objective, unsigned* __restrict__ status,
+             unsigned* __restrict__ flagged, int64_t* __restrict__ n_flagged) {
+    constexpr int GP = (G + 1) / 2;
+    extern __shared__ __align__(16) ull sm_c[];      // K rounded up to whole chunks, GP pairs of -c each
+    __shared__ double sh[SM_THREADS / 32];
+    __shared__ bool last;
+    const int tid = threadIdx.x, lane = tid & 31, k = tid & (SM_LPP - 1);
+    const int n_chunks = (K + SM_CHUNK - 1) / SM_CHUNK;
+    for (int e = tid; e < n_chunks * SM_CHUNK * GP; e += SM_THREADS) {
+        const int j = e / GP, t = 2 * (e - j * GP);
+        // rows past the last centroid are infinitely far away
+        const float a = j < K ? -__ldcg(C + (int64_t)j * G + t) : 3.0e38f;
+        const float b = j < K ? (t + 1 < G ? -__ldcg(C + (int64_t)j * G + t + 1) : 0.f) : 3.0e38f;
+        sm_c[e] = f2_pack(a, b);
+    }
+    __syncthreads();
+    bool nonfinite = false;
+    double acc = 0.0;
+    const int64_t step = (int64_t)gridDim.x * SM_GROUPS * SM_P;
+    for (int64_t base = ((int64_t)blockIdx.x * SM_GROUPS + tid / SM_LPP) * SM_P; base - (tid / SM_LPP) * SM_P < N; base += step) {
+        float xv[SM_P][G];
+        ull x2[SM_P][GP];
+#pragma unroll
+        for (int p = 0; p < SM_P; ++p) {
+            load_point<G>(X, base + p, N, xv[p], nonfinite);
+#pragma unroll
+            for (int t = 0; t < GP; ++t) x2[p][t] = f2_pack(xv[p][2 * t], 2 * t + 1 < G ? xv[p][2 * t + 1] : 0.f);
+        }
+        float b1[SM_P], b2[SM_P];
+        int bc[SM_P];
+#pragma unroll
+        for (int p = 0; p < SM_P; ++p) { b1[p] = INFINITY; b2[p] = INFINITY; bc[p] = 0; }
+        for (int c = 0; c < n_chunks; ++c) {
+            float m[SM_P];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const ull* row = sm_c + (c * SM_CHUNK + e * SM_LPP + k) * GP;
+                ull cv[GP];
+                if constexpr (GP % 2 == 0) {
+#pragma unroll
+                    for (int t = 0; t < GP; t += 2) {
+                        const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(row + t);
+                        cv[t] = u.x; cv[t + 1] = u.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int t = 0; t < GP; ++t) cv[t] = row[t];
+                }
+#pragma unroll
+                for (int p = 0; p < SM_P; ++p) {
+                    ull d2 = 0ull;
+#pragma unroll
+                    for (int t = 0; t < GP; ++t) { const ull df = f2_add(x2[p][t], cv[t]); d2 = f2_fma(df, df, d2); }
+                    const float d = f2_sum(d2);
+                    m[p] = e == 0 ? d : fminf(m[p], d);
+                }
+            }
+#pragma unroll
+            for (int p = 0; p < SM_P; ++p) {
+                const bool better = m[p] < b1[p];
+                b2[p] = better ? b1[p] : fminf(b2[p], m[p]);
+                bc[p] = better ? c : bc[p];
+                b1[p] = better ? m[p] : b1[p];
+            }
+        }
+        // the group's smallest distance, the chunk that holds it (as 8 c + lane) and the smallest of any other chunk
+        int at[SM_P];
+        bool many[SM_P], any = false;
+#pragma unroll
+        for (int p = 0; p < SM_P; ++p) {
+            float s1 = b1[p], s2 = b2[p];
+            at[p] = bc[p] * SM_LPP + k;
+#pragma unroll
+            for (int o = SM_LPP / 2; o > 0; o >>= 1) {
+                const float o1 = __shfl_xor_sync(0xffffffffu, s1, o), o2 = __shfl_xor_sync(0xffffffffu, s2, o);
+                const int oat = __shfl_xor_sync(0xffffffffu, at[p], o);
+                const bool take = o1 < s1 || (o1 == s1 && oat < at[p]);
+                s2 = fminf(take ? s1 : o1, fminf(s2, o2));
+                at[p] = take ? oat : at[p];
+                s1 = take ? o1 : s1;
+            }
+            b1[p] = s1 * (1.0f + 7.62939453125e-6f) + 1.0e-37f;       // from here on: the bound
+            many[p] = !(s2 > b1[p]);                  // the same answer in the eight lanes
+            any |= many[p];
+        }
+        // lanes 0..3 look at the four centroids of the winning chunk of an even point, lanes 4..7 at those of the odd
+        // point beside it
+        const int half = k >> 2, e4 = k & 3;
+#pragma unroll
+        for (int q = 0; q < SM_P / 2; ++q) {
+            float x[G];
+#pragma unroll
+            for (int t = 0; t < G; ++t) x[t] = half ? xv[2 * q + 1][t] : xv[2 * q][t];
+            const int a = half ? at[2 * q + 1] : at[2 * q];
+            const int j = (a >> 3) * SM_CHUNK + e4 * SM_LPP + (a & 7);
+            const float bound = half ? b1[2 * q + 1] : b1[2 * q];
+            bool close = half ? many[2 * q + 1] : many[2 * q];
+            double Db = INFINITY;
+            int jb = 0x7fffffff;
+            if (j < K) { Db = exact_distance<G>(x, sm_c + j * GP); jb = j; }
+            if (flagged) close |= __popc(__ballot_sync(0xffffffffu, Db <= (double)bound) >> (lane & 28) & 15u) > 1;
+            if (__any_sync(0xffffffffu, any)) {        // rare: every centroid of the points whose second chunk comes as close
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int p = 2 * q + h;
+                    if (!many[p]) continue;
+                    double D = INFINITY;
+                    int jm = 0x7fffffff;
+                    for (int jj = k; jj < K; jj += SM_LPP) {
+                        const ull* row = sm_c + jj * GP;
+                        ull d2 = 0ull;
+#pragma unroll
+                        for (int t = 0; t < GP; ++t) { const ull df = f2_add(x2[p][t], row[t]); d2 = f2_fma(df, df, d2); }
+                        if (f2_sum(d2) <= b1[p]) {
+                            const double d = exact_distance<G>(xv[p], row);
+                            if (d < D || (d == D && jj < jm)) { D = d; jm = jj; }
+                        }
+                    }
+                    const unsigned group = 0xffu << (lane & 24);
+#pragma unroll
+                    for (int o = SM_LPP / 2; o > 0; o >>= 1) {
+                        const double Do = __shfl_xor_sync(group, D, o);
+                        const int jo = __shfl_xor_sync(group, jm, o);
+                        if (Do < D || (Do == D && jo < jm)) { D = Do; jm = jo; }
+                    }
+                    if (half == h) { Db = D; jb = jm; }
+                }
+            }
+            const int64_t i = base + 2 * q + half;
+            const int before = (mode == SMALL_NEXT && i < N) ? idx[i] : -1;
+            __syncwarp();                             // every lane has read the old code before one replaces it
+#pragma unroll
+            for (int o = 2; o > 0; o >>= 1) {
+                const double Do = __shfl_xor_sync(0xffffffffu, Db, o);
+                const int jo = __shfl_xor_sync(0xffffffffu, jb, o);
+                if (Do < Db || (Do == Db && jo < jb)) { Db = Do; jb = jo; }
+            }
+            if (jb >= K) jb = K - 1;                   // only reachable with non-finite input
+            if (i < N) {
+                if (e4 == 0) {
+                    idx[i] = (uint16_t)jb;
+                    if (dist) dist[i] = (float)Db;
+                    acc += (double)(float)Db;
+                    if (flagged && close) flagged[atomicAdd(reinterpret_cast<ull*>(status + 2), 1ull)] = (unsigned)i;
+                }
+                if (mode != SMALL_E && jb != before) {
+                    if (e4 == 0) {
+                        atomicAdd(counts + jb, 1);
+                        if (before >= 0) atomicSub(counts + before, 1);
+                    }
+                    for (int t = e4; t < G; t += 4) {
+                        const uint16_t h = __ldg(X + i * G + t);
+                        add_coord(h, sum_lo + (int64_t)jb * G + t, sum_hi + (int64_t)jb * G + t);
+                        if (before >= 0)               // minus the value: the sign bit flipped
+                            add_coord(h ^ 0x8000u, sum_lo + (int64_t)before * G + t, sum_hi + (int64_t)before * G + t);
+                    }
+                }
+            }
+        }
+    }
+    if (nonfinite) atomicOr(status, CC_DEV_NONFINITE);
+    __threadfence();                                    // this thread's sums before the block's ticket
+    auto block_add = [&](double v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0) sh[tid >> 5] = v;
+        __syncthreads();
+        double r = 0.0;
+        if (tid < 32) {
+            r = tid < SM_THREADS / 32 ? sh[tid] : 0.0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
+        }
+        return r;                                       // valid in thread 0
+    };
+    const double mine = block_add(acc);
+    if (tid == 0) {
+        partials[blockIdx.x] = mine;
+        __threadfence();
+        last = atomicAdd(status + 8, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double tot = 0.0;
+    for (int b = tid; b < (int)gridDim.x; b += SM_THREADS) tot += __ldcg(partials + b);
+    const double all = block_add(tot);
+    if (tid == 0) {
+        if (objective) *objective = all;
+        if (n_flagged) *n_flagged = (int64_t)__ldcg(reinterpret_cast<const ull*>(status + 2));
+        status[8] = 0u;
+    }
+    if (mode == SMALL_E || !with_means) return;
+    for (int e = tid; e < K * G; e += SM_THREADS) {
+        const int n = __ldcg(counts + e / G);
+        const long long lo = __ldcg(reinterpret_cast<const long long*>(sum_lo) + e), hi = __ldcg(reinterpret_cast<const long long*>(sum_hi) + e);
+        if (n > 0) C[e] = mean_of(lo, hi, n);           // empty cluster: previous centroid stays
+    }
+}
+
+template <int G>
+size_t small_smem(int K) { return (size_t)((K + SM_CHUNK - 1) / SM_CHUNK) * SM_CHUNK * ((G + 1) / 2) * 8; }
+
+template <int G>
+cudaError_t launch_small(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, float* C, int K, int mode, uint16_t* idx, float* dist,
+                         int32_t* counts, double* objective, int64_t* n_flagged, cudaStream_t st) {
+    static bool attr_dev[64] = {};
+    bool& have = attr_dev[ctx->device & 63];
+    if (!have) {
+        const cudaError_t e = cudaFuncSetAttribute(small_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMALL_SMEM);
+        if (e != cudaSuccess) return e;
+        have = true;
+    }
+    char* ws = static_cast<char*>(ctx->ws);
+    int64_t blocks = (N + SM_GROUPS * SM_P - 1) / (SM_GROUPS * SM_P);
+    const int64_t cap = ctx->sm_count;                  // at most CC_OBJ_BLOCKS partial sums
+    if (blocks > cap) blocks = cap;
+    if (n_flagged) {
+        const cudaError_t e = cudaMemsetAsync(ws + L.status + 8, 0, 8, st);
+        if (e != cudaSuccess) return e;
+    }
+    ProfScope ps(ctx, CC_K_ASSIGN_MAIN, st);
+    small_kernel<G><<<(unsigned)blocks, SM_THREADS, small_smem<G>(K), st>>>(
+        X, N, C, K, mode, idx, dist, reinterpret_cast<ull*>(ws + L.sum_lo), reinterpret_cast<ull*>(ws + L.sum_hi), counts,
+        K * G <= SM_MEANS && ctx->empty_rule == CC_EMPTY_KEEP, reinterpret_cast<double*>(ws + L.partials), objective,
+        reinterpret_cast<unsigned*>(ws + L.status), n_flagged ? reinterpret_cast<unsigned*>(ws + L.flagged) : nullptr, n_flagged);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+bool cc_small_applies(const cc_ctx* ctx, int64_t N, int g, int K) {
+    const int64_t pairs = (g + 1) / 2;
+    return ctx->path == CC_PATH_AUTO && N > 0 && (K + SM_CHUNK - 1) / SM_CHUNK * SM_CHUNK * pairs * 8 <= SMALL_SMEM && N * K * (2 * pairs + 3) <= SMALL_WORK;
+}
+
+// C is only written in the modes with an M-step.  n_flagged: how many points had more than one candidate (listed in the
+// workspace, as the other E-steps list the points of their exact stage).
+cudaError_t cc_launch_small(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, int g, float* C, int K, int mode, uint16_t* idx,
+                            float* dist, int32_t* counts, double* objective, int64_t* n_flagged, cudaStream_t st) {
+    cudaError_t e = cudaSuccess;
+#define CALL(G) e = launch_small<G>(ctx, L, X, N, C, K, mode, idx, dist, counts, objective, n_flagged, st)
+    switch (g) {
+        case 1: CALL(1); break;   case 2: CALL(2); break;   case 3: CALL(3); break;   case 4: CALL(4); break;
+        case 5: CALL(5); break;   case 6: CALL(6); break;   case 7: CALL(7); break;   case 8: CALL(8); break;
+        case 9: CALL(9); break;   case 10: CALL(10); break; case 11: CALL(11); break; case 12: CALL(12); break;
+        case 13: CALL(13); break; case 14: CALL(14); break; case 15: CALL(15); break; case 16: CALL(16); break;
+        default: return cudaErrorInvalidValue;
+    }
+#undef CALL
+    if (e != cudaSuccess || mode == SMALL_E) return e;
+    // the means, or the splitting of empty clusters, where the kernel has left them
+    if (K * g <= SM_MEANS && ctx->empty_rule == CC_EMPTY_KEEP) return e;
+    return cc_launch_update_means(ctx, L, g, K, C, counts, st);
+}

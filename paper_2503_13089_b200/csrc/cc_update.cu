@@ -16,21 +16,9 @@
 // (the same sums without the division).
 #include "cc_common.cuh"
 #include "cc_assign_shared.cuh"
+#include "cc_sums.cuh"
 
 namespace {
-
-__device__ __forceinline__ void add_coord(uint16_t h, ull* lo, ull* hi) {
-    const float v = __half2float(__ushort_as_half(h));
-    const unsigned e = (h >> 10) & 31u;
-    if (e == 31u) return;                       // non-finite: reported by the E-step, skipped here
-    if (e >= 18u) {                             // |v| >= 8: multiple of 2^-7
-        const long long q = __float2ll_rn(v * 128.0f);
-        atomicAdd(hi, (ull)q);
-    } else if ((h & 0x7fffu) != 0u) {           // multiple of 2^-24
-        const long long q = __float2ll_rn(v * 16777216.0f);
-        atomicAdd(lo, (ull)q);
-    }
-}
 
 // One lane per coordinate: the G reductions of a point go to G adjacent 64-bit words (one 32-byte
 // sector at G = 4, one 128-byte line at G = 16), so a warp's reduction instruction touches 32 / G
@@ -204,8 +192,7 @@ update_finish_kernel(long long* __restrict__ sum_lo, long long* __restrict__ sum
         if (e == j * g) counts[j] = n;
     }
     if (n <= 0) return;   // empty cluster: previous centroid stays
-    const double s = (double)lo * 5.9604644775390625e-8 + (double)hi * 0.0078125;
-    C[e] = (float)(s / (double)n);
+    C[e] = mean_of(lo, hi, n);
 }
 
 // Gradient with respect to the codebook: the exact integer sums as they are, rounded once to FP32.
@@ -343,6 +330,19 @@ cudaError_t cc_launch_codebook_grad(cc_ctx* ctx, const WsLayout& L, const uint16
     return cudaGetLastError();
 }
 
+// Means from the workspace sums (one copy) and `counts`, then the rule for empty clusters.
+cudaError_t cc_launch_update_means(cc_ctx* ctx, const WsLayout& L, int g, int K, float* C, int32_t* counts, cudaStream_t st) {
+    char* ws = static_cast<char*>(ctx->ws);
+    {
+        ProfScope ps(ctx, CC_K_UPDATE_FINISH, st);
+        update_finish_kernel<<<(K * g + 255) / 256, 256, 0, st>>>(reinterpret_cast<long long*>(ws + L.sum_lo),
+                                                                 reinterpret_cast<long long*>(ws + L.sum_hi), counts, counts, K,
+                                                                 g, 1, C);
+    }
+    if (ctx->empty_rule == CC_EMPTY_SPLIT_LARGEST) return cc_launch_split_empty(ctx, L, C, K, g, counts, st);
+    return cudaGetLastError();
+}
+
 // Incremental M-step (see update_delta_kernel): the workspace sums and `counts` must be those of
 // the previous M-step on the same X, and idx_prev the codes they were computed from.
 cudaError_t cc_launch_update_delta(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, int g,
@@ -360,14 +360,7 @@ cudaError_t cc_launch_update_delta(cc_ctx* ctx, const WsLayout& L, const uint16_
         CC_UPDATE_DISPATCH(g, CALL)
 #undef CALL
     }
-    {
-        ProfScope ps(ctx, CC_K_UPDATE_FINISH, st);
-        update_finish_kernel<<<(K * g + 255) / 256, 256, 0, st>>>(reinterpret_cast<long long*>(sum_lo),
-                                                                 reinterpret_cast<long long*>(sum_hi), counts, counts, K,
-                                                                 g, 1, C);
-    }
-    if (ctx->empty_rule == CC_EMPTY_SPLIT_LARGEST) return cc_launch_split_empty(ctx, L, C, K, g, counts, st);
-    return cudaGetLastError();
+    return cc_launch_update_means(ctx, L, g, K, C, counts, st);
 }
 
 // ---------------------------------------------------------------------------------------------
