@@ -215,6 +215,13 @@ cudaError_t assign_any(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_
         return e;
     }
     if (!dist) dist = reinterpret_cast<float*>(static_cast<char*>(ctx->ws) + L.dist_tmp);
+    if (ctx->path == CC_PATH_AUTO && cc_prune_applies(N, K) && (objective || n_resolved)) {
+        // the same sum as behind the pruned E-step: a fit's objectives do not depend on which of the two an iteration ran
+        cudaError_t e = cc_launch_assign_tensor(ctx, L, X, N, g, C, K, idx, dist, nullptr, nullptr, st);
+        PruneBuffers b = prune_buffers(ctx, L, N, g, K);
+        b.dist_s = dist;
+        return e == cudaSuccess ? cc_launch_sum_exact(ctx, b, false, objective, n_resolved, st) : e;
+    }
     if (use_tensor_path(ctx, g, K))
         return cc_launch_assign_tensor(ctx, L, X, N, g, C, K, idx, dist, objective, n_resolved, st);
     return cc_launch_assign_ffma(ctx, L, X, N, g, C, K, idx, dist, objective, n_resolved, st);
