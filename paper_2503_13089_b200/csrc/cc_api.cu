@@ -28,7 +28,7 @@ WsLayout cc_ws_layout(int64_t N, int g, int K) {
     L.tensor = take(Kpad * (size_t)(64 + 1) * 4);
     L.tstate = take((size_t)N * 8);
     L.idx_prev = take((size_t)N * 2);
-    const bool pr = cc_prune_applies(N, K);
+    const bool pr = cc_prune_applies(N, g, K);
     auto take_if = [&](size_t bytes) { size_t o = off; if (pr) off += cc_align_up(bytes, 256); return o; };
     const size_t n_chunks = cc_align_up((size_t)(K + 63) / 64, 8), groups = (size_t)((N + 511) / 512);
     const size_t Kp = (size_t)cc_tree_positions(K);
@@ -51,8 +51,8 @@ WsLayout cc_ws_layout(int64_t N, int g, int K) {
     return L;
 }
 
-// Pruned E-step: worth its preparation (tree, sort, lists) from this many distances on.
-bool cc_prune_applies(int64_t N, int K) { return N >= 32768 && K >= 2048 && N * (int64_t)K >= (int64_t)1 << 33; }
+// Sizes for which a call may run the pruned E-step (see prune_pays): the workspace has room for it.
+bool cc_prune_applies(int64_t N, int g, int K) { return g <= CC_PRUNE_G && N >= 32768 && K >= 4096 && N * (int64_t)K >= (int64_t)1 << 33; }
 
 // Words of the per (row block, chunk) gaps kept between the iterations of a fit; none where they would take
 // more than 4 GB (few chunks near a point there: the bounding boxes alone rule nearly all out).
@@ -194,11 +194,32 @@ cudaError_t prune_order(cc_ctx* ctx, const PruneBuffers& b, const uint16_t* X, i
     return cc_launch_sort_points(ctx, X, b.N, g, b.tree, levels, reinterpret_cast<uint16_t*>(b.tstate), b.pos, b.first, b.Xs, st);
 }
 
-// Up to this sub-vector length the bounding boxes alone leave well under all chunks to a first E-step.
-constexpr int PRUNE_COLD_G = 6;
+// Whether `steps` E-steps in a row on N points are faster with chunks ruled out, by the length of the sub-vectors.  In
+// more dimensions a box or a gap rules out less and the preparation has to be paid back over more iterations; with
+// fewer centroids there are fewer chunks to rule out.  Measured, pruned against exhaustive, on heavy-tailed points (time
+// of the call as a fraction of the exhaustive one): one step, g = 2, 4 M x 4096 0.95; g = 4, 4 M x 8192 0.92, 1 M x 65536
+// 0.47, 0.26 M x 65536 1.25; g = 5, 2 M x 32768 0.82, 4 M x 16384 1.05; g = 6, 2 M x 65536 0.95, 0.5 M x 65536 1.16.
+// A fit, g = 2, 4 M x 4096, 5 iterations 0.62; g = 4, 5 iterations: 1 M x 8192 1.10, 4 M x 8192 0.74, 0.26 M x 65536 0.77;
+// 20: 2 M x 4096 0.95, 4 M x 2048 1.17; g = 5, 4 M x 16384, 5 iterations 0.81, 1 M x 8700, 20 0.88, 5 1.27; g = 6, 5
+// iterations: 2 M x 32768 1.03, 2 M x 65536 0.79, 0.14 M x 65536 0.84; 10: x 32768 0.86, x 16384 1.03; 20: x 16384 0.90,
+// x 8192 1.15; g = 7, x 65536: 10 iterations 1.00, 20 0.80; x 32768, 20 0.98; g = 8, x 65536: 10 1.03, 20 0.83; x 32768 0.99.
+struct PruneRule { int g_max, steps, K; double scores, scores_all; };   // from so many steps, centroids, N K and N K steps on
+constexpr PruneRule PRUNE_RULES[] = {
+    {3, 1, 4096, 1.6e10, 0},  {3, 2, 4096, 8.5e9, 4e10},  {4, 1, 8192, 3.2e10, 0},  {4, 2, 8192, 8.5e9, 5e10}, {4, 16, 4096, 8.5e9, 0},
+    {5, 1, 32768, 3.2e10, 0}, {5, 4, 16384, 3e10, 0},     {5, 16, 8192, 8.5e9, 0},
+    {6, 1, 60000, 1.2e11, 0}, {6, 5, 49152, 8.5e9, 0},    {6, 10, 32768, 3e10, 0},  {6, 16, 16384, 8.5e9, 0},
+    {7, 16, 40000, 8.5e9, 0}, {8, 16, 49152, 8.5e9, 0},
+};
 
-bool use_pruned(const cc_ctx* ctx, int64_t N, int g, int K, int e_steps) {
-    return ctx->path == CC_PATH_AUTO && cc_prune_applies(N, K) && (g <= PRUNE_COLD_G || (g <= 8 && e_steps >= 4));
+bool prune_pays(int64_t N, int g, int K, int steps) {
+    const double scores = (double)N * (double)K;
+    for (const PruneRule& r : PRUNE_RULES)
+        if (g <= r.g_max && steps >= r.steps && K >= r.K && scores >= r.scores && scores * steps >= r.scores_all) return true;
+    return false;
+}
+
+bool use_pruned(const cc_ctx* ctx, int64_t N, int g, int K, int steps) {
+    return ctx->path == CC_PATH_AUTO && cc_prune_applies(N, g, K) && prune_pays(N, g, K, steps);
 }
 
 cudaError_t assign_any(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, int g, const float* C, int K,
@@ -215,7 +236,7 @@ cudaError_t assign_any(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_
         return e;
     }
     if (!dist) dist = reinterpret_cast<float*>(static_cast<char*>(ctx->ws) + L.dist_tmp);
-    if (ctx->path == CC_PATH_AUTO && cc_prune_applies(N, K) && (objective || n_resolved)) {
+    if (ctx->path == CC_PATH_AUTO && cc_prune_applies(N, g, K) && (objective || n_resolved)) {
         // the same sum as behind the pruned E-step: a fit's objectives do not depend on which of the two an iteration ran
         cudaError_t e = cc_launch_assign_tensor(ctx, L, X, N, g, C, K, idx, dist, nullptr, nullptr, st);
         PruneBuffers b = prune_buffers(ctx, L, N, g, K);
@@ -235,7 +256,7 @@ cudaError_t fit_pruned(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_
     cudaError_t e = prune_order(ctx, b, X, g, C, st);
     for (int it = 0; it < iters && e == cudaSuccess; ++it) {
         bool have_max = true;
-        if (it == 0 && g > PRUNE_COLD_G) {
+        if (it == 0 && !prune_pays(N, g, K, 1)) {            // nothing known of the points yet
             e = cc_launch_assign_tensor(ctx, L, b.Xs, N, g, C, K, b.idx_s, b.dist_s, nullptr, nullptr, st);
             have_max = false;
         } else {

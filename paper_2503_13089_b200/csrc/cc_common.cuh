@@ -163,7 +163,8 @@ cudaError_t cc_launch_assign_tail(cc_ctx*, const WsLayout&, const uint16_t* X, i
                                   cudaStream_t);
 
 // Spatial order and pruned E-step.
-bool cc_prune_applies(int64_t N, int K);
+bool cc_prune_applies(int64_t N, int g, int K);
+constexpr int CC_PRUNE_G = 8;          // longest sub-vectors for which it is ever the faster
 size_t cc_prune_gap_words(int64_t N, int K);
 int cc_tree_positions(int K);
 cudaError_t cc_launch_tree(cc_ctx*, const float* C, int K, int g, unsigned* order, unsigned* scratch, unsigned* tree, cudaStream_t);

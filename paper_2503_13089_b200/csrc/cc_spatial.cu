@@ -402,10 +402,7 @@ cudaError_t cc_launch_tree(cc_ctx* ctx, const float* C, int K, int g, unsigned* 
     switch (g) {                                                                                    \
         case 1: CALL(1); break;   case 2: CALL(2); break;   case 3: CALL(3); break;                 \
         case 4: CALL(4); break;   case 5: CALL(5); break;   case 6: CALL(6); break;                 \
-        case 7: CALL(7); break;   case 8: CALL(8); break;   case 9: CALL(9); break;                 \
-        case 10: CALL(10); break; case 11: CALL(11); break; case 12: CALL(12); break;               \
-        case 13: CALL(13); break; case 14: CALL(14); break; case 15: CALL(15); break;               \
-        case 16: CALL(16); break;                                                                   \
+        case 7: CALL(7); break;   case 8: CALL(8); break;                                           \
         default: return cudaErrorInvalidValue;                                                      \
     }
 

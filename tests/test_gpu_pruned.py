@@ -39,9 +39,9 @@ def _fit(X, g, K, iters, C0, path):
 
 
 @pytest.mark.parametrize("N,g,K,iters,kind", [
-    (4194304, 4, 2048, 3, "heavy"), (2100001, 4, 4097, 4, "ties"), (1000003, 3, 9000, 4, "heavy"), (400129, 6, 24003, 5, "clumps"),
-    (2200000, 2, 4100, 3, "heavy"), (300031, 1, 30000, 3, "heavy"), (150001, 7, 65500, 5, "heavy"), (150000, 8, 65536, 5, "ties"),
-    (262144, 5, 32833, 6, "heavy"), (140000, 6, 65535, 4, "ties"),
+    (2100001, 4, 4097, 17, "ties"), (1000003, 4, 16385, 4, "heavy"), (2000003, 3, 9001, 2, "heavy"), (400129, 6, 24003, 17, "clumps"),
+    (2200000, 2, 4100, 5, "heavy"), (300031, 1, 30000, 5, "heavy"), (150001, 7, 65500, 17, "heavy"), (150000, 8, 65536, 17, "ties"),
+    (524288, 5, 65535, 5, "heavy"), (140000, 6, 65535, 6, "ties"), (4000001, 4, 8193, 2, "clumps"), (2000003, 6, 61000, 5, "heavy"),
 ])
 def test_pruned_fit_equals_exhaustive_fit(N, g, K, iters, kind):
     from paper_2503_13089_b200 import binding as cc
@@ -71,7 +71,7 @@ def test_pruned_fit_equals_exhaustive_fit(N, g, K, iters, kind):
 
 
 def test_objectives_of_a_longer_fit_start_with_those_of_a_shorter_one():
-    """g = 8: three iterations run exhaustively, four in spatial order; the first three objectives have the same bits."""
+    """g = 8: fifteen iterations run exhaustively, sixteen in spatial order; the first objectives have the same bits."""
     from paper_2503_13089_b200 import binding as cc
     from tests import gpu_util as u
     N, g, K = 150000, 8, 60001
@@ -79,14 +79,14 @@ def test_objectives_of_a_longer_fit_start_with_those_of_a_shorter_one():
     X = _points(N, g, K, "heavy")
     C0 = torch.empty((K, g), device="cuda")
     cc.cc_init_codebook(u.ctx(), X, N, g, K, 1, C0)
-    t3, t4 = _fit(X, g, K, 3, C0, cc.PATH_AUTO)[4], _fit(X, g, K, 4, C0, cc.PATH_AUTO)[4]
-    assert torch.equal(t3, t4[:3])
+    shorter, longer = _fit(X, g, K, 15, C0, cc.PATH_AUTO)[4], _fit(X, g, K, 16, C0, cc.PATH_AUTO)[4]
+    assert torch.equal(shorter, longer[:15])
 
 
 def test_pruned_non_finite_input_is_reported():
     from paper_2503_13089_b200 import binding as cc
     from tests import gpu_util as u
-    N, g, K = 150000, 4, 60000
+    N, g, K = 600000, 4, 60000
     u.ctx().ensure_workspace(N, g, K)
     X = _points(N, g, K, "heavy")
     C0 = torch.empty((K, g), device="cuda")
