@@ -7,25 +7,9 @@ namespace {
 
 constexpr int TD = 64;   // transpose tile edge (elements)
 
-// PAPER_T reshape is a 2-D transpose with zero padding: X viewed as d_in x out_pad holds W^T.
-// 64 x 64 tiles go through shared memory so that both the reads (along d_in) and the writes
-// (along out_pad) are contiguous.
-__global__ void __launch_bounds__(256)
-reshape_transpose_kernel(const uint16_t* __restrict__ W, int64_t d_out, int64_t d_in, int64_t out_pad,
-                         uint16_t* __restrict__ X) {
-    __shared__ uint16_t tile[TD][TD + 2];
-    const int64_t i0 = (int64_t)blockIdx.x * TD, o0 = (int64_t)blockIdx.y * TD;
-    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
-    for (int r = ty; r < TD; r += 4) {          // r: out_feature within the tile, tx: in_feature
-        const int64_t o = o0 + r, i = i0 + tx;
-        tile[r][tx] = (o < d_out && i < d_in) ? W[o * d_in + i] : (uint16_t)0;
-    }
-    __syncthreads();
-    for (int r = ty; r < TD; r += 4) {          // r: in_feature within the tile, tx: out_feature
-        const int64_t i = i0 + r, o = o0 + tx;
-        if (i < d_in && o < out_pad) X[i * out_pad + o] = tile[tx][r];
-    }
-}
+// PAPER_T reshape is a 2-D transpose with zero padding: X viewed as d_in x out_pad holds W^T; decode is the other
+// way round.  64 x 64 tiles go through shared memory so that both the reads (along one dimension) and the writes (along
+// the other) are contiguous.
 
 // ---- 16-byte versions of the two transposing kernels (taken when every row is a whole number of
 // 8-element groups).  A 64 x 64 tile goes through shared memory as 32-bit words (two elements),
@@ -118,6 +102,132 @@ decode_transpose_vec_kernel(const uint16_t* __restrict__ C16, const uint16_t* __
             if (o < d_out) *reinterpret_cast<uint4*>(W_hat + o * d_in + i) = even;
             if (o + 1 < d_out) *reinterpret_cast<uint4*>(W_hat + (o + 1) * d_in + i) = odd;
         }
+    }
+}
+
+// ---- Any row length: the same tiles, global memory in 32-bit words of two elements.
+// Elements 0..63 of a run that starts at element `off` (any parity) of `base` (4-byte aligned): lane l holds elements
+// 2l, 2l + 1 and the first n of them are stored.  Called by whole warps.
+__device__ __forceinline__ void store_run(uint16_t* __restrict__ base, int64_t off, int n, unsigned w, int lane) {
+    const unsigned next = __shfl_down_sync(0xffffffffu, w, 1);
+    if ((off & 1) == 0) {
+        if (2 * lane + 1 < n) *reinterpret_cast<unsigned*>(base + off + 2 * lane) = w;
+        else if (2 * lane < n) base[off + 2 * lane] = (uint16_t)w;
+    } else {                                    // words hold elements 2l + 1, 2l + 2
+        if (lane == 0 && n > 0) base[off] = (uint16_t)w;
+        if (lane < 31 && 2 * lane + 2 < n) *reinterpret_cast<unsigned*>(base + off + 2 * lane + 1) = __byte_perm(w, next, 0x5432);
+        else if (2 * lane + 1 < n) base[off + 2 * lane + 1] = (uint16_t)(w >> 16);
+    }
+}
+
+// Rows 2 rp, 2 rp + 1 of the transposed tile (columns of the tile as it lies in shared memory), elements 2l, 2l + 1.
+__device__ __forceinline__ void tile_columns(const unsigned* tile, int rp, int lane, unsigned& even, unsigned& odd) {
+    const unsigned a = tile[tile_row(2 * lane) + rp], b = tile[tile_row(2 * lane + 1) + rp];
+    even = __byte_perm(a, b, 0x5410);
+    odd = __byte_perm(a, b, 0x7632);
+}
+
+// 8192 x 8192, g = 6, reshape and codebook gradient together (element by element 341 us): 255 us.
+__global__ void __launch_bounds__(256)
+reshape_transpose_any_kernel(const uint16_t* __restrict__ W, int64_t d_out, int64_t d_in, int64_t out_pad,
+                             uint16_t* __restrict__ X) {
+    __shared__ unsigned tile[TILE_WORDS];
+    const int64_t i0 = (int64_t)blockIdx.x * TD, o0 = (int64_t)blockIdx.y * TD;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if ((d_in & 7) == 0) {
+        const int c = threadIdx.x & 7, r0 = threadIdx.x >> 3;
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const int r = r0 + 32 * p;
+            const int64_t o = o0 + r, i = i0 + 8 * c;
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (o < d_out && i < d_in) v = __ldg(reinterpret_cast<const uint4*>(W + o * d_in + i));
+            tile_put8(tile, r, c, v);
+        }
+    } else {
+        const int64_t i = i0 + 2 * lane;
+        unsigned w[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            const int64_t o = o0 + warp + 8 * m;
+            w[m] = 0u;
+            if (o < d_out && i < d_in) {
+                const uint16_t* src = W + o * d_in + i;
+                if ((d_in & 1) == 0) w[m] = __ldg(reinterpret_cast<const unsigned*>(src));
+                else w[m] = (unsigned)__ldg(src) | (i + 1 < d_in ? (unsigned)__ldg(src + 1) << 16 : 0u);
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < 8; ++m) tile[tile_row(warp + 8 * m) + lane] = w[m];
+    }
+    __syncthreads();
+    const int n = (int)(out_pad - o0 < TD ? out_pad - o0 : TD);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        unsigned even, odd;
+        tile_columns(tile, warp + 8 * m, lane, even, odd);
+        const int64_t i = i0 + 2 * (warp + 8 * m);
+        if (i < d_in) store_run(X, i * out_pad + o0, n, even, lane);
+        if (i + 1 < d_in) store_run(X, (i + 1) * out_pad + o0, n, odd, lane);
+    }
+}
+
+// A lane owns out_features 2l, 2l + 1 of the tile, so that its place inside the codebook row is found once; with even g the
+// two are one word of one row, with odd g two values of one row or of two.
+// 8192 x 8192, K = 65536 (element by element 179 us, most of it in a 64-bit division for each): g = 6 76 us, g = 7
+// 88 us.
+template <bool EVEN_G>
+__global__ void __launch_bounds__(256)
+decode_transpose_any_kernel(const uint16_t* __restrict__ C16, int K, int g, const uint16_t* __restrict__ idx, int64_t d_out,
+                            int64_t d_in, int64_t out_pad, uint16_t* __restrict__ W_hat) {
+    __shared__ unsigned tile[TILE_WORDS];
+    const int64_t i0 = (int64_t)blockIdx.x * TD, o0 = (int64_t)blockIdx.y * TD;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned kmax = (unsigned)K - 1u;
+    {
+        const int64_t opg = out_pad / g;
+        const unsigned o = (unsigned)o0 + 2u * lane, grp0 = o / (unsigned)g, t0 = o - grp0 * (unsigned)g;
+        const unsigned grp1 = t0 + 1 == (unsigned)g ? grp0 + 1 : grp0, t1 = t0 + 1 == (unsigned)g ? 0u : t0 + 1;
+        const bool live0 = o < out_pad, live1 = o + 1 < out_pad;
+        unsigned c0[8], c1[8], w[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            const int64_t i = i0 + warp + 8 * m;
+            const uint16_t* row = idx + i * opg;
+            c0[m] = (live0 && i < d_in) ? (unsigned)__ldg(row + grp0) : 0u;
+            if constexpr (!EVEN_G) c1[m] = (live1 && i < d_in) ? (unsigned)__ldg(row + grp1) : 0u;
+        }
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {            // a code beyond the codebook must not leave it
+            if constexpr (EVEN_G) {
+                w[m] = __ldg(reinterpret_cast<const unsigned*>(C16 + (int64_t)min(c0[m], kmax) * g + t0));
+            } else {
+                w[m] = (unsigned)__ldg(C16 + (int64_t)min(c0[m], kmax) * g + t0) | (unsigned)__ldg(C16 + (int64_t)min(c1[m], kmax) * g + t1) << 16;
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < 8; ++m) tile[tile_row(warp + 8 * m) + lane] = w[m];
+    }
+    __syncthreads();
+    if ((d_in & 7) == 0) {
+        const int c = threadIdx.x & 7, r0 = threadIdx.x >> 3;
+        uint4 even, odd;
+        tile_column8x2(tile, c, r0, even, odd);
+        const int64_t o = o0 + 2 * r0, i = i0 + 8 * c;
+        if (i < d_in) {
+            if (o < d_out) *reinterpret_cast<uint4*>(W_hat + o * d_in + i) = even;
+            if (o + 1 < d_out) *reinterpret_cast<uint4*>(W_hat + (o + 1) * d_in + i) = odd;
+        }
+        return;
+    }
+    const int n = (int)(d_in - i0 < TD ? d_in - i0 : TD);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        unsigned even, odd;
+        tile_columns(tile, warp + 8 * m, lane, even, odd);
+        const int64_t o = o0 + 2 * (warp + 8 * m);
+        if (o < d_out) store_run(W_hat, o * d_in + i0, n, even, lane);
+        if (o + 1 < d_out) store_run(W_hat, (o + 1) * d_in + i0, n, odd, lane);
     }
 }
 
@@ -442,31 +552,6 @@ reshape_rows_kernel(const uint16_t* __restrict__ W, int64_t d_out, int64_t d_in,
     }
 }
 
-// PAPER_T decode: W_hat[o][i] = C16[idx[(i*out_pad + o) / g]][(i*out_pad + o) % g].  The gather
-// runs along o (contiguous in the codes and in each codebook row), the store along i.
-__global__ void __launch_bounds__(256)
-decode_transpose_kernel(const uint16_t* __restrict__ C16, int g, const uint16_t* __restrict__ idx, int64_t d_out,
-                        int64_t d_in, int64_t out_pad, uint16_t* __restrict__ W_hat) {
-    __shared__ uint16_t tile[TD][TD + 2];
-    const int64_t i0 = (int64_t)blockIdx.x * TD, o0 = (int64_t)blockIdx.y * TD;
-    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
-    for (int r = ty; r < TD; r += 4) {          // r: in_feature, tx: out_feature
-        const int64_t i = i0 + r, o = o0 + tx;
-        uint16_t v = 0;
-        if (i < d_in && o < d_out) {
-            const int64_t flat = i * out_pad + o;
-            const int64_t n = flat / g;
-            v = __ldg(C16 + (int64_t)__ldg(idx + n) * g + (flat - n * g));
-        }
-        tile[r][tx] = v;
-    }
-    __syncthreads();
-    for (int r = ty; r < TD; r += 4) {          // r: out_feature, tx: in_feature
-        const int64_t o = o0 + r, i = i0 + tx;
-        if (o < d_out && i < d_in) W_hat[o * d_in + i] = tile[tx][r];
-    }
-}
-
 // ROWS decode: W_hat[o][i] = C16[idx[(o*in_pad + i) / g]][(o*in_pad + i) % g].
 __global__ void __launch_bounds__(256)
 decode_rows_kernel(const uint16_t* __restrict__ C16, int g, const uint16_t* __restrict__ idx, int64_t d_out,
@@ -521,7 +606,7 @@ cudaError_t cc_launch_reshape(cc_ctx* ctx, const uint16_t* W, int64_t d_out, int
         if (d_in % 8 == 0 && out_pad % 8 == 0)
             reshape_transpose_vec_kernel<<<grid, 256, 0, st>>>(W, d_out, d_in, out_pad, X);
         else
-            reshape_transpose_kernel<<<grid, 256, 0, st>>>(W, d_out, d_in, out_pad, X);
+            reshape_transpose_any_kernel<<<grid, 256, 0, st>>>(W, d_out, d_in, out_pad, X);
     } else {
         const int64_t in_pad = pad_to(d_in, g);
         int64_t blocks = (d_out * in_pad + 255) / 256;
@@ -556,7 +641,8 @@ cudaError_t cc_launch_decode(cc_ctx* ctx, const uint16_t* C16, int K, int g, con
         if (vec && g == 4) decode_transpose_vec_kernel<4><<<grid, 256, 0, st>>>(C16, idx, d_out, d_in, out_pad, W_hat);
         else if (vec && g == 8) decode_transpose_vec_kernel<8><<<grid, 256, 0, st>>>(C16, idx, d_out, d_in, out_pad, W_hat);
         else if (vec && g == 16) decode_transpose_vec_kernel<16><<<grid, 256, 0, st>>>(C16, idx, d_out, d_in, out_pad, W_hat);
-        else decode_transpose_kernel<<<grid, 256, 0, st>>>(C16, g, idx, d_out, d_in, out_pad, W_hat);
+        else if (g % 2 == 0) decode_transpose_any_kernel<true><<<grid, 256, 0, st>>>(C16, K, g, idx, d_out, d_in, out_pad, W_hat);
+        else decode_transpose_any_kernel<false><<<grid, 256, 0, st>>>(C16, K, g, idx, d_out, d_in, out_pad, W_hat);
     } else {
         const int64_t in_pad = pad_to(d_in, g);
         int64_t blocks = (d_out * d_in + 255) / 256;
