@@ -10,6 +10,10 @@ one JSON line; it also carries, under "workloads", a short run of every other co
 With N > 1 every rank clusters its own matrices (different seeds) and no data crosses ranks: the
 paper's "clustering of different matrices is independent".
 
+The unit counts distances that are evaluated, so the headline, its rooflines and the other configurations run the
+exhaustive E-step on the tensor cores.  The library's default path rules centroids out without evaluating them where that is
+faster and gives the same codes, centroids and distances; its times stand beside them under "default_path".
+
 `--kernel` runs one entry point a few times on a synthetic case of the given size and prints the
 mean device time per kernel class (the small cases the ncu summaries under profiles/ were taken on).
 """
@@ -98,7 +102,7 @@ class ClockSampler:
 
 def contraction_columns(g: int) -> int:
     """Length of the FP16 contraction the tensor-core scan runs for sub-vector dimension g (the
-    library's choice of operand pieces: see TcCfg in csrc/cc_assign_tensor.cu)."""
+    library's choice of operand pieces: see TcCfg in csrc/cc_assign_tensor.cuh)."""
     kd34, kd24, kd22 = ((3 * g + 4 + 15) // 16 * 16, (2 * g + 4 + 15) // 16 * 16, (2 * g + 2 + 15) // 16 * 16)
     return kd34 if (kd34 <= 48 and kd34 <= min(kd24, kd22)) else min(kd24, kd22)
 
@@ -523,7 +527,8 @@ def main():
 
     ctx = cc.Context(local_rank)
     path = {"auto": cc.PATH_AUTO, "ffma": cc.PATH_FFMA, "tensor": cc.PATH_TENSOR}[args.path]
-    cc.cc_set_path(ctx, path)
+    exhaustive = cc.PATH_TENSOR if args.path == "auto" else path
+    cc.cc_set_path(ctx, exhaustive)
     layout = cc.LAYOUT_PAPER_T
     peaks = measured_peaks()
     flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")   # > L2 (126 MB)
@@ -560,9 +565,20 @@ def main():
     resolved = run.near_ties()
     cc.cc_poll_status(ctx)
     ms_local = sum(ms_steps) / len(ms_steps)
+    default_ms = default_e2e_ms = None
+    if args.path == "auto":
+        cc.cc_set_path(ctx, cc.PATH_AUTO)
+        run.step()
+        default_ms = run.timed(args.steps, flush, barrier)[0]
+        cc.cc_poll_status(ctx)
+        cc.cc_set_path(ctx, exhaustive)
     run.free_device()
     e2e_ms, h2d, d2h = run.e2e(args.steps, 1, flush, barrier)
     e2e_local = sum(e2e_ms) / len(e2e_ms)
+    if args.path == "auto":
+        cc.cc_set_path(ctx, cc.PATH_AUTO)
+        default_e2e_ms = run.e2e(args.steps, 1, flush, barrier)[0]
+        cc.cc_set_path(ctx, exhaustive)
 
     # ---------------- max over ranks
     evals_step_local = sum(N * w.K * (w.iters + 1) for N in run.Ns)   # iters E-steps + the final one
@@ -636,10 +652,18 @@ def main():
                 c2 = s2.stop()
                 nt2 = r2.near_ties()
                 cc.cc_poll_status(ctx)
+                default2 = None
+                if args.path == "auto":
+                    cc.cc_set_path(ctx, cc.PATH_AUTO)
+                    r2.step()
+                    default2 = r2.timed(2, flush, barrier)[0]
+                    cc.cc_poll_status(ctx)
+                    cc.cc_set_path(ctx, exhaustive)
                 sm2 = summarise(w2, r2.Ns, ph2, 1, peaks, ceiling_for(w2.g), args.path)
                 ms2m = sum(ms2) / len(ms2)
                 others.append({"workload": name, "g": w2.g, "K": w2.K, "iters": w2.iters, "N_per_matrix": r2.Ns,
                                "steps": 2, "warmup": 1, "ms_per_step": ms2m,
+                               "default_path": {"ms_per_step": sum(default2) / len(default2)} if default2 else None,
                                "value": sum(N * w2.K * (w2.iters + 1) for N in r2.Ns) / (ms2m * 1e-3),
                                "s_per_lloyd_iteration": sm2["s_per_lloyd_iteration"],
                                "scan": sm2["scan"], "e_step": sm2["e_step"],
@@ -678,7 +702,7 @@ def main():
             "dtype": "f32", "data": "synthetic",
             "config": {"workload": w.name, "matrices_per_rank": len(specs), "g": g, "K": K, "iters": iters,
                        "N_per_matrix": Ns_head,
-                       "layout": "paper_transpose", "path": args.path,
+                       "layout": "paper_transpose", "path": "tensor" if args.path == "auto" else args.path,
                        "l2": "flushed between timed steps (256 MB write)",
                        "step": "reshape + init + %d x (assign + update) + finalize + decode per matrix" % iters},
             "s_per_lloyd_iteration": summ["s_per_lloyd_iteration"],
@@ -690,6 +714,9 @@ def main():
                     "api": "cc_compress_host: pinned host W in; FP16 codebook, codes, objective trace and the decoded "
                            "matrix out (the same work as the device-resident step plus the copies); its device buffer "
                            "is allocated by one untimed call"},
+            "default_path": {"ms_per_step": sum(default_ms) / len(default_ms), "e2e_ms_per_step": sum(default_e2e_ms) / len(default_e2e_ms),
+                             "note": "this rank; the same step with the library's own choice of E-step: same codes, centroids and "
+                                     "distances, not every distance evaluated"} if default_ms else None,
             "gpu_launches": launches,
             "roofline": roofline,
             "hbm_kernels": summ["hbm_kernels"],
