@@ -118,11 +118,11 @@ constexpr int CC_OBJ_BLOCKS = 1024;    // partial sums of the objective reductio
 
 WsLayout cc_ws_layout(int64_t N, int g, int K);
 
-// Copies of the M-step's sums (small codebooks only: at most CC_SUM_COPY_ELEMS words per array).
+// Copies of the M-step's sums (at most CC_SUM_COPY_ELEMS words per array).
 #ifndef CC_SUM_COPIES_MAX
 #define CC_SUM_COPIES_MAX 16
 #endif
-constexpr int CC_SUM_COPY_ELEMS = 262144;
+constexpr int CC_SUM_COPY_ELEMS = 1048576;
 static inline int cc_sum_copies(int K, int g) {
     const int r = CC_SUM_COPY_ELEMS / (K * g);
     return r < 1 ? 1 : (r > CC_SUM_COPIES_MAX ? CC_SUM_COPIES_MAX : r);

@@ -24,7 +24,9 @@ namespace {
 // sector at G = 4, one 128-byte line at G = 16), so a warp's reduction instruction touches 32 / G
 // sectors instead of 32.  With few clusters the same words are hit by many points at once and the
 // reductions queue up in L2; the sums are then kept in R copies (copy = block % R, one after the
-// other, `copy_elems` words apart; the counts likewise, K apart) which the finish kernel adds up.
+// other, `copy_elems` words apart; the counts likewise, K apart) which the finish kernel adds up.  With many clusters
+// of uneven size four copies still pay: 4.2 M points, g = 4, K = 65536, the popular quarter of the codes used by half of
+// the points 65 us with one copy, 47 with four (codes all used alike 42 and 43).
 // COUNT: the gradient with respect to the codebook needs no counts, and a point's count is a request of its own beside
 // the one or two of its sums.
 template <int G, bool COUNT>
@@ -280,10 +282,8 @@ cudaError_t accumulate_all(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, in
     }
     int32_t* cc = R > 1 ? reinterpret_cast<int32_t*>(ws + L.count_copies) : counts;
     *count_copies = cc;
-    const size_t used = sizeof(ull) * (size_t)K * g * R;
-    cudaError_t e;
-    if ((e = cudaMemsetAsync(sum_lo, 0, used, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(sum_hi, 0, used, st)) != cudaSuccess) return e;
+    cudaError_t e;       // the two arrays lie one behind the other
+    if ((e = cudaMemsetAsync(sum_lo, 0, L.sum_hi - L.sum_lo + sizeof(ull) * (size_t)K * g * R, st)) != cudaSuccess) return e;
     if (!want_counts) cc = nullptr;
     else if ((e = cudaMemsetAsync(cc, 0, sizeof(int32_t) * (size_t)K * R, st)) != cudaSuccess) return e;
     if (N > 0) {
