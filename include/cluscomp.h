@@ -61,14 +61,15 @@ typedef enum {
                                in_features zero-padded to a multiple of g.                   */
 
 /* Which E-step kernel family cc_assign uses. */
-#define CC_PATH_AUTO 0   /* the faster path: measured, the tensor-core one for every g */
+#define CC_PATH_AUTO 0   /* by size: exhaustive on the tensor cores, chunks of centroids ruled out first, or direct */
 #define CC_PATH_FFMA 1   /* FP32 FMA pipes, register-tiled                             */
 #define CC_PATH_TENSOR 2 /* tcgen05 tensor cores with TMEM accumulators                */
 
 typedef struct cc_ctx cc_ctx; /* opaque; one per device and per concurrent user */
 
 /* Context.  cc_create binds to `device` (cudaSetDevice is called inside every entry point).
- * cc_destroy frees host state and the buffer of cc_compress_host; the workspace stays the caller's. */
+ * cc_destroy frees host state and the buffers of cc_compress_host (device, and 512 KB of page-locked host memory);
+ * the workspace stays the caller's. */
 cc_status cc_create(cc_ctx** out, int device);
 cc_status cc_destroy(cc_ctx* ctx);
 const char* cc_status_string(cc_status s);
@@ -336,14 +337,15 @@ cc_status cc_decode(cc_ctx* ctx, const uint16_t* C16, int K, int g, const uint16
 
 /* Forward of the compressed linear layer, appendix listing (ClusCompLinear.forward):
  *   weight = codebook[code].view(in_features, -1) with the padded columns dropped;  y = x . weight (+ bias).
- * The decoded weight is never written to memory: codebook rows are gathered straight into the
- * shared-memory operand of a tensor-core GEMM (FP16 inputs, FP32 accumulation).
+ * Up to a few hundred tokens the decoded weight is never written to memory: codebook rows are looked up in, or gathered
+ * straight into, shared memory (FP16 inputs, FP32 accumulation).  From there on it is decoded once per call into tiles
+ * in the workspace (at most 128 MB at a time) and multiplied by a tensor-core GEMM.
  * x: M x d_in FP16 row-major (M tokens).  C16: K x g FP16.  idx: cc_num_subvectors(d_out, d_in, g,
  * CC_LAYOUT_PAPER_T) codes, each < K.  bias (may be NULL): d_out FP32.  y (out): M x d_out FP32
  * row-major.  The listing keeps every tensor in a 16-bit type; here the accumulator is handed out
  * unrounded.  Scratch: cc_linear_workspace_bytes(M, d_out, d_in) bytes of the context's workspace
- * (cc_set_workspace; used when the in_features are split across thread blocks, which happens for
- * small M; the partial sums are added in a fixed order, so the result is the same on every call).
+ * (cc_set_workspace; partial sums where the in_features are split across thread blocks, the tiles of many tokens; sums are
+ * added in a fixed order, so the result is the same on every call).
  * 1 <= M < 2^31 / d_out; x, C16, y 16-byte aligned. */
 size_t cc_linear_workspace_bytes(cc_ctx* ctx, int64_t M, int64_t d_out, int64_t d_in);
 cc_status cc_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, const uint16_t* C16, int K, int g,

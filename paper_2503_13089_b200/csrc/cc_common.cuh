@@ -188,7 +188,7 @@ cudaError_t cc_launch_small(cc_ctx*, const WsLayout&, const uint16_t* X, int64_t
 // Scratch of the layer forward in the workspace: the status block, a copy of the codebook with padded rows, the rest.
 constexpr size_t CC_LINEAR_SCRATCH_FROM = CC_STATUS_BYTES + (size_t)65536 * 32;
 
-// Compressed linear layer: y = x . decode(C16, idx)^T (+ bias), the decoded weight never stored.
+// Compressed linear layer: y = x . decode(C16, idx)^T (+ bias).
 size_t cc_linear_scratch_bytes(int64_t M, int64_t d_out, int64_t d_in, int sm_count);
 int cc_linear_q_table_max(void);
 // The same for many tokens (cc_linear_wide.cu): the weight is decoded once into tiles in the workspace.

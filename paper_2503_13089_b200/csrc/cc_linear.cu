@@ -1,5 +1,7 @@
 // Forward of the compressed linear layer (appendix listing): out = x . weight (+ bias) with
 // weight = codebook[code] viewed as (in_features, out_features + pad), the padded columns dropped.
+// Three ways: a few tokens look the codes up in shared memory (linear_gemv_kernel below), many multiply a weight decoded
+// once (cc_linear_wide.cu), those in between take the kernel described here.
 // The decoded weight is never written to memory: the kernel gathers codebook rows straight into the
 // shared-memory operand of a tcgen05 GEMM.
 //
