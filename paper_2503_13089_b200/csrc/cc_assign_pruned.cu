@@ -411,7 +411,9 @@ pruned_list_kernel(const ListArgs a) {
 // an MMA, a further one 45, the MMA and its commit together 48 (N = 64); a waiting warp is back at work about 90
 // cycles after the arrival.  What counts is therefore the chain of a pair: announcement, load of the accumulator, its
 // release, next MMA.  Per 128 x 64 block and SM: one issuer for four tiles 335 cycles, one issuer per tile 222; a
-// pipeline per tile with a handshake per chunk 217, per pair 167 with one accumulator and both chunks by the same warp.
+// pipeline per tile with a handshake per chunk 217, per pair 167 with one accumulator and both chunks by the same warp
+// (2.8 M points, K = 65,500, g = 6, twenty iterations 87 ms); there the thread that issued and copied took 700 cycles a
+// pair, and with both waits in one round trip, the copies on a warp of their own and two accumulators 83.5 ms.
 constexpr int PS_EPI = 8;
 constexpr int PS_THREADS = (PS_EPI + 2) * 32;
 constexpr int PS_BLOCKS = 2;             // resident per SM
@@ -421,7 +423,7 @@ constexpr int PS_RING = 8;
 template <int G> struct PrCfg {
     using Cfg = TcCfg<G>;
     static constexpr int CH_BYTES = PR_CHUNK * Cfg::KD * 2;
-    static constexpr int STAGES = Cfg::KD == 16 ? 10 : Cfg::KD == 32 ? 6 : 4;   // pairs of chunks
+    static constexpr int STAGES = Cfg::KD == 16 ? 10 : 6;   // pairs of chunks
     static constexpr int SMEM = 2 * Cfg::A_TILE + STAGES * 2 * CH_BYTES + PS_LISTS * PR_MAX_CHUNKS * 2 + 2 * 3 * TM * 4 + 512;
 };
 

@@ -2,7 +2,7 @@
 //
 // cc_linear.cu gathers codebook rows straight into the operand of the MMA, once per block of tokens.  Every gather
 // is a request for one L2 sector, and an SM gets about 0.73 of those through per clock; at 4096 tokens that, not the
-// product, was the time (8 gathers per weight group: 440 us for 4096 x 4096, g = 4, K = 65536, 142 us this way; the product alone takes
+// product, was the time (8 gathers per weight group: 440 us for 4096 x 4096, g = 4, K = 65536, 138 us this way; the product alone takes
 // 82 us at the rate a library GEMM reaches).  From a few hundred tokens on it is cheaper to gather once:
 //   1. linear_prepare_kernel  decodes the weight into FP16 tiles that are the byte image of the MMA's operand (128
 //                             out_features x 64 in_features, canonical K-major layout without swizzle), and lays x out in
@@ -122,22 +122,31 @@ linear_prepare_kernel(const uint16_t* __restrict__ C16, bool padded, const unsig
     uint4* dst = reinterpret_cast<uint4*>(x_tiles + (int64_t)b * NT * (WKB * 2));
     const int m0 = m_first + tt * NT;
     const bool vec = (d_in & 7) == 0;
-    for (int s = tid; s < NT * (WKB / 8); s += PREP_THREADS) {
-        const int kc = s & 7, r = s >> 3;
-        const int m = m0 + r, i = c * WKB + kc * 8;
-        uint4 w = make_uint4(0u, 0u, 0u, 0u);
-        if (m < M && i < d_in) {
-            const uint16_t* src = x + (int64_t)m * d_in + i;
-            if (vec) {
-                w = __ldg(reinterpret_cast<const uint4*>(src));
-            } else {
-                unsigned h[8];
+    constexpr int BATCH = 4;                         // loads under way per thread
+    for (int s0 = tid; s0 < NT * (WKB / 8); s0 += BATCH * PREP_THREADS) {
+        uint4 w[BATCH];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) h[u] = i + u < d_in ? (unsigned)__ldg(src + u) : 0u;
-                w = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, h[6] | h[7] << 16);
+        for (int u = 0; u < BATCH; ++u) {
+            const int s = s0 + u * PREP_THREADS, kc = s & 7, r = s >> 3;
+            const int m = m0 + r, i = c * WKB + kc * 8;
+            w[u] = make_uint4(0u, 0u, 0u, 0u);
+            if (r < NT && m < M && i < d_in) {
+                const uint16_t* src = x + (int64_t)m * d_in + i;
+                if (vec) {
+                    w[u] = __ldg(reinterpret_cast<const uint4*>(src));
+                } else {
+                    unsigned h[8];
+#pragma unroll
+                    for (int v = 0; v < 8; ++v) h[v] = i + v < d_in ? (unsigned)__ldg(src + v) : 0u;
+                    w[u] = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, h[6] | h[7] << 16);
+                }
             }
         }
-        dst[kc * NT + r] = w;
+#pragma unroll
+        for (int u = 0; u < BATCH; ++u) {
+            const int s = s0 + u * PREP_THREADS, kc = s & 7, r = s >> 3;
+            if (r < NT) dst[kc * NT + r] = w[u];
+        }
     }
 }
 
