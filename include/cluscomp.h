@@ -77,6 +77,10 @@ const char* cc_status_string(cc_status s);
 /* Scratch memory needed by any call on a problem of this size, in bytes (0 on bad arguments).
  * The workspace must stay valid and unshared while calls using it are in flight. */
 size_t cc_workspace_bytes(int64_t N, int g, int K);
+/* The size with which cc_assign, cc_fit and cc_finalize can also take the E-step that rules centroids out first (same results,
+ * up to nine times faster on large problems; it keeps the points in spatial order and lists of what may matter, up to about
+ * (50 + 2 g) bytes per point and a further 4 GB).  Never less than cc_workspace_bytes, with which every call runs. */
+size_t cc_workspace_bytes_preferred(int64_t N, int g, int K);
 cc_status cc_set_workspace(cc_ctx* ctx, void* workspace, size_t bytes);
 
 /* CC_PATH_* override for cc_assign / cc_fit / cc_finalize (default CC_PATH_AUTO).

@@ -35,6 +35,7 @@ SIGNATURES = {
     "cc_destroy": (_i32, [_vp]),
     "cc_status_string": (ct.c_char_p, [_i32]),
     "cc_workspace_bytes": (_sz, [_i64, _i32, _i32]),
+    "cc_workspace_bytes_preferred": (_sz, [_i64, _i32, _i32]),
     "cc_set_workspace": (_i32, [_vp, _vp, _sz]),
     "cc_set_path": (_i32, [_vp, _i32]),
     "cc_launch_count": (_i64, [_vp]),
@@ -141,11 +142,18 @@ class Context:
             pass
 
     def ensure_workspace(self, N: int, g: int, K: int, at_least: int = 0) -> None:
+        """A workspace of the preferred size, or, where memory does not reach that far, of the needed one."""
         need = max(cc_workspace_bytes(N, g, K), at_least)
         if need == 0:
             raise CCError(2, "cc_workspace_bytes")
-        if self._ws is None or self._ws.numel() < need:
-            self._ws = torch.empty(need, dtype=torch.uint8, device="cuda:%d" % self.device)
+        want = max(cc_workspace_bytes_preferred(N, g, K), need)
+        if self._ws is None or self._ws.numel() < want:
+            try:
+                self._ws = torch.empty(want, dtype=torch.uint8, device="cuda:%d" % self.device)
+            except torch.OutOfMemoryError:
+                if self._ws is not None and self._ws.numel() >= need:
+                    return
+                self._ws = torch.empty(need, dtype=torch.uint8, device="cuda:%d" % self.device)
             cc_set_workspace(self, self._ws, self._ws.numel())
 
 
@@ -155,6 +163,10 @@ def cc_status_string(status: int) -> str:
 
 def cc_workspace_bytes(N: int, g: int, K: int) -> int:
     return int(load().cc_workspace_bytes(N, g, K))
+
+
+def cc_workspace_bytes_preferred(N: int, g: int, K: int) -> int:
+    return int(load().cc_workspace_bytes_preferred(N, g, K))
 
 
 def cc_set_workspace(ctx: Context, workspace: Optional[torch.Tensor], nbytes: int) -> None:

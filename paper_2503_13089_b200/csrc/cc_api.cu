@@ -28,6 +28,7 @@ WsLayout cc_ws_layout(int64_t N, int g, int K) {
     L.tensor = take(Kpad * (size_t)(64 + 1) * 4);
     L.tstate = take((size_t)N * 8);
     L.idx_prev = take((size_t)N * 2);
+    L.total = off;
     const bool pr = cc_prune_applies(N, g, K);
     auto take_if = [&](size_t bytes) { size_t o = off; if (pr) off += cc_align_up(bytes, 256); return o; };
     const size_t n_chunks = cc_align_up((size_t)(K + 63) / 64, 8), groups = (size_t)((N + 511) / 512);
@@ -47,11 +48,11 @@ WsLayout cc_ws_layout(int64_t N, int g, int K) {
     L.c_prev = take_if((size_t)K * g * 4);
     L.boxes = take_if(n_chunks * (4 * g + 3) * 4);
     L.moved = take_if(n_chunks * 4);
-    L.total = off;
+    L.total_preferred = off;
     return L;
 }
 
-// Sizes for which a call may run the pruned E-step (see prune_pays): the workspace has room for it.
+// Sizes for which a call may run the pruned E-step (see prune_pays), if the workspace is of the preferred size.
 bool cc_prune_applies(int64_t N, int g, int K) { return g <= CC_PRUNE_G && N >= 32768 && K >= 4096 && N * (int64_t)K >= (int64_t)1 << 33; }
 
 // Words of the per (row block, chunk) gaps kept between the iterations of a fit; none where they would take
@@ -218,15 +219,15 @@ bool prune_pays(int64_t N, int g, int K, int steps) {
     return false;
 }
 
-bool use_pruned(const cc_ctx* ctx, int64_t N, int g, int K, int steps) {
-    return ctx->path == CC_PATH_AUTO && cc_prune_applies(N, g, K) && prune_pays(N, g, K, steps);
+bool use_pruned(const cc_ctx* ctx, const WsLayout& L, int64_t N, int g, int K, int steps) {
+    return ctx->path == CC_PATH_AUTO && cc_prune_applies(N, g, K) && ctx->ws_bytes >= L.total_preferred && prune_pays(N, g, K, steps);
 }
 
 cudaError_t assign_any(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, int g, const float* C, int K,
                        uint16_t* idx, float* dist, double* objective, int64_t* n_resolved, cudaStream_t st) {
     if (cc_small_applies(ctx, N, g, K))
         return cc_launch_small(ctx, L, X, N, g, const_cast<float*>(C), K, SMALL_E, idx, dist, nullptr, objective, n_resolved, st);
-    if (use_pruned(ctx, N, g, K, 1)) {
+    if (use_pruned(ctx, L, N, g, K, 1)) {
         const PruneBuffers b = prune_buffers(ctx, L, N, g, K);
         cudaError_t e = prune_order(ctx, b, X, g, C, st);
         if (e == cudaSuccess) e = cc_launch_assign_pruned(ctx, b, g, C, CC_PRUNE_COLD, st);
@@ -364,6 +365,10 @@ cc_status cc_destroy(cc_ctx* ctx) {
 size_t cc_workspace_bytes(int64_t N, int g, int K) {
     if (g < 1 || g > 16 || K < 1 || K > 65536 || N < 0 || N >= (int64_t)1 << 31) return 0;
     return cc_ws_layout(N, g, K).total;
+}
+
+size_t cc_workspace_bytes_preferred(int64_t N, int g, int K) {
+    return cc_workspace_bytes(N, g, K) ? cc_ws_layout(N, g, K).total_preferred : 0;
 }
 
 cc_status cc_set_workspace(cc_ctx* ctx, void* workspace, size_t bytes) {
@@ -559,7 +564,7 @@ cc_status cc_fit(cc_ctx* ctx, const uint16_t* X, int64_t N, int g, int K, int it
     if (cudaSetDevice(ctx->device) != cudaSuccess) return CC_ERR_CUDA;
     const WsLayout L = cc_ws_layout(N, g, K);
     cudaStream_t st = (cudaStream_t)stream;
-    if (iters > 0 && use_pruned(ctx, N, g, K, iters))
+    if (iters > 0 && use_pruned(ctx, L, N, g, K, iters))
         return from_cuda(fit_pruned(ctx, L, X, N, g, K, iters, C, idx, dist, counts, objective_trace, st));
     if (iters > 0 && cc_small_applies(ctx, N, g, K))
         return from_cuda(fit_small(ctx, L, X, N, g, K, iters, C, idx, dist, counts, objective_trace, st));
@@ -777,20 +782,25 @@ cc_status cc_compress_host(cc_ctx* ctx, const uint16_t* W_host, int64_t d_out, i
     cudaStream_t st = (cudaStream_t)stream;
 
     const size_t w_bytes = (size_t)d_out * d_in * 2, x_bytes = (size_t)N * g * 2;
-    const size_t ws_bytes = cc_ws_layout(N, g, K).total;
-    // one allocation, carved: W | X | C | C16 | idx | trace | workspace | dist | counts; the results and the status word
-    // at the head of the workspace lie in a row
+    const WsLayout L = cc_ws_layout(N, g, K);
+    // one allocation, carved: W | X | C | dist | counts | C16 | idx | trace | workspace; the small results and the status
+    // word at the head of the workspace lie in a row
     size_t off = 0;
     auto take = [&](size_t b) { size_t o = off; off += cc_align_up(b, 256); return o; };
-    const size_t oW = take(w_bytes), oX = take(x_bytes), oC = take((size_t)K * g * 4), oC16 = take((size_t)K * g * 2),
-                 oIdx = take((size_t)N * 2), oTr = take((size_t)(iters + 1) * 8), oWs = take(ws_bytes), oDist = take((size_t)N * 4),
-                 oCnt = take((size_t)K * 4);
-    if (ctx->e2e_bytes < off) {          // grown on demand and kept: repeated calls allocate nothing
+    const size_t oW = take(w_bytes), oX = take(x_bytes), oC = take((size_t)K * g * 4), oDist = take((size_t)N * 4),
+                 oCnt = take((size_t)K * 4), oC16 = take((size_t)K * g * 2), oIdx = take((size_t)N * 2),
+                 oTr = take((size_t)(iters + 1) * 8), oWs = take(0);
+    size_t ws_bytes = L.total_preferred;
+    if (ctx->e2e_bytes < oWs + ws_bytes) {          // grown on demand and kept: repeated calls allocate nothing
         if (ctx->e2e_buf) cudaFree(ctx->e2e_buf);
         ctx->e2e_buf = nullptr;
         ctx->e2e_bytes = 0;
-        if (cudaMalloc(&ctx->e2e_buf, off) != cudaSuccess) return CC_ERR_CUDA;
-        ctx->e2e_bytes = off;
+        if (cudaMalloc(&ctx->e2e_buf, oWs + ws_bytes) != cudaSuccess) {
+            cudaGetLastError();
+            ws_bytes = L.total;                     // less memory: what every call needs
+            if (cudaMalloc(&ctx->e2e_buf, oWs + ws_bytes) != cudaSuccess) return CC_ERR_CUDA;
+        }
+        ctx->e2e_bytes = oWs + ws_bytes;
     }
     char* base = static_cast<char*>(ctx->e2e_buf);
     void* saved_ws = ctx->ws;

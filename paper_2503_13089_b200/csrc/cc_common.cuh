@@ -80,6 +80,7 @@ struct WsLayout {
     size_t tensor;     // staging of the tensor-core E-step (split codebook operand)
     size_t tstate;     // float2 N: (second-best chunk minimum, best chunk id) from the tensor-core scan
     size_t idx_prev;   // u16 N: codes of the previous M-step inside cc_fit
+    size_t total;      // what every call needs
     // pruned E-step (nothing where it does not apply, see cc_prune_applies)
     size_t xs;         // u16 N x g: points in spatial order
     size_t pos;        // u32 N: point -> position
@@ -96,7 +97,7 @@ struct WsLayout {
     size_t c_prev;     // float K x g: codebook of the last E-step
     size_t boxes;      // float chunks x (2 g + 2 g + 3)
     size_t moved;      // float chunks
-    size_t total;
+    size_t total_preferred;
 };
 
 // Buffers of the pruned E-step (cc_assign_pruned.cu), carved from the workspace.

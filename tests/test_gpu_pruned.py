@@ -96,3 +96,29 @@ def test_pruned_non_finite_input_is_reported():
         _fit(X, g, K, 2, C0, cc.PATH_AUTO)
     assert e.value.status == 8
     cc.cc_set_path(u.ctx(), cc.PATH_AUTO)
+
+
+def test_fit_in_the_smaller_workspace_gives_the_same():
+    """cc_workspace_bytes is enough for every call; with cc_workspace_bytes_preferred the same fit may be pruned."""
+    from paper_2503_13089_b200 import binding as cc
+    N, g, K, iters = 1000003, 3, 9000, 5
+    assert cc.cc_workspace_bytes_preferred(N, g, K) > cc.cc_workspace_bytes(N, g, K)
+    assert cc.cc_workspace_bytes_preferred(N, 9, K) == cc.cc_workspace_bytes(N, 9, K)
+    assert cc.cc_workspace_bytes_preferred(N, 17, K) == 0
+    X = _points(N, g, K, "heavy")
+    out = []
+    for size in (cc.cc_workspace_bytes, cc.cc_workspace_bytes_preferred):
+        c = cc.Context(0)
+        ws = torch.empty(size(N, g, K), dtype=torch.uint8, device="cuda")
+        cc.cc_set_workspace(c, ws, ws.numel())
+        C = torch.empty((K, g), device="cuda")
+        cc.cc_init_codebook(c, X, N, g, K, 3, C)
+        idx, dist = torch.empty(N, dtype=torch.uint16, device="cuda"), torch.empty(N, device="cuda")
+        counts, trace = torch.empty(K, dtype=torch.int32, device="cuda"), torch.zeros(iters, dtype=torch.float64, device="cuda")
+        before = cc.cc_launch_count(c)
+        cc.cc_fit(c, X, N, g, K, iters, C, idx, dist, counts, trace)
+        cc.cc_poll_status(c)
+        out.append((C, idx.view(torch.int16), dist, counts, trace, cc.cc_launch_count(c) - before))
+        torch.cuda.synchronize()
+    assert out[0][5] != out[1][5]                        # two different ways
+    assert all(torch.equal(x, y) for x, y in zip(out[0][:5], out[1][:5]))
