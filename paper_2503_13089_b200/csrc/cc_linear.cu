@@ -27,6 +27,7 @@
 
 #include "cc_common.cuh"
 #include "cc_tcgen05.cuh"
+#include "cc_linear_plan.h"
 #include "cc_linear_rows.cuh"
 
 namespace {
@@ -379,11 +380,6 @@ linear_reduce_kernel(const float* __restrict__ partial, int splits, int64_t n, i
 // slab); the slabs are added in order by the CTA that finishes last, or by linear_reduce_kernel: the same bits
 // on every call.
 // blockIdx.x: block of 64 code groups; y: range of rows_per_split in_features; z: slice of slice_rows codebook rows.
-constexpr int LG_THREADS = 1024, LG_GRPS = 64, LG_SUB = 16, LG_M_MAX = 4;
-constexpr int LG_X_MAX = 16 * 1024;                    // bytes of x (FP32) beside the table
-constexpr int LG_SMEM = 226 * 1024, LG_SLICE = LG_SMEM - 128 - LG_X_MAX - 64;   // bytes of a slice
-constexpr int LG_SLICES_MAX = 5;
-
 template <int G>
 __device__ __forceinline__ void gemv_levels(const unsigned char* row, unsigned (&lv)[G]) {
     if constexpr (G == 4) {
@@ -433,14 +429,6 @@ __device__ __forceinline__ void gemv_row(const unsigned char* table, unsigned ro
 #pragma unroll
     for (int t = 0; t < G; ++t) c[t] = __half2float(__ushort_as_half((unsigned short)((t & 1) ? w[t / 2] >> 16 : w[t / 2] & 0xffffu)));
 }
-
-// Rows of codes a thread requests together; the next ones are under way while these are used.
-__host__ __device__ constexpr int gemv_batch(int g, int mt) { return g * mt <= 8 ? 8 : 4; }
-// Neighbouring code groups per thread: two codes come in one word and share the loads of x.  For short rows of the FP16
-// codebook and layers of many codes: one token, g = 4, K = 65536, 11008 x 4096 39.8 -> 33.7 us, 4096 x 4096 18.7 -> 17.2;
-// with few codes the wider exchange at the end costs more (g = 3, 700 x 900 7.7 -> 9.3; g = 8, 4096 x 4096 16.2 -> 17.1).
-__host__ __device__ constexpr bool gemv_pair(int g, bool quant) { return g <= 4 && !quant; }
-constexpr int64_t LG_PAIR_FROM = 1 << 21;              // codes
 
 // PW: code groups per thread, 1 or 2 (2 wants an even number of groups and the codes on a word boundary).
 template <int G, int MT, bool QUANT, int PW>
@@ -641,40 +629,6 @@ linear_pad_rows_kernel(const uint16_t* __restrict__ C16, int K, int g, int pad, 
 // (33 tokens, g = 6, K = 1024: 512 x 512 17.4 us without, 21.5 with it).
 constexpr int64_t LINEAR_PAD_FROM = 400000;
 
-struct GemvPlan { int pw, o_blocks, slices, slice_rows, splits, rows_per_split; size_t smem; };
-
-// Slices of the codebook as its bytes ask for, splits of the in_features by a count of clocks: a CTA pays for its
-// table (about 40 bytes a clock), some 4000 for its beginning and end, and 10 a row of codes; CTAs come in waves of one per SM.
-GemvPlan gemv_plan(int64_t d_in, int out_groups, int sm_count, int K, int g, int mt, bool quant, bool words) {
-    GemvPlan p;
-    p.pw = (words && out_groups % 2 == 0 && gemv_pair(g, quant) && out_groups * d_in >= LG_PAIR_FROM) ? 2 : 1;
-    p.o_blocks = (out_groups / p.pw + LG_GRPS - 1) / LG_GRPS;
-    const size_t row = quant ? (size_t)(g / 2) : (size_t)(2 * g);
-    p.slices = (int)(((size_t)K * row + LG_SLICE - 1) / LG_SLICE);
-    p.slice_rows = (K + p.slices - 1) / p.slices;
-    p.slice_rows = (p.slice_rows + 15) / 16 * 16;
-    p.slices = (K + p.slice_rows - 1) / p.slice_rows;
-    const int step = gemv_batch(g, mt) * LG_SUB, rows_max = LG_X_MAX / (4 * mt) / step * step;
-    const int ctas = p.o_blocks * p.slices;
-    int most = 3 * sm_count / ctas, least = (int)((d_in + rows_max - 1) / rows_max);
-    if ((int64_t)most * LG_SUB > d_in) most = (int)((d_in + LG_SUB - 1) / LG_SUB);   // at least 16 in_features per CTA
-    if (most < least) most = least;
-    double best = 0.0;
-    p.splits = 0;
-    for (int s = least; s <= most; ++s) {
-        const int64_t rows = (d_in + s - 1) / s;
-        const double t = (double)((ctas * s + sm_count - 1) / sm_count) * ((double)(p.slice_rows * row) / 40.0 + 4000.0 + 8.0 * p.pw * (double)rows);
-        if (p.splits == 0 || t < best) { best = t; p.splits = s; }
-    }
-    p.rows_per_split = (int)((d_in + p.splits - 1) / p.splits);
-    p.splits = (int)((d_in + p.rows_per_split - 1) / p.rows_per_split);
-    size_t tail = (size_t)p.slice_rows * row + (quant ? 0 : row + 4);
-    const size_t red = (size_t)(LG_SUB - 1) * g * p.pw * LG_GRPS * 4;
-    if (tail < red) tail = red;
-    p.smem = 128 + (size_t)((p.rows_per_split + step - 1) / step * step) * mt * 4 + (tail + 15) / 16 * 16;
-    return p;
-}
-
 // Tokens from which decoding the weight once and multiplying it afterwards (cc_linear_wide.cu) is the faster way
 // (4096 x 4096, g = 4, K = 65536: 128 tokens 42 against 46 us, 192 tokens 52 against 46, 512 tokens 85 against 52), earlier
 // where the tiles of this kernel fill the SMs by themselves, so that its waves are the coarser (11008 x 4096, g = 8,
@@ -737,12 +691,8 @@ size_t cc_linear_scratch_bytes(int64_t M, int64_t d_out, int64_t d_in, int sm_co
     if (splits > chunks / 4) splits = chunks / 4;
     if (splits < 2) splits = 0;    // a single CTA per tile writes y itself
     if (M <= LG_M_MAX) {
-        // the few-token kernel: three CTAs per SM at the most, or as many splits as x asks for (see gemv_plan); the most
-        // slabs come with the fewest blocks of code groups, i.e. at g = 16
-        const int o_blocks = (int)((d_out / 32 + LG_GRPS - 1) / LG_GRPS);
-        const int64_t least = LG_SLICES_MAX * ((d_in + 511) / 512);
-        const int64_t most = 3 * sm_count / (o_blocks < 1 ? 1 : o_blocks) + LG_SLICES_MAX;
-        if (splits < (most > least ? most : least)) splits = (int)(most > least ? most : least);
+        const int64_t slabs = gemv_slabs_most(d_out, d_in, sm_count);
+        if (splits < slabs) splits = (int)slabs;
     }
     const size_t own = CC_LINEAR_SCRATCH_FROM + (size_t)splits * (size_t)M * (size_t)d_out * 4;
     const size_t wide = M >= LINEAR_WIDE_FEWEST ? cc_linear_wide_bytes(M, d_out, d_in) : 0;
@@ -811,17 +761,6 @@ cudaError_t launch_linear(cc_ctx* ctx, const LinearPlan& p, const uint16_t* x, i
 
 namespace {
 
-// Where the look-up kernel is the faster one.  M x g accumulators must fit the registers of 1024 threads per SM; the
-// FP16 codebook is read once per slice, which costs the less the fewer gathers it saves (4096 x 4096: g = 4, K = 65536
-// 26.9 -> 17.2 us at one token, 26.7 -> 25.7 at four; g = 6, K = 65500, four slices 30.8 -> 22.2 at one, on 11008 x 4096
-// 98 -> 94 at four, where the tensor kernel with padded rows takes 70; g = 16, K = 20000, three slices, two tokens 20.2
-// -> 24.4, not used).
-constexpr int gemv_tokens(int g) { return g <= 8 ? 4 : 2; }                  // 4-bit codebook
-bool gemv_fp16(int64_t M, int K, int g) {
-    return M <= (g <= 4 ? 4 : 2) && (size_t)K * (2 * g) <= (size_t)(g <= 8 ? 4 : 2) * LG_SLICE;
-}
-constexpr int gemv_pad(int64_t M) { return M <= 2 ? (int)M : 4; }
-
 template <int G, int MT, bool QUANT, int PW>
 cudaError_t launch_gemv_w(cc_ctx* ctx, const GemvPlan& p, const uint16_t* x, int M, const void* book,
                         const float* qscale, int K, const uint16_t* idx, int d_out, int d_in, int out_groups, float* out,
@@ -877,9 +816,11 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
     const int out_groups = (int)((d_out + g - 1) / g);
     const int64_t n = M * d_out;
     cudaError_t e = cudaSuccess;
-    if (qtab ? M <= gemv_tokens(g) : gemv_fp16(M, K, g)) {
+    GemvPlan v = {};
+    if (gemv_applies(M, K, g, qtab != nullptr))
+        v = gemv_plan(d_in, out_groups, ctx->sm_count, K, g, gemv_pad(M), qtab != nullptr, (reinterpret_cast<uintptr_t>(idx) & 3u) == 0);
+    if (v.fits) {
         // a handful of tokens: the shared-memory look-up kernel, then the same reduction (it also adds the bias)
-        const GemvPlan v = gemv_plan(d_in, out_groups, ctx->sm_count, K, g, gemv_pad(M), qtab != nullptr, (reinterpret_cast<uintptr_t>(idx) & 3u) == 0);
         const int slabs_n = v.splits * v.slices;
         unsigned* arrived = nullptr;
         {

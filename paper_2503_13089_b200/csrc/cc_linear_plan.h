@@ -1,0 +1,99 @@
+// Host-side plan of the few-token layer forward (linear_gemv_kernel in cc_linear.cu).  No CUDA in here: what a plan asks
+// for can be checked against the kernel's limits without a device.
+#pragma once
+
+#include <stddef.h>
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define CC_PLAN_FN __host__ __device__
+#else
+#define CC_PLAN_FN
+#endif
+
+namespace {
+
+constexpr int LG_THREADS = 1024, LG_GRPS = 64, LG_SUB = 16, LG_M_MAX = 4;
+constexpr int LG_SMEM = 226 * 1024;                    // bytes of shared memory the kernel may have
+constexpr int LG_HEAD = 128;                           // barrier, flag, 4-bit levels
+constexpr int LG_X_MAX = 16 * 1024;                    // bytes of x (FP32) beside the table
+constexpr int LG_SLICES_MAX = 4;
+constexpr int LG_SPLITS_MAX = 65535;                   // gridDim.y
+
+// Rows of codes a thread requests together; the next ones are under way while these are used.
+CC_PLAN_FN constexpr int gemv_batch(int g, int mt) { return g * mt <= 8 ? 8 : 4; }
+// Neighbouring code groups per thread: two codes come in one word and share the loads of x.  For short rows of the FP16
+// codebook and layers of many codes: one token, g = 4, K = 65536, 11008 x 4096 39.8 -> 33.7 us, 4096 x 4096 18.7 -> 17.2;
+// with few codes the wider exchange at the end costs more (g = 3, 700 x 900 7.7 -> 9.3; g = 8, 4096 x 4096 16.2 -> 17.1).
+constexpr bool gemv_pair(int g, bool quant) { return g <= 4 && !quant; }
+constexpr int64_t LG_PAIR_FROM = 1 << 21;              // codes
+
+// Bytes of a codebook row, and of what lies behind the rows of a slice: a row of zeros and a word that the loads of odd rows
+// may touch.
+constexpr size_t gemv_row_bytes(int g, bool quant) { return quant ? (size_t)(g / 2) : (size_t)(2 * g); }
+constexpr size_t gemv_tail_bytes(int g, bool quant) { return quant ? 0 : gemv_row_bytes(g, quant) + 4; }
+
+// Rows of a slice: whole groups of 16 (so that a slice starts on a 16-byte boundary), as many as leave room for a full x.
+constexpr int gemv_slice_most(int g, bool quant) {
+    return (int)((LG_SMEM - LG_HEAD - LG_X_MAX - 15 - gemv_tail_bytes(g, quant)) / gemv_row_bytes(g, quant) / 16 * 16);
+}
+
+// Where the look-up kernel is the faster one.  M x g accumulators must fit the registers of 1024 threads per SM; the
+// FP16 codebook is read once per slice, which costs the less the fewer gathers it saves (4096 x 4096: g = 4, K = 65536
+// 26.9 -> 18.4 us at one token, 26.7 -> 25.7 at four; g = 6, K = 65500, four slices 30.8 -> 22.2 at one, on 11008 x 4096
+// 98 -> 94 at four, where the tensor kernel with padded rows takes 70; g = 16, K = 20000, three slices, two tokens 20.2
+// -> 24.4, not used).
+constexpr int gemv_tokens(int g) { return g <= 8 ? 4 : 2; }                  // 4-bit codebook
+inline bool gemv_applies(int64_t M, int K, int g, bool quant) {
+    if (quant) return M <= gemv_tokens(g);
+    return M <= (g <= 4 ? 4 : 2) && K <= (g <= 8 ? LG_SLICES_MAX : 2) * gemv_slice_most(g, false);
+}
+constexpr int gemv_pad(int64_t M) { return M <= 2 ? (int)M : 4; }
+
+// fits: within what a launch may ask for; where not, the tensor kernel takes the call.
+struct GemvPlan { int pw, o_blocks, slices, slice_rows, splits, rows_per_split; size_t smem; bool fits; };
+
+// Slices of the codebook as its bytes ask for, splits of the in_features by a count of clocks: a CTA pays for its
+// table (about 40 bytes a clock), some 4000 for its beginning and end, and 8 a row of codes (16 where a thread has two
+// groups); CTAs come in waves of one per SM.  mt: tokens rounded up to 1, 2 or 4; words: the codes start on a word boundary.
+inline GemvPlan gemv_plan(int64_t d_in, int out_groups, int sm_count, int K, int g, int mt, bool quant, bool words) {
+    GemvPlan p;
+    p.pw = (words && out_groups % 2 == 0 && gemv_pair(g, quant) && out_groups * d_in >= LG_PAIR_FROM) ? 2 : 1;
+    p.o_blocks = (out_groups / p.pw + LG_GRPS - 1) / LG_GRPS;
+    const size_t row = gemv_row_bytes(g, quant);
+    const int slice_most = gemv_slice_most(g, quant);
+    p.slices = (K + slice_most - 1) / slice_most;
+    p.slice_rows = ((K + p.slices - 1) / p.slices + 15) / 16 * 16;          // at most slice_most
+    p.slices = (K + p.slice_rows - 1) / p.slice_rows;
+    const int step = gemv_batch(g, mt) * LG_SUB, rows_max = LG_X_MAX / (4 * mt) / step * step;
+    const int ctas = p.o_blocks * p.slices;
+    int most = 3 * sm_count / ctas, least = (int)((d_in + rows_max - 1) / rows_max);
+    if ((int64_t)most * LG_SUB > d_in) most = (int)((d_in + LG_SUB - 1) / LG_SUB);   // at least 16 in_features per CTA
+    if (most < least) most = least;
+    double best = 0.0;
+    p.splits = 0;
+    for (int s = least; s <= most; ++s) {
+        const int64_t rows = (d_in + s - 1) / s;
+        const double t = (double)(((int64_t)ctas * s + sm_count - 1) / sm_count) * ((double)(p.slice_rows * row) / 40.0 + 4000.0 + 8.0 * p.pw * (double)rows);
+        if (p.splits == 0 || t < best) { best = t; p.splits = s; }
+    }
+    p.rows_per_split = (int)((d_in + p.splits - 1) / p.splits);
+    p.splits = (int)((d_in + p.rows_per_split - 1) / p.rows_per_split);
+    size_t table = (size_t)p.slice_rows * row + gemv_tail_bytes(g, quant);
+    const size_t red = (size_t)(LG_SUB - 1) * g * p.pw * LG_GRPS * 4;       // the exchange takes the table's place
+    if (table < red) table = red;
+    p.smem = LG_HEAD + (size_t)((p.rows_per_split + step - 1) / step * step) * mt * 4 + (table + 15) / 16 * 16;
+    p.fits = p.smem <= (size_t)LG_SMEM && p.splits <= LG_SPLITS_MAX;
+    return p;
+}
+
+// Slabs of partial sums that any plan of such a layer may write: three CTAs per SM at the most, or as many splits as x asks
+// for.  The most come with the fewest blocks of code groups, i.e. at g = 16.
+inline int64_t gemv_slabs_most(int64_t d_out, int64_t d_in, int sm_count) {
+    const int o_blocks = (int)((d_out / 32 + LG_GRPS - 1) / LG_GRPS);
+    const int64_t least = LG_SLICES_MAX * ((d_in + 511) / 512);
+    const int64_t most = 3 * sm_count / (o_blocks < 1 ? 1 : o_blocks) + LG_SLICES_MAX;
+    return most > least ? most : least;
+}
+
+}  // namespace
