@@ -430,6 +430,8 @@ __device__ __forceinline__ void gemv_row(const unsigned char* table, unsigned ro
     for (int t = 0; t < G; ++t) c[t] = __half2float(__ushort_as_half((unsigned short)((t & 1) ? w[t / 2] >> 16 : w[t / 2] & 0xffffu)));
 }
 
+template <bool V> struct GemvChecked { static constexpr bool value = V; };
+
 // PW: code groups per thread, 1 or 2 (2 wants an even number of groups and the codes on a word boundary).
 template <int G, int MT, bool QUANT, int PW>
 __global__ void __launch_bounds__(LG_THREADS, 1)
@@ -494,11 +496,16 @@ linear_gemv_kernel(const uint16_t* __restrict__ x, int M, const unsigned char* _
     } else {
         if (tid < ROWB + 4) qt[bytes + tid] = 0;                                 // the row of zeros
     }
+    bool mine_odd = false;
     for (int e = tid; e < rows_whole * MT; e += LG_THREADS) {
         const int r = e / MT, m = e - r * MT;
-        xs[e] = (m < M && r < rows) ? __half2float(__ushort_as_half(__ldg(x + (int64_t)m * d_in + i0 + r))) : 0.f;
+        const float v = (m < M && r < rows) ? __half2float(__ushort_as_half(__ldg(x + (int64_t)m * d_in + i0 + r))) : 0.f;
+        if constexpr (!QUANT) mine_odd |= !(fabsf(v) < INFINITY);
+        xs[e] = v;
     }
-    __syncthreads();
+    bool odd_x = false;                                                          // an infinite or undefined x among them
+    if constexpr (QUANT) __syncthreads();
+    else odd_x = __syncthreads_or(mine_odd);
     const bool ok = mbar_wait(smem_u32(qbar), 0, abort_flag);                    // nobody goes on before the table has landed
 
     float acc[MT][GE];
@@ -507,7 +514,9 @@ linear_gemv_kernel(const uint16_t* __restrict__ x, int M, const unsigned char* _
 #pragma unroll
         for (int t = 0; t < GE; ++t) acc[m][t] = 0.f;
     const unsigned kmax = (unsigned)K - 1u;
-    if (live && ok) {
+    // checked: rows outside the slice are left out instead of added as zeros, which an infinite x would not survive
+    auto look_up = [&](auto checked) {
+        constexpr bool CHECKED = decltype(checked)::value;
         for (int r0 = sub; r0 < rows; r0 += STEP) {
             unsigned now[RB];
 #pragma unroll
@@ -537,7 +546,9 @@ linear_gemv_kernel(const uint16_t* __restrict__ x, int M, const unsigned char* _
 #pragma unroll
                         for (int t = 0; t < G; ++t) c[t] = lut16[lv[t]];
                     } else {
-                        gemv_row<G>(qt, r < rows ? min(one - lo, n_rows) : n_rows, c);   // outside the slice, or past the last row: zeros
+                        const unsigned row = r < rows ? min(one - lo, n_rows) : n_rows;  // outside the slice, or past the last row: zeros
+                        if constexpr (CHECKED) { if (row == n_rows) continue; }
+                        gemv_row<G>(qt, row, c);
                     }
 #pragma unroll
                     for (int m = 0; m < MT; ++m)
@@ -546,6 +557,10 @@ linear_gemv_kernel(const uint16_t* __restrict__ x, int M, const unsigned char* _
                 }
             }
         }
+    };
+    if (live && ok) {
+        if (odd_x) look_up(GemvChecked<!QUANT>{});
+        else look_up(GemvChecked<false>{});
     }
     // ---- the sub-slices meet, one token at a time (the exchange area takes the table's place)
     __syncthreads();
