@@ -873,8 +873,11 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
     const int64_t codes = (d_out + g - 1) / g * d_in;
     // the codebook's own rows take one load (the widest wants them on 32-byte boundaries)
     bool padded = row_pad(g) == g && (g < 16 || (reinterpret_cast<uintptr_t>(C16) & 31u) == 0);
-    if (!qtab && !padded && codes >= LINEAR_PAD_FROM && codes >= 4 * (int64_t)K) {
-        uint16_t* table = reinterpret_cast<uint16_t*>(ws + CC_STATUS_BYTES);
+    size_t table_at = 0;
+    if (!qtab && !padded && codes >= LINEAR_PAD_FROM && codes >= 4 * (int64_t)K)
+        table_at = padded_table_at(reinterpret_cast<uintptr_t>(ws), CC_STATUS_BYTES, CC_LINEAR_SCRATCH_FROM, K, row_pad(g));
+    if (table_at) {
+        uint16_t* table = reinterpret_cast<uint16_t*>(ws + table_at);
         ProfScope ps(ctx, CC_K_OTHER, st);
         linear_pad_rows_kernel<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(C16, K, g, row_pad(g), table);
         C16 = table;

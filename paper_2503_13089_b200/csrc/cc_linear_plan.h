@@ -1,5 +1,5 @@
-// Host-side plan of the few-token layer forward (linear_gemv_kernel in cc_linear.cu).  No CUDA in here: what a plan asks
-// for can be checked against the kernel's limits without a device.
+// Host-side plans of the layer forward (cc_linear.cu): the few-token kernel's launch, the place of the padded codebook.  No
+// CUDA in here: what a plan asks for can be checked against the kernels' limits without a device.
 #pragma once
 
 #include <stddef.h>
@@ -94,6 +94,13 @@ inline int64_t gemv_slabs_most(int64_t d_out, int64_t d_in, int sm_count) {
     const int64_t least = LG_SLICES_MAX * ((d_in + 511) / 512);
     const int64_t most = 3 * sm_count / (o_blocks < 1 ? 1 : o_blocks) + LG_SLICES_MAX;
     return most > least ? most : least;
+}
+
+// Where a copy of the codebook with rows of `pad` values goes between byte `from` and byte `to` of a workspace at address `ws`,
+// which need only be on a 16-byte boundary while a row of 16 values is one load of 32 bytes: its offset, or 0 if it does not fit.
+inline size_t padded_table_at(uintptr_t ws, size_t from, size_t to, int K, int pad) {
+    const size_t at = ((ws + from + 31) & ~(uintptr_t)31) - ws;
+    return at + (size_t)K * pad * 2 <= to ? at : 0;
 }
 
 }  // namespace

@@ -1,8 +1,10 @@
 """The layer forward where a plan or a load meets its limit: codebooks whose slices end within a few rows of what shared memory
-holds beside a full x, and infinite activations.  Same bound as in test_gpu_linear_paths: (d_in + 64) 2^-23 sum |x w|.
+holds beside a full x, infinite activations, and workspaces that start on any 16-byte
+boundary.  Same bound as in test_gpu_linear_paths: (d_in + 64) 2^-23 sum |x w|.
 """
 import numpy as np
 import pytest
+import torch
 
 from tests.test_gpu_linear_paths import _case, _run, _want
 
@@ -38,3 +40,28 @@ def test_infinite_activations(M, d_out, d_in, g, K, q4):
     odd = ~np.isfinite(want)
     assert np.array_equal(np.isnan(y), np.isnan(want)) and np.array_equal(y[odd & ~np.isnan(want)], want[odd & ~np.isnan(want)])
     assert odd[0].all() and np.isfinite(y[~odd]).all()
+
+
+@pytest.mark.parametrize("M,d_out,d_in,g,K,q4", [
+    (6, 1700, 4096, 16, 3000, False), (5, 2500, 1600, 9, 20001, False), (20, 2100, 2100, 11, 65536, False), (200, 2100, 2100, 13, 16000, False),
+    (7, 2048, 2048, 6, 65536, False), (1, 700, 900, 4, 60000, False), (2, 700, 900, 4, 60000, True), (300, 516, 260, 16, 16384, True),
+])
+@pytest.mark.parametrize("shift", [16, 48])
+def test_workspace_on_a_16_byte_boundary(M, d_out, d_in, g, K, q4, shift):
+    from paper_2503_13089_b200 import binding as cc
+    from tests import gpu_util as u
+    x, C16, idx, bias = _case(M, d_out, d_in, g, K, shift)
+    c = cc.Context(0)
+    room = torch.zeros(cc.cc_linear_workspace_bytes(c, M, d_out, d_in) + 64, dtype=torch.uint8, device="cuda")
+    cc.cc_set_workspace(c, room[shift:], room.numel() - 64)
+    book, codes, y = u.half_dev(C16), u.dev(idx.view(np.int16)).view(torch.uint16), torch.full((M, d_out), float("nan"), device="cuda")
+    if q4:
+        q, s, deq = torch.zeros((K * g + 1) // 2, dtype=torch.uint8, device="cuda"), torch.zeros(1, device="cuda"), torch.zeros((K, g), dtype=torch.float16, device="cuda")
+        cc.cc_quantize_codebook(c, book, K, g, 4, q, s, deq)
+        cc.cc_linear_forward_q4(c, u.half_dev(x), M, q, s, K, g, codes, d_out, d_in, u.dev(bias), y)
+        C16 = deq.cpu().numpy()
+    else:
+        cc.cc_linear_forward(c, u.half_dev(x), M, book, K, g, codes, d_out, d_in, u.dev(bias), y)
+    cc.cc_poll_status(c)
+    want, bound = _want(x, C16, idx, d_out, d_in, bias)
+    assert np.all(np.abs(y.cpu().numpy() - want) <= bound)

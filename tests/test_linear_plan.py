@@ -1,5 +1,6 @@
 """The few-token layer forward's launch plan, walked on the host: no plan may ask for more shared memory than its kernel's limit,
-more slabs than the scratch is sized for, or slices that leave out a row of the codebook.  Numbers of centroids are taken
+more slabs than the scratch is sized for, or slices that leave out a row of the codebook; the padded codebook starts where its widest
+load may, whatever the workspace starts at.  Numbers of centroids are taken
 densely around the ends of every slice, where rounding to whole groups of 16 rows decides."""
 import os
 import subprocess
@@ -48,6 +49,15 @@ int main() {
     // more in_features than a grid has rows of blocks for: the plan says so
     const GemvPlan far = gemv_plan((int64_t)1 << 30, 1, 148, 100, 1, 1, false, false);
     if (far.fits) { printf("a plan of %d splits fits\n", far.splits); ++bad; }
+    // the padded codebook: rows of 16 values are loads of 32 bytes, a workspace starts on any 16-byte boundary
+    const size_t from = 4096, to = from + 65536 * 32;
+    for (uintptr_t ws = 1 << 20; ws < (1 << 20) + 256; ws += 16)
+        for (int K = 1; K <= 65536; K += K < 65000 ? 97 : 1)
+            for (int pad = 4; pad <= 16; pad *= 2) {
+                const size_t at = padded_table_at(ws, from, to, K, pad);
+                const bool must = from + 16 + (size_t)K * pad * 2 <= to;
+                if (at ? (ws + at) % 32 || at < from || at + (size_t)K * pad * 2 > to : must) { printf("table at %zu, K=%d pad=%d\n", at, K, pad); ++bad; }
+            }
     printf("%ld plans, %ld bad\n", plans, bad);
     return bad || plans < 100000;
 }
