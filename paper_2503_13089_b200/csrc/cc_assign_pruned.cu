@@ -857,9 +857,10 @@ pruned_finish_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __r
             L1 += fabsf(x_own[t]);
         }
         if (live) {
+            const float d = D == D ? (float)D : INFINITY;    // an undefined point is infinitely far away, as in the exhaustive E-step
             idx[i] = (uint16_t)__ldg(order + p1);
-            dist[i] = (float)D;
-            far = fmaxf(far, (float)D);
+            dist[i] = d;
+            far = fmaxf(far, d);
             const double Au = (double)A * 1.0001;
             const double bound = 2.0 * ((double)TcCfg<G>::ERR_UNITS * 5.9604644775390625e-8 *
                                             (3.0 * Au + 4.0 * sqrt(Au * D) * 1.0000001 + 2.0 * D)
@@ -902,6 +903,7 @@ pruned_resolve_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __
             const double df = __dsub_rn((double)x[t], (double)__ldg(C + (int64_t)jb * G + t));
             Db = __dadd_rn(Db, __dmul_rn(df, df));
         }
+        if (!(Db == Db)) Db = INFINITY;
         float bound = __double2float_ru(Db * (1.0 + 3.814697265625e-6));
         const uint16_t* L = list + tile * ld;
         const int n = (int)list_n[tile];

@@ -122,3 +122,30 @@ def test_fit_in_the_smaller_workspace_gives_the_same():
         torch.cuda.synchronize()
     assert out[0][5] != out[1][5]                        # two different ways
     assert all(torch.equal(x, y) for x, y in zip(out[0][:5], out[1][:5]))
+
+
+@pytest.mark.parametrize("size", ["preferred", "needed"])
+def test_an_undefined_point_is_infinitely_far_away(size):
+    """Points that are not numbers have no nearest centroid; their distances and the objective are infinite whichever E-step ran,
+    and the other points keep theirs."""
+    from paper_2503_13089_b200 import binding as cc
+    N, g, K = 600000, 4, 60000
+    c = cc.Context(0)
+    ws = torch.empty((cc.cc_workspace_bytes_preferred if size == "preferred" else cc.cc_workspace_bytes)(N, g, K), dtype=torch.uint8, device="cuda")
+    cc.cc_set_workspace(c, ws, ws.numel())
+    X = _points(N, g, K, "heavy")
+    C = torch.empty((K, g), device="cuda")
+    cc.cc_init_codebook(c, X, N, g, K, 1, C)
+    X[77, 1], X[N - 1, 3], X[4000, 0] = float("nan"), float("nan"), float("inf")
+    out = {}
+    for path in (cc.PATH_AUTO, cc.PATH_TENSOR):
+        cc.cc_set_path(c, path)
+        idx, dist = torch.empty(N, dtype=torch.uint16, device="cuda"), torch.empty(N, device="cuda")
+        obj = torch.zeros(1, dtype=torch.float64, device="cuda")
+        cc.cc_assign(c, X, N, g, C, K, idx, dist, obj, None)
+        with pytest.raises(cc.CCError):
+            cc.cc_poll_status(c)
+        assert obj.item() == float("inf") and torch.equal(torch.isinf(dist).nonzero().flatten().cpu(), torch.tensor([77, 4000, N - 1]))
+        out[path] = (idx.view(torch.int16), dist)
+    fine = torch.isfinite(out[cc.PATH_TENSOR][1])
+    assert int(fine.sum()) == N - 3 and all(torch.equal(a[fine], b[fine]) for a, b in zip(out[cc.PATH_AUTO], out[cc.PATH_TENSOR]))
