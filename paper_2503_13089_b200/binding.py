@@ -129,6 +129,7 @@ class Context:
         _check(load().cc_create(ct.byref(self._h), device), "cc_create")
         self.device = device
         self._ws = None
+        self._ws_refused = None      # smallest workspace that was refused for want of memory
 
     def close(self):
         if self._h:
@@ -147,11 +148,16 @@ class Context:
         if need == 0:
             raise CCError(2, "cc_workspace_bytes")
         want = max(cc_workspace_bytes_preferred(N, g, K), need)
-        if self._ws is None or self._ws.numel() < want:
+        have = 0 if self._ws is None else self._ws.numel()
+        ask = self._ws_refused is None or want < self._ws_refused     # a size that was refused is not asked for again
+        if have < (want if ask else need):
             try:
-                self._ws = torch.empty(want, dtype=torch.uint8, device="cuda:%d" % self.device)
+                self._ws = torch.empty(want if ask else need, dtype=torch.uint8, device="cuda:%d" % self.device)
             except torch.OutOfMemoryError:
-                if self._ws is not None and self._ws.numel() >= need:
+                if not ask or want == need:
+                    raise
+                self._ws_refused = want
+                if have >= need:
                     return
                 self._ws = torch.empty(need, dtype=torch.uint8, device="cuda:%d" % self.device)
             cc_set_workspace(self, self._ws, self._ws.numel())

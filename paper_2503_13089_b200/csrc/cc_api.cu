@@ -339,6 +339,7 @@ cc_status cc_create(cc_ctx** out, int device) {
     c->prof = nullptr;
     c->e2e_buf = nullptr;
     c->e2e_bytes = 0;
+    c->e2e_refused = 0;
     c->stage = nullptr;
     c->empty_rule = CC_EMPTY_KEEP;
     *out = c;
@@ -790,18 +791,29 @@ cc_status cc_compress_host(cc_ctx* ctx, const uint16_t* W_host, int64_t d_out, i
     const size_t oW = take(w_bytes), oX = take(x_bytes), oC = take((size_t)K * g * 4), oDist = take((size_t)N * 4),
                  oCnt = take((size_t)K * 4), oC16 = take((size_t)K * g * 2), oIdx = take((size_t)N * 2),
                  oTr = take((size_t)(iters + 1) * 8), oWs = take(0);
-    size_t ws_bytes = L.total_preferred;
-    if (ctx->e2e_bytes < oWs + ws_bytes) {          // grown on demand and kept: repeated calls allocate nothing
+    // Grown on demand and kept: repeated calls allocate nothing.  Where memory does not reach to the preferred size, what every call
+    // needs; the context remembers it and keeps its buffer.
+    const size_t want = oWs + L.total_preferred, need = oWs + L.total;
+    size_t free_bytes = 0, all_bytes = 0;
+    if (ctx->e2e_bytes >= need && ctx->e2e_bytes < want && (!ctx->e2e_refused || want < ctx->e2e_refused) &&
+        cudaMemGetInfo(&free_bytes, &all_bytes) == cudaSuccess && free_bytes + ctx->e2e_bytes < want)
+        ctx->e2e_refused = want;                        // nothing to be had by giving up the buffer that is there
+    const bool ask = !ctx->e2e_refused || want < ctx->e2e_refused;
+    if (ctx->e2e_bytes < (ask ? want : need)) {
         if (ctx->e2e_buf) cudaFree(ctx->e2e_buf);
         ctx->e2e_buf = nullptr;
         ctx->e2e_bytes = 0;
-        if (cudaMalloc(&ctx->e2e_buf, oWs + ws_bytes) != cudaSuccess) {
+        size_t got = want;
+        if (!ask || cudaMalloc(&ctx->e2e_buf, want) != cudaSuccess) {
             cudaGetLastError();
-            ws_bytes = L.total;                     // less memory: what every call needs
-            if (cudaMalloc(&ctx->e2e_buf, oWs + ws_bytes) != cudaSuccess) return CC_ERR_CUDA;
+            ctx->e2e_buf = nullptr;
+            if (ask) ctx->e2e_refused = want;
+            got = need;
+            if (cudaMalloc(&ctx->e2e_buf, need) != cudaSuccess) { ctx->e2e_buf = nullptr; return CC_ERR_CUDA; }
         }
-        ctx->e2e_bytes = oWs + ws_bytes;
+        ctx->e2e_bytes = got;
     }
+    const size_t ws_bytes = ctx->e2e_bytes >= want ? L.total_preferred : L.total;
     char* base = static_cast<char*>(ctx->e2e_buf);
     void* saved_ws = ctx->ws;
     const size_t saved_bytes = ctx->ws_bytes;

@@ -33,6 +33,7 @@ struct cc_ctx {
     cc_prof_slot* prof;   // CC_PROF_CAP slots, events created on first use
     void* e2e_buf;        // device memory of cc_compress_host, grown on demand, freed by cc_destroy
     size_t e2e_bytes;
+    size_t e2e_refused;   // smallest size that was refused for want of memory (0: none yet); not asked for again
     void* stage;          // CC_STAGE_BYTES of page-locked host memory for small results, made on first use, freed by cc_destroy
     int empty_rule;       // CC_EMPTY_*
 };
