@@ -430,7 +430,50 @@ __device__ __forceinline__ void gemv_row(const unsigned char* table, unsigned ro
     for (int t = 0; t < G; ++t) c[t] = __half2float(__ushort_as_half((unsigned short)((t & 1) ? w[t / 2] >> 16 : w[t / 2] & 0xffffu)));
 }
 
-template <bool V> struct GemvChecked { static constexpr bool value = V; };
+// Adds x times the rows of one batch of codes (in_features r0, r0 + LG_SUB, ..) to a thread's sums.  CHECKED: rows outside the
+// slice are left out instead of added as zeros, which an infinite x would not survive.
+template <int G, int MT, bool QUANT, int PW, bool CHECKED, int RB>
+__device__ __forceinline__ void gemv_add(float (&acc)[MT][G * PW], const unsigned (&code)[RB], int r0, int rows, const float* xs,
+                                         const unsigned char* qt, const float* lut16, unsigned kmax, unsigned lo, unsigned n_rows) {
+#pragma unroll
+    for (int u = 0; u < RB; ++u) {
+        const int r = r0 + u * LG_SUB;
+        if (QUANT && r >= rows) break;
+        float xv[MT];
+        if constexpr (MT == 4) {
+            const float4 v = *reinterpret_cast<const float4*>(xs + r * 4);
+            xv[0] = v.x; xv[1] = v.y; xv[2] = v.z; xv[3] = v.w;
+        } else if constexpr (MT == 2) {
+            const float2 v = *reinterpret_cast<const float2*>(xs + r * 2);
+            xv[0] = v.x; xv[1] = v.y;
+        } else {
+            xv[0] = xs[r];
+        }
+#pragma unroll
+        for (int p = 0; p < PW; ++p) {
+            const unsigned one = PW == 1 ? code[u] : (p ? code[u] >> 16 : code[u] & 0xffffu);
+            if constexpr (QUANT) {
+                unsigned lv[G];
+                gemv_levels<G>(qt + (size_t)min(one, kmax) * (G / 2), lv);       // a code beyond the codebook must not leave it
+#pragma unroll
+                for (int t = 0; t < G; ++t) {
+                    const float c = lut16[lv[t]];
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) acc[m][p * G + t] = fmaf(xv[m], c, acc[m][p * G + t]);
+                }
+            } else {
+                const unsigned row = r < rows ? min(one - lo, n_rows) : n_rows;  // outside the slice, or past the last row: zeros
+                if (CHECKED && row == n_rows) continue;
+                float c[G];
+                gemv_row<G>(qt, row, c);
+#pragma unroll
+                for (int m = 0; m < MT; ++m)
+#pragma unroll
+                    for (int t = 0; t < G; ++t) acc[m][p * G + t] = fmaf(xv[m], c[t], acc[m][p * G + t]);
+            }
+        }
+    }
+}
 
 // PW: code groups per thread, 1 or 2 (2 wants an even number of groups and the codes on a word boundary).
 template <int G, int MT, bool QUANT, int PW>
@@ -514,53 +557,26 @@ linear_gemv_kernel(const uint16_t* __restrict__ x, int M, const unsigned char* _
 #pragma unroll
         for (int t = 0; t < GE; ++t) acc[m][t] = 0.f;
     const unsigned kmax = (unsigned)K - 1u;
-    // checked: rows outside the slice are left out instead of added as zeros, which an infinite x would not survive
-    auto look_up = [&](auto checked) {
-        constexpr bool CHECKED = decltype(checked)::value;
-        for (int r0 = sub; r0 < rows; r0 += STEP) {
-            unsigned now[RB];
-#pragma unroll
-            for (int u = 0; u < RB; ++u) now[u] = code[u];
-            request(r0 + STEP);
-#pragma unroll
-            for (int u = 0; u < RB; ++u) {
-                const int r = r0 + u * LG_SUB;
-                if (QUANT && r >= rows) break;
-                float xv[MT];
-                if constexpr (MT == 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(xs + r * 4);
-                    xv[0] = v.x; xv[1] = v.y; xv[2] = v.z; xv[3] = v.w;
-                } else if constexpr (MT == 2) {
-                    const float2 v = *reinterpret_cast<const float2*>(xs + r * 2);
-                    xv[0] = v.x; xv[1] = v.y;
-                } else {
-                    xv[0] = xs[r];
-                }
-#pragma unroll
-                for (int p = 0; p < PW; ++p) {
-                    const unsigned one = PW == 1 ? now[u] : (p ? now[u] >> 16 : now[u] & 0xffffu);
-                    float c[G];
-                    if constexpr (QUANT) {
-                        unsigned lv[G];
-                        gemv_levels<G>(qt + (size_t)min(one, kmax) * ROWB, lv);  // a code beyond the codebook must not leave it
-#pragma unroll
-                        for (int t = 0; t < G; ++t) c[t] = lut16[lv[t]];
-                    } else {
-                        const unsigned row = r < rows ? min(one - lo, n_rows) : n_rows;  // outside the slice, or past the last row: zeros
-                        if constexpr (CHECKED) { if (row == n_rows) continue; }
-                        gemv_row<G>(qt, row, c);
-                    }
-#pragma unroll
-                    for (int m = 0; m < MT; ++m)
-#pragma unroll
-                        for (int t = 0; t < G; ++t) acc[m][p * G + t] = fmaf(xv[m], c[t], acc[m][p * G + t]);
-                }
-            }
-        }
-    };
     if (live && ok) {
-        if (odd_x) look_up(GemvChecked<!QUANT>{});
-        else look_up(GemvChecked<false>{});
+        unsigned now[RB];
+        int r0 = sub;
+#define CC_GEMV_ADD(CHECKED, CODES) gemv_add<G, MT, QUANT, PW, CHECKED, RB>(acc, CODES, r0, rows, xs, qt, lut16, kmax, lo, n_rows)
+#define CC_GEMV_WALK(CHECKED)                                                                          \
+        for (; r0 + STEP < rows; r0 += STEP) {                                                         \
+            _Pragma("unroll") for (int u = 0; u < RB; ++u) now[u] = code[u];                           \
+            request(r0 + STEP);                                                                        \
+            CC_GEMV_ADD(CHECKED, now);                                                                 \
+        }                                                                                              \
+        if (r0 < rows) CC_GEMV_ADD(CHECKED, code)              /* nothing left to request */
+        if constexpr (QUANT) {
+            CC_GEMV_WALK(false);
+        } else if (odd_x) {
+            CC_GEMV_WALK(true);
+        } else {
+            CC_GEMV_WALK(false);
+        }
+#undef CC_GEMV_WALK
+#undef CC_GEMV_ADD
     }
     // ---- the sub-slices meet, one token at a time (the exchange area takes the table's place)
     __syncthreads();
