@@ -850,7 +850,7 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
     GemvPlan v = {};
     if (gemv_applies(M, K, g, qtab != nullptr))
         v = gemv_plan(d_in, out_groups, ctx->sm_count, K, g, gemv_pad(M), qtab != nullptr, (reinterpret_cast<uintptr_t>(idx) & 3u) == 0);
-    if (v.fits) {
+    if (v.fits && v.pays) {
         // a handful of tokens: the shared-memory look-up kernel, then the same reduction (it also adds the bias)
         const int slabs_n = v.splits * v.slices;
         unsigned* arrived = nullptr;

@@ -50,8 +50,28 @@ inline bool gemv_applies(int64_t M, int K, int g, bool quant) {
 }
 constexpr int gemv_pad(int64_t M) { return M <= 2 ? (int)M : 4; }
 
-// fits: within what a launch may ask for; where not, the tensor kernel takes the call.
-struct GemvPlan { int pw, o_blocks, slices, slice_rows, splits, rows_per_split; size_t smem; bool fits; };
+// fits: within what a launch may ask for; pays: not slower than the tensor kernel.  Where not both, that kernel takes the call.
+struct GemvPlan { int pw, o_blocks, slices, slice_rows, splits, rows_per_split; size_t smem; bool fits, pays; };
+
+// Whether a plan for the FP16 codebook beats the tensor kernel.  What costs is its end, where one CTA adds up the slabs of a
+// block of code groups, eight loads a thread at a time: `tail` counts those rounds.  A layer with few code groups has few
+// blocks and many slabs, and the tensor kernel is quick on it where a row of the codebook is one load.  One and two tokens, look-up / tensor
+// kernel in us (tail): 1024 x 4096, g = 16, K = 4096 13.7 / 9.5 (19) and 21.1 / 9.5 (38), g = 9, K = 20000 12.0 / 12.2 (10) and 15.9 /
+// 12.3 (20); 128 x 4096, K = 256 (19) g = 8 9.7 / 8.8 and 11.1 / 8.8, g = 4 9.1 / 8.8 and 10.9 / 8.8, g = 2 8.5 / 9.4 and 10.0 / 9.4;
+// 512 x 512, g = 16, K = 4096 8.7 / 8.3 (2) and 11.2 / 8.5 (4); one token, g = 16: 2048 x 2048, K = 5000 12.0 / 9.6, 700 x 900 9.3 /
+// 10.5; four, 1536 x 6144, g = 4, K = 300 14.7 / 12.3 (14).  Slices read every code once more each, which a layer of about a
+// million codes does not make up for: 1024 x 4096, g = 4, K = 65536 10.4 / 12.0 and, at four tokens, 13.9 / 12.0, g = 8, K = 20000 10.7 /
+// 10.0 and 12.1 / 10.1; but 700 x 900, g = 4, K = 65536, four tokens 10.3 / 14.0.
+inline bool gemv_pays(const GemvPlan& p, int64_t d_in, int out_groups, int g, int mt) {
+    const int slabs = p.splits * p.slices, groups = out_groups < LG_GRPS * p.pw ? out_groups : LG_GRPS * p.pw;
+    const int tail = (slabs + 7) / 8 * ((mt * g * groups + LG_THREADS - 1) / LG_THREADS);
+    if (tail >= 20) return false;
+    if (g != 4 && g != 8 && g != 16) return true;                           // several loads a row, or two values
+    if (mt * g >= 8 && tail >= 14) return false;
+    if (g == 16 && p.o_blocks <= 2 && (mt > 1 || d_in % 8 == 0)) return false;   // x in 16-byte pieces there
+    const int64_t codes = out_groups * d_in;
+    return !(p.slices > 1 && mt * g * p.slices >= 32 && codes >= 500000 && codes <= 1100000);
+}
 
 // Slices of the codebook as its bytes ask for, splits of the in_features by a count of clocks: a CTA pays for its
 // table (about 40 bytes a clock), some 4000 for its beginning and end, and 8 a row of codes (16 where a thread has two
@@ -84,6 +104,7 @@ inline GemvPlan gemv_plan(int64_t d_in, int out_groups, int sm_count, int K, int
     if (table < red) table = red;
     p.smem = LG_HEAD + (size_t)((p.rows_per_split + step - 1) / step * step) * mt * 4 + (table + 15) / 16 * 16;
     p.fits = p.smem <= (size_t)LG_SMEM && p.splits <= LG_SPLITS_MAX;
+    p.pays = quant || gemv_pays(p, d_in, out_groups, g, mt);
     return p;
 }
 

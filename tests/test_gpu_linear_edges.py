@@ -1,5 +1,5 @@
 """The layer forward where a plan or a load meets its limit: codebooks whose slices end within a few rows of what shared memory
-holds beside a full x, infinite activations, and workspaces that start on any 16-byte
+holds beside a full x, layers of few code groups, infinite activations, and workspaces that start on any 16-byte
 boundary.  Same bound as in test_gpu_linear_paths: (d_in + 64) 2^-23 sum |x w|.
 """
 import numpy as np
@@ -14,8 +14,11 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("M,d_out,d_in,g,K", [
     (4, 14336, 2048, 4, 53700), (2, 11008, 2048, 8, 53696), (2, 11008, 2048, 8, 53700), (2, 8192, 2048, 7, 61380), (1, 11008, 4096, 7, 61385),
     (1, 11008, 4096, 7, 61376), (2, 11008, 4096, 8, 40280),
+    # few code groups: either side of where the tensor kernel takes over
+    (1, 1024, 4096, 16, 4096), (2, 1024, 4096, 16, 256), (1, 2048, 4096, 16, 256), (2, 512, 512, 16, 300), (2, 1024, 4096, 9, 20000),
+    (4, 1024, 4096, 4, 65536), (2, 1024, 4096, 4, 65536), (3, 128, 4096, 4, 256), (1, 128, 4096, 2, 256),
 ])
-def test_slices_that_fill_shared_memory(M, d_out, d_in, g, K):
+def test_slices_and_layers_at_their_limits(M, d_out, d_in, g, K):
     x, C16, idx, bias = _case(M, d_out, d_in, g, K, K)
     y, _ = _run(x, C16, idx, d_out, d_in, bias)
     want, bound = _want(x, C16, idx, d_out, d_in, bias)
