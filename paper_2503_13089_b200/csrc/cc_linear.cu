@@ -656,9 +656,12 @@ linear_pad_rows_kernel(const uint16_t* __restrict__ C16, int K, int g, int pad, 
     }
 }
 
-// Codes from which the copy pays: as a launch it takes about 4 us, and it saves some 12 us a million codes at g = 6
-// (33 tokens, g = 6, K = 1024: 512 x 512 17.4 us without, 21.5 with it).
-constexpr int64_t LINEAR_PAD_FROM = 400000;
+// Gathers (codes times blocks of tokens) from which the copy pays: as a launch it takes one to two us.  33 tokens, with / without, in
+// us: 1024 x 4096, g = 6 (0.7 M) K = 256 12.8 / 10.8, K = 16000 13.7 / 13.0; 2048 x 2048, g = 5 (0.8 M) 12.5 / 11.1 and 13.7 / 13.6;
+// 4096 x 4096, g = 9 (1.9 M) 20.8 / 21.4 and 25.6 / 31.4, g = 6 (2.8 M) 21.5 / 20.2 and 25.8 / 28.4; 11008 x 4096, g = 6 (7.5 M) 47.8 / 48.1
+// and 58.9 / 69.9.  320 tokens, 1024 x 4096, g = 6, K = 65536 (1.4 M) 29.2 / 32.1.
+constexpr int64_t LINEAR_PAD_FROM = 1200000, LINEAR_PAD_FROM_SMALL = 3200000;   // the latter for even g and codebooks that L1 holds
+constexpr int LINEAR_PAD_SMALL = 512;                                           // rows
 
 // Tokens from which decoding the weight once and multiplying it afterwards (cc_linear_wide.cu) is the faster way
 // (4096 x 4096, g = 4, K = 65536: 128 tokens 42 against 46 us, 192 tokens 52 against 46, 512 tokens 85 against 52), earlier
@@ -886,11 +889,12 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
     // beside the table: token blocks of 64 with four stages, or, from LQ_WIDE_FROM tokens on, of 256 with two
     const LinearPlan p = qtab ? linear_plan(M, d_out, d_in, ctx->sm_count, M >= LQ_WIDE_FROM ? LNT_MAX : LQ_NT_MAX, (size_t)K * (g / 2), g)
                               : linear_plan(M, d_out, d_in, ctx->sm_count, LNT_MAX, 0, g);
-    const int64_t codes = (d_out + g - 1) / g * d_in;
+    const bool wide = M >= (p.fill == 1 ? LINEAR_WIDE_FEWEST : LINEAR_WIDE_FROM) && cc_linear_wide_applies(M, d_out, d_in, p.fill, ctx->sm_count);
+    const int64_t codes = (d_out + g - 1) / g * d_in, gathers = codes * (wide ? 1 : p.tok_blocks);
     // the codebook's own rows take one load (the widest wants them on 32-byte boundaries)
     bool padded = row_pad(g) == g && (g < 16 || (reinterpret_cast<uintptr_t>(C16) & 31u) == 0);
     size_t table_at = 0;
-    if (!qtab && !padded && codes >= LINEAR_PAD_FROM && codes >= 4 * (int64_t)K)
+    if (!qtab && !padded && gathers >= (g % 2 == 0 && K <= LINEAR_PAD_SMALL ? LINEAR_PAD_FROM_SMALL : LINEAR_PAD_FROM) && codes >= 4 * (int64_t)K)
         table_at = padded_table_at(reinterpret_cast<uintptr_t>(ws), CC_STATUS_BYTES, CC_LINEAR_SCRATCH_FROM, K, row_pad(g));
     if (table_at) {
         uint16_t* table = reinterpret_cast<uint16_t*>(ws + table_at);
@@ -899,7 +903,7 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
         C16 = table;
         padded = true;
     }
-    if (M >= (p.fill == 1 ? LINEAR_WIDE_FEWEST : LINEAR_WIDE_FROM) && cc_linear_wide_applies(M, d_out, d_in, p.fill, ctx->sm_count))
+    if (wide)
         return cc_launch_linear_wide(ctx, x, M, C16, padded, qtab, qscale, K, g, idx, d_out, d_in, bias, y, p.fill, st);
     bool fused = false;
     {

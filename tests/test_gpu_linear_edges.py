@@ -46,8 +46,8 @@ def test_infinite_activations(M, d_out, d_in, g, K, q4):
 
 
 @pytest.mark.parametrize("M,d_out,d_in,g,K,q4", [
-    (6, 1700, 4096, 16, 3000, False), (5, 2500, 1600, 9, 20001, False), (20, 2100, 2100, 11, 65536, False), (200, 2100, 2100, 13, 16000, False),
-    (7, 2048, 2048, 6, 65536, False), (1, 700, 900, 4, 60000, False), (2, 700, 900, 4, 60000, True), (300, 516, 260, 16, 16384, True),
+    (6, 1700, 4096, 16, 3000, False), (5, 2500, 4400, 9, 20001, False), (20, 3700, 3700, 11, 65536, False), (200, 4000, 4000, 13, 16000, False),
+    (7, 3000, 3000, 6, 65536, False), (3, 4100, 4800, 16, 777, False), (1, 700, 900, 4, 60000, False), (2, 700, 900, 4, 60000, True), (300, 516, 260, 16, 16384, True),
 ])
 @pytest.mark.parametrize("shift", [16, 48])
 def test_workspace_on_a_16_byte_boundary(M, d_out, d_in, g, K, q4, shift):
