@@ -659,15 +659,27 @@ linear_pad_rows_kernel(const uint16_t* __restrict__ C16, int K, int g, int pad, 
 // Gathers (codes times blocks of tokens) from which the copy pays: as a launch it takes one to two us.  33 tokens, with / without, in
 // us: 1024 x 4096, g = 6 (0.7 M) K = 256 12.8 / 10.8, K = 16000 13.7 / 13.0; 2048 x 2048, g = 5 (0.8 M) 12.5 / 11.1 and 13.7 / 13.6;
 // 4096 x 4096, g = 9 (1.9 M) 20.8 / 21.4 and 25.6 / 31.4, g = 6 (2.8 M) 21.5 / 20.2 and 25.8 / 28.4; 11008 x 4096, g = 6 (7.5 M) 47.8 / 48.1
-// and 58.9 / 69.9.  320 tokens, 1024 x 4096, g = 6, K = 65536 (1.4 M) 29.2 / 32.1.
-constexpr int64_t LINEAR_PAD_FROM = 1200000, LINEAR_PAD_FROM_SMALL = 3200000;   // the latter for even g and codebooks that L1 holds
-constexpr int LINEAR_PAD_SMALL = 512;                                           // rows
+// and 58.9 / 69.9.  320 tokens, 1024 x 4096, K = 65536: g = 6 (1.4 M) 29.2 / 32.1, g = 9 (0.9 M) 27.3 / 30.0.
+constexpr int64_t LINEAR_PAD_ODD = 900000, LINEAR_PAD_EVEN = 1200000, LINEAR_PAD_EVEN_SMALL = 3200000;   // the last for codebooks that L1 holds
+constexpr int LINEAR_PAD_SMALL = 512;                                                                   // rows
+int64_t linear_pad_from(int g, int K) {
+    return g % 2 ? LINEAR_PAD_ODD : K <= LINEAR_PAD_SMALL ? LINEAR_PAD_EVEN_SMALL : LINEAR_PAD_EVEN;
+}
 
-// Tokens from which decoding the weight once and multiplying it afterwards (cc_linear_wide.cu) is the faster way
-// (4096 x 4096, g = 4, K = 65536: 128 tokens 42 against 46 us, 192 tokens 52 against 46, 512 tokens 85 against 52), earlier
-// where the tiles of this kernel fill the SMs by themselves, so that its waves are the coarser (11008 x 4096, g = 8,
-// 128 tokens: 95 against 67 us; g = 6, 33 tokens: 83 against about 80).
-constexpr int LINEAR_WIDE_FROM = 192, LINEAR_WIDE_FEWEST = 96;
+// Tokens from which decoding the weight once and multiplying it afterwards (cc_linear_wide.cu) is the faster way, gathering /
+// decoding in us: 4096 x 4096, g = 4, K = 65536, 128 tokens 42 / 46, 192 tokens 52 / 46, 512 tokens 85 / 52.  Earlier where
+// the tiles of this kernel fill the SMs by themselves, so that its waves are the coarser (11008 x 4096, g = 8, 128 tokens
+// 95 / 67; g = 6, 33 tokens 83 / about 80).  Later where it splits the in_features and so keeps the SMs busier than the few whole
+// tiles of the product do: from 224 tokens on for long in_features and short rows (4096 x 11008, g = 4: K = 256, 192 tokens 58 / 67,
+// K = 8000 65 / 71, at 224 tokens 82 / 71; g = 8, K = 16000, 192 tokens 82 / 75), from 256 on for the 4-bit codebook in shared
+// memory with four splits or more (1024 x 4096, g = 6, 192 tokens 19 / 26, 224 tokens 23 / 26; FP16, 2048 x 2048, eight splits, g = 8,
+// 224 tokens 19 / 16).
+constexpr int LINEAR_WIDE_FEWEST = 96, LINEAR_WIDE_FROM = 192, LINEAR_WIDE_LONG = 224, LINEAR_WIDE_Q4 = 256;
+int linear_wide_from(int fill, int64_t d_in, int g, bool quant) {
+    if (fill == 1) return LINEAR_WIDE_FEWEST;
+    if (quant && fill >= 4) return LINEAR_WIDE_Q4;
+    return !quant && fill > 2 && g <= 6 && d_in > 8192 ? LINEAR_WIDE_LONG : LINEAR_WIDE_FROM;
+}
 
 constexpr int LINEAR_SPLITS_MORE = 8;   // splits beyond those that fill the SMs once are tried up to this many
 
@@ -889,12 +901,12 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
     // beside the table: token blocks of 64 with four stages, or, from LQ_WIDE_FROM tokens on, of 256 with two
     const LinearPlan p = qtab ? linear_plan(M, d_out, d_in, ctx->sm_count, M >= LQ_WIDE_FROM ? LNT_MAX : LQ_NT_MAX, (size_t)K * (g / 2), g)
                               : linear_plan(M, d_out, d_in, ctx->sm_count, LNT_MAX, 0, g);
-    const bool wide = M >= (p.fill == 1 ? LINEAR_WIDE_FEWEST : LINEAR_WIDE_FROM) && cc_linear_wide_applies(M, d_out, d_in, p.fill, ctx->sm_count);
+    const bool wide = M >= linear_wide_from(p.fill, d_in, g, qtab != nullptr) && cc_linear_wide_applies(M, d_out, d_in, p.fill, ctx->sm_count);
     const int64_t codes = (d_out + g - 1) / g * d_in, gathers = codes * (wide ? 1 : p.tok_blocks);
     // the codebook's own rows take one load (the widest wants them on 32-byte boundaries)
     bool padded = row_pad(g) == g && (g < 16 || (reinterpret_cast<uintptr_t>(C16) & 31u) == 0);
     size_t table_at = 0;
-    if (!qtab && !padded && gathers >= (g % 2 == 0 && K <= LINEAR_PAD_SMALL ? LINEAR_PAD_FROM_SMALL : LINEAR_PAD_FROM) && codes >= 4 * (int64_t)K)
+    if (!qtab && !padded && gathers >= linear_pad_from(g, K) && codes >= 4 * (int64_t)K)
         table_at = padded_table_at(reinterpret_cast<uintptr_t>(ws), CC_STATUS_BYTES, CC_LINEAR_SCRATCH_FROM, K, row_pad(g));
     if (table_at) {
         uint16_t* table = reinterpret_cast<uint16_t*>(ws + table_at);
