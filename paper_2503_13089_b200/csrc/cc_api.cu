@@ -567,7 +567,7 @@ cc_status cc_fit(cc_ctx* ctx, const uint16_t* X, int64_t N, int g, int K, int it
     cudaStream_t st = (cudaStream_t)stream;
     if (iters > 0 && use_pruned(ctx, L, N, g, K, iters))
         return from_cuda(fit_pruned(ctx, L, X, N, g, K, iters, C, idx, dist, counts, objective_trace, st));
-    if (iters > 0 && cc_small_applies(ctx, N, g, K))
+    if (iters > 0 && cc_small_fit_applies(ctx, N, g, K))
         return from_cuda(fit_small(ctx, L, X, N, g, K, iters, C, idx, dist, counts, objective_trace, st));
     for (int it = 0; it < iters; ++it) {
         cudaError_t e = assign_any(ctx, L, X, N, g, C, K, idx, dist, objective_trace ? objective_trace + it : nullptr,

@@ -184,6 +184,7 @@ enum { SMALL_E = 0, SMALL_FIRST = 1, SMALL_NEXT = 2 };
 constexpr int SMALL_SMEM = 96 * 1024;                // bytes of codebook
 constexpr int64_t SMALL_WORK = 350000000;            // point-centroid pairs times instructions each
 bool cc_small_applies(const cc_ctx*, int64_t N, int g, int K);
+bool cc_small_fit_applies(const cc_ctx*, int64_t N, int g, int K);   // whole iterations
 cudaError_t cc_launch_small(cc_ctx*, const WsLayout&, const uint16_t* X, int64_t N, int g, float* C, int K, int mode, uint16_t* idx,
                             float* dist, int32_t* counts, double* objective, int64_t* n_flagged, cudaStream_t);
 

@@ -287,6 +287,18 @@ bool cc_small_applies(const cc_ctx* ctx, int64_t N, int g, int K) {
     return ctx->path == CC_PATH_AUTO && N > 0 && (K + SM_CHUNK - 1) / SM_CHUNK * SM_CHUNK * pairs * 8 <= SMALL_SMEM && N * K * (2 * pairs + 3) <= SMALL_WORK;
 }
 
+// The M-step adds every point to its cluster's words in L2.  With very few clusters, or few words a cluster, those additions queue
+// up, and summing in shared memory behind the E-step (cc_launch_update) is faster.  Three iterations, one launch each against the tensor-core
+// path with that M-step: K = 1, g = 16 20,000 points 0.63 times its time, 60,000 1.21, 600,000 3.2; K = 1, g = 4 60,000 0.68, 300,000 1.56;
+// g = 1, K = 64 200,000 0.88, 300,000 1.40; g = 2, K = 64 300,000 0.92, 600,000 1.75; g = 8, K = 2 300,000 0.76, 2 M 1.54; g = 3,
+// K = 8 200,000 0.74, 2 M 1.13; but g = 4, K = 2, 24 M 0.65, K = 8, 6 M 0.47, g = 1, K = 128, 531,000 0.93.
+bool cc_small_fit_applies(const cc_ctx* ctx, int64_t N, int g, int K) {
+    if (!cc_small_applies(ctx, N, g, K)) return false;
+    if (K == 1) return N <= 100000 && N * g <= 500000;
+    if ((g <= 2 && K <= 64) || (g == 3 && K <= 8)) return N <= 250000;
+    return K > 2 || g <= 4 || N <= 400000;
+}
+
 // C is only written in the modes with an M-step.  n_flagged: how many points had more than one candidate (listed in the
 // workspace, as the other E-steps list the points of their exact stage).
 cudaError_t cc_launch_small(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, int g, float* C, int K, int mode, uint16_t* idx,

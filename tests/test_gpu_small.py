@@ -17,6 +17,8 @@ pytestmark = pytest.mark.gpu
     (1, 4, 1, 2), (5, 3, 5, 2), (255, 4, 31, 4), (256, 4, 32, 4), (257, 4, 33, 4), (1023, 1, 9, 3), (3001, 2, 64, 4),
     (9000, 5, 65, 3), (4000, 6, 1025, 3), (5000, 7, 100, 3), (2500, 8, 1500, 3), (3000, 9, 257, 3), (2000, 16, 1536, 2),
     (1700, 15, 300, 3), (38000, 4, 200, 3), (80001, 4, 130, 2), (7000, 4, 6144, 2),
+    # few clusters, many points: either side of where the sums have a kernel of their own
+    (40000, 16, 1, 2), (100001, 3, 1, 2), (250001, 8, 2, 3), (250000, 1, 64, 3), (260000, 2, 33, 3), (250003, 3, 8, 3),
 ])
 def test_small_fit_matches_oracle(N, g, K, iters):
     from paper_2503_13089_b200 import binding as cc
