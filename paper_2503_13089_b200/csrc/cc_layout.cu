@@ -405,7 +405,12 @@ cudaError_t launch_decode_pipe(int sm_count, const uint16_t* C16, const uint16_t
 // One CTA per SM, four groups of 256 threads, each with a tile and a barrier of its own; the codes of tile k + 2 and
 // the rows of tile k + 1 are under way while tile k is transposed and stored.
 constexpr int RES_GROUPS = 4, RES_THREADS = RES_GROUPS * 256;
-constexpr int RES_TILES = 24;                        // tiles per CTA from which filling the table is paid for
+// Tiles per CTA from which this is the faster way: a short codebook is in L1 soon, and the plain kernels have more threads.  Plain /
+// this, in us, g = 4: 4096 x 4096 (28 tiles a CTA) K = 256 10.3 / 11.6, K = 4096 11.7 / 12.1, K = 8192 12.6 / 12.3, K = 20000
+// 16.3 / 13.4; 4096 x 8192 (55) K = 256 19.7 / 20.7, K = 4096 22.0 / 21.3; 4096 x 11008 (74) K = 16 29.4 / 23.8, K = 4096 32.8 / 28.1; g = 8:
+// 4096 x 8192 K = 1000 19.4 / 21.2, 4096 x 11008 29.2 / 27.8.
+constexpr int RES_TILES = 24, RES_TILES_SHORT = 64;
+constexpr int RES_SHORT = 6000;                      // rows of a short codebook
 constexpr int RES_SMEM = 226 * 1024, RES_TABLE = RES_SMEM - RES_GROUPS * kTileBytes;
 constexpr int RES_SMEM_PART = 194 * 1024, RES_TABLE_PART = RES_SMEM_PART - RES_GROUPS * kTileBytes;
 
@@ -629,7 +634,7 @@ cudaError_t cc_launch_decode(cc_ctx* ctx, const uint16_t* C16, int K, int g, con
         // stays in L1: there the chain of latencies bounds a tile.  A larger codebook is bound by the
         // L2 sectors its gathers move, and more resident threads (the kernel below) serve it better.
         // Many tiles: the codebook's head in shared memory (see the kernel above).
-        if (vec && n_tiles >= (int64_t)ctx->sm_count * RES_TILES && res_applies(K, g)) {
+        if (vec && n_tiles >= (int64_t)ctx->sm_count * (K < RES_SHORT ? RES_TILES_SHORT : RES_TILES) && res_applies(K, g)) {
             if (g == 4) return launch_decode_resident<4>(ctx, C16, idx, K, d_out, d_in, out_pad, W_hat, (int)grid.x, (int)grid.y, st);
             return launch_decode_resident<8>(ctx, C16, idx, K, d_out, d_in, out_pad, W_hat, (int)grid.x, (int)grid.y, st);
         }
