@@ -130,7 +130,15 @@ static inline int cc_sum_copies(int K, int g) {
     return r < 1 ? 1 : (r > CC_SUM_COPIES_MAX ? CC_SUM_COPIES_MAX : r);
 }
 
-static inline size_t cc_align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+// Copies for N points: few points do not queue up, and every copy is cleared and added up (8192 points, g = 16, K = 4096 with
+// four copies 9.1 us, with sixteen 12.2; 65,000 points, g = 12 12.9 and 15.5; but 524,000 points, g = 8, K = 20000 with one 33.5, with
+// six 22.9; 4.2 M points, g = 4, K = 65536 with one 65, with four 47).
+constexpr int CC_SUM_COPY_FEW = 262144;              // words an array up to CC_SUM_COPY_POINTS points
+constexpr int64_t CC_SUM_COPY_POINTS = 131072;
+static inline int cc_sum_copies_for(int64_t N, int K, int g) {
+    const int most = cc_sum_copies(K, g), few = CC_SUM_COPY_FEW / (K * g) < 1 ? 1 : CC_SUM_COPY_FEW / (K * g);
+    return N > CC_SUM_COPY_POINTS || few > most ? most : few;
+}
 
 // Launchers (each returns cudaGetLastError() of its launches and bumps ctx->launches).
 cudaError_t cc_launch_reshape(cc_ctx*, const uint16_t* W, int64_t d_out, int64_t d_in, int g, int layout,

@@ -282,8 +282,11 @@ cudaError_t accumulate_all(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, in
     }
     int32_t* cc = R > 1 ? reinterpret_cast<int32_t*>(ws + L.count_copies) : counts;
     *count_copies = cc;
-    cudaError_t e;       // the two arrays lie one behind the other
-    if ((e = cudaMemsetAsync(sum_lo, 0, L.sum_hi - L.sum_lo + sizeof(ull) * (size_t)K * g * R, st)) != cudaSuccess) return e;
+    const size_t used = sizeof(ull) * (size_t)K * g * R;
+    const bool one = L.sum_lo + cc_align_up(used, 256) == L.sum_hi;      // the two arrays lie one behind the other
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(sum_lo, 0, one ? L.sum_hi - L.sum_lo + used : used, st)) != cudaSuccess) return e;
+    if (!one && (e = cudaMemsetAsync(sum_hi, 0, used, st)) != cudaSuccess) return e;
     if (!want_counts) cc = nullptr;
     else if ((e = cudaMemsetAsync(cc, 0, sizeof(int32_t) * (size_t)K * R, st)) != cudaSuccess) return e;
     if (N > 0) {
@@ -300,7 +303,7 @@ cudaError_t accumulate_all(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, in
 cudaError_t cc_launch_update(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, int g, const uint16_t* idx,
                              int K, float* C, int32_t* counts, cudaStream_t st) {
     char* ws = static_cast<char*>(ctx->ws);
-    int R = cc_sum_copies(K, g);
+    int R = cc_sum_copies_for(N, K, g);
     int32_t* count_copies = nullptr;
     const cudaError_t e = accumulate_all(ctx, L, X, N, g, idx, K, counts, R, &count_copies, true, st);
     if (e != cudaSuccess) return e;
@@ -320,7 +323,7 @@ cudaError_t cc_launch_codebook_grad(cc_ctx* ctx, const WsLayout& L, const uint16
                                     const uint16_t* idx, int K, float* dC, cudaStream_t st) {
     char* ws = static_cast<char*>(ctx->ws);
     int32_t* counts = reinterpret_cast<int32_t*>(ws + L.positions);
-    int R = cc_sum_copies(K, g);
+    int R = cc_sum_copies_for(N, K, g);
     int32_t* count_copies = nullptr;
     const cudaError_t e = accumulate_all(ctx, L, dX, N, g, idx, K, counts, R, &count_copies, false, st);
     if (e != cudaSuccess) return e;
