@@ -140,6 +140,8 @@ static inline int cc_sum_copies_for(int64_t N, int K, int g) {
     return N > CC_SUM_COPY_POINTS || few > most ? most : few;
 }
 
+static inline size_t cc_align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
 // Launchers (each returns cudaGetLastError() of its launches and bumps ctx->launches).
 cudaError_t cc_launch_reshape(cc_ctx*, const uint16_t* W, int64_t d_out, int64_t d_in, int g, int layout,
                               uint16_t* X, cudaStream_t);
