@@ -198,17 +198,20 @@ cudaError_t prune_order(cc_ctx* ctx, const PruneBuffers& b, const uint16_t* X, i
 // Whether `steps` E-steps in a row on N points are faster with chunks ruled out, by the length of the sub-vectors.  In
 // more dimensions a box or a gap rules out less and the preparation has to be paid back over more iterations; with
 // fewer centroids there are fewer chunks to rule out.  Measured, pruned against exhaustive, on heavy-tailed points (time
-// of the call as a fraction of the exhaustive one): one step, g = 2, 4 M x 4096 0.95; g = 4, 4 M x 8192 0.92, 1 M x 65536
-// 0.47, 0.26 M x 65536 1.25; g = 5, 2 M x 32768 0.82, 4 M x 16384 1.05; g = 6, 2 M x 65536 0.95, 0.5 M x 65536 1.16.
-// A fit, g = 2, 4 M x 4096, 5 iterations 0.62; g = 4, 5 iterations: 1 M x 8192 1.10, 4 M x 8192 0.74, 0.26 M x 65536 0.77;
-// 20: 2 M x 4096 0.95, 4 M x 2048 1.17; g = 5, 4 M x 16384, 5 iterations 0.81, 1 M x 8700, 20 0.88, 5 1.27; g = 6, 5
-// iterations: 2 M x 32768 1.03, 2 M x 65536 0.79, 0.14 M x 65536 0.84; 10: x 32768 0.86, x 16384 1.03; 20: x 16384 0.90,
-// x 8192 1.15; g = 7, x 65536: 10 iterations 1.00, 20 0.80; x 32768, 20 0.98; g = 8, x 65536: 10 1.03, 20 0.83; x 32768 0.99.
+// of the call as a fraction of the exhaustive one; normal and uniform points do better):
+// one step: g = 2, 4 M x 4096 0.95; g = 3, x 4096 4 M 1.21, 15.6 M 1.02, 2 M x 8192 0.86; g = 4, 4 M x 8192 0.92, 1 M x 65536 0.47,
+// 0.26 M x 65536 1.25; g = 5, 2 M x 32768 0.82, 4 M x 16384 1.05; g = 6, 2 M x 65536 0.95, 0.5 M x 65536 1.16.
+// A fit: g = 2, 4 M x 4096, 5 iterations 0.62; g = 4, 2 iterations 1.6 M x 16384 1.14, 2.3 M 0.73, 3.1 M x 8192 1.15, 4.7 M 0.90, 5
+// iterations 1 M x 8192 1.10, 4 M x 8192 0.74, 0.26 M x 65536 0.77, 20 iterations 2 M x 4096 0.95, 4 M x 2048 1.17; g = 5, 4 M x 16384,
+// 5 iterations 0.81, 1 M x 8700, 20 0.88, 5 1.27; g = 6, 5 iterations 0.13 M x 65536 1.29, 0.15 M 1.06, 0.5 M 0.90, 2 M x 32768 1.03, 2 M x
+// 65536 0.79, 10 iterations x 32768 0.86, x 16384 1.03, 20 iterations x 16384 0.90, x 8192 1.15; g = 7, x 65536 10 iterations
+// 1.00, 20 0.80, x 32768, 20 0.98; g = 8, x 65536 10 1.03, 20 0.83, x 32768 0.99.
 struct PruneRule { int g_max, steps, K; double scores, scores_all; };   // from so many steps, centroids, N K and N K steps on
 constexpr PruneRule PRUNE_RULES[] = {
-    {3, 1, 4096, 1.6e10, 0},  {3, 2, 4096, 8.5e9, 4e10},  {4, 1, 8192, 3.2e10, 0},  {4, 2, 8192, 8.5e9, 5e10}, {4, 16, 4096, 8.5e9, 0},
+    {3, 1, 4096, 6e10, 0},    {3, 1, 8192, 1.6e10, 0},    {3, 2, 4096, 8.5e9, 4e10},
+    {4, 1, 8192, 3.2e10, 0},  {4, 2, 8192, 8.5e9, 7e10},  {4, 16, 4096, 8.5e9, 0},
     {5, 1, 32768, 3.2e10, 0}, {5, 4, 16384, 3e10, 0},     {5, 16, 8192, 8.5e9, 0},
-    {6, 1, 60000, 1.2e11, 0}, {6, 5, 49152, 8.5e9, 0},    {6, 10, 32768, 3e10, 0},  {6, 16, 16384, 8.5e9, 0},
+    {6, 1, 60000, 1.2e11, 0}, {6, 5, 49152, 1.2e10, 0},   {6, 10, 32768, 3e10, 0},  {6, 16, 16384, 8.5e9, 0},
     {7, 16, 40000, 8.5e9, 0}, {8, 16, 49152, 8.5e9, 0},
 };
 
@@ -218,6 +221,10 @@ bool prune_pays(int64_t N, int g, int K, int steps) {
         if (g <= r.g_max && steps >= r.steps && K >= r.K && scores >= r.scores && scores * steps >= r.scores_all) return true;
     return false;
 }
+
+// Whether the first E-step of a pruned fit starts from the tree.  With up to three dimensions earlier than for a step by itself, as the
+// points are sorted anyway (g = 3, 5 M x 4096, two iterations: 2.68 ms, with an exhaustive first step 3.19).
+bool first_pruned(int64_t N, int g, int K) { return prune_pays(N, g, K, 1) || (g <= 3 && (double)N * (double)K >= 1.6e10); }
 
 bool use_pruned(const cc_ctx* ctx, const WsLayout& L, int64_t N, int g, int K, int steps) {
     return ctx->path == CC_PATH_AUTO && cc_prune_applies(N, g, K) && ctx->ws_bytes >= L.total_preferred && prune_pays(N, g, K, steps);
@@ -257,7 +264,7 @@ cudaError_t fit_pruned(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_
     cudaError_t e = prune_order(ctx, b, X, g, C, st);
     for (int it = 0; it < iters && e == cudaSuccess; ++it) {
         bool have_max = true;
-        if (it == 0 && !prune_pays(N, g, K, 1)) {            // nothing known of the points yet
+        if (it == 0 && !first_pruned(N, g, K)) {            // nothing known of the points yet
             e = cc_launch_assign_tensor(ctx, L, b.Xs, N, g, C, K, b.idx_s, b.dist_s, nullptr, nullptr, st);
             have_max = false;
         } else {

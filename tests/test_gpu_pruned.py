@@ -42,6 +42,7 @@ def _fit(X, g, K, iters, C0, path):
     (2100001, 4, 4097, 17, "ties"), (1000003, 4, 16385, 4, "heavy"), (2000003, 3, 9001, 2, "heavy"), (400129, 6, 24003, 17, "clumps"),
     (2200000, 2, 4100, 5, "heavy"), (300031, 1, 30000, 5, "heavy"), (150001, 7, 65500, 17, "heavy"), (150000, 8, 65536, 17, "ties"),
     (524288, 5, 65535, 5, "heavy"), (140000, 6, 65535, 6, "ties"), (4000001, 4, 8193, 2, "clumps"), (2000003, 6, 61000, 5, "heavy"),
+    (190001, 6, 65535, 6, "ties"), (4400001, 4, 8193, 2, "clumps"), (1990001, 3, 8200, 2, "heavy"),
 ])
 def test_pruned_fit_equals_exhaustive_fit(N, g, K, iters, kind):
     from paper_2503_13089_b200 import binding as cc
