@@ -42,7 +42,7 @@ order_init_kernel(unsigned* __restrict__ order, int K, int Kp) {
 __global__ void __launch_bounds__(KT_THREADS, 1)
 tree_split_kernel(const float* __restrict__ C, int K, int g, int n, const unsigned* __restrict__ in,
                   unsigned* __restrict__ out, unsigned* __restrict__ tree) {
-    extern __shared__ uint16_t keys[];                       // n
+    extern __shared__ __align__(16) uint16_t keys[];                       // n
     __shared__ float part[16][32][2];
     __shared__ int cnt[2][32];
     __shared__ int axis_sh;
@@ -142,7 +142,7 @@ tree_finish_kernel(const float* __restrict__ C, int K, int g, int n0, unsigned* 
                    int first) {
     __shared__ unsigned long long key[KB_MAX];
     __shared__ unsigned char axes[KB_MAX / 2];
-    extern __shared__ float var[];                           // (n0 / n) x g of one level, at most n0 / 2 x g words
+    extern __shared__ __align__(16) float var[];                           // (n0 / n) x g of one level, at most n0 / 2 x g words
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int start = blockIdx.x * n0;
     for (int e = tid; e < n0; e += KT_THREADS) key[e] = order[start + e];
@@ -223,7 +223,7 @@ template <int G>
 __global__ void __launch_bounds__(1024, 1)
 point_leaf_kernel(const uint16_t* __restrict__ X, int64_t N, const unsigned* __restrict__ tree, int levels,
                   uint16_t* __restrict__ leaf, unsigned* __restrict__ rank, unsigned* __restrict__ hist) {
-    extern __shared__ unsigned st[];
+    extern __shared__ __align__(16) unsigned st[];
     const int in_smem = (1 << levels) < PK_SMEM_NODES ? (1 << levels) : PK_SMEM_NODES;
     for (int e = threadIdx.x; e < in_smem; e += 1024) st[e] = tree[e];
     __syncthreads();
