@@ -6,13 +6,14 @@
 
 One "step" is one pass of the whole path over the synthetic weight matrices of the workload
 (default: the 8192x28672, g=4, K=65536, 10-iteration configuration, the largest one).  Rank 0 prints
-one JSON line; it also carries, under "workloads", a short run of every other configuration.
+one JSON line, short enough for a reader that keeps only the end of the output; what explains it (kernel classes, the rooflines, a
+short run of every other configuration, the layer forward) goes to standard error as one line that starts with "detail".
 With N > 1 every rank clusters its own matrices (different seeds) and no data crosses ranks: the
 paper's "clustering of different matrices is independent".
 
 The unit counts distances that are evaluated, so the headline, its rooflines and the other configurations run the
 exhaustive E-step on the tensor cores.  The library's default path rules centroids out without evaluating them where that is
-faster and gives the same codes, centroids and distances; its times stand beside them under "default_path".
+faster and gives the same codes, centroids and distances; its times stand in the line under "default_path".
 
 `--kernel` runs one entry point a few times on a synthetic case of the given size and prints the
 mean device time per kernel class (the small cases the ncu summaries under profiles/ were taken on).
@@ -706,18 +707,25 @@ def main():
                        "l2": "flushed between timed steps (256 MB write)",
                        "step": "reshape + init + %d x (assign + update) + finalize + decode per matrix" % iters},
             "s_per_lloyd_iteration": summ["s_per_lloyd_iteration"],
+            "e2e": {"value": total_evals / (e2e_step * 1e-3), "unit": "distance evaluations/s",
+                    "ms_per_step": e2e_step, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
+                    "api": "cc_compress_host, pinned host buffers"},
+            "default_path": {"ms_per_step": sum(default_ms) / len(default_ms),
+                             "e2e_ms_per_step": sum(default_e2e_ms) / len(default_e2e_ms)} if default_ms else None,
+            "gpu_launches": launches,
+            "roofline": {k: roofline.get(k) for k in ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic", "avg_launch_ms",
+                                                      "launches")},
+            "clocks": clocks,
+            "cpu_baseline": cpu_baseline,
+        }
+        detail = {
             "e_step_ms": summ["e_step_ms"], "m_step_ms": summ["m_step_ms"], "final_e_step_ms": summ["final_e_step_ms"],
             "near_tie_points_per_assign": resolved,
             "ms_steps": ms_steps,
-            "e2e": {"value": total_evals / (e2e_step * 1e-3), "unit": "distance evaluations/s",
-                    "ms_per_step": e2e_step, "steps": len(e2e_ms), "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
-                    "api": "cc_compress_host: pinned host W in; FP16 codebook, codes, objective trace and the decoded "
-                           "matrix out (the same work as the device-resident step plus the copies); its device buffer "
-                           "is allocated by one untimed call"},
-            "default_path": {"ms_per_step": sum(default_ms) / len(default_ms), "e2e_ms_per_step": sum(default_e2e_ms) / len(default_e2e_ms),
-                             "note": "this rank; the same step with the library's own choice of E-step: same codes, centroids and "
-                                     "distances, not every distance evaluated"} if default_ms else None,
-            "gpu_launches": launches,
+            "e2e_note": "FP16 codebook, codes, objective trace and the decoded matrix out (the same work as the device-resident "
+                        "step plus the copies); its device buffer is allocated by one untimed call",
+            "default_path_note": "this rank; the same step with the library's own choice of E-step: same codes, centroids and "
+                                 "distances, not every distance evaluated",
             "roofline": roofline,
             "hbm_kernels": summ["hbm_kernels"],
             "kernels": summ["kernel_classes"],
@@ -727,10 +735,9 @@ def main():
             "probes": {"min_rate_lane_instr_per_clk_per_sm": min_rate, "probe_sm_mhz": probe_mhz,
                        "probe_distinct_sms": probe_sms, "fp32_fma_tflops_scalar": fp32_scalar,
                        "fp32_fma_tflops_packed": fp32_packed},
-            "clocks": clocks,
-            "cpu_baseline": cpu_baseline,
             "context": {"paper_70B_clustering_hours_1gpu": 25.6},
         }
+        sys.stderr.write("detail " + json.dumps(detail) + "\n")
         print(json.dumps(line))
     if world > 1:
         dist.destroy_process_group()
