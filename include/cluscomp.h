@@ -79,7 +79,9 @@ const char* cc_status_string(cc_status s);
 size_t cc_workspace_bytes(int64_t N, int g, int K);
 /* The size with which cc_assign, cc_fit and cc_finalize can also take the E-step that rules centroids out first (same results,
  * up to nine times faster on large problems; it keeps the points in spatial order and lists of what may matter, up to about
- * (50 + 2 g) bytes per point and a further 4 GB).  Never less than cc_workspace_bytes, with which every call runs. */
+ * (50 + 2 g) bytes per point and a further 4 GB).  Never less than cc_workspace_bytes, with which every call runs.
+ * cc_compress_host takes the preferred size where device memory reaches that far; a size that was refused once is not
+ * asked for again by that context. */
 size_t cc_workspace_bytes_preferred(int64_t N, int g, int K);
 cc_status cc_set_workspace(cc_ctx* ctx, void* workspace, size_t bytes);
 
@@ -343,7 +345,7 @@ cc_status cc_decode(cc_ctx* ctx, const uint16_t* C16, int K, int g, const uint16
  *   weight = codebook[code].view(in_features, -1) with the padded columns dropped;  y = x . weight (+ bias).
  * Up to a few hundred tokens the decoded weight is never written to memory: codebook rows are looked up in, or gathered
  * straight into, shared memory (FP16 inputs, FP32 accumulation).  From there on it is decoded once per call into tiles
- * in the workspace (at most 128 MB at a time) and multiplied by a tensor-core GEMM.
+ * in the workspace (at most 128 MB at a time, or two rows of tiles) and multiplied by a tensor-core GEMM.
  * x: M x d_in FP16 row-major (M tokens).  C16: K x g FP16.  idx: cc_num_subvectors(d_out, d_in, g,
  * CC_LAYOUT_PAPER_T) codes, each < K.  bias (may be NULL): d_out FP32.  y (out): M x d_out FP32
  * row-major.  The listing keeps every tensor in a 16-bit type; here the accumulator is handed out

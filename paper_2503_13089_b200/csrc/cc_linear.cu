@@ -374,7 +374,7 @@ linear_reduce_kernel(const float* __restrict__ partial, int splits, int64_t n, i
 // FP16 codebook: a table that does not fit is cut into slices, a CTA for each.  It reads all the codes of its range and
 // adds up those inside its slice; the others read a row of zeros behind it.  Reading every code once per slice is
 // cheap (coalesced, about 12 instructions each) beside a gather from L2, of which an SM gets 0.73 a clock through: one
-// token, 4096 x 4096, g = 4, K = 65536 (512 KB, three slices) 26.9 us as gathers, 17.2 so.
+// token, 4096 x 4096, g = 4, K = 65536 (512 KB, three slices) 26.9 us as gathers, 18.4 so.
 // CTA = 64 threads' code groups x 16 interleaved sub-slices of the in_features; the sixteen partial sums meet in
 // shared memory in a fixed order, and the CTA writes its slab of partial sums (y itself when there is a single
 // slab); the slabs are added in order by the CTA that finishes last, or by linear_reduce_kernel: the same bits
@@ -691,7 +691,8 @@ LinearPlan linear_plan(int64_t M, int64_t d_out, int64_t d_in, int sm_count, int
     LinearPlan p;
     const int64_t mt = M < nt_max ? M : nt_max;
     p.NT = (int)((mt + 15) / 16 * 16);
-    // FP16 codebook with rows of at most 8 bytes, many tokens: the gathers of the weight tile bound a stage, so
+    // FP16 codebook with rows of at most 8 bytes, many tokens (of a layer too narrow for cc_linear_wide.cu, which the figures here
+    // were taken before): the gathers of the weight tile bound a stage, so
     // one tile serves 512 tokens (two MMAs of 256 columns, all 512 TMEM columns) and the pipeline has two stages
     // of that size: 4096 x 4096, g 4, 4096 tokens 0.571 -> 0.464 ms.  With 16-byte rows (g = 8) there are half as
     // many gathers per weight and the coarser grid costs more than the reuse saves (1.62 -> 1.70 ms on 8192 x 8192).

@@ -23,7 +23,8 @@ constexpr int LG_SPLITS_MAX = 65535;                   // gridDim.y
 // Rows of codes a thread requests together; the next ones are under way while these are used.
 CC_PLAN_FN constexpr int gemv_batch(int g, int mt) { return g * mt <= 8 ? 8 : 4; }
 // Neighbouring code groups per thread: two codes come in one word and share the loads of x.  For short rows of the FP16
-// codebook and layers of many codes: one token, g = 4, K = 65536, 11008 x 4096 39.8 -> 33.7 us, 4096 x 4096 18.7 -> 17.2;
+// codebook and layers of many codes (calls back to back, codes in L2): one token, g = 4, K = 65536, 11008 x 4096 39.8 -> 33.7 us, 4096 x
+// 4096 18.7 -> 17.2;
 // with few codes the wider exchange at the end costs more (g = 3, 700 x 900 7.7 -> 9.3; g = 8, 4096 x 4096 16.2 -> 17.1).
 constexpr bool gemv_pair(int g, bool quant) { return g <= 4 && !quant; }
 constexpr int64_t LG_PAIR_FROM = 1 << 21;              // codes
