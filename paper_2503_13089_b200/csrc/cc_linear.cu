@@ -658,14 +658,17 @@ linear_pad_rows_kernel(const uint16_t* __restrict__ C16, int K, int g, int pad, 
     }
 }
 
-// Gathers (codes times blocks of tokens) from which the copy pays: as a launch it takes one to two us.  33 tokens, with / without, in
-// us: 1024 x 4096, g = 6 (0.7 M) K = 256 12.8 / 10.8, K = 16000 13.7 / 13.0; 2048 x 2048, g = 5 (0.8 M) 12.5 / 11.1 and 13.7 / 13.6;
-// 4096 x 4096, g = 9 (1.9 M) 20.8 / 21.4 and 25.6 / 31.4, g = 6 (2.8 M) 21.5 / 20.2 and 25.8 / 28.4; 11008 x 4096, g = 6 (7.5 M) 47.8 / 48.1
-// and 58.9 / 69.9.  320 tokens, 1024 x 4096, K = 65536: g = 6 (1.4 M) 29.2 / 32.1, g = 9 (0.9 M) 27.3 / 30.0.
-constexpr int64_t LINEAR_PAD_ODD = 900000, LINEAR_PAD_EVEN = 1200000, LINEAR_PAD_EVEN_SMALL = 3200000;   // the last for codebooks that L1 holds
+// Gathers (codes times blocks of tokens) from which the copy pays: as a launch it takes one to two us.  With / without, in us.  Even g, 33
+// tokens: 1024 x 4096, g = 6 (0.7 M) K = 256 12.8 / 10.8, K = 16000 13.7 / 13.0; 4096 x 4096, g = 6 (2.8 M) 21.5 / 20.2 and 25.8 / 28.4;
+// 11008 x 4096, g = 6 (7.5 M) 47.8 / 48.1 and 58.9 / 69.9; 320 tokens, 1024 x 4096, g = 6, K = 65536 (1.4 M) 29.2 / 32.1.  Odd g, whose
+// rows start in either half of a word: 33 tokens, 2048 x 2048, g = 5 (0.8 M), K = 256 12.5 / 11.1, K = 16000 13.7 / 13.6; 1408 x 2368,
+// g = 7 (0.5 M), K = 19472 16.1 / 21.3; 10 tokens, 852 x 3703, g = 7 (0.5 M), K = 36751 19.0 / 25.1.
+constexpr int64_t LINEAR_PAD_ODD = 400000, LINEAR_PAD_EVEN = 1200000;
+constexpr int64_t LINEAR_PAD_ODD_SMALL = 900000, LINEAR_PAD_EVEN_SMALL = 3200000;                       // for codebooks that L1 holds
 constexpr int LINEAR_PAD_SMALL = 512;                                                                   // rows
 int64_t linear_pad_from(int g, int K) {
-    return g % 2 ? LINEAR_PAD_ODD : K <= LINEAR_PAD_SMALL ? LINEAR_PAD_EVEN_SMALL : LINEAR_PAD_EVEN;
+    if (K <= LINEAR_PAD_SMALL) return g % 2 ? LINEAR_PAD_ODD_SMALL : LINEAR_PAD_EVEN_SMALL;
+    return g % 2 ? LINEAR_PAD_ODD : LINEAR_PAD_EVEN;
 }
 
 // Tokens from which decoding the weight once and multiplying it afterwards (cc_linear_wide.cu) is the faster way, gathering /
