@@ -1,0 +1,33 @@
+"""All iterations of a small fit in one launch against the same iterations one launch each: the same bits."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("N,g,K,iters", [
+    (1, 3, 1, 3), (255, 4, 7, 4), (257, 4, 256, 5), (32768, 4, 1024, 7),          # one block, two, every block one step; K g at the bound
+    (120000, 4, 257, 3), (70001, 1, 300, 6), (5000, 16, 256, 2),                  # several steps a block; odd sizes; long sub-vectors
+])
+def test_small_fit_in_one_launch(N, g, K, iters):
+    from paper_2503_13089_b200 import binding as cc
+    from tests import gpu_util as u
+    rng = np.random.default_rng(N + g + K)
+    X = u.half_dev(rng.standard_t(3.0, (N, g)).astype(np.float16))
+    c = u.ctx()
+    c.ensure_workspace(N, g, K)
+    C0 = torch.empty((K, g), device="cuda")
+    cc.cc_init_codebook(c, X, N, g, K, 5, C0)
+
+    def buffers():
+        return (C0.clone(), torch.zeros(N, dtype=torch.uint16, device="cuda"), torch.empty(N, device="cuda"),
+                torch.empty(K, dtype=torch.int32, device="cuda"), torch.zeros(iters, dtype=torch.float64, device="cuda"))
+
+    a, b = buffers(), buffers()
+    cc.cc_fit(c, X, N, g, K, iters, *a)
+    for it in range(iters):
+        cc.cc_fit(c, X, N, g, K, 1, *b[:4], b[4][it:])
+    cc.cc_poll_status(c)
+    for x, y in zip(a, b):
+        assert x.cpu().numpy().tobytes() == y.cpu().numpy().tobytes()
