@@ -59,6 +59,23 @@ struct ProfScope {
     ~ProfScope() { if (slot) cudaEventRecord(slot->b, st); }
 };
 
+// Launch that may begin before the kernel in front of it has ended; what it needs of that one stands behind
+// griddepcontrol.wait.
+template <class... Args, class... Given>
+cudaError_t launch_after(dim3 grid, dim3 block, size_t smem, cudaStream_t st, void (*kernel)(Args...), Given... args) {
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args>(args)...);
+}
+
 // Status block at the start of every workspace: cleared by cc_set_workspace.
 constexpr size_t CC_STATUS_BYTES = 4096;
 constexpr int CC_ARRIVAL_WORD = 64, CC_ARRIVAL_COUNTERS = 960;
@@ -205,7 +222,8 @@ cudaError_t cc_launch_small_loop(cc_ctx*, const WsLayout&, const uint16_t* X, in
 constexpr size_t CC_LINEAR_SCRATCH_FROM = CC_STATUS_BYTES + (size_t)65536 * 32;
 
 // Compressed linear layer: y = x . decode(C16, idx)^T (+ bias).
-size_t cc_linear_scratch_bytes(int64_t M, int64_t d_out, int64_t d_in, int sm_count);
+size_t cc_linear_scratch_bytes(int64_t M, int64_t d_out, int64_t d_in, int sm_count);             // what every call needs
+size_t cc_linear_scratch_bytes_preferred(int64_t M, int64_t d_out, int64_t d_in, int sm_count);   // what every way of a call needs
 int cc_linear_q_table_max(void);
 // The same for many tokens (cc_linear_wide.cu): the weight is decoded once into tiles in the workspace.
 bool cc_linear_wide_applies(int64_t M, int64_t d_out, int64_t d_in, int splits, int sm_count);

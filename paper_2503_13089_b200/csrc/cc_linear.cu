@@ -1,7 +1,8 @@
 // Forward of the compressed linear layer (appendix listing): out = x . weight (+ bias) with
 // weight = codebook[code] viewed as (in_features, out_features + pad), the padded columns dropped.
-// Three ways: a few tokens look the codes up in shared memory (linear_gemv_kernel below), many multiply a weight decoded
-// once (cc_linear_wide.cu), those in between take the kernel described here.
+// Four ways: a few tokens look the codes up in shared memory (linear_gemv_kernel below), a batch of them looks them up
+// coordinate by coordinate into the operand of a product (cc_linear_planes.cu), many tokens multiply a weight decoded
+// once (cc_linear_wide.cu); where none of these is the faster one, the kernel described here.
 // The decoded weight is never written to memory: the kernel gathers codebook rows straight into the
 // shared-memory operand of a tcgen05 GEMM.
 //
@@ -29,6 +30,10 @@
 #include "cc_tcgen05.cuh"
 #include "cc_linear_plan.h"
 #include "cc_linear_rows.cuh"
+
+cudaError_t cc_launch_linear_planes(cc_ctx* ctx, const PlanesPlan& p, const uint16_t* x, int M, const uint16_t* C16, const unsigned char* qtab,
+                                    const float* qscale, int K, int g, const uint16_t* idx, int d_out, int d_in, const float* bias, float* y,
+                                    cudaStream_t st);
 
 namespace {
 
@@ -686,6 +691,8 @@ int linear_wide_from(int fill, int64_t d_in, int g, bool quant) {
     return !quant && fill > 2 && g <= 6 && d_in > 8192 ? LINEAR_WIDE_LONG : LINEAR_WIDE_FROM;
 }
 
+constexpr int PLANES_CHAIN_MOST = 16;
+
 constexpr int LINEAR_SPLITS_MORE = 8;   // splits beyond those that fill the SMs once are tried up to this many
 
 struct LinearPlan { int NT, a_pad, stages, tmem_cols, o_tiles, tok_blocks, splits, chunks_per_split, fill; size_t smem; };   // fill: splits that fill the SMs once
@@ -749,6 +756,23 @@ size_t cc_linear_scratch_bytes(int64_t M, int64_t d_out, int64_t d_in, int sm_co
     const size_t own = CC_LINEAR_SCRATCH_FROM + (size_t)splits * (size_t)M * (size_t)d_out * 4;
     const size_t wide = M >= LINEAR_WIDE_FEWEST ? cc_linear_wide_bytes(M, d_out, d_in) : 0;
     return own > wide ? own : wide;
+}
+
+// Stages of 64 in_features that the planes' kernel may add up in one accumulator: no longer a chain than the tensor
+// kernel would have had (its splits), and at most 16.
+static int planes_chain(int64_t M, int64_t d_out, int64_t d_in, int sm_count, int g) {
+    const LinearPlan p = linear_plan(M, d_out, d_in, sm_count, LNT_MAX, 0, g);
+    return p.chunks_per_split < PLANES_CHAIN_MOST ? p.chunks_per_split : PLANES_CHAIN_MOST;
+}
+
+size_t cc_linear_scratch_bytes_preferred(int64_t M, int64_t d_out, int64_t d_in, int sm_count) {
+    size_t most = cc_linear_scratch_bytes(M, d_out, d_in, sm_count);
+    if (M > PL_NT_MAX) return most;
+    for (int g = 1; g <= 16; ++g) {
+        const size_t b = CC_LINEAR_SCRATCH_FROM + planes_bytes_most(M, d_out, d_in, g, planes_chain(M, d_out, d_in, sm_count, g));
+        if (b > most) most = b;
+    }
+    return most;
 }
 
 int cc_linear_q_table_max(void) { return LQ_TABLE_MAX; }
@@ -903,6 +927,12 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
         if (blocks > cap) blocks = cap;
         linear_reduce_kernel<<<(unsigned)blocks, 256, 0, st>>>(partial, slabs_n, n, (int)d_out, bias, y);
         return cudaGetLastError();
+    }
+    {
+        PlanesPlan pl = {};
+        if (M <= PL_NT_MAX) pl = planes_plan(M, d_out, d_in, ctx->sm_count, K, g, planes_chain(M, d_out, d_in, ctx->sm_count, g));
+        if (pl.fits && planes_pay(pl, M, out_groups * d_in, g, qtab != nullptr) && ctx->ws_bytes >= CC_LINEAR_SCRATCH_FROM + pl.bytes)
+            return cc_launch_linear_planes(ctx, pl, x, (int)M, C16, qtab, qscale, K, g, idx, (int)d_out, (int)d_in, bias, y, st);
     }
     // beside the table: token blocks of 64 with four stages, or, from LQ_WIDE_FROM tokens on, of 256 with two
     const LinearPlan p = qtab ? linear_plan(M, d_out, d_in, ctx->sm_count, M >= LQ_WIDE_FROM ? LNT_MAX : LQ_NT_MAX, (size_t)K * (g / 2), g)

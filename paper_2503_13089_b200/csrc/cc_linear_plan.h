@@ -11,6 +11,11 @@
 #define CC_PLAN_FN
 #endif
 
+// ---- Layer forward plane by plane (cc_linear_planes.cu).
+// PP: coordinates side by side in a table row; groups: plane groups (a table each); ctas: per plane group; an item is a tile of
+// 128 / PP code groups and one of `splits` parts of the in_features.
+struct PlanesPlan { int PP, groups, ctas, tiles, splits, NT, nt_cols, stages, tmem_cols; size_t smem, x_bytes, bytes; bool fits; double clocks; };
+
 namespace {
 
 constexpr int LG_THREADS = 1024, LG_GRPS = 64, LG_SUB = 16, LG_M_MAX = 4;
@@ -123,6 +128,94 @@ inline int64_t gemv_slabs_most(int64_t d_out, int64_t d_in, int sm_count) {
 inline size_t padded_table_at(uintptr_t ws, size_t from, size_t to, int K, int pad) {
     const size_t at = ((ws + from + 31) & ~(uintptr_t)31) - ws;
     return at + (size_t)K * pad * 2 <= to ? at : 0;
+}
+
+// ---- Layer forward plane by plane.
+constexpr int PL_ROWS = 128, PL_KB = 64, PL_NT_MAX = 256, PL_SPLITS_MAX = 64;
+constexpr size_t PL_SMEM = 226 * 1024, PL_HEAD = 256;
+
+// Clocks of an SM for a stage of 64 in_features: its 2 CW look-ups by 32 lanes take 3.5 clocks each (rows of 2 or 4 bytes) or 6.2
+// (8 bytes), half a clock goes to the codes and half to each 16-byte piece of the operand.
+constexpr double planes_stage_clocks(int PP) { return 2.0 * (PL_ROWS / PP) * ((PP == 4 ? 6.2 : 3.5) + 0.5 + 0.5 * PP); }
+
+constexpr size_t PL_SLABS_MOST = 48u << 20;           // bytes of partial sums, unless the shortest chains ask for more
+
+// chain: stages of 64 in_features that may be added up in one accumulator.
+inline PlanesPlan planes_plan(int64_t M, int64_t d_out, int64_t d_in, int sm_count, int K, int g, int chain) {
+    PlanesPlan best = {};
+    const int chunks = (int)((d_in + PL_KB - 1) / PL_KB);
+    const int out_groups = (int)((d_out + g - 1) / g);
+    if (M > PL_NT_MAX) return best;
+    for (int PP = 1; PP <= 4; PP *= 2) {
+        PlanesPlan p = {};
+        p.PP = PP;
+        p.groups = (g + PP - 1) / PP;
+        if (PP > 1 && p.groups == (g + PP / 2 - 1) / (PP / 2)) continue;      // no fewer tables than with shorter rows
+        p.NT = (int)((M + 15) / 16 * 16);
+        p.nt_cols = (p.NT + 31) / 32 * 32;
+        const size_t table = ((size_t)K * PP * 2 + 15) / 16 * 16, stage = PL_ROWS * PL_KB * 2 + (size_t)p.NT * PL_KB * 2;
+        p.stages = 4 * stage + table + PL_HEAD <= PL_SMEM ? 4 : 2;
+        p.smem = p.stages * stage + table + PL_HEAD;
+        if (p.smem > PL_SMEM) continue;
+        p.tmem_cols = 64;
+        while (p.tmem_cols < 2 * p.nt_cols) p.tmem_cols *= 2;
+        const int cw = PL_ROWS / PP, most_ctas = sm_count / p.groups;
+        if (most_ctas < 1) continue;
+        p.tiles = (out_groups + cw - 1) / cw;
+        int least = (chunks + chain - 1) / chain, most = chunks < PL_SPLITS_MAX ? chunks : PL_SPLITS_MAX;
+        if (least < 1) least = 1;
+        if (most < least) most = least;
+        p.x_bytes = (size_t)p.NT * chunks * (PL_KB * 2);
+        p.fits = true;
+        for (int s = least; s <= most; ++s) {
+            const int64_t items = (int64_t)p.tiles * s;
+            const size_t slabs = (size_t)p.groups * items * p.NT * PL_ROWS * 4;
+            if (s > least && slabs > PL_SLABS_MOST) break;
+            const int rounds = (int)((items + most_ctas - 1) / most_ctas);
+            const double t = rounds * ((double)chunks / s * planes_stage_clocks(PP) + 400.0 + 4.0 * p.NT) +
+                             (double)s * p.tiles * p.groups * p.NT * PL_ROWS * 8.0 / 4000.0 + (double)table / 50.0;
+            if (best.fits && t >= best.clocks) continue;
+            p.splits = s;
+            p.clocks = t;
+            p.ctas = items < most_ctas ? (int)items : most_ctas;
+            p.bytes = p.x_bytes + slabs;
+            best = p;
+        }
+    }
+    return best;
+}
+
+// Whether the planes' three launches beat the kernels they stand in for.  The planes win where the look-ups are many for each table
+// an SM loads and each launch, and lose where a code costs more look-ups than gathers would take from L2.  Old / planes in us:
+//   g >= 10 with fewer than four coordinates a look-up (33 tokens, 4096 x 4096, g = 16, K = 65536 20 / 34; with four:
+//     119 tokens, 3008 x 10368, K = 4880 44 / 29);
+//   one coordinate a look-up (K > 51,000 or so): 4096 x 4096, 33 tokens, g = 4 27 / 23, 11008 x 4096 68 / 44, g = 6 65 / 50, g = 8 53 / 49,
+//     but 4096 x 4096, g = 8 22 / 27 and, few codes, 22 tokens, 1344 x 4992, g = 5 18 / 24, 153 tokens, 1024 x 1024, g = 6 13 / 17;
+//   many parts of the in_features, i.e. few out_features: 57 tokens, 640 x 9707, g = 6, K = 12893 17 / 20, 25 tokens, 640 x 6893,
+//     g = 4, K = 27278 12 / 15; with four coordinates a look-up 12 tokens, 832 x 1984, g = 4, K = 1137 14 / 10;
+//   the 4-bit codebook from 192 tokens on, where the weight is decoded once: 215 tokens, 8064 x 2191, g = 8 24 / 41;
+//   many tokens on few codes: 224 tokens, 768 x 512, g = 4, K = 17749 12.9 / 14.3.
+// Over 162 drawn layers of 5 to 256 tokens the planes alone are 1.22 times as fast in the mean, with these bounds 1.24.
+// Up to 64 tokens the answer may not depend on the form of the codebook (both give the same bits there).
+inline bool planes_pay(const PlanesPlan& p, int64_t M, int64_t codes, int g, bool quant) {
+    if (g >= 10 && p.PP < 4) return false;
+    if (p.PP == 1 && (g >= 8 || codes < 2000000)) return false;
+    if (p.PP < 4 && p.splits > 16) return false;
+    return !(quant && M > 192) && !(M > 128 && codes < 200000);
+}
+
+// At least the scratch of any such plan for this g, whatever the codebook's size.
+inline size_t planes_bytes_most(int64_t M, int64_t d_out, int64_t d_in, int g, int chain) {
+    const int64_t chunks = (d_in + PL_KB - 1) / PL_KB, out_groups = (d_out + g - 1) / g, NT = (M + 15) / 16 * 16;
+    const int64_t least = (chunks + chain - 1) / chain;
+    size_t most = 0;
+    for (int PP = 1; PP <= 4; PP *= 2) {
+        const int64_t tiles = (out_groups + PL_ROWS / PP - 1) / (PL_ROWS / PP) * ((g + PP - 1) / PP);
+        const size_t one = (size_t)tiles * NT * PL_ROWS * 4, lo = one * least, hi = one * PL_SPLITS_MAX;
+        const size_t cut = hi < PL_SLABS_MOST ? hi : PL_SLABS_MOST, b = lo > cut ? lo : cut;
+        if (b > most) most = b;
+    }
+    return most + (size_t)NT * chunks * (PL_KB * 2);
 }
 
 }  // namespace

@@ -204,6 +204,7 @@ linear_gemm_kernel(const unsigned char* __restrict__ w_tiles, const unsigned cha
     if (warp == GW) {
         // ------------------------------------------------------------ copies
         if (elect_one()) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");       // the tiles
             int st = 0, total = 0;
             uint32_t ph = 0;
             const unsigned char* bsrc = x_tiles + (int64_t)blockIdx.y * chunks * NT * (WKB * 2);
@@ -372,9 +373,8 @@ cudaError_t launch_gemm(cc_ctx* ctx, const WidePlan& p, const unsigned char* w_t
     const int stages = gemm_stages(ROWS, p.NT);
     const dim3 grid((unsigned)((row_tiles + ROWS - 1) / ROWS), (unsigned)((m_end - m_first + p.NT - 1) / p.NT));
     ProfScope ps(ctx, CC_K_LINEAR, st);
-    linear_gemm_kernel<ROWS><<<grid, GEMM_THREADS, stages * gemm_stage_bytes(ROWS, p.NT), st>>>(
-        w_tiles, x_tiles, chunks, p.NT, stages, p.segs, row_tiles, o_first, (int)d_out, (int)m_first, (int)m_end, bias, y, status);
-    return cudaGetLastError();
+    return launch_after(grid, dim3(GEMM_THREADS), (size_t)stages * gemm_stage_bytes(ROWS, p.NT), st, linear_gemm_kernel<ROWS>,
+                        w_tiles, x_tiles, chunks, p.NT, stages, p.segs, row_tiles, o_first, (int)d_out, (int)m_first, (int)m_end, bias, y, status);
 }
 
 template <int G, bool QUANT>

@@ -1,0 +1,50 @@
+"""The planes' layer forward (cc_linear_planes.cu): its launch plans, walked on the host.  No plan may ask for more shared memory or
+tensor memory than there is, more scratch than cc_linear_workspace_bytes answers, longer chains than allowed, or blocks without work."""
+import os
+import subprocess
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2503_13089_b200", "csrc")
+
+WALK = r"""
+#include <cstdio>
+#include <initializer_list>
+#include "cc_linear_plan.h"
+
+int main() {
+    long plans = 0, bad = 0;
+    const int64_t layers[][2] = {{28672, 8192}, {11008, 4096}, {128256, 4096}, {4096, 4096}, {1024, 11008}, {700, 900}, {1, 1}, {65, 30000}, {512, 513}};
+    const int tokens[] = {1, 5, 16, 17, 33, 48, 64, 65, 100, 128, 192, 255, 256};
+    const int books[] = {1, 2, 300, 4096, 12287, 12288, 16384, 24575, 32768, 32769, 50000, 65535, 65536};
+    for (const auto& l : layers)
+        for (int g = 1; g <= 16; ++g)
+            for (int M : tokens)
+                for (int K : books)
+                    for (int chain : {1, 3, 16}) {
+                        const PlanesPlan p = planes_plan(M, l[0], l[1], 148, K, g, chain);
+                        const int chunks = (int)((l[1] + 63) / 64);
+                        const size_t table = ((size_t)K * p.PP * 2 + 15) / 16 * 16;
+                        bool ok = p.fits && p.PP * p.groups >= g && p.PP * (p.groups - 1) < g && p.NT >= M && p.NT % 16 == 0 && p.nt_cols >= p.NT &&
+                                  p.nt_cols % 32 == 0 && 2 * p.nt_cols <= p.tmem_cols && p.tmem_cols <= 512 && (p.stages == 2 || p.stages == 4);
+                        ok = ok && p.smem <= PL_SMEM && p.smem >= table + p.stages * (size_t)(128 * 64 * 2 + p.NT * 128) + PL_HEAD;
+                        const int64_t out_groups = (l[0] + g - 1) / g, items = (int64_t)p.tiles * p.splits;
+                        ok = ok && (int64_t)p.tiles * (128 / p.PP) >= out_groups && p.ctas >= 1 && p.ctas <= items && p.ctas * p.groups <= 148;
+                        ok = ok && p.splits >= 1 && p.splits <= chunks && (chunks + p.splits - 1) / p.splits <= chain;
+                        ok = ok && p.bytes == p.x_bytes + (size_t)p.groups * items * p.NT * 512 && p.x_bytes == (size_t)p.NT * chunks * 128;
+                        ok = ok && p.bytes <= planes_bytes_most(M, l[0], l[1], g, chain);
+                        ++plans;
+                        if (!ok && bad++ < 10)
+                            printf("M=%d %ldx%ld g=%d K=%d chain=%d: PP %d groups %d ctas %d tiles %d splits %d NT %d stages %d smem %zu\n", M, (long)l[0],
+                                   (long)l[1], g, K, chain, p.PP, p.groups, p.ctas, p.tiles, p.splits, p.NT, p.stages, p.smem);
+                    }
+    printf("%ld plans, %ld bad\n", plans, bad);
+    return bad != 0;
+}
+"""
+
+
+def test_no_plan_of_the_planes_exceeds_its_limits(tmp_path):
+    src, exe = tmp_path / "walk.cpp", tmp_path / "walk"
+    src.write_text(WALK)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    out = subprocess.run([str(exe)], stdout=subprocess.PIPE, text=True)
+    assert out.returncode == 0, out.stdout
