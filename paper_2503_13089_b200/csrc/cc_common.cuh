@@ -164,6 +164,10 @@ cudaError_t cc_launch_reshape(cc_ctx*, const uint16_t* W, int64_t d_out, int64_t
                               uint16_t* X, cudaStream_t);
 cudaError_t cc_launch_decode(cc_ctx*, const uint16_t* C16, int K, int g, const uint16_t* idx, int64_t d_out,
                              int64_t d_in, int layout, uint16_t* W_hat, cudaStream_t);
+// The same by coordinates (cc_decode_planes.cu).
+bool cc_decode_planes_applies(int K, int g, int64_t d_out, int64_t d_in, const void* W_hat);
+cudaError_t cc_launch_decode_planes(cc_ctx*, const uint16_t* C16, int K, int g, const uint16_t* idx, int64_t d_out, int64_t d_in,
+                                    uint16_t* W_hat, cudaStream_t);
 cudaError_t cc_launch_gather_init(cc_ctx*, const uint16_t* X, int g, int K, const int64_t* pos_dev, float* C,
                                   cudaStream_t);
 constexpr int CC_INIT_ARGS = 480;      // initial positions that travel as a kernel argument instead of a copy

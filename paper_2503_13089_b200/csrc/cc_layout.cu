@@ -623,6 +623,8 @@ cudaError_t cc_launch_reshape(cc_ctx* ctx, const uint16_t* W, int64_t d_out, int
 
 cudaError_t cc_launch_decode(cc_ctx* ctx, const uint16_t* C16, int K, int g, const uint16_t* idx, int64_t d_out,
                              int64_t d_in, int layout, uint16_t* W_hat, cudaStream_t st) {
+    if (layout == CC_LAYOUT_PAPER_T && cc_decode_planes_applies(K, g, d_out, d_in, W_hat))
+        return cc_launch_decode_planes(ctx, C16, K, g, idx, d_out, d_in, W_hat, st);
     ProfScope ps(ctx, CC_K_DECODE, st);
     if (layout == CC_LAYOUT_PAPER_T) {
         const int64_t out_pad = pad_to(d_out, g);
