@@ -72,6 +72,8 @@ template <int G> struct FfmaCfg {
 template <int G>
 __global__ void prep_ffma_kernel(const float* __restrict__ C, int K, int Kpad, float4* __restrict__ prep,
                                  unsigned* __restrict__ status) {
+    let_next_start();
+    after_previous();
     int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q == 0) {  // reset the flagged-point counter of this E-step
         *reinterpret_cast<ull*>(status + 2) = 0ull;
@@ -107,6 +109,8 @@ __global__ void __launch_bounds__(kThreads, FfmaCfg<G>::MIN_BLOCKS)
 assign_ffma_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __restrict__ C, int K, int Kpad,
                    const float4* __restrict__ prep, uint16_t* __restrict__ idx, float* __restrict__ dist,
                    unsigned* __restrict__ status, unsigned* __restrict__ flagged) {
+    let_next_start();
+    after_previous();
     using Cfg = FfmaCfg<G>;
     constexpr int P = Cfg::P, TILE = Cfg::TILE, CHUNK = Cfg::CHUNK, ROW4 = Cfg::ROW4;
     constexpr bool PACKED = Cfg::PACKED;
@@ -282,6 +286,8 @@ resolve_scan_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __re
                     const unsigned* __restrict__ status, const unsigned* __restrict__ flagged,
                     ResolveEntry* __restrict__ scratch, int64_t cap_entries, uint16_t* __restrict__ idx,
                     float* __restrict__ dist) {
+    let_next_start();
+    after_previous();
     ull F = *reinterpret_cast<const ull*>(status + 2);
     if (F > (ull)N) F = (ull)N;
     if (F == 0) return;
@@ -371,6 +377,8 @@ __global__ void __launch_bounds__(128)
 resolve_merge_kernel(int64_t N, int K, const unsigned* __restrict__ status, const unsigned* __restrict__ flagged,
                      const ResolveEntry* __restrict__ scratch, int64_t cap_entries, ull scan_threads,
                      uint16_t* __restrict__ idx, float* __restrict__ dist) {
+    let_next_start();
+    after_previous();
     ull F = *reinterpret_cast<const ull*>(status + 2);
     if (F > (ull)N) F = (ull)N;
     if (F == 0) return;
@@ -422,6 +430,8 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 __global__ void __launch_bounds__(256)
 objective_kernel(const float* __restrict__ dist, int64_t N, double* __restrict__ partials, unsigned* __restrict__ status,
                  double* __restrict__ objective, int64_t* __restrict__ n_resolved) {
+    let_next_start();
+    after_previous();
     __shared__ double sh[8];
     __shared__ bool last;
     const int64_t per = (N + gridDim.x - 1) / gridDim.x;
@@ -464,8 +474,8 @@ cudaError_t launch_ffma(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64
         const int64_t per_block = (int64_t)kThreads * FfmaCfg<G>::P;
         const int64_t blocks = (N + per_block - 1) / per_block;
         ProfScope ps(ctx, CC_K_ASSIGN_MAIN, st);
-        assign_ffma_kernel<G><<<(unsigned)blocks, kThreads, 0, st>>>(X, N, C, K, Kpad, prep, idx, dist, status,
-                                                                     flagged);
+        launch_after(dim3((unsigned)blocks), dim3(kThreads), 0, st, assign_ffma_kernel<G>,
+                    X, N, C, K, Kpad, prep, idx, dist, status, flagged);
     }
     return cudaGetLastError();
 }
@@ -484,17 +494,20 @@ cudaError_t launch_tail(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64
         const int blocks = ctx->sm_count * 16;
         {
             ProfScope ps(ctx, CC_K_RESOLVE, st);
-            resolve_scan_kernel<G><<<blocks, 128, 0, st>>>(X, N, C, K, status, flagged, scratch, cap_entries, idx, dist);
+            launch_after(dim3(blocks), dim3(128), 0, st, resolve_scan_kernel<G>,
+                    X, N, C, K, status, flagged, scratch, cap_entries, idx, dist);
         }
         ProfScope ps(ctx, CC_K_RESOLVE, st);
-        resolve_merge_kernel<<<blocks, 128, 0, st>>>(N, K, status, flagged, scratch, cap_entries, (ull)blocks * 128, idx, dist);
+        launch_after(dim3(blocks), dim3(128), 0, st, resolve_merge_kernel,
+                    N, K, status, flagged, scratch, cap_entries, (ull)blocks * 128, idx, dist);
     }
     if (objective || n_resolved) {
         int blocks = (int)((N + 4095) / 4096);
         if (blocks > CC_OBJ_BLOCKS) blocks = CC_OBJ_BLOCKS;
         if (blocks < 1) blocks = 1;
         ProfScope ps(ctx, CC_K_OBJECTIVE, st);
-        objective_kernel<<<blocks, 256, 0, st>>>(dist, N, partials, status, objective, n_resolved);
+        launch_after(dim3(blocks), dim3(256), 0, st, objective_kernel,
+                    dist, N, partials, status, objective, n_resolved);
     }
     return cudaGetLastError();
 }
@@ -504,8 +517,8 @@ cudaError_t launch_prep(cc_ctx* ctx, const WsLayout& L, const float* C, int K, c
     char* ws = static_cast<char*>(ctx->ws);
     const int Kpad = (int)cc_align_up((size_t)K, CC_KPAD);
     ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
-    prep_ffma_kernel<G><<<(Kpad / 4 + 127) / 128, 128, 0, st>>>(C, K, Kpad, reinterpret_cast<float4*>(ws + L.cprep),
-                                                                reinterpret_cast<unsigned*>(ws + L.status));
+    launch_after(dim3((Kpad / 4 + 127) / 128), dim3(128), 0, st, prep_ffma_kernel<G>,
+                    C, K, Kpad, reinterpret_cast<float4*>(ws + L.cprep), reinterpret_cast<unsigned*>(ws + L.status));
     return cudaGetLastError();
 }
 

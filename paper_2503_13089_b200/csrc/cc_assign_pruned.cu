@@ -65,6 +65,8 @@ __global__ void __launch_bounds__(256)
 pruned_prep_kernel(const float* __restrict__ C, int K, int n_pos, const unsigned* __restrict__ order,
                    TcParams* __restrict__ params, unsigned char* __restrict__ gB, float* __restrict__ rescan,
                    float* __restrict__ Cs, unsigned* __restrict__ status) {
+    let_next_start();
+    after_previous();
     constexpr int KD = TcCfg<G>::KD;
     const float S = scale_from_range(params->cmax_bits, params->qmax_bits);
     const int ne = norm_exponent(S, params->qmax_bits);
@@ -103,6 +105,8 @@ __global__ void __launch_bounds__(256)
 chunk_bounds_kernel(const float* __restrict__ C, int K, const unsigned* __restrict__ order, int n_chunks,
                     float* __restrict__ C_prev, int have_prev, float* __restrict__ box_t, float* __restrict__ box_c,
                     float* __restrict__ moved) {
+    let_next_start();
+    after_previous();
     const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (c >= n_chunks) return;
     float lo[G], hi[G], far2 = 0.f;
@@ -176,6 +180,8 @@ enum { PL_COLD, PL_NOGAP, PL_RESTART, PL_NEXT };
 template <int G, int MODE>
 __global__ void __launch_bounds__(PR_GROUP)
 pruned_list_kernel(const ListArgs a) {
+    let_next_start();
+    after_previous();
     constexpr bool GAP = MODE == PL_RESTART || MODE == PL_NEXT;
     __shared__ float wlo[PR_ROWS][G], whi[PR_ROWS][G], wub[PR_ROWS];
     __shared__ float glo_s[G], ghi_s[G], gub_s;
@@ -503,6 +509,8 @@ __device__ __forceinline__ float word_norm(const unsigned* w) {
 template <int G, bool GAP>
 __global__ void __launch_bounds__(PS_THREADS, PS_BLOCKS)
 assign_pruned_kernel(const ScanArgs a) {
+    let_next_start();
+    after_previous();
     using Cfg = TcCfg<G>;
     constexpr int KD = Cfg::KD, A_TILE = Cfg::A_TILE, CH = PrCfg<G>::CH_BYTES, STAGES = PrCfg<G>::STAGES;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -779,6 +787,8 @@ pruned_finish_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __r
                      const float* __restrict__ rescan, const unsigned* __restrict__ order, const float2* __restrict__ tstate,
                      const TcParams* __restrict__ params, uint16_t* __restrict__ idx, float* __restrict__ dist,
                      unsigned* __restrict__ status, unsigned* __restrict__ flagged) {
+    let_next_start();
+    after_previous();
     const int k = threadIdx.x & (LPP - 1);
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -884,6 +894,8 @@ pruned_resolve_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __
                       const unsigned* __restrict__ order, const uint16_t* __restrict__ list, const unsigned* __restrict__ list_n,
                       int ld, const unsigned* __restrict__ status, const unsigned* __restrict__ flagged,
                       uint16_t* __restrict__ idx, float* __restrict__ dist) {
+    let_next_start();
+    after_previous();
     __shared__ double sD[4];
     __shared__ int sJ[4];
     ull F = *reinterpret_cast<const ull*>(status + 2);
@@ -954,6 +966,8 @@ pruned_resolve_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __
 __global__ void __launch_bounds__(256)
 sum_exact_kernel(const float* __restrict__ dist, int64_t N, unsigned* __restrict__ status, long long* __restrict__ acc,
                  double* __restrict__ objective, int64_t* __restrict__ n_resolved) {
+    let_next_start();
+    after_previous();
     __shared__ long long sh[3][8];
     __shared__ bool last;
     const unsigned top = status[40];
@@ -1007,6 +1021,8 @@ sum_exact_kernel(const float* __restrict__ dist, int64_t N, unsigned* __restrict
 // Largest distance into status word 40, for E-steps whose finish kernel did not leave it there.
 __global__ void __launch_bounds__(256)
 dist_max_kernel(const float* __restrict__ dist, int64_t N, unsigned* __restrict__ status) {
+    let_next_start();
+    after_previous();
     float m = 0.f;
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < N; i += (int64_t)gridDim.x * 256) m = fmaxf(m, dist[i]);
     m = redux_max(m);
@@ -1032,16 +1048,19 @@ cudaError_t run_pruned(cc_ctx* ctx, const PruneBuffers& b, const float* C, int m
     if ((e = cudaMemsetAsync(b.status + 2, 0, 120 + sizeof(TcParams), st)) != cudaSuccess) return e;
     {
         ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
-        tensor_range_kernel<<<(K + 255) / 256, 256, 0, st>>>(C, K, G, params);
+        launch_after(dim3((K + 255) / 256), dim3(256), 0, st, tensor_range_kernel,
+                    C, K, G, params);
     }
     {
         ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
         const int n = n_chunks * PR_CHUNK * (Cfg::KD / 8);
-        pruned_prep_kernel<G><<<(n + 255) / 256, 256, 0, st>>>(C, K, n_chunks * PR_CHUNK, b.order, params, b.gB, b.rescan, b.Cs, b.status);
+        launch_after(dim3((n + 255) / 256), dim3(256), 0, st, pruned_prep_kernel<G>,
+                    C, K, n_chunks * PR_CHUNK, b.order, params, b.gB, b.rescan, b.Cs, b.status);
     }
     {
         ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
-        chunk_bounds_kernel<G><<<(n_chunks * 32 + 255) / 256, 256, 0, st>>>(C, K, b.order, n_chunks, b.C_prev, restart ? 0 : 1, b.box_t, b.box_c, b.moved);
+        launch_after(dim3((n_chunks * 32 + 255) / 256), dim3(256), 0, st, chunk_bounds_kernel<G>,
+                    C, K, b.order, n_chunks, b.C_prev, restart ? 0 : 1, b.box_t, b.box_c, b.moved);
     }
     const bool use_gap = b.gap != nullptr && !cold;
     {
@@ -1053,10 +1072,14 @@ cudaError_t run_pruned(cc_ctx* ctx, const PruneBuffers& b, const float* C, int m
         a.list = b.list; a.list_n = b.list_n; a.status = b.status;
         ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
         const unsigned blocks = (unsigned)n_groups;
-        if (cold) pruned_list_kernel<G, PL_COLD><<<blocks, PR_GROUP, 0, st>>>(a);
-        else if (!use_gap) pruned_list_kernel<G, PL_NOGAP><<<blocks, PR_GROUP, 0, st>>>(a);
-        else if (restart) pruned_list_kernel<G, PL_RESTART><<<blocks, PR_GROUP, 0, st>>>(a);
-        else pruned_list_kernel<G, PL_NEXT><<<blocks, PR_GROUP, 0, st>>>(a);
+        if (cold) launch_after(dim3(blocks), dim3(PR_GROUP), 0, st, pruned_list_kernel<G, PL_COLD>,
+                    a);
+        else if (!use_gap) launch_after(dim3(blocks), dim3(PR_GROUP), 0, st, pruned_list_kernel<G, PL_NOGAP>,
+                    a);
+        else if (restart) launch_after(dim3(blocks), dim3(PR_GROUP), 0, st, pruned_list_kernel<G, PL_RESTART>,
+                    a);
+        else launch_after(dim3(blocks), dim3(PR_GROUP), 0, st, pruned_list_kernel<G, PL_NEXT>,
+                    a);
     }
     {
         ScanArgs a;
@@ -1066,21 +1089,23 @@ cudaError_t run_pruned(cc_ctx* ctx, const PruneBuffers& b, const float* C, int m
         const unsigned most = (unsigned)ctx->sm_count * PS_BLOCKS;
         const unsigned grid = (unsigned)a.n_tiles < most ? (unsigned)a.n_tiles : most;
         ProfScope ps(ctx, CC_K_ASSIGN_MAIN, st);
-        if (use_gap) assign_pruned_kernel<G, true><<<grid, PS_THREADS, PrCfg<G>::SMEM, st>>>(a);
-        else assign_pruned_kernel<G, false><<<grid, PS_THREADS, PrCfg<G>::SMEM, st>>>(a);
+        if (use_gap) launch_after(dim3(grid), dim3(PS_THREADS), PrCfg<G>::SMEM, st, assign_pruned_kernel<G, true>,
+                    a);
+        else launch_after(dim3(grid), dim3(PS_THREADS), PrCfg<G>::SMEM, st, assign_pruned_kernel<G, false>,
+                    a);
     }
     {
         ProfScope ps(ctx, CC_K_ASSIGN_FINISH, st);
         int64_t blocks = (b.N + 255) / 256;
         const int64_t cap = (int64_t)ctx->sm_count * 32;
         if (blocks > cap) blocks = cap;
-        pruned_finish_kernel<G><<<(unsigned)blocks, 256, 0, st>>>(b.Xs, b.N, b.Cs, K, n_chunks, b.rescan, b.order, b.tstate, params,
-                                                                  b.idx_s, b.dist_s, b.status, b.flagged);
+        launch_after(dim3((unsigned)blocks), dim3(256), 0, st, pruned_finish_kernel<G>,
+                    b.Xs, b.N, b.Cs, K, n_chunks, b.rescan, b.order, b.tstate, params, b.idx_s, b.dist_s, b.status, b.flagged);
     }
     {
         ProfScope ps(ctx, CC_K_RESOLVE, st);
-        pruned_resolve_kernel<G><<<ctx->sm_count * 16, 128, 0, st>>>(b.Xs, b.N, C, b.Cs, K, b.order, b.list, b.list_n, b.ld, b.status,
-                                                                     b.flagged, b.idx_s, b.dist_s);
+        launch_after(dim3(ctx->sm_count * 16), dim3(128), 0, st, pruned_resolve_kernel<G>,
+                    b.Xs, b.N, C, b.Cs, K, b.order, b.list, b.list_n, b.ld, b.status, b.flagged, b.idx_s, b.dist_s);
     }
     return cudaGetLastError();
 }
@@ -1108,9 +1133,11 @@ cudaError_t cc_launch_sum_exact(cc_ctx* ctx, const PruneBuffers& b, bool have_ma
         const cudaError_t e = cudaMemsetAsync(b.status + 40, 0, sizeof(unsigned), st);
         if (e != cudaSuccess) return e;
         ProfScope ps(ctx, CC_K_OBJECTIVE, st);
-        dist_max_kernel<<<(unsigned)blocks, 256, 0, st>>>(b.dist_s, b.N, b.status);
+        launch_after(dim3((unsigned)blocks), dim3(256), 0, st, dist_max_kernel,
+                    b.dist_s, b.N, b.status);
     }
     ProfScope ps(ctx, CC_K_OBJECTIVE, st);
-    sum_exact_kernel<<<(unsigned)blocks, 256, 0, st>>>(b.dist_s, b.N, b.status, b.acc, objective, n_resolved);
+    launch_after(dim3((unsigned)blocks), dim3(256), 0, st, sum_exact_kernel,
+                    b.dist_s, b.N, b.status, b.acc, objective, n_resolved);
     return cudaGetLastError();
 }

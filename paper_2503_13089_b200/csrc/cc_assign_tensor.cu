@@ -53,6 +53,8 @@ template <int G>
 __global__ void __launch_bounds__(256)
 prep_tensor_kernel(const float* __restrict__ C, int K, int Kpad, TcParams* __restrict__ params,
                    uint16_t* __restrict__ gB, float* __restrict__ rescan) {
+    let_next_start();
+    after_previous();
     using Cfg = TcCfg<G>;
     constexpr int KD = Cfg::KD;
     const float S = scale_from_range(params->cmax_bits, params->qmax_bits);
@@ -126,6 +128,8 @@ assign_tensor_kernel(const uint16_t* __restrict__ X, int64_t N, const uint16_t* 
                      int na_per_cta, int64_t tile_offset, const TcParams* __restrict__ params,
                      float2* __restrict__ tstate, unsigned* __restrict__ status, float* __restrict__ dump,
                      int64_t dump_ld) {
+    let_next_start();
+    after_previous();
     using Cfg = TcCfg<G>;
     constexpr int KD = Cfg::KD, STAGES = Cfg::STAGES;
     constexpr int A_TILE = Cfg::A_TILE, B_TILE = Cfg::B_TILE;
@@ -349,6 +353,8 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
 assign_tensor_persistent_kernel(const uint16_t* __restrict__ X, int64_t N, const uint16_t* __restrict__ gB, int n_btiles,
                                 int n_groups, const TcParams* __restrict__ params, float2* __restrict__ tstate,
                                 unsigned* __restrict__ status) {
+    let_next_start();
+    after_previous();
     using Cfg = TcCfg<G>;
     constexpr int KD = Cfg::KD, STAGES = Cfg::STAGES;
     constexpr int A_TILE = Cfg::A_TILE, B_TILE = Cfg::B_TILE, A_SET = NA * A_TILE;
@@ -594,6 +600,8 @@ finish_tensor_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __r
                      const float* __restrict__ rescan, const float2* __restrict__ tstate,
                      const TcParams* __restrict__ params, uint16_t* __restrict__ idx, float* __restrict__ dist,
                      unsigned* __restrict__ status, unsigned* __restrict__ flagged) {
+    let_next_start();
+    after_previous();
     const int k = threadIdx.x & (LPP - 1);
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -722,12 +730,14 @@ cudaError_t launch_tensor(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int
     if ((e = cudaMemsetAsync(status + 2, 0, 120 + sizeof(TcParams), st)) != cudaSuccess) return e;
     {
         ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
-        tensor_range_kernel<<<(K + 255) / 256, 256, 0, st>>>(C, K, G, params);
+        launch_after(dim3((K + 255) / 256), dim3(256), 0, st, tensor_range_kernel,
+                    C, K, G, params);
     }
     {
         ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
         const int n = Kpad * (Cfg::KD / 8);
-        prep_tensor_kernel<G><<<(n + 255) / 256, 256, 0, st>>>(C, K, Kpad, params, gB, dump ? nullptr : rescan);
+        launch_after(dim3((n + 255) / 256), dim3(256), 0, st, prep_tensor_kernel<G>,
+                    C, K, Kpad, params, gB, dump ? nullptr : rescan);
     }
     if (N > 0) {
         const int64_t n_tiles = (N + TM - 1) / TM;
@@ -745,8 +755,8 @@ cudaError_t launch_tensor(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int
         if (dump) {
             const int64_t blocks = (n_tiles + na_per_cta - 1) / na_per_cta;
             ProfScope ps(ctx, CC_K_OTHER, st);
-            assign_tensor_kernel<G, true, false><<<(unsigned)blocks, TC_THREADS, Cfg::SMEM, st>>>(
-                X, N, gB, Kpad / TN, (int)na_per_cta, 0, params, tstate, status, dump, dump_ld);
+            launch_after(dim3((unsigned)blocks), dim3(TC_THREADS), Cfg::SMEM, st, assign_tensor_kernel<G, true, false>,
+                     X, N, gB, Kpad / TN, (int)na_per_cta, 0, params, tstate, status, dump, dump_ld);
             return cudaGetLastError();
         }
         if (!scan_in) {
@@ -760,16 +770,16 @@ cudaError_t launch_tensor(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int
                     if ((e = cudaFuncSetAttribute(assign_tensor_persistent_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, PersistCfg<G>::SMEM)) != cudaSuccess) return e;
                     attr_p = true;
                 }
-                assign_tensor_persistent_kernel<G><<<ctx->sm_count, PERSIST_THREADS, PersistCfg<G>::SMEM, st>>>(
-                    X, N, gB, Kpad / TN, (int)full_blocks, params, tstate, status);
+                launch_after(dim3(ctx->sm_count), dim3(PERSIST_THREADS), PersistCfg<G>::SMEM, st, assign_tensor_persistent_kernel<G>,
+                     X, N, gB, Kpad / TN, (int)full_blocks, params, tstate, status);
             } else if (full_blocks > 0)
-                assign_tensor_kernel<G, false, true><<<(unsigned)full_blocks, TC_THREADS, Cfg::SMEM, st>>>(
-                    X, N, gB, Kpad / TN, NA, 0, params, tstate, status, nullptr, 0);
+                launch_after(dim3((unsigned)full_blocks), dim3(TC_THREADS), Cfg::SMEM, st, assign_tensor_kernel<G, false, true>,
+                     X, N, gB, Kpad / TN, NA, 0, params, tstate, status, nullptr, 0);
             const int64_t rest_tiles = n_tiles - full_blocks * NA;
             if (rest_tiles > 0) {
                 const int64_t blocks = (rest_tiles + na_per_cta - 1) / na_per_cta;
-                assign_tensor_kernel<G, false, false><<<(unsigned)blocks, TC_THREADS, Cfg::SMEM, st>>>(
-                    X, N, gB, Kpad / TN, (int)na_per_cta, full_blocks * NA, params, tstate, status, nullptr, 0);
+                launch_after(dim3((unsigned)blocks), dim3(TC_THREADS), Cfg::SMEM, st, assign_tensor_kernel<G, false, false>,
+                     X, N, gB, Kpad / TN, (int)na_per_cta, full_blocks * NA, params, tstate, status, nullptr, 0);
             }
         }
         {
@@ -777,9 +787,8 @@ cudaError_t launch_tensor(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int
             int64_t fblocks = (N + 255) / 256;            // a warp takes 32 points per round
             const int64_t cap = (int64_t)ctx->sm_count * 32;
             if (fblocks > cap) fblocks = cap;
-            finish_tensor_kernel<G><<<(unsigned)fblocks, 256, 0, st>>>(
-                X, N, C, K, Kpad / TCHUNK, rescan, tstate, params, idx, dist, status,
-                reinterpret_cast<unsigned*>(ws + L.flagged));
+            launch_after(dim3((unsigned)fblocks), dim3(256), 0, st, finish_tensor_kernel<G>,
+                     X, N, C, K, Kpad / TCHUNK, rescan, tstate, params, idx, dist, status, reinterpret_cast<unsigned*>(ws + L.flagged));
         }
     }
     return cudaGetLastError();

@@ -100,6 +100,8 @@ __device__ __forceinline__ float qconst(int p, int e) {
 // Largest |c| and largest ||c||^2 of the codebook (params zeroed beforehand).
 __global__ void __launch_bounds__(256)
 tensor_range_kernel(const float* __restrict__ C, int K, int g, TcParams* __restrict__ params) {
+    let_next_start();
+    after_previous();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     float cm = 0.f, qm = 0.f;
     if (j < K) {

@@ -59,8 +59,16 @@ struct ProfScope {
     ~ProfScope() { if (slot) cudaEventRecord(slot->b, st); }
 };
 
+// In a kernel that launch_after starts: everything in front of it has ended and is visible from here on; and the next such kernel may
+// start (its blocks take the places that become free, and wait here in turn).  Calls back to back save about a
+// microsecond each.
+#ifdef __CUDACC__
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+
 // Launch that may begin before the kernel in front of it has ended; what it needs of that one stands behind
-// griddepcontrol.wait.
+// after_previous().
 template <class... Args, class... Given>
 cudaError_t launch_after(dim3 grid, dim3 block, size_t smem, cudaStream_t st, void (*kernel)(Args...), Given... args) {
     cudaLaunchAttribute at = {};

@@ -28,6 +28,8 @@ template <int MODE>
 __global__ void __launch_bounds__(DP_THREADS, 1)
 decode_planes_kernel(const uint16_t* __restrict__ C16, int K, int g, const uint16_t* __restrict__ idx, int out_groups, int d_out, int d_in,
                      uint16_t* __restrict__ W_hat) {
+    let_next_start();
+    after_previous();
     constexpr int QS = DP_GROUPS / 2, PASSES = R / 16;
     extern __shared__ __align__(16) unsigned char dp_smem[];
     unsigned char* table = dp_smem;
@@ -114,8 +116,8 @@ cudaError_t launch(cc_ctx* ctx, const uint16_t* C16, int K, int g, const uint16_
     const int groups = (g + PP - 1) / PP;
     const dim3 grid((unsigned)(ctx->sm_count / groups < 1 ? 1 : ctx->sm_count / groups), (unsigned)groups);
     ProfScope ps(ctx, CC_K_DECODE, st);
-    decode_planes_kernel<MODE><<<grid, DP_THREADS, (size_t)plane_table_bytes(K, PP) + DP_WARPS * DP_STAGE, st>>>(C16, K, g, idx, out_groups, d_out,
-                                                                                                                 d_in, W_hat);
+    launch_after(dim3(grid), dim3(DP_THREADS), (size_t)plane_table_bytes(K, PP) + DP_WARPS * DP_STAGE, st, decode_planes_kernel<MODE>,
+                    C16, K, g, idx, out_groups, d_out, d_in, W_hat);
     return cudaGetLastError();
 }
 

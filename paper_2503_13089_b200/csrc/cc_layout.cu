@@ -41,6 +41,8 @@ __device__ __forceinline__ void tile_column8x2(const unsigned* tile, int c, int 
 __global__ void __launch_bounds__(256)
 reshape_transpose_vec_kernel(const uint16_t* __restrict__ W, int64_t d_out, int64_t d_in, int64_t out_pad,
                              uint16_t* __restrict__ X) {
+    let_next_start();
+    after_previous();
     __shared__ unsigned tile[TILE_WORDS];
     const int64_t i0 = (int64_t)blockIdx.x * TD, o0 = (int64_t)blockIdx.y * TD;
     const int c = threadIdx.x & 7, r0 = threadIdx.x >> 3;
@@ -71,6 +73,8 @@ template <int G>
 __global__ void __launch_bounds__(256)
 decode_transpose_vec_kernel(const uint16_t* __restrict__ C16, const uint16_t* __restrict__ idx, int64_t d_out,
                             int64_t d_in, int64_t out_pad, uint16_t* __restrict__ W_hat) {
+    let_next_start();
+    after_previous();
     __shared__ unsigned tile[TILE_WORDS];
     const int64_t i0 = (int64_t)blockIdx.x * TD, o0 = (int64_t)blockIdx.y * TD;
     const int c = threadIdx.x & 7, r0 = threadIdx.x >> 3;
@@ -131,6 +135,8 @@ __device__ __forceinline__ void tile_columns(const unsigned* tile, int rp, int l
 __global__ void __launch_bounds__(256)
 reshape_transpose_any_kernel(const uint16_t* __restrict__ W, int64_t d_out, int64_t d_in, int64_t out_pad,
                              uint16_t* __restrict__ X) {
+    let_next_start();
+    after_previous();
     __shared__ unsigned tile[TILE_WORDS];
     const int64_t i0 = (int64_t)blockIdx.x * TD, o0 = (int64_t)blockIdx.y * TD;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -180,6 +186,8 @@ template <bool EVEN_G>
 __global__ void __launch_bounds__(256)
 decode_transpose_any_kernel(const uint16_t* __restrict__ C16, int K, int g, const uint16_t* __restrict__ idx, int64_t d_out,
                             int64_t d_in, int64_t out_pad, uint16_t* __restrict__ W_hat) {
+    let_next_start();
+    after_previous();
     __shared__ unsigned tile[TILE_WORDS];
     const int64_t i0 = (int64_t)blockIdx.x * TD, o0 = (int64_t)blockIdx.y * TD;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -313,6 +321,8 @@ template <int G, bool TABLE>
 __global__ void __launch_bounds__(256, 4)
 decode_transpose_pipe_kernel(const uint16_t* __restrict__ C16, const uint16_t* __restrict__ idx, int K, int64_t d_out,
                              int64_t d_in, int64_t out_pad, uint16_t* __restrict__ W_hat, int tiles_x, int tiles_y) {
+    let_next_start();
+    after_previous();
     extern __shared__ __align__(16) unsigned char decode_smem[];
     unsigned* tile = reinterpret_cast<unsigned*>(decode_smem);
     const uint16_t* table = C16;
@@ -383,11 +393,11 @@ cudaError_t launch_decode_pipe(int sm_count, const uint16_t* C16, const uint16_t
         const cudaError_t e = cudaFuncSetAttribute(decode_transpose_pipe_kernel<G, true>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        decode_transpose_pipe_kernel<G, true><<<(unsigned)grid, 256, smem, st>>>(C16, idx, K, d_out, d_in, out_pad,
-                                                                                 W_hat, tiles_x, tiles_y);
+        launch_after(dim3((unsigned)grid), dim3(256), smem, st, decode_transpose_pipe_kernel<G, true>,
+                    C16, idx, K, d_out, d_in, out_pad, W_hat, tiles_x, tiles_y);
     } else {
-        decode_transpose_pipe_kernel<G, false><<<(unsigned)grid, 256, smem, st>>>(C16, idx, K, d_out, d_in, out_pad,
-                                                                                  W_hat, tiles_x, tiles_y);
+        launch_after(dim3((unsigned)grid), dim3(256), smem, st, decode_transpose_pipe_kernel<G, false>,
+                    C16, idx, K, d_out, d_in, out_pad, W_hat, tiles_x, tiles_y);
     }
     return cudaGetLastError();
 }
@@ -478,6 +488,8 @@ template <int G>
 __global__ void __launch_bounds__(RES_THREADS, 1)
 decode_transpose_resident_kernel(const uint16_t* __restrict__ C16, const uint16_t* __restrict__ idx, int K, int head_rows,
                                  int64_t d_out, int64_t d_in, int64_t out_pad, uint16_t* __restrict__ W_hat, int tiles_x, int tiles_y) {
+    let_next_start();
+    after_previous();
     extern __shared__ __align__(16) unsigned char decode_smem[];
     const int group = threadIdx.x >> 8, tid = threadIdx.x & 255;
     unsigned* tile = reinterpret_cast<unsigned*>(decode_smem + group * kTileBytes);
@@ -541,8 +553,8 @@ cudaError_t launch_decode_resident(cc_ctx* ctx, const uint16_t* C16, const uint1
         have = true;
     }
     const int head = res_head(K, G);
-    decode_transpose_resident_kernel<G><<<(unsigned)ctx->sm_count, RES_THREADS, RES_GROUPS * kTileBytes + head * 2 * G, st>>>(
-        C16, idx, K, head, d_out, d_in, out_pad, W_hat, tiles_x, tiles_y);
+    launch_after(dim3((unsigned)ctx->sm_count), dim3(RES_THREADS), RES_GROUPS * kTileBytes + head * 2 * G, st, decode_transpose_resident_kernel<G>,
+                     C16, idx, K, head, d_out, d_in, out_pad, W_hat, tiles_x, tiles_y);
     return cudaGetLastError();
 }
 
@@ -550,6 +562,8 @@ cudaError_t launch_decode_resident(cc_ctx* ctx, const uint16_t* C16, const uint1
 __global__ void __launch_bounds__(256)
 reshape_rows_kernel(const uint16_t* __restrict__ W, int64_t d_out, int64_t d_in, int64_t in_pad,
                     uint16_t* __restrict__ X) {
+    let_next_start();
+    after_previous();
     const int64_t total = d_out * in_pad;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t o = e / in_pad, i = e - o * in_pad;
@@ -561,6 +575,8 @@ reshape_rows_kernel(const uint16_t* __restrict__ W, int64_t d_out, int64_t d_in,
 __global__ void __launch_bounds__(256)
 decode_rows_kernel(const uint16_t* __restrict__ C16, int g, const uint16_t* __restrict__ idx, int64_t d_out,
                    int64_t d_in, int64_t in_pad, uint16_t* __restrict__ W_hat) {
+    let_next_start();
+    after_previous();
     const int64_t total = d_out * d_in;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t o = e / d_in, i = e - o * d_in;
@@ -572,6 +588,8 @@ decode_rows_kernel(const uint16_t* __restrict__ C16, int g, const uint16_t* __re
 
 __global__ void gather_init_kernel(const uint16_t* __restrict__ X, int g, int K, const int64_t* __restrict__ pos,
                                    float* __restrict__ C) {
+    let_next_start();
+    after_previous();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= K * g) return;
     const int k = e / g, t = e - k * g;
@@ -581,6 +599,8 @@ __global__ void gather_init_kernel(const uint16_t* __restrict__ X, int g, int K,
 struct InitArgs { int64_t pos[CC_INIT_ARGS]; };
 
 __global__ void gather_init_args_kernel(const uint16_t* __restrict__ X, int g, int K, const __grid_constant__ InitArgs a, float* __restrict__ C) {
+    let_next_start();
+    after_previous();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= K * g) return;
     const int k = e / g, t = e - k * g;
@@ -591,6 +611,8 @@ __global__ void gather_init_args_kernel(const uint16_t* __restrict__ X, int g, i
 // the stored codebook are computed against).
 __global__ void to_half_kernel(const float* __restrict__ C, int64_t n, uint16_t* __restrict__ C16,
                                float* __restrict__ widened) {
+    let_next_start();
+    after_previous();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n) return;
     const __half h = __float2half_rn(C[e]);
@@ -609,14 +631,17 @@ cudaError_t cc_launch_reshape(cc_ctx* ctx, const uint16_t* W, int64_t d_out, int
         const int64_t out_pad = pad_to(d_out, g);
         dim3 grid((unsigned)((d_in + TD - 1) / TD), (unsigned)((out_pad + TD - 1) / TD));
         if (d_in % 8 == 0 && out_pad % 8 == 0)
-            reshape_transpose_vec_kernel<<<grid, 256, 0, st>>>(W, d_out, d_in, out_pad, X);
+            launch_after(dim3(grid), dim3(256), 0, st, reshape_transpose_vec_kernel,
+                    W, d_out, d_in, out_pad, X);
         else
-            reshape_transpose_any_kernel<<<grid, 256, 0, st>>>(W, d_out, d_in, out_pad, X);
+            launch_after(dim3(grid), dim3(256), 0, st, reshape_transpose_any_kernel,
+                    W, d_out, d_in, out_pad, X);
     } else {
         const int64_t in_pad = pad_to(d_in, g);
         int64_t blocks = (d_out * in_pad + 255) / 256;
         if (blocks > (int64_t)ctx->sm_count * 32) blocks = (int64_t)ctx->sm_count * 32;
-        reshape_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>(W, d_out, d_in, in_pad, X);
+        launch_after(dim3((unsigned)blocks), dim3(256), 0, st, reshape_rows_kernel,
+                    W, d_out, d_in, in_pad, X);
     }
     return cudaGetLastError();
 }
@@ -645,16 +670,22 @@ cudaError_t cc_launch_decode(cc_ctx* ctx, const uint16_t* C16, int K, int g, con
             if (g == 8) return launch_decode_pipe<8>(ctx->sm_count, C16, idx, K, d_out, d_in, out_pad, W_hat, (int)grid.x, (int)grid.y, st);
             return launch_decode_pipe<16>(ctx->sm_count, C16, idx, K, d_out, d_in, out_pad, W_hat, (int)grid.x, (int)grid.y, st);
         }
-        if (vec && g == 4) decode_transpose_vec_kernel<4><<<grid, 256, 0, st>>>(C16, idx, d_out, d_in, out_pad, W_hat);
-        else if (vec && g == 8) decode_transpose_vec_kernel<8><<<grid, 256, 0, st>>>(C16, idx, d_out, d_in, out_pad, W_hat);
-        else if (vec && g == 16) decode_transpose_vec_kernel<16><<<grid, 256, 0, st>>>(C16, idx, d_out, d_in, out_pad, W_hat);
-        else if (g % 2 == 0) decode_transpose_any_kernel<true><<<grid, 256, 0, st>>>(C16, K, g, idx, d_out, d_in, out_pad, W_hat);
-        else decode_transpose_any_kernel<false><<<grid, 256, 0, st>>>(C16, K, g, idx, d_out, d_in, out_pad, W_hat);
+        if (vec && g == 4) launch_after(dim3(grid), dim3(256), 0, st, decode_transpose_vec_kernel<4>,
+                    C16, idx, d_out, d_in, out_pad, W_hat);
+        else if (vec && g == 8) launch_after(dim3(grid), dim3(256), 0, st, decode_transpose_vec_kernel<8>,
+                    C16, idx, d_out, d_in, out_pad, W_hat);
+        else if (vec && g == 16) launch_after(dim3(grid), dim3(256), 0, st, decode_transpose_vec_kernel<16>,
+                    C16, idx, d_out, d_in, out_pad, W_hat);
+        else if (g % 2 == 0) launch_after(dim3(grid), dim3(256), 0, st, decode_transpose_any_kernel<true>,
+                    C16, K, g, idx, d_out, d_in, out_pad, W_hat);
+        else launch_after(dim3(grid), dim3(256), 0, st, decode_transpose_any_kernel<false>,
+                    C16, K, g, idx, d_out, d_in, out_pad, W_hat);
     } else {
         const int64_t in_pad = pad_to(d_in, g);
         int64_t blocks = (d_out * d_in + 255) / 256;
         if (blocks > (int64_t)ctx->sm_count * 32) blocks = (int64_t)ctx->sm_count * 32;
-        decode_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>(C16, g, idx, d_out, d_in, in_pad, W_hat);
+        launch_after(dim3((unsigned)blocks), dim3(256), 0, st, decode_rows_kernel,
+                    C16, g, idx, d_out, d_in, in_pad, W_hat);
     }
     return cudaGetLastError();
 }
@@ -662,7 +693,8 @@ cudaError_t cc_launch_decode(cc_ctx* ctx, const uint16_t* C16, int K, int g, con
 cudaError_t cc_launch_gather_init(cc_ctx* ctx, const uint16_t* X, int g, int K, const int64_t* pos_dev, float* C,
                                   cudaStream_t st) {
     ProfScope ps(ctx, CC_K_OTHER, st);
-    gather_init_kernel<<<(K * g + 255) / 256, 256, 0, st>>>(X, g, K, pos_dev, C);
+    launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, gather_init_kernel,
+                    X, g, K, pos_dev, C);
     return cudaGetLastError();
 }
 
@@ -672,13 +704,15 @@ cudaError_t cc_launch_gather_init_args(cc_ctx* ctx, const uint16_t* X, int g, in
     InitArgs a;
     for (int k = 0; k < CC_INIT_ARGS; ++k) a.pos[k] = k < K ? pos_host[k] : 0;
     ProfScope ps(ctx, CC_K_OTHER, st);
-    gather_init_args_kernel<<<(K * g + 255) / 256, 256, 0, st>>>(X, g, K, a, C);
+    launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, gather_init_args_kernel,
+                    X, g, K, a, C);
     return cudaGetLastError();
 }
 
 cudaError_t cc_launch_to_half(cc_ctx* ctx, const float* C, int64_t n, uint16_t* C16, float* C_widened,
                               cudaStream_t st) {
     ProfScope ps(ctx, CC_K_OTHER, st);
-    to_half_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(C, n, C16, C_widened);
+    launch_after(dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, to_half_kernel,
+                    C, n, C16, C_widened);
     return cudaGetLastError();
 }

@@ -103,6 +103,8 @@ linear_forward_kernel(const uint16_t* __restrict__ x, int M, const uint16_t* __r
     uint32_t* lut2 = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(bars) + 256);   // QUANT only
     unsigned char* qt = reinterpret_cast<unsigned char*>(lut2 + 256);                            // QUANT only
 
+    let_next_start();
+    after_previous();
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int o0 = blockIdx.x * LM;
     const int m0 = blockIdx.y * NT;
@@ -363,6 +365,8 @@ linear_forward_kernel(const uint16_t* __restrict__ x, int M, const uint16_t* __r
 __global__ void __launch_bounds__(256)
 linear_reduce_kernel(const float* __restrict__ partial, int splits, int64_t n, int d_out, const float* __restrict__ bias,
                      float* __restrict__ y) {
+    let_next_start();
+    after_previous();
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         float s = bias ? __ldg(bias + (int)(e % d_out)) : 0.f;
         for (int k = 0; k < splits; ++k) s += partial[(int64_t)k * n + e];
@@ -505,10 +509,14 @@ linear_gemv_kernel(const uint16_t* __restrict__ x, int M, const unsigned char* _
     const unsigned n_rows = K - (int)lo < slice_rows ? K - lo : (unsigned)slice_rows;
     const int bytes = (int)n_rows * ROWB;
     const unsigned char* src_book = book + (size_t)lo * ROWB;
+    let_next_start();
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(qbar)));
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    after_previous();
+    if (tid == 0) {
         const uint32_t bulk = (uint32_t)bytes & ~15u, bar = smem_u32(qbar);
         if (bulk) {
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bulk) : "memory");
@@ -651,6 +659,8 @@ linear_gemv_kernel(const uint16_t* __restrict__ x, int M, const unsigned char* _
 // Copy of the codebook with rows of `pad` values, a power of two, so that a gather is one load (load_row_padded).
 __global__ void __launch_bounds__(256)
 linear_pad_rows_kernel(const uint16_t* __restrict__ C16, int K, int g, int pad, uint16_t* __restrict__ table) {
+    let_next_start();
+    after_previous();
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= K) return;
     const uint16_t* src = C16 + (int64_t)j * g;
@@ -810,11 +820,7 @@ cudaError_t launch_linear_s(cc_ctx* ctx, const LinearPlan& p, const uint16_t* x,
         have = true;
     }
     const dim3 grid(p.o_tiles, p.tok_blocks, p.splits);
-    linear_forward_kernel<G, QUANT, PADDED, STAGES><<<grid, LTHREADS, p.smem, st>>>(x, M, C16, qtab, qscale, K, idx, d_out, d_in,
-                                                                            out_groups, p.NT, p.a_pad, p.tmem_cols,
-                                                                            p.chunks_per_split, out, split_stride, bias, status, arrived,
-                                                                            bias_final, y_final);
-    return cudaGetLastError();
+    return launch_after(grid, dim3(LTHREADS), p.smem, st, linear_forward_kernel<G, QUANT, PADDED, STAGES>, x, M, C16, qtab, qscale, K, idx, d_out, d_in, out_groups, p.NT, p.a_pad, p.tmem_cols, p.chunks_per_split, out, split_stride, bias, status, arrived, bias_final, y_final);
 }
 
 // Two stages exist where the plan can ask for them: beside the 4-bit table, and for rows of at most 8 bytes.
@@ -850,10 +856,7 @@ cudaError_t launch_gemv_w(cc_ctx* ctx, const GemvPlan& p, const uint16_t* x, int
         have = true;
     }
     const dim3 grid(p.o_blocks, p.splits, p.slices);
-    linear_gemv_kernel<G, MT, QUANT, PW><<<grid, LG_THREADS, p.smem, st>>>(
-        x, M, static_cast<const unsigned char*>(book), qscale, K, p.slice_rows, idx, d_out, d_in, out_groups, p.rows_per_split, out,
-        split_stride, status, arrived, bias, y, p.splits * p.slices == 1);
-    return cudaGetLastError();
+    return launch_after(grid, dim3(LG_THREADS), p.smem, st, linear_gemv_kernel<G, MT, QUANT, PW>, x, M, static_cast<const unsigned char*>(book), qscale, K, p.slice_rows, idx, d_out, d_in, out_groups, p.rows_per_split, out, split_stride, status, arrived, bias, y, p.splits * p.slices == 1);
 }
 
 template <int G, int MT, bool QUANT>
@@ -925,8 +928,7 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
         int64_t blocks = (n + 255) / 256;
         const int64_t cap = (int64_t)ctx->sm_count * 8;
         if (blocks > cap) blocks = cap;
-        linear_reduce_kernel<<<(unsigned)blocks, 256, 0, st>>>(partial, slabs_n, n, (int)d_out, bias, y);
-        return cudaGetLastError();
+        return launch_after(dim3((unsigned)blocks), dim3(256), 0, st, linear_reduce_kernel, partial, slabs_n, n, (int)d_out, bias, y);
     }
     {
         PlanesPlan pl = {};
@@ -947,7 +949,8 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
     if (table_at) {
         uint16_t* table = reinterpret_cast<uint16_t*>(ws + table_at);
         ProfScope ps(ctx, CC_K_OTHER, st);
-        linear_pad_rows_kernel<<<(unsigned)((K + 255) / 256), 256, 0, st>>>(C16, K, g, row_pad(g), table);
+        e = launch_after(dim3((unsigned)((K + 255) / 256)), dim3(256), 0, st, linear_pad_rows_kernel, C16, K, g, row_pad(g), table);
+        if (e != cudaSuccess) return e;
         C16 = table;
         padded = true;
     }
@@ -985,8 +988,7 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
         int64_t blocks = (n + 255) / 256;
         const int64_t cap = (int64_t)ctx->sm_count * 8;
         if (blocks > cap) blocks = cap;
-        linear_reduce_kernel<<<(unsigned)blocks, 256, 0, st>>>(partial, p.splits, n, (int)d_out, bias, y);
-        e = cudaGetLastError();
+        e = launch_after(dim3((unsigned)blocks), dim3(256), 0, st, linear_reduce_kernel, partial, p.splits, n, (int)d_out, bias, y);
     }
     return e;
 }

@@ -32,7 +32,8 @@ __global__ void __launch_bounds__(PREP_BLOCK)
 planes_prepare_kernel(const uint16_t* __restrict__ C16, const unsigned char* __restrict__ qtab, const float* __restrict__ qscale,
                       int K, int g, int PP, int book_blocks, unsigned char* __restrict__ planes, const uint16_t* __restrict__ x,
                       int M, int d_in, int NT, unsigned char* __restrict__ x_tiles) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    after_previous();
+    let_next_start();                                // the product may read the codes at once, so not before this
     const int tid = threadIdx.x;
     if ((int)blockIdx.x < book_blocks) {
         const int k = blockIdx.x * PREP_BLOCK + tid;
@@ -121,7 +122,7 @@ linear_planes_kernel(const unsigned char* __restrict__ planes, int K, const uint
     const unsigned char* my_plane = planes + (int64_t)blockIdx.y * table_bytes;
     float* my_slabs = slabs + (int64_t)blockIdx.y * items * NT * PM;
 
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    let_next_start();
     if (tid == 0) {
         auto init = [&](uint64_t* b, int n) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(n)); };
         for (int s = 0; s < STAGES; ++s) { init(full + s, WPS + 1); init(empty + s, 1); }
@@ -235,7 +236,7 @@ linear_planes_kernel(const unsigned char* __restrict__ planes, int K, const uint
     } else if (warp == 5) {
         // ------------------------------------------------------------ copies: the table, then x tile by tile
         if (elect_one()) {
-            asm volatile("griddepcontrol.wait;" ::: "memory");
+            after_previous();
             const uint32_t lb = smem_u32(landed), tb = smem_u32(table);
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(lb), "r"((uint32_t)table_bytes) : "memory");
             for (uint32_t off = 0; off < (uint32_t)table_bytes; off += 16384u) {
@@ -306,7 +307,8 @@ planes_reduce_kernel(const float* __restrict__ slabs, int PP, int groups_n, int 
     const int o0 = tile * CW * g;
     int width = d_out - o0;
     width = width < CW * g ? width : CW * g;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    let_next_start();
+    after_previous();
     const int64_t slab = (int64_t)NT * PM;
     for (int e = threadIdx.x; e < groups_n * PM; e += RED_THREADS) {
         const int pg = e / PM, row = e % PM, q = row % half, pb = row / half;
@@ -366,13 +368,13 @@ cudaError_t cc_launch_linear_planes(cc_ctx* ctx, const PlanesPlan& p, const uint
     unsigned char* x_tiles = reinterpret_cast<unsigned char*>(ws + CC_LINEAR_SCRATCH_FROM);
     float* slabs = reinterpret_cast<float*>(x_tiles + p.x_bytes);
     const int out_groups = (d_out + g - 1) / g, chunks = (d_in + PKB - 1) / PKB, book_blocks = (K + PREP_BLOCK - 1) / PREP_BLOCK;
+    cudaError_t e;
     {
         ProfScope ps(ctx, CC_K_OTHER, st);
         const unsigned blocks = (unsigned)(book_blocks + chunks);
-        if (qtab) planes_prepare_kernel<true><<<blocks, PREP_BLOCK, 0, st>>>(C16, qtab, qscale, K, g, p.PP, book_blocks, planes, x, M, d_in, p.NT, x_tiles);
-        else planes_prepare_kernel<false><<<blocks, PREP_BLOCK, 0, st>>>(C16, qtab, qscale, K, g, p.PP, book_blocks, planes, x, M, d_in, p.NT, x_tiles);
+        e = qtab ? launch_after(dim3(blocks), dim3(PREP_BLOCK), 0, st, planes_prepare_kernel<true>, C16, qtab, qscale, K, g, p.PP, book_blocks, planes, x, M, d_in, p.NT, x_tiles)
+                 : launch_after(dim3(blocks), dim3(PREP_BLOCK), 0, st, planes_prepare_kernel<false>, C16, qtab, qscale, K, g, p.PP, book_blocks, planes, x, M, d_in, p.NT, x_tiles);
     }
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     e = p.PP == 1 ? launch_planes_s<1>(ctx, p, planes, K, idx, out_groups, d_in, x_tiles, slabs, status, st)
       : p.PP == 2 ? launch_planes_s<2>(ctx, p, planes, K, idx, out_groups, d_in, x_tiles, slabs, status, st)

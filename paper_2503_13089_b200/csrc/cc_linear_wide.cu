@@ -67,6 +67,8 @@ linear_prepare_kernel(const uint16_t* __restrict__ C16, bool padded, const unsig
     __shared__ __align__(16) uint4 stage[TILES * (WKB / 8) * (WM / 8) * PREP_PAD];
     __shared__ uint32_t lut[QUANT ? 256 : 1];
     const int tid = threadIdx.x;
+    let_next_start();
+    after_previous();
     if ((int)blockIdx.x < w_blocks) {
         const int per_row = (chunks + TILES - 1) / TILES;
         const int row = (int)blockIdx.x / per_row, c0 = ((int)blockIdx.x - row * per_row) * TILES;
@@ -204,7 +206,7 @@ linear_gemm_kernel(const unsigned char* __restrict__ w_tiles, const unsigned cha
     if (warp == GW) {
         // ------------------------------------------------------------ copies
         if (elect_one()) {
-            asm volatile("griddepcontrol.wait;" ::: "memory");       // the tiles
+            after_previous();                                        // the tiles
             int st = 0, total = 0;
             uint32_t ph = 0;
             const unsigned char* bsrc = x_tiles + (int64_t)blockIdx.y * chunks * NT * (WKB * 2);
@@ -384,9 +386,8 @@ cudaError_t launch_prepare(cc_ctx* ctx, const uint16_t* C16, bool padded, const 
     const int w_blocks = row_tiles * ((chunks + prep_tiles(G) - 1) / prep_tiles(G));
     const int x_blocks = with_x ? (int)((m_end - m_first + NT - 1) / NT) * chunks : 0;
     ProfScope ps(ctx, CC_K_DECODE, st);
-    linear_prepare_kernel<G, QUANT><<<(unsigned)(w_blocks + x_blocks), PREP_THREADS, 0, st>>>(
-        C16, padded, qtab, qscale, K, idx, (int)d_in, out_groups, o_first, chunks, w_blocks, w_tiles, x, (int)m_first, (int)m_end, NT, x_tiles);
-    return cudaGetLastError();
+    return launch_after(dim3((unsigned)(w_blocks + x_blocks)), dim3(PREP_THREADS), 0, st, linear_prepare_kernel<G, QUANT>,
+                        C16, padded, qtab, qscale, K, idx, (int)d_in, out_groups, o_first, chunks, w_blocks, w_tiles, x, (int)m_first, (int)m_end, NT, x_tiles);
 }
 
 }  // namespace

@@ -31,6 +31,8 @@ constexpr int KB_MAX = 4096;                 // positions of the subtree that on
 
 __global__ void __launch_bounds__(256)
 order_init_kernel(unsigned* __restrict__ order, int K, int Kp) {
+    let_next_start();
+    after_previous();
     const int p = blockIdx.x * 256 + threadIdx.x;
     if (p < Kp) order[p] = p < K ? (unsigned)p : 0xffffffffu;
 }
@@ -42,6 +44,8 @@ order_init_kernel(unsigned* __restrict__ order, int K, int Kp) {
 __global__ void __launch_bounds__(KT_THREADS, 1)
 tree_split_kernel(const float* __restrict__ C, int K, int g, int n, const unsigned* __restrict__ in,
                   unsigned* __restrict__ out, unsigned* __restrict__ tree) {
+    let_next_start();
+    after_previous();
     extern __shared__ __align__(16) uint16_t keys[];                       // n
     __shared__ float part[16][32][2];
     __shared__ int cnt[2][32];
@@ -140,6 +144,8 @@ tree_split_kernel(const float* __restrict__ C, int K, int g, int n, const unsign
 __global__ void __launch_bounds__(KT_THREADS, 1)
 tree_finish_kernel(const float* __restrict__ C, int K, int g, int n0, unsigned* __restrict__ order, unsigned* __restrict__ tree,
                    int first) {
+    let_next_start();
+    after_previous();
     __shared__ unsigned long long key[KB_MAX];
     __shared__ unsigned char axes[KB_MAX / 2];
     extern __shared__ __align__(16) float var[];                           // (n0 / n) x g of one level, at most n0 / 2 x g words
@@ -223,6 +229,8 @@ template <int G>
 __global__ void __launch_bounds__(1024, 1)
 point_leaf_kernel(const uint16_t* __restrict__ X, int64_t N, const unsigned* __restrict__ tree, int levels,
                   uint16_t* __restrict__ leaf, unsigned* __restrict__ rank, unsigned* __restrict__ hist) {
+    let_next_start();
+    after_previous();
     extern __shared__ __align__(16) unsigned st[];
     const int in_smem = (1 << levels) < PK_SMEM_NODES ? (1 << levels) : PK_SMEM_NODES;
     for (int e = threadIdx.x; e < in_smem; e += 1024) st[e] = tree[e];
@@ -259,6 +267,8 @@ point_leaf_kernel(const uint16_t* __restrict__ X, int64_t N, const unsigned* __r
 // Exclusive prefix sums of `bins` (<= 65536) counters, in place; one thread block.
 __global__ void __launch_bounds__(1024)
 leaf_offsets_kernel(unsigned* __restrict__ hist, int bins) {
+    let_next_start();
+    after_previous();
     __shared__ unsigned wsum[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned carry = 0;
@@ -287,6 +297,8 @@ template <int G>
 __global__ void __launch_bounds__(256)
 point_move_kernel(const uint16_t* __restrict__ X, int64_t N, const uint16_t* __restrict__ leaf, unsigned* __restrict__ pos,
                   const unsigned* __restrict__ offset, uint16_t* __restrict__ Xs) {
+    let_next_start();
+    after_previous();
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < N; i += (int64_t)gridDim.x * 256) {
         const unsigned p = __ldg(offset + leaf[i]) + pos[i];
         const uint16_t* src = X + i * G;
@@ -314,6 +326,8 @@ __global__ void __launch_bounds__(256)
 unsort_kernel(const unsigned* __restrict__ pos, int64_t N, const uint16_t* __restrict__ idx_s, const float* __restrict__ dist_s,
               uint16_t* __restrict__ idx, float* __restrict__ dist, const unsigned* __restrict__ marks, unsigned* __restrict__ count,
               unsigned* __restrict__ flagged) {
+    let_next_start();
+    after_previous();
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < N; i += (int64_t)gridDim.x * 256) {
         const unsigned p = pos[i];
         idx[i] = __ldg(idx_s + p);
@@ -324,6 +338,8 @@ unsort_kernel(const unsigned* __restrict__ pos, int64_t N, const uint16_t* __res
 
 __global__ void __launch_bounds__(256)
 mark_kernel(const unsigned* __restrict__ flagged, int64_t N, const unsigned* __restrict__ status, unsigned* __restrict__ marks) {
+    let_next_start();
+    after_previous();
     ull F = *reinterpret_cast<const ull*>(status + 2);
     if (F > (ull)N) F = (ull)N;
     for (ull f = (ull)blockIdx.x * 256 + threadIdx.x; f < F; f += (ull)gridDim.x * 256) atomicOr(marks + (flagged[f] >> 5), 1u << (flagged[f] & 31u));
@@ -345,16 +361,19 @@ cudaError_t sort_points(cc_ctx* ctx, const uint16_t* X, int64_t N, const unsigne
         ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
         int64_t blocks = (N + 1023) / 1024;
         if (blocks > ctx->sm_count) blocks = ctx->sm_count;
-        point_leaf_kernel<G><<<(unsigned)blocks, 1024, nodes * 4, st>>>(X, N, tree, levels, leaf, pos, hist);
+        launch_after(dim3((unsigned)blocks), dim3(1024), nodes * 4, st, point_leaf_kernel<G>,
+                    X, N, tree, levels, leaf, pos, hist);
     }
     {
         ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
-        leaf_offsets_kernel<<<1, 1024, 0, st>>>(hist, 1 << levels);
+        launch_after(dim3(1), dim3(1024), 0, st, leaf_offsets_kernel,
+                    hist, 1 << levels);
     }
     ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
     int64_t blocks = (N + 255) / 256;
     if (blocks > (int64_t)ctx->sm_count * 32) blocks = (int64_t)ctx->sm_count * 32;
-    point_move_kernel<G><<<(unsigned)blocks, 256, 0, st>>>(X, N, leaf, pos, hist, Xs);
+    launch_after(dim3((unsigned)blocks), dim3(256), 0, st, point_move_kernel<G>,
+                    X, N, leaf, pos, hist, Xs);
     return cudaGetLastError();
 }
 
@@ -384,17 +403,20 @@ cudaError_t cc_launch_tree(cc_ctx* ctx, const float* C, int K, int g, unsigned* 
     unsigned* b = (splits & 1) ? order : scratch;
     {
         ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
-        order_init_kernel<<<(Kp + 255) / 256, 256, 0, st>>>(a, K, Kp);
+        launch_after(dim3((Kp + 255) / 256), dim3(256), 0, st, order_init_kernel,
+                    a, K, Kp);
     }
     int nodes = 1;
     for (int n = Kp; n > KB_MAX; n >>= 1, nodes <<= 1) {
         ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
-        tree_split_kernel<<<nodes, KT_THREADS, n * 2, st>>>(C, K, g, n, a, b, tree);
+        launch_after(dim3(nodes), dim3(KT_THREADS), n * 2, st, tree_split_kernel,
+                    C, K, g, n, a, b, tree);
         unsigned* t = a; a = b; b = t;
     }
     ProfScope ps(ctx, CC_K_ASSIGN_PREP, st);
     const int n0 = Kp / nodes;
-    tree_finish_kernel<<<nodes, KT_THREADS, (size_t)n0 / 2 * g * 4, st>>>(C, K, g, n0, a, tree, nodes);
+    launch_after(dim3(nodes), dim3(KT_THREADS), (size_t)n0 / 2 * g * 4, st, tree_finish_kernel,
+                    C, K, g, n0, a, tree, nodes);
     return cudaGetLastError();
 }
 
@@ -425,11 +447,13 @@ cudaError_t cc_launch_unsort(cc_ctx* ctx, const unsigned* pos, int64_t N, const 
         if ((e = cudaMemsetAsync(marks, 0, (size_t)(N + 31) / 32 * 4, st)) != cudaSuccess) return e;
         if ((e = cudaMemsetAsync(status + 41, 0, sizeof(unsigned), st)) != cudaSuccess) return e;
         ProfScope ps(ctx, CC_K_RESOLVE, st);
-        mark_kernel<<<ctx->sm_count, 256, 0, st>>>(flagged, N, status, marks);
+        launch_after(dim3(ctx->sm_count), dim3(256), 0, st, mark_kernel,
+                    flagged, N, status, marks);
     }
     ProfScope ps(ctx, CC_K_ASSIGN_FINISH, st);
     int64_t blocks = (N + 255) / 256;
     if (blocks > (int64_t)ctx->sm_count * 32) blocks = (int64_t)ctx->sm_count * 32;
-    unsort_kernel<<<(unsigned)blocks, 256, 0, st>>>(pos, N, idx_s, dist_s, idx, dist, marks, status + 41, flagged);
+    launch_after(dim3((unsigned)blocks), dim3(256), 0, st, unsort_kernel,
+                    pos, N, idx_s, dist_s, idx, dist, marks, status + 41, flagged);
     return cudaGetLastError();
 }

@@ -33,6 +33,8 @@ template <int G, bool COUNT>
 __global__ void __launch_bounds__(256)
 update_accumulate_kernel(const uint16_t* __restrict__ X, int64_t N, const uint16_t* __restrict__ idx, int K,
                          ull* __restrict__ sum_lo, ull* __restrict__ sum_hi, int* __restrict__ counts, int R) {
+    let_next_start();
+    after_previous();
     const int copy = (int)(blockIdx.x % (unsigned)R);
     sum_lo += (int64_t)copy * K * G;
     sum_hi += (int64_t)copy * K * G;
@@ -83,6 +85,8 @@ template <int G>
 __global__ void __launch_bounds__(UP_THREADS, 1)
 update_private_kernel(const uint16_t* __restrict__ X, int64_t N, const uint16_t* __restrict__ idx, int K,
                       ull* __restrict__ sum_lo, ull* __restrict__ sum_hi, int* __restrict__ counts) {
+    let_next_start();
+    after_previous();
     extern __shared__ __align__(16) uint32_t up_sm[];
     // coordinate-major (word t K + j): at step t a warp's 32 points hit banks j mod 32, spread over all
     // banks, where the cluster-major order would confine them to the banks t mod G
@@ -145,6 +149,8 @@ __global__ void __launch_bounds__(256)
 update_delta_kernel(const uint16_t* __restrict__ X, int64_t N, const uint16_t* __restrict__ idx,
                     uint16_t* __restrict__ idx_prev, int K, ull* __restrict__ sum_lo, ull* __restrict__ sum_hi,
                     int* __restrict__ counts) {
+    let_next_start();
+    after_previous();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
         const int jn = idx[i], jo = idx_prev[i];
         if (jn == jo || jn >= K || jo >= K) continue;
@@ -177,6 +183,8 @@ update_delta_kernel(const uint16_t* __restrict__ X, int64_t N, const uint16_t* _
 __global__ void __launch_bounds__(256)
 update_finish_kernel(long long* __restrict__ sum_lo, long long* __restrict__ sum_hi, const int* count_copies,
                      int* counts, int K, int g, int R, float* __restrict__ C) {
+    let_next_start();
+    after_previous();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     const int KG = K * g;
     if (e >= KG) return;
@@ -201,6 +209,8 @@ update_finish_kernel(long long* __restrict__ sum_lo, long long* __restrict__ sum
 __global__ void __launch_bounds__(256)
 grad_finish_kernel(const long long* __restrict__ sum_lo, const long long* __restrict__ sum_hi, int n, int R,
                    float* __restrict__ dC) {
+    let_next_start();
+    after_previous();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n) return;
     long long lo = 0, hi = 0;
@@ -230,8 +240,8 @@ cudaError_t launch_accumulate(int sm_count, const uint16_t* X, int64_t N, const 
     int64_t blocks = (N * G + 255) / 256;
     const int64_t cap = (int64_t)sm_count * 16;
     if (blocks > cap) blocks = cap;
-    if (counts) update_accumulate_kernel<G, true><<<(unsigned)blocks, 256, 0, st>>>(X, N, idx, K, sum_lo, sum_hi, counts, R);
-    else update_accumulate_kernel<G, false><<<(unsigned)blocks, 256, 0, st>>>(X, N, idx, K, sum_lo, sum_hi, nullptr, R);
+    if (counts) launch_after(dim3((unsigned)blocks), dim3(256), 0, st, update_accumulate_kernel<G, true>, X, N, idx, K, sum_lo, sum_hi, counts, R);
+    else launch_after(dim3((unsigned)blocks), dim3(256), 0, st, update_accumulate_kernel<G, false>, X, N, idx, K, sum_lo, sum_hi, nullptr, R);
     return cudaGetLastError();
 }
 
@@ -253,7 +263,7 @@ cudaError_t launch_private(cc_ctx* ctx, const uint16_t* X, int64_t N, const uint
         attr = true;
     }
     const size_t smem = (size_t)K * (8 * (size_t)G + 4);
-    update_private_kernel<G><<<ctx->sm_count, UP_THREADS, smem, st>>>(X, N, idx, K, sum_lo, sum_hi, counts);
+    launch_after(dim3(ctx->sm_count), dim3(UP_THREADS), smem, st, update_private_kernel<G>, X, N, idx, K, sum_lo, sum_hi, counts);
     return cudaGetLastError();
 }
 
@@ -309,9 +319,7 @@ cudaError_t cc_launch_update(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, 
     if (e != cudaSuccess) return e;
     {
         ProfScope ps(ctx, CC_K_UPDATE_FINISH, st);
-        update_finish_kernel<<<(K * g + 255) / 256, 256, 0, st>>>(reinterpret_cast<long long*>(ws + L.sum_lo),
-                                                                 reinterpret_cast<long long*>(ws + L.sum_hi),
-                                                                 count_copies, counts, K, g, R, C);
+        launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, update_finish_kernel, reinterpret_cast<long long*>(ws + L.sum_lo), reinterpret_cast<long long*>(ws + L.sum_hi), count_copies, counts, K, g, R, C);
     }
     if (ctx->empty_rule == CC_EMPTY_SPLIT_LARGEST) return cc_launch_split_empty(ctx, L, C, K, g, counts, st);
     return cudaGetLastError();
@@ -328,8 +336,7 @@ cudaError_t cc_launch_codebook_grad(cc_ctx* ctx, const WsLayout& L, const uint16
     const cudaError_t e = accumulate_all(ctx, L, dX, N, g, idx, K, counts, R, &count_copies, false, st);
     if (e != cudaSuccess) return e;
     ProfScope ps(ctx, CC_K_UPDATE_FINISH, st);
-    grad_finish_kernel<<<(K * g + 255) / 256, 256, 0, st>>>(reinterpret_cast<long long*>(ws + L.sum_lo),
-                                                           reinterpret_cast<long long*>(ws + L.sum_hi), K * g, R, dC);
+    launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, grad_finish_kernel, reinterpret_cast<long long*>(ws + L.sum_lo), reinterpret_cast<long long*>(ws + L.sum_hi), K * g, R, dC);
     return cudaGetLastError();
 }
 
@@ -338,9 +345,7 @@ cudaError_t cc_launch_update_means(cc_ctx* ctx, const WsLayout& L, int g, int K,
     char* ws = static_cast<char*>(ctx->ws);
     {
         ProfScope ps(ctx, CC_K_UPDATE_FINISH, st);
-        update_finish_kernel<<<(K * g + 255) / 256, 256, 0, st>>>(reinterpret_cast<long long*>(ws + L.sum_lo),
-                                                                 reinterpret_cast<long long*>(ws + L.sum_hi), counts, counts, K,
-                                                                 g, 1, C);
+        launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, update_finish_kernel, reinterpret_cast<long long*>(ws + L.sum_lo), reinterpret_cast<long long*>(ws + L.sum_hi), counts, counts, K, g, 1, C);
     }
     if (ctx->empty_rule == CC_EMPTY_SPLIT_LARGEST) return cc_launch_split_empty(ctx, L, C, K, g, counts, st);
     return cudaGetLastError();
@@ -359,7 +364,7 @@ cudaError_t cc_launch_update_delta(cc_ctx* ctx, const WsLayout& L, const uint16_
         const int64_t cap = (int64_t)ctx->sm_count * 16;
         if (blocks > cap) blocks = cap;
         ProfScope ps(ctx, CC_K_UPDATE_DELTA, st);
-#define CALL(G) update_delta_kernel<G><<<(unsigned)blocks, 256, 0, st>>>(X, N, idx, idx_prev, K, sum_lo, sum_hi, counts)
+#define CALL(G) launch_after(dim3((unsigned)blocks), dim3(256), 0, st, update_delta_kernel<G>, X, N, idx, idx_prev, K, sum_lo, sum_hi, counts)
         CC_UPDATE_DISPATCH(g, CALL)
 #undef CALL
     }
@@ -429,8 +434,6 @@ extern "C" cc_status cc_update_static(int device, const uint16_t* X, int64_t N, 
 #undef CALL
         if (e != cudaSuccess) return CC_ERR_CUDA;
     }
-    update_finish_kernel<<<(K * g + 255) / 256, 256, 0, st>>>(reinterpret_cast<long long*>(sum_lo),
-                                                             reinterpret_cast<long long*>(sum_hi), counts, counts, K, g,
-                                                             1, C);
+    launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, update_finish_kernel, reinterpret_cast<long long*>(sum_lo), reinterpret_cast<long long*>(sum_hi), counts, counts, K, g, 1, C);
     return cudaGetLastError() == cudaSuccess ? CC_OK : CC_ERR_CUDA;
 }
