@@ -302,7 +302,7 @@ constexpr int RED_THREADS = 256;
 __global__ void __launch_bounds__(RED_THREADS)
 planes_reduce_kernel(const float* __restrict__ slabs, int PP, int groups_n, int tiles, int splits, int NT, int g, int d_out,
                      const float* __restrict__ bias, float* __restrict__ y) {
-    extern __shared__ float red_row[];                               // CW x g outputs
+    extern __shared__ __align__(16) float red_row[];                 // CW x g outputs
     const int CW = PM / PP, half = CW / 2, tile = blockIdx.x, m = blockIdx.y;
     const int o0 = tile * CW * g;
     int width = d_out - o0;
