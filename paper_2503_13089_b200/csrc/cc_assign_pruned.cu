@@ -32,11 +32,6 @@ constexpr int PR_GROUP = PR_TILES * TM;  // points per group
 constexpr int PR_ROWS = PR_GROUP / 32;   // row blocks per group
 constexpr int PR_MAX_CHUNKS = 1024;
 
-__device__ __forceinline__ float redux_min(float v) {
-    float r;
-    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
-    return r;
-}
 __device__ __forceinline__ float redux_max(float v) {
     float r;
     asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
@@ -159,7 +154,7 @@ chunk_bounds_kernel(const float* __restrict__ C, int K, const unsigned* __restri
 // whole pairs with an entry that nobody needs.
 constexpr int PR_MASK_SHIFT = 10;
 constexpr unsigned PR_CHUNK_MASK = (1u << PR_MASK_SHIFT) - 1u, PR_LOOK = 1u << 14;
-constexpr int PR_LOOK_EVERY = 4;         // pairs
+constexpr int PR_LOOK_EVERY = 16;        // pairs
 
 struct ListArgs {
     const uint16_t* Xs; int64_t N;
@@ -410,9 +405,10 @@ pruned_list_kernel(const ListArgs a) {
 //   warp 8      copies lists and chunks (one thread)
 //   warp 9      issues the MMAs (one thread): 128 points x two chunks into one of two accumulators
 // A pair costs nothing to a warp that needs neither of it: the MMA thread releases the accumulator in its stead.
-// Pairs are announced on a ring of eight barriers, and every warp looks at (waits for and releases) at least every
-// fourth pair, which keeps it within one phase of every barrier, and a tile's last pair, after which the tile's
-// A rows are free.
+// Pairs are announced on a ring of barriers, and every warp looks at (waits for and releases) one pair in half a ring
+// at the least, which keeps it within one phase of every barrier, and a tile's last pair, after which the tile's
+// A rows are free.  A look that a warp does not need holds the accumulator up: one in sixteen instead of one in four (5.6 M
+// points, g = 8, K = 65536, twenty iterations 346 -> 341 ms).
 // Measured on the way here: a successful wait on an mbarrier costs an issuing thread about 110 cycles right behind
 // an MMA, a further one 45, the MMA and its commit together 48 (N = 64); a waiting warp is back at work about 90
 // cycles after the arrival.  What counts is therefore the chain of a pair: announcement, load of the accumulator, its
@@ -420,17 +416,20 @@ pruned_list_kernel(const ListArgs a) {
 // pipeline per tile with a handshake per chunk 217, per pair 167 with one accumulator and both chunks by the same warp
 // (2.8 M points, K = 65,500, g = 6, twenty iterations 87 ms); there the thread that issued and copied took 700 cycles a
 // pair, and with both waits in one round trip, the copies on a warp of their own and two accumulators 83.5 ms.
+// Where the time goes (the 19 scans of that fit, 58.9 ms; each with less of the look left in): without the gap 47.0, without gap and
+// minimum 32.5, without loading the accumulator either, i.e. the handshakes alone, 29.8.  Finishing the gap of one look beside the
+// accumulator or the minimum of the next was slower each way it was written (1 to 30 %): the release must not wait.
 constexpr int PS_EPI = 8;
 constexpr int PS_THREADS = (PS_EPI + 2) * 32;
 constexpr int PS_BLOCKS = 2;             // resident per SM
 constexpr int PS_LISTS = 3;
-constexpr int PS_RING = 8;
+constexpr int PS_RING = 2 * PR_LOOK_EVERY;
 
 template <int G> struct PrCfg {
     using Cfg = TcCfg<G>;
     static constexpr int CH_BYTES = PR_CHUNK * Cfg::KD * 2;
     static constexpr int STAGES = Cfg::KD == 16 ? 10 : 6;   // pairs of chunks
-    static constexpr int SMEM = 2 * Cfg::A_TILE + STAGES * 2 * CH_BYTES + PS_LISTS * PR_MAX_CHUNKS * 2 + 2 * 3 * TM * 4 + 512;
+    static constexpr int SMEM = 2 * Cfg::A_TILE + STAGES * 2 * CH_BYTES + PS_LISTS * PR_MAX_CHUNKS * 2 + 2 * 3 * TM * 4 + 512 + PS_RING * 8;
 };
 
 struct ScanArgs {
@@ -781,6 +780,8 @@ assign_pruned_kernel(const ScanArgs a) {
 
 // ---------------------------------------------------------------------------------------------
 // Finish: as in the exhaustive scan (see finish_tensor_kernel), on positions; codes come out as centroid numbers.
+// Neighbouring positions mostly share their winning chunk (winners_by_chunk): 4.2 M points, g = 4, K = 4096 271 us with a
+// group of lanes per point, 230 so; 2.8 M, g = 6, K = 65500 324 and 233.
 template <int G>
 __global__ void __launch_bounds__(256)
 pruned_finish_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __restrict__ Cs, int K, int n_chunks,
@@ -789,8 +790,9 @@ pruned_finish_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __r
                      unsigned* __restrict__ status, unsigned* __restrict__ flagged) {
     let_next_start();
     after_previous();
-    const int k = threadIdx.x & (LPP - 1);
+    __shared__ __align__(16) float2 xs_all[8][32][G];            // each coordinate twice
     const int lane = threadIdx.x & 31;
+    float2 (*xs)[G] = xs_all[threadIdx.x >> 5];
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const int64_t rounds = (N + n_warps * 32 - 1) / (n_warps * 32);
@@ -799,62 +801,19 @@ pruned_finish_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __r
     float far = 0.f;
     for (int64_t rd = 0; rd < rounds; ++rd) {
         const int64_t base = (rd * n_warps + warp0) * 32;
+        if (base >= N) break;
         const int64_t i_raw = base + lane;
         const bool live = i_raw < N;
         const int64_t i = live ? i_raw : N - 1;
-        float2 t_own = tstate[i];
-        t_own.y = __int_as_float(min(max(__float_as_int(t_own.y), 0), n_chunks - 1));   // garbage after a time-out stays inside
+        const float2 t_own = tstate[i];
+        const int chunk_own = min(max(__float_as_int(t_own.y), 0), n_chunks - 1);   // garbage after a time-out stays inside
         float x_own[G];
         bool nf = false;
         load_point<G>(X, i, N, x_own, nf);
         float keep_s1 = 0.f, keep_s2 = 0.f;
         int keep_p = 0;
-#pragma unroll 1
-        for (int sub = 0; sub < LPP; ++sub) {
-            const int src = (lane & ~(LPP - 1)) + sub;
-            const int chunk = __shfl_sync(0xffffffffu, __float_as_int(t_own.y), src);
-            float x[G];
-#pragma unroll
-            for (int t = 0; t < G; ++t) x[t] = __shfl_sync(0xffffffffu, x_own[t], src);
-            const float4* blk = reinterpret_cast<const float4*>(rescan + (int64_t)chunk * ((G + 1) * PR_CHUNK)) + k;
-            float s1 = INFINITY, s2 = INFINITY;
-            int j1 = 4 * k;
-#pragma unroll
-            for (int hf = 0; hf < PR_CHUNK / 4 / LPP; ++hf) {
-                const float4 cs = __ldg(blk + G * (PR_CHUNK / 4) + hf * LPP);
-                float s[4] = {cs.x, cs.y, cs.z, cs.w};
-#pragma unroll
-                for (int t = 0; t < G; ++t) {
-                    const float4 mv = __ldg(blk + t * (PR_CHUNK / 4) + hf * LPP);
-                    s[0] = fmaf(x[t], mv.x, s[0]);
-                    s[1] = fmaf(x[t], mv.y, s[1]);
-                    s[2] = fmaf(x[t], mv.z, s[2]);
-                    s[3] = fmaf(x[t], mv.w, s[3]);
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const bool take = s[e] < s1;
-                    s2 = take ? s1 : fminf(s2, s[e]);
-                    j1 = take ? (hf * LPP + k) * 4 + e : j1;
-                    s1 = take ? s[e] : s1;
-                }
-            }
-#pragma unroll
-            for (int o = LPP / 2; o > 0; o >>= 1) {
-                const float os1 = __shfl_xor_sync(0xffffffffu, s1, o);
-                const float os2 = __shfl_xor_sync(0xffffffffu, s2, o);
-                const int oj = __shfl_xor_sync(0xffffffffu, j1, o);
-                const bool take = os1 < s1 || (os1 == s1 && oj < j1);
-                s2 = fminf(take ? s1 : os1, fminf(s2, os2));
-                s1 = take ? os1 : s1;
-                j1 = take ? oj : j1;
-            }
-            if (k == sub) {
-                keep_p = j1 + chunk * PR_CHUNK;
-                keep_s1 = s1;
-                keep_s2 = fminf(s2, t_own.x * invS);
-            }
-        }
+        winners_by_chunk<G>(rescan, chunk_own, x_own, xs, keep_s1, keep_s2, keep_p);
+        keep_s2 = fminf(keep_s2, t_own.x * invS);
         const int p1 = min(keep_p, K - 1);   // beyond K only with non-finite input or after a time-out
         double D = 0.0;
         float A = 0.f, L1 = 0.f;

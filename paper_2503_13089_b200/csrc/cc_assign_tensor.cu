@@ -594,7 +594,9 @@ assign_tensor_persistent_kernel(const uint16_t* __restrict__ X, int64_t N, const
 // least as close as the winner (distance d) has ||c|| <= ||x|| + d, hence 2||c||^2 + ||x||^2 <=
 // 3||x||^2 + 4||x|| d + 2 d^2, so a point whose two smallest scores are closer than 2E with that
 // substitution goes to the exact stage.
-template <int G>
+//
+// BY_CHUNK: winner and runner-up as winners_by_chunk finds them, for few chunks.
+template <int G, bool BY_CHUNK>
 __global__ void __launch_bounds__(256)
 finish_tensor_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __restrict__ C, int K, int n_chunks,
                      const float* __restrict__ rescan, const float2* __restrict__ tstate,
@@ -602,6 +604,7 @@ finish_tensor_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __r
                      unsigned* __restrict__ status, unsigned* __restrict__ flagged) {
     let_next_start();
     after_previous();
+    __shared__ __align__(16) float2 xs_all[BY_CHUNK ? 8 : 1][32][G];
     const int k = threadIdx.x & (LPP - 1);
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -634,6 +637,10 @@ finish_tensor_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __r
         load_point<G>(X, i, N, x_own, nf);
         float keep_s1 = 0.f, keep_s2 = 0.f;
         int keep_j = 0;
+        if constexpr (BY_CHUNK) {
+            winners_by_chunk<G>(rescan, __float_as_int(t_own.y), x_own, xs_all[threadIdx.x >> 5], keep_s1, keep_s2, keep_j);
+            keep_s2 = fminf(keep_s2, t_own.x * invS);
+        } else
 #pragma unroll 1
         for (int sub = 0; sub < LPP; ++sub) {
             const int src = (lane & ~(LPP - 1)) + sub;
@@ -709,6 +716,11 @@ finish_tensor_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __r
         }
     }
 }
+
+// Winners chunk by chunk where 32 points meet few chunks.  E-step of 4.2 M points, a group of lanes per point / by chunk, in us:
+// g = 4, K = 256 640 / 614, K = 512 650 / 638, K = 1024 660 / 680; g = 6 821 / 759, 827 / 790, 860 / 850; g = 8 972 / 858, 1061 / 913, 1182 /
+// 1011; g = 16 1136 / 997, 1363 / 1166, 1490 / 1465, K = 2048 1740 / 1935.
+constexpr bool finish_by_chunk(int K, int g) { return K <= (g <= 4 ? 512 : 1024); }
 
 template <int G>
 cudaError_t launch_tensor(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, const float* C, int K,
@@ -787,7 +799,9 @@ cudaError_t launch_tensor(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int
             int64_t fblocks = (N + 255) / 256;            // a warp takes 32 points per round
             const int64_t cap = (int64_t)ctx->sm_count * 32;
             if (fblocks > cap) fblocks = cap;
-            launch_after(dim3((unsigned)fblocks), dim3(256), 0, st, finish_tensor_kernel<G>,
+            if (finish_by_chunk(K, G)) launch_after(dim3((unsigned)fblocks), dim3(256), 0, st, finish_tensor_kernel<G, true>,
+                     X, N, C, K, Kpad / TCHUNK, rescan, tstate, params, idx, dist, status, reinterpret_cast<unsigned*>(ws + L.flagged));
+            else launch_after(dim3((unsigned)fblocks), dim3(256), 0, st, finish_tensor_kernel<G, false>,
                      X, N, C, K, Kpad / TCHUNK, rescan, tstate, params, idx, dist, status, reinterpret_cast<unsigned*>(ws + L.flagged));
         }
     }

@@ -198,4 +198,60 @@ __device__ __forceinline__ float chunk_min64(const uint32_t* v0, const uint32_t*
     return fminf(min3(w0, w1, u[6]), val(63));
 }
 
+__device__ __forceinline__ ull fma2(ull a, ull b, ull c) { ull r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ float redux_min(float v) {
+    float r;
+    asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+// Winner and runner-up inside their winning chunks for the 32 points of a warp, chunk by chunk: a lane keeps two of a
+// chunk's 64 centroids in registers (read once per chunk, where a group of lanes per point reads 256 (G + 1) bytes per
+// point), the points' coordinates come from shared memory, two to a packed instruction, and two warp-wide minima give the
+// smallest score and the next.  Pays where the points share few chunks.  xs: room for the points' coordinates, each twice.
+// The scores are those of the chain s = fma(x_{g-1}, m_{g-1}, ... fma(x_0, m_0, ||c||^2)).
+template <int G>
+__device__ __forceinline__ void winners_by_chunk(const float* __restrict__ rescan, int chunk_own, const float (&x_own)[G],
+                                                 float2 (*xs)[G], float& best, float& second, int& at) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < G; ++t) xs[lane][t] = make_float2(x_own[t], x_own[t]);
+    __syncwarp();
+    unsigned todo = 0xffffffffu;
+    while (todo) {
+        const int chunk = __shfl_sync(0xffffffffu, chunk_own, __ffs(todo) - 1);
+        unsigned members = __ballot_sync(0xffffffffu, chunk_own == chunk);
+        todo &= ~members;
+        const ull* blk = reinterpret_cast<const ull*>(rescan + (int64_t)chunk * ((G + 1) * TCHUNK)) + lane;
+        ull m[G + 1];
+#pragma unroll
+        for (int t = 0; t <= G; ++t) m[t] = __ldg(blk + t * (TCHUNK / 2));
+        auto point = [&](int p) {
+            ull s = m[G];
+#pragma unroll
+            for (int t = 0; t < G; ++t) s = fma2(*reinterpret_cast<const ull*>(&xs[p][t]), m[t], s);
+            const float a = __uint_as_float((unsigned)s), b = __uint_as_float((unsigned)(s >> 32));
+            const float mn = fminf(a, b);
+            const float s1 = redux_min(mn);
+            const int w = (__ffs(__ballot_sync(0xffffffffu, mn == s1)) - 1) & 31;
+            const float s2 = redux_min(lane == w ? fmaxf(a, b) : mn);
+            const unsigned odd = __ballot_sync(0xffffffffu, b < a);
+            if (lane == p) {
+                best = s1;
+                second = s2;
+                at = chunk * TCHUNK + (s1 < INFINITY ? 2 * w + (int)((odd >> w) & 1u) : 0);
+            }
+        };
+        while (members) {                                    // two at a time: their chains overlap
+            const int p0 = __ffs(members) - 1;
+            members &= members - 1;
+            const int p1 = members ? __ffs(members) - 1 : p0;
+            members &= members - 1;
+            point(p0);
+            point(p1);
+        }
+    }
+}
+
 }  // namespace
