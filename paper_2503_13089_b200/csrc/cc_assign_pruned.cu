@@ -508,7 +508,6 @@ __device__ __forceinline__ float word_norm(const unsigned* w) {
 template <int G, bool GAP>
 __global__ void __launch_bounds__(PS_THREADS, PS_BLOCKS)
 assign_pruned_kernel(const ScanArgs a) {
-    let_next_start();
     after_previous();
     using Cfg = TcCfg<G>;
     constexpr int KD = Cfg::KD, A_TILE = Cfg::A_TILE, CH = PrCfg<G>::CH_BYTES, STAGES = PrCfg<G>::STAGES;

@@ -128,7 +128,6 @@ assign_tensor_kernel(const uint16_t* __restrict__ X, int64_t N, const uint16_t* 
                      int na_per_cta, int64_t tile_offset, const TcParams* __restrict__ params,
                      float2* __restrict__ tstate, unsigned* __restrict__ status, float* __restrict__ dump,
                      int64_t dump_ld) {
-    let_next_start();
     after_previous();
     using Cfg = TcCfg<G>;
     constexpr int KD = Cfg::KD, STAGES = Cfg::STAGES;
@@ -353,7 +352,6 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
 assign_tensor_persistent_kernel(const uint16_t* __restrict__ X, int64_t N, const uint16_t* __restrict__ gB, int n_btiles,
                                 int n_groups, const TcParams* __restrict__ params, float2* __restrict__ tstate,
                                 unsigned* __restrict__ status) {
-    let_next_start();
     after_previous();
     using Cfg = TcCfg<G>;
     constexpr int KD = Cfg::KD, STAGES = Cfg::STAGES;

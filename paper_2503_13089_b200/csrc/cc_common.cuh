@@ -61,7 +61,8 @@ struct ProfScope {
 
 // In a kernel that launch_after starts: everything in front of it has ended and is visible from here on; and the next such kernel may
 // start (its blocks take the places that become free, and wait here in turn).  Calls back to back save about a
-// microsecond each.
+// microsecond each.  Kernels that fill an SM's shared memory do not let the next one start before they end where that lives off
+// L1: its blocks would keep the small L1 they found (35,000 points, g = 16, K = 6971, twelve iterations 1189 -> 1294 us).
 #ifdef __CUDACC__
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -28,7 +28,6 @@ template <int MODE>
 __global__ void __launch_bounds__(DP_THREADS, 1)
 decode_planes_kernel(const uint16_t* __restrict__ C16, int K, int g, const uint16_t* __restrict__ idx, int out_groups, int d_out, int d_in,
                      uint16_t* __restrict__ W_hat) {
-    let_next_start();
     after_previous();
     constexpr int QS = DP_GROUPS / 2, PASSES = R / 16;
     extern __shared__ __align__(16) unsigned char dp_smem[];

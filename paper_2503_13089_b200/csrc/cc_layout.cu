@@ -321,7 +321,6 @@ template <int G, bool TABLE>
 __global__ void __launch_bounds__(256, 4)
 decode_transpose_pipe_kernel(const uint16_t* __restrict__ C16, const uint16_t* __restrict__ idx, int K, int64_t d_out,
                              int64_t d_in, int64_t out_pad, uint16_t* __restrict__ W_hat, int tiles_x, int tiles_y) {
-    let_next_start();
     after_previous();
     extern __shared__ __align__(16) unsigned char decode_smem[];
     unsigned* tile = reinterpret_cast<unsigned*>(decode_smem);
@@ -488,7 +487,6 @@ template <int G>
 __global__ void __launch_bounds__(RES_THREADS, 1)
 decode_transpose_resident_kernel(const uint16_t* __restrict__ C16, const uint16_t* __restrict__ idx, int K, int head_rows,
                                  int64_t d_out, int64_t d_in, int64_t out_pad, uint16_t* __restrict__ W_hat, int tiles_x, int tiles_y) {
-    let_next_start();
     after_previous();
     extern __shared__ __align__(16) unsigned char decode_smem[];
     const int group = threadIdx.x >> 8, tid = threadIdx.x & 255;

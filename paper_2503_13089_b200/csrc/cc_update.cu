@@ -85,7 +85,6 @@ template <int G>
 __global__ void __launch_bounds__(UP_THREADS, 1)
 update_private_kernel(const uint16_t* __restrict__ X, int64_t N, const uint16_t* __restrict__ idx, int K,
                       ull* __restrict__ sum_lo, ull* __restrict__ sum_hi, int* __restrict__ counts) {
-    let_next_start();
     after_previous();
     extern __shared__ __align__(16) uint32_t up_sm[];
     // coordinate-major (word t K + j): at step t a warp's 32 points hit banks j mod 32, spread over all
