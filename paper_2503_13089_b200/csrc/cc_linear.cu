@@ -933,7 +933,7 @@ cudaError_t cc_launch_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, 
     {
         PlanesPlan pl = {};
         if (M <= PL_NT_MAX) pl = planes_plan(M, d_out, d_in, ctx->sm_count, K, g, planes_chain(M, d_out, d_in, ctx->sm_count, g));
-        if (pl.fits && planes_pay(pl, M, out_groups * d_in, g, qtab != nullptr) && ctx->ws_bytes >= CC_LINEAR_SCRATCH_FROM + pl.bytes)
+        if (pl.fits && planes_pay(pl, M, d_out, d_in, g, qtab != nullptr) && ctx->ws_bytes >= CC_LINEAR_SCRATCH_FROM + pl.bytes)
             return cc_launch_linear_planes(ctx, pl, x, (int)M, C16, qtab, qscale, K, g, idx, (int)d_out, (int)d_in, bias, y, st);
     }
     // beside the table: token blocks of 64 with four stages, or, from LQ_WIDE_FROM tokens on, of 256 with two

@@ -194,13 +194,17 @@ inline PlanesPlan planes_plan(int64_t M, int64_t d_out, int64_t d_in, int sm_cou
 //   many parts of the in_features, i.e. few out_features: 57 tokens, 640 x 9707, g = 6, K = 12893 17 / 20, 25 tokens, 640 x 6893,
 //     g = 4, K = 27278 12 / 15; with four coordinates a look-up 12 tokens, 832 x 1984, g = 4, K = 1137 14 / 10;
 //   the 4-bit codebook from 192 tokens on, where the weight is decoded once: 215 tokens, 8064 x 2191, g = 8 24 / 41;
+//   few in_features for many out_features, whose tiles keep the SMs busy without parts: 101 tokens, 6848 x 1011, g = 8, K = 2499, 4 bits 16.4 /
+//     18.0, 5 tokens, 10624 x 686, g = 4, K = 39870 13.9 / 15.2 (odd g: 66 tokens, 8000 x 896, g = 5 22 / 18);
 //   many tokens on few codes: 224 tokens, 768 x 512, g = 4, K = 17749 12.9 / 14.3.
 // Over 162 drawn layers of 5 to 256 tokens the planes alone are 1.22 times as fast in the mean, with these bounds 1.24.
 // Up to 64 tokens the answer may not depend on the form of the codebook (both give the same bits there).
-inline bool planes_pay(const PlanesPlan& p, int64_t M, int64_t codes, int g, bool quant) {
+inline bool planes_pay(const PlanesPlan& p, int64_t M, int64_t d_out, int64_t d_in, int g, bool quant) {
+    const int64_t codes = (d_out + g - 1) / g * d_in;
     if (g >= 10 && p.PP < 4) return false;
     if (p.PP == 1 && (g >= 8 || codes < 2000000)) return false;
     if (p.PP < 4 && p.splits > 16) return false;
+    if (g % 2 == 0 && d_in <= 1152 && d_out >= 4 * d_in) return false;
     return !(quant && M > 192) && !(M > 128 && codes < 200000);
 }
 
