@@ -133,6 +133,23 @@ inline size_t padded_table_at(uintptr_t ws, size_t from, size_t to, int K, int p
 // ---- Layer forward plane by plane.
 constexpr int PL_ROWS = 128, PL_KB = 64, PL_NT_MAX = 256, PL_SPLITS_MAX = 64;
 constexpr size_t PL_SMEM = 226 * 1024, PL_HEAD = 256;
+constexpr int PL_LOOK_WARPS = 16;
+
+// How the look-up warps share out a stage.  The warps of a stage are PL_LOOK_WARPS / stages; a thread of them has one pair of
+// neighbouring code groups and blocks of eight in_features first, first + step, ...  With four coordinates a look-up and two stages
+// there are twice as many threads as blocks: half of them have none, their first is behind the last of the stage.
+struct PlaneShare { int pair, first, step; };
+CC_PLAN_FN constexpr PlaneShare plane_share(int PP, int stages, int thread) {
+    const int pairs = PL_ROWS / PP / 2;
+    return {thread % pairs, thread / pairs, PL_LOOK_WARPS / stages * 32 / pairs};
+}
+
+// In_features of block `block` of stage `stage` whose codes may be asked for: 8, fewer at the end of the layer, 0 where there is no
+// such block (past the layer, or past the stage).
+CC_PLAN_FN constexpr int plane_block_rows(int stage, int block, int d_in) {
+    const int left = d_in - (stage * PL_KB + block * 8);
+    return block >= PL_KB / 8 || left <= 0 ? 0 : (left < 8 ? left : 8);
+}
 
 // Clocks of an SM for a stage of 64 in_features: its 2 CW look-ups by 32 lanes take 3.5 clocks each (rows of 2 or 4 bytes) or 6.2
 // (8 bytes), half a clock goes to the codes and half to each 16-byte piece of the operand.

@@ -22,7 +22,7 @@ constexpr int PM = PL_ROWS;                             // operand rows = TMEM l
 constexpr int PKB = PL_KB;                           // in_features per stage
 constexpr int P_A_STAGE = PM * PKB * 2;
 constexpr int P_STAGES_MAX = 4;
-constexpr int P_LOOK_WARPS = 16;
+constexpr int P_LOOK_WARPS = PL_LOOK_WARPS;
 constexpr int P_THREADS = (4 + 2 + P_LOOK_WARPS) * 32;
 constexpr int PREP_BLOCK = 256;
 
@@ -104,7 +104,7 @@ linear_planes_kernel(const unsigned char* __restrict__ planes, int K, const uint
                      int NT, int nt_cols, int items, int splits, int tmem_cols, const unsigned char* __restrict__ x_tiles,
                      float* __restrict__ slabs, unsigned* __restrict__ status) {
     constexpr int CW = PM / PP, PAIRS_W = CW / 2;
-    constexpr int WPS = P_LOOK_WARPS / STAGES, STAGE_THREADS = WPS * 32;                // warps and threads that fill one
+    constexpr int WPS = P_LOOK_WARPS / STAGES;                      // warps that fill a stage
     extern __shared__ __align__(1024) unsigned char pl_smem[];
     const int b_stage = NT * PKB * 2;
     unsigned char* table = pl_smem;                                 // first, so that look-ups have a constant base
@@ -149,16 +149,17 @@ linear_planes_kernel(const unsigned char* __restrict__ planes, int K, const uint
         for (int s = 0; s < sg && w.more(); ++s) w.step();
         const unsigned kmax2 = (unsigned)(K - 1) * 0x10001u, row = (unsigned)out_groups * 2u;
         const unsigned char* codes = reinterpret_cast<const unsigned char*>(idx);
-        // A thread's look-ups of a stage: one pair of code groups, blocks of eight in_features rb0, rb0 + RB_STEP, ..
-        constexpr int RB_STEP = STAGE_THREADS / PAIRS_W;
-        const int q = ptid % PAIRS_W, rb0 = ptid / PAIRS_W;
+        constexpr int RB_STEP = plane_share(PP, STAGES, 0).step;
+        const PlaneShare mine = plane_share(PP, STAGES, ptid);
+        const int q = mine.pair, rb0 = mine.first;
         PlaneCodes<MODE> coming;                                     // of the next block to look up, requested early
         auto request = [&](const PlaneWalk& at, int rb) {
             const unsigned grp = at.tile * CW + 2 * q;
-            if ((int)grp >= out_groups) return;
+            const int rows = plane_block_rows(at.c, rb, d_in);       // never past the end of the codes
+            if ((int)grp >= out_groups || rows == 0) return;
             const unsigned i = at.c * PKB + rb * 8, off = i * row + grp * 2u, second = (int)grp + 1 < out_groups ? 2u : 0u;
-            if ((at.c + 1) * PKB <= d_in) coming.request(codes, off, row, second);
-            else if ((int)i < d_in) coming.request_some(codes, off, row, second, d_in - (int)i);
+            if (rows == 8) coming.request(codes, off, row, second);
+            else coming.request_some(codes, off, row, second, rows);
         };
         if (w.more()) request(w, rb0);
         bool ok = mbar_wait(smem_u32(landed), 0, abort_flag);

@@ -48,3 +48,56 @@ def test_no_plan_of_the_planes_exceeds_its_limits(tmp_path):
     subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
     out = subprocess.run([str(exe)], stdout=subprocess.PIPE, text=True)
     assert out.returncode == 0, out.stdout
+
+
+REQUESTS = r"""
+#include <cstdio>
+#include <vector>
+#include "cc_linear_plan.h"
+
+// The look-up threads' requests in the order of linear_planes_kernel: the first block of a thread's first stage before the loop, in the loop
+// always the next one; `item` starts at any stage.  No request may lie past the layer, and every in_feature has to have been asked for.
+int main() {
+    long asked = 0, bad = 0;
+    for (int PP = 1; PP <= 4; PP *= 2)
+        for (int stages = 2; stages <= 4; stages += 2)
+            for (int d_in : {1, 7, 8, 63, 64, 65, 72, 127, 128, 130, 191, 192, 200, 256, 515, 4491, 2380})
+                for (int from = 0; from < (d_in + 63) / 64; ++from) {
+                    const int chunks = (d_in + 63) / 64, pairs = 64 / PP, threads = PL_LOOK_WARPS / stages * 32;
+                    std::vector<int> seen((size_t)pairs * d_in, 0);
+                    auto request = [&](int stage, const PlaneShare& t, int block) {
+                        const int rows = plane_block_rows(stage, block, d_in);
+                        for (int r = 0; r < rows; ++r) {
+                            const int i = stage * 64 + block * 8 + r;
+                            ++asked;
+                            if (i < 0 || i >= d_in || i >= (stage + 1) * 64) { if (bad++ < 10) printf("PP=%d stages=%d d_in=%d: row %d\n", PP, stages, d_in, i); }
+                            else ++seen[(size_t)t.pair * d_in + i];
+                        }
+                    };
+                    for (int sg = 0; sg < stages; ++sg)
+                        for (int thread = 0; thread < threads; ++thread) {
+                            const PlaneShare t = plane_share(PP, stages, thread);
+                            int c = from + sg;
+                            if (t.pair < 0 || t.pair >= pairs || t.step < 1) { ++bad; continue; }
+                            if (c < chunks) request(c, t, t.first);
+                            for (; c < chunks; c += stages)
+                                for (int b = t.first; b < 8; b += t.step) {
+                                    if (b + t.step < 8) request(c, t, b + t.step);
+                                    else if (c + stages < chunks) request(c + stages, t, t.first);
+                                }
+                        }
+                    for (size_t e = 0; e < seen.size(); ++e)
+                        if (seen[e] != ((int)(e % d_in) >= from * 64 ? 1 : 0) && bad++ < 10) printf("PP=%d stages=%d d_in=%d: %d times\n", PP, stages, d_in, seen[e]);
+                }
+    printf("%ld requests, %ld bad\n", asked, bad);
+    return bad != 0;
+}
+"""
+
+
+def test_no_look_up_thread_asks_for_codes_past_the_layer(tmp_path):
+    src, exe = tmp_path / "requests.cpp", tmp_path / "requests"
+    src.write_text(REQUESTS)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    out = subprocess.run([str(exe)], stdout=subprocess.PIPE, text=True)
+    assert out.returncode == 0, out.stdout
