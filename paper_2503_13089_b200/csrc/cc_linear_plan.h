@@ -144,12 +144,8 @@ CC_PLAN_FN constexpr PlaneShare plane_share(int PP, int stages, int thread) {
     return {thread % pairs, thread / pairs, PL_LOOK_WARPS / stages * 32 / pairs};
 }
 
-// In_features of block `block` of stage `stage` whose codes may be asked for: 8, fewer at the end of the layer, 0 where there is no
-// such block (past the layer, or past the stage).
-CC_PLAN_FN constexpr int plane_block_rows(int stage, int block, int d_in) {
-    const int left = d_in - (stage * PL_KB + block * 8);
-    return block >= PL_KB / 8 || left <= 0 ? 0 : (left < 8 ? left : 8);
-}
+// Whether a stage has the block, i.e. whether its codes may be asked for (those of its in_features that exist).
+CC_PLAN_FN constexpr bool plane_has_block(int step, int block) { return step <= PL_KB / 8 || block < PL_KB / 8; }
 
 // Clocks of an SM for a stage of 64 in_features: its 2 CW look-ups by 32 lanes take 3.5 clocks each (rows of 2 or 4 bytes) or 6.2
 // (8 bytes), half a clock goes to the codes and half to each 16-byte piece of the operand.

@@ -150,16 +150,14 @@ linear_planes_kernel(const unsigned char* __restrict__ planes, int K, const uint
         const unsigned kmax2 = (unsigned)(K - 1) * 0x10001u, row = (unsigned)out_groups * 2u;
         const unsigned char* codes = reinterpret_cast<const unsigned char*>(idx);
         constexpr int RB_STEP = plane_share(PP, STAGES, 0).step;
-        const PlaneShare mine = plane_share(PP, STAGES, ptid);
-        const int q = mine.pair, rb0 = mine.first;
+        const int q = plane_share(PP, STAGES, ptid).pair, rb0 = plane_share(PP, STAGES, ptid).first;
         PlaneCodes<MODE> coming;                                     // of the next block to look up, requested early
         auto request = [&](const PlaneWalk& at, int rb) {
             const unsigned grp = at.tile * CW + 2 * q;
-            const int rows = plane_block_rows(at.c, rb, d_in);       // never past the end of the codes
-            if ((int)grp >= out_groups || rows == 0) return;
+            if ((int)grp >= out_groups || !plane_has_block(RB_STEP, rb)) return;
             const unsigned i = at.c * PKB + rb * 8, off = i * row + grp * 2u, second = (int)grp + 1 < out_groups ? 2u : 0u;
-            if (rows == 8) coming.request(codes, off, row, second);
-            else coming.request_some(codes, off, row, second, rows);
+            if ((at.c + 1) * PKB <= d_in) coming.request(codes, off, row, second);
+            else if ((int)i < d_in) coming.request_some(codes, off, row, second, d_in - (int)i);
         };
         if (w.more()) request(w, rb0);
         bool ok = mbar_wait(smem_u32(landed), 0, abort_flag);

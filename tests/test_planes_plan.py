@@ -66,9 +66,10 @@ int main() {
                     const int chunks = (d_in + 63) / 64, pairs = 64 / PP, threads = PL_LOOK_WARPS / stages * 32;
                     std::vector<int> seen((size_t)pairs * d_in, 0);
                     auto request = [&](int stage, const PlaneShare& t, int block) {
-                        const int rows = plane_block_rows(stage, block, d_in);
-                        for (int r = 0; r < rows; ++r) {
+                        if (!plane_has_block(t.step, block)) return;
+                        for (int r = 0; r < 8; ++r) {
                             const int i = stage * 64 + block * 8 + r;
+                            if ((stage + 1) * 64 > d_in && i >= d_in) break;       // a stage that is not whole is looked at row by row
                             ++asked;
                             if (i < 0 || i >= d_in || i >= (stage + 1) * 64) { if (bad++ < 10) printf("PP=%d stages=%d d_in=%d: row %d\n", PP, stages, d_in, i); }
                             else ++seen[(size_t)t.pair * d_in + i];
