@@ -385,7 +385,7 @@ def linear_rows(cc, torch, ctx, peaks):
     for M in (1, 16, 256, 4096):
         x = (torch.randn((M, d_in), device="cuda", generator=gen) * 0.5).to(torch.float16)
         y = torch.empty((M, d_out), dtype=torch.float32, device="cuda")
-        ctx.ensure_workspace(N, g, K, at_least=cc.cc_linear_workspace_bytes(ctx, M, d_out, d_in))
+        ctx.ensure_workspace(N, g, K, at_least=cc.cc_linear_workspace_bytes_preferred(ctx, M, d_out, d_in, g, K))
         reps = 20
 
         def timed(call):
@@ -421,7 +421,7 @@ def run_kernel_mode(a):
     N, g, K = a.N, a.g, a.K
     ctx = cc.Context(0)
     d_out, d_in = g * 1024, N // 1024
-    ctx.ensure_workspace(N, g, K, at_least=cc.cc_linear_workspace_bytes(ctx, a.M, d_out, max(d_in, 1)) if a.kernel in ("linear", "linear_q4") else 0)
+    ctx.ensure_workspace(N, g, K, at_least=cc.cc_linear_workspace_bytes_preferred(ctx, a.M, d_out, max(d_in, 1), g, K) if a.kernel in ("linear", "linear_q4") else 0)
     cc.cc_set_path(ctx, {"auto": 0, "ffma": 1, "tensor": 2}[a.path])
     Xn = wl.make_points(N, g, 1)
     X = torch.from_numpy(Xn.view(np.int16)).cuda().view(torch.float16)

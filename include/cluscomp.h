@@ -350,10 +350,15 @@ cc_status cc_decode(cc_ctx* ctx, const uint16_t* C16, int K, int g, const uint16
  * CC_LAYOUT_PAPER_T) codes, each < K.  bias (may be NULL): d_out FP32.  y (out): M x d_out FP32
  * row-major.  The listing keeps every tensor in a 16-bit type; here the accumulator is handed out
  * unrounded.  Scratch: cc_linear_workspace_bytes(M, d_out, d_in) bytes of the context's workspace
- * (cc_set_workspace; partial sums where the in_features are split across thread blocks, the tiles of many tokens; sums are
- * added in a fixed order, so the result is the same on every call).
+ * (cc_set_workspace; partial sums where the in_features are split across thread blocks, the tiles of many tokens).  Sums are
+ * added in a fixed order, so the result is the same on every call with a workspace of the same size.
  * 1 <= M < 2^31 / d_out; x, C16, y 16-byte aligned. */
 size_t cc_linear_workspace_bytes(cc_ctx* ctx, int64_t M, int64_t d_out, int64_t d_in);
+/* The size with which the forward of such a layer can also take the kernel that looks the codes up coordinate by coordinate
+ * (up to 256 tokens, up to twice as fast; the sums come in another order): never less than cc_linear_workspace_bytes, with which
+ * every call runs, and the same where that kernel is not the faster one.  33 tokens, 11008 x 4096, g = 6, K = 65500: 20 MB instead
+ * of 14; 256 tokens, 8192 x 28672, g = 4, K = 16000: 252 MB instead of 149.  0 on bad arguments. */
+size_t cc_linear_workspace_bytes_preferred(cc_ctx* ctx, int64_t M, int64_t d_out, int64_t d_in, int g, int K);
 cc_status cc_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, const uint16_t* C16, int K, int g,
                             const uint16_t* idx, int64_t d_out, int64_t d_in, const float* bias, float* y,
                             void* stream);
@@ -369,7 +374,7 @@ cc_status cc_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, const uin
  * requests to L2 into shared-memory reads.  For a handful of tokens (M <= 4; M <= 2 when g > 8) a
  * kernel without the tensor core runs: table look-ups and FP32 multiply-adds, partial sums added in a
  * fixed order (the same bits on every call).  g even (2..16; other g: CC_ERR_UNSUPPORTED_G); a larger
- * codebook: CC_ERR_SHAPE; q 16-byte aligned; workspace as for cc_linear_forward.  Calls on one context
+ * codebook: CC_ERR_SHAPE; q 16-byte aligned; workspace (either size) as for cc_linear_forward.  Calls on one context
  * must not overlap on the device (they share the workspace and its counters). */
 cc_status cc_linear_forward_q4(cc_ctx* ctx, const uint16_t* x, int64_t M, const uint8_t* q, const float* scale, int K,
                                int g, const uint16_t* idx, int64_t d_out, int64_t d_in, const float* bias, float* y,

@@ -69,6 +69,7 @@ SIGNATURES = {
     "cc_finalize": (_i32, [_vp, _vp, _i64, _i32, _vp, _i32, _vp, _vp, _vp, _vp, _vp]),
     "cc_decode": (_i32, [_vp, _vp, _i32, _i32, _vp, _i64, _i64, _i32, _vp, _vp]),
     "cc_linear_workspace_bytes": (_sz, [_vp, _i64, _i64, _i64]),
+    "cc_linear_workspace_bytes_preferred": (_sz, [_vp, _i64, _i64, _i64, _i32, _i32]),
     "cc_linear_forward": (_i32, [_vp, _vp, _i64, _vp, _i32, _i32, _vp, _i64, _i64, _vp, _vp, _vp]),
     "cc_linear_forward_q4": (_i32, [_vp, _vp, _i64, _vp, _vp, _i32, _i32, _vp, _i64, _i64, _vp, _vp, _vp]),
     "cc_poll_status": (_i32, [_vp, _vp]),
@@ -372,6 +373,10 @@ def cc_decode(ctx, C16, K, g, idx, d_out, d_in, layout, W_hat, stream=None) -> N
 
 def cc_linear_workspace_bytes(ctx, M: int, d_out: int, d_in: int) -> int:
     return int(load().cc_linear_workspace_bytes(ctx._h, M, d_out, d_in))
+
+
+def cc_linear_workspace_bytes_preferred(ctx, M: int, d_out: int, d_in: int, g: int, K: int) -> int:
+    return int(load().cc_linear_workspace_bytes_preferred(ctx._h, M, d_out, d_in, g, K))
 
 
 def cc_linear_forward(ctx, x, M, C16, K, g, idx, d_out, d_in, bias, y, stream=None) -> None:

@@ -732,7 +732,12 @@ cc_status cc_decode(cc_ctx* ctx, const uint16_t* C16, int K, int g, const uint16
 
 size_t cc_linear_workspace_bytes(cc_ctx* ctx, int64_t M, int64_t d_out, int64_t d_in) {
     if (!ctx || M < 1 || d_out < 1 || d_in < 1 || M * d_out >= (int64_t)1 << 31 || d_in >= (int64_t)1 << 31) return 0;
-    return cc_linear_scratch_bytes_preferred(M, d_out, d_in, ctx->sm_count);
+    return cc_linear_scratch_bytes(M, d_out, d_in, ctx->sm_count);
+}
+
+size_t cc_linear_workspace_bytes_preferred(cc_ctx* ctx, int64_t M, int64_t d_out, int64_t d_in, int g, int K) {
+    if (!cc_linear_workspace_bytes(ctx, M, d_out, d_in) || g < 1 || g > 16 || K < 1 || K > 65536) return 0;
+    return cc_linear_scratch_bytes_preferred(M, d_out, d_in, ctx->sm_count, K, g);
 }
 
 cc_status cc_linear_forward(cc_ctx* ctx, const uint16_t* x, int64_t M, const uint16_t* C16, int K, int g,

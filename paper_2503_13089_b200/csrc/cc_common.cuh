@@ -236,7 +236,7 @@ constexpr size_t CC_LINEAR_SCRATCH_FROM = CC_STATUS_BYTES + (size_t)65536 * 32;
 
 // Compressed linear layer: y = x . decode(C16, idx)^T (+ bias).
 size_t cc_linear_scratch_bytes(int64_t M, int64_t d_out, int64_t d_in, int sm_count);             // what every call needs
-size_t cc_linear_scratch_bytes_preferred(int64_t M, int64_t d_out, int64_t d_in, int sm_count);   // what every way of a call needs
+size_t cc_linear_scratch_bytes_preferred(int64_t M, int64_t d_out, int64_t d_in, int sm_count, int K, int g);   // what the fastest way needs
 int cc_linear_q_table_max(void);
 // The same for many tokens (cc_linear_wide.cu): the weight is decoded once into tiles in the workspace.
 bool cc_linear_wide_applies(int64_t M, int64_t d_out, int64_t d_in, int splits, int sm_count);

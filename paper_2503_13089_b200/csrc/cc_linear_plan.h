@@ -1,5 +1,6 @@
-// Host-side plans of the layer forward (cc_linear.cu): the few-token kernel's launch, the place of the padded codebook.  No
-// CUDA in here: what a plan asks for can be checked against the kernels' limits without a device.
+// Host-side plans of the layer forward: the few-token kernel's launch, the tensor kernel's (both cc_linear.cu), the one by planes
+// (cc_linear_planes.cu), the place of the padded codebook.  No CUDA in here: what a plan asks for can be checked against the kernels'
+// limits without a device.
 #pragma once
 
 #include <stddef.h>
@@ -114,6 +115,15 @@ inline GemvPlan gemv_plan(int64_t d_in, int out_groups, int sm_count, int K, int
     return p;
 }
 
+// The plan with which the look-up kernel takes a call; .fits is false where it does not.
+inline GemvPlan gemv_for(int64_t M, int64_t d_out, int64_t d_in, int sm_count, int K, int g, bool quant, bool words) {
+    GemvPlan p = {};
+    if (!gemv_applies(M, K, g, quant)) return p;
+    p = gemv_plan(d_in, (int)((d_out + g - 1) / g), sm_count, K, g, gemv_pad(M), quant, words);
+    p.fits = p.fits && p.pays;
+    return p;
+}
+
 // Slabs of partial sums that any plan of such a layer may write: three CTAs per SM at the most, or as many splits as x asks
 // for.  The most come with the fewest blocks of code groups, i.e. at g = 16.
 inline int64_t gemv_slabs_most(int64_t d_out, int64_t d_in, int sm_count) {
@@ -128,6 +138,81 @@ inline int64_t gemv_slabs_most(int64_t d_out, int64_t d_in, int sm_count) {
 inline size_t padded_table_at(uintptr_t ws, size_t from, size_t to, int K, int pad) {
     const size_t at = ((ws + from + 31) & ~(uintptr_t)31) - ws;
     return at + (size_t)K * pad * 2 <= to ? at : 0;
+}
+
+// ---- The tensor kernel.
+constexpr int LM = 128;                 // out_features per CTA = MMA M = TMEM lanes
+constexpr int LKB = 64;                 // in_features per pipeline stage
+constexpr int LSTAGES = 4;              // at most; two where the 4-bit table leaves room for no more wide tiles
+constexpr int LPROD = 512;              // producer threads (16 warps); warps 0..3 also run the epilogue
+constexpr int LTHREADS = LPROD + 32;    // + the MMA warp
+constexpr int LNT_MAX = 256;            // tokens per CTA = MMA N
+// Operand tiles in shared memory: the K-major no-swizzle layout of 8 x 16-byte core matrices, with the two
+// strides of the descriptor chosen against bank conflicts of the producers' 16-byte stores.  Neighbouring
+// lanes of an A-tile store hold neighbouring code groups, i.e. rows g apart in one column of core matrices:
+// 144 instead of 128 bytes between 8-row groups puts row r at 16-byte slot 9 (r / 8) + r % 8, and the eight
+// lanes of a store phase then fall into eight different slots mod 8 for g = 2, 4, 8 (two by two for g = 16;
+// at 128 bytes they all shared one or two).  Neighbouring lanes of a B-tile store hold neighbouring
+// 8-column pieces of one token's row: 16 bytes more between the columns of core matrices does the same.
+// Measured (4096 x 4096, g 4, K 65536): the B stride alone 0.772 -> 0.585 ms at 4096 tokens, 64 -> 50 us at
+// 256; the A stride on top 35.7 -> 33.6 us at 64 tokens (87 -> 64 us at g = 8 on 8192 x 8192, 16 tokens) but
+// 0.585 -> 0.807 ms at 4096 tokens, where the MMA's own reads of the wider-spaced A tile come to matter:
+// the A tile is widened for token blocks of at most 64 only, and never beside the 4-bit table (no room).
+CC_PLAN_FN constexpr int a_sbo(bool pad) { return pad ? 144 : 128; }
+CC_PLAN_FN constexpr int a_lbo(bool pad) { return (LM / 8) * a_sbo(pad); }
+CC_PLAN_FN constexpr int a_stage(bool pad) { return (LKB / 8) * a_lbo(pad); }   // bytes
+CC_PLAN_FN constexpr int b_lbo(int nt) { return nt * 16 + 16; }
+CC_PLAN_FN constexpr int b_stage_bytes(int nt) { return (LKB / 8) * b_lbo(nt); }
+// Quantised codebook (4 bits per value, two values per byte, low nibble first; Section 5.3): the whole
+// table sits in shared memory, and a 256-entry table turns a byte into its two dequantised FP16 values.
+constexpr int LQ_TABLE_MAX = 128 * 1024;   // bytes of packed codebook that fit beside the stages
+constexpr int LQ_BULK_PIECE = 32 * 1024;   // bytes per bulk copy of the table
+constexpr int LQ_WIDE_FROM = 256;
+constexpr int LQ_NT_MAX = 64;              // tokens per CTA when the table takes most of the shared memory
+
+constexpr int LINEAR_SPLITS_MORE = 8;   // splits beyond those that fill the SMs once are tried up to this many
+
+struct LinearPlan { int NT, a_pad, stages, tmem_cols, o_tiles, tok_blocks, splits, chunks_per_split, fill; size_t smem; };   // fill: splits that fill the SMs once
+
+// nt_max: tokens per CTA (256, or 64 with a quantised codebook in shared memory); table_bytes: that codebook.
+inline LinearPlan linear_plan(int64_t M, int64_t d_out, int64_t d_in, int sm_count, int nt_max = LNT_MAX, size_t table_bytes = 0,
+                       int g = 4) {
+    LinearPlan p;
+    const int64_t mt = M < nt_max ? M : nt_max;
+    p.NT = (int)((mt + 15) / 16 * 16);
+    // FP16 codebook with rows of at most 8 bytes, many tokens (of a layer too narrow for cc_linear_wide.cu, which the figures here
+    // were taken before): the gathers of the weight tile bound a stage, so
+    // one tile serves 512 tokens (two MMAs of 256 columns, all 512 TMEM columns) and the pipeline has two stages
+    // of that size: 4096 x 4096, g 4, 4096 tokens 0.571 -> 0.464 ms.  With 16-byte rows (g = 8) there are half as
+    // many gathers per weight and the coarser grid costs more than the reuse saves (1.62 -> 1.70 ms on 8192 x 8192).
+    const bool wide = table_bytes == 0 && nt_max == LNT_MAX && M >= 2 * LNT_MAX && g <= 4;
+    if (wide) p.NT = 2 * LNT_MAX;
+    p.tmem_cols = 32;
+    while (p.tmem_cols < p.NT) p.tmem_cols *= 2;
+    p.o_tiles = (int)((d_out + LM - 1) / LM);
+    p.tok_blocks = (int)((M + p.NT - 1) / p.NT);
+    const int chunks = (int)((d_in + LKB - 1) / LKB);
+    int splits = sm_count / (p.o_tiles * p.tok_blocks);             // fill the SMs when there are few tiles
+    if (splits > chunks / 4) splits = chunks / 4;                   // at least four stages of work per CTA
+    if (splits < 1) splits = 1;
+    p.fill = splits;
+    // More splits where the last wave would leave most SMs idle (86 tiles on 148 SMs: five splits make 2.9 waves of a
+    // fifth each; 33 tokens, 11008 x 4096, g = 6: 80 -> 62 us): clocks of a wave count as its stages, two stages' worth of
+    // setting up, and the slabs' traffic.  A stage is 8192 / g gathers at 0.73 a clock.
+    const double stage_clk = 8192.0 / g / 0.73 + 4.0 * p.NT, slab_clk = (double)M * (double)d_out * 8.0 / 2000.0;
+    double least = 0.0;
+    const int most = chunks / 4 < LINEAR_SPLITS_MORE ? chunks / 4 : LINEAR_SPLITS_MORE;
+    for (int cand = splits; cand <= most || cand == splits; ++cand) {
+        const int cps = (chunks + cand - 1) / cand, real = (chunks + cps - 1) / cps;
+        const int64_t ctas = (int64_t)p.o_tiles * p.tok_blocks * real;
+        const double t = (double)((ctas + sm_count - 1) / sm_count) * (cps + 2) * stage_clk + (real > 1 ? 4000.0 + real * slab_clk : 0.0);
+        if (cand == splits || t < 0.95 * least) { least = t; p.splits = real; p.chunks_per_split = cps; }
+    }
+    p.a_pad = (table_bytes == 0 && p.NT <= 64) ? 1 : 0;
+    p.stages = (wide || (table_bytes != 0 && p.NT > LQ_NT_MAX)) ? 2 : LSTAGES;
+    p.smem = (size_t)p.stages * (a_stage(p.a_pad) + (size_t)b_stage_bytes(p.NT)) + 256;
+    if (table_bytes) p.smem += 1024 + (table_bytes + 15) / 16 * 16;
+    return p;
 }
 
 // ---- Layer forward plane by plane.
@@ -221,18 +306,21 @@ inline bool planes_pay(const PlanesPlan& p, int64_t M, int64_t d_out, int64_t d_
     return !(quant && M > 192) && !(M > 128 && codes < 200000);
 }
 
-// At least the scratch of any such plan for this g, whatever the codebook's size.
-inline size_t planes_bytes_most(int64_t M, int64_t d_out, int64_t d_in, int g, int chain) {
-    const int64_t chunks = (d_in + PL_KB - 1) / PL_KB, out_groups = (d_out + g - 1) / g, NT = (M + 15) / 16 * 16;
-    const int64_t least = (chunks + chain - 1) / chain;
-    size_t most = 0;
-    for (int PP = 1; PP <= 4; PP *= 2) {
-        const int64_t tiles = (out_groups + PL_ROWS / PP - 1) / (PL_ROWS / PP) * ((g + PP - 1) / PP);
-        const size_t one = (size_t)tiles * NT * PL_ROWS * 4, lo = one * least, hi = one * PL_SPLITS_MAX;
-        const size_t cut = hi < PL_SLABS_MOST ? hi : PL_SLABS_MOST, b = lo > cut ? lo : cut;
-        if (b > most) most = b;
-    }
-    return most + (size_t)NT * chunks * (PL_KB * 2);
+// Stages of 64 in_features that the planes' kernel may add up in one accumulator: no longer a chain than the tensor
+// kernel would have had (its splits), and at most 16.
+constexpr int PLANES_CHAIN_MOST = 16;
+inline int planes_chain(int64_t M, int64_t d_out, int64_t d_in, int sm_count, int g) {
+    const LinearPlan p = linear_plan(M, d_out, d_in, sm_count, LNT_MAX, 0, g);
+    return p.chunks_per_split < PLANES_CHAIN_MOST ? p.chunks_per_split : PLANES_CHAIN_MOST;
+}
+
+// The plan with which the planes take a call that the look-up kernel does not; .fits is false where they do not.
+inline PlanesPlan planes_for(int64_t M, int64_t d_out, int64_t d_in, int sm_count, int K, int g, bool quant) {
+    PlanesPlan p = {};
+    if (M > PL_NT_MAX) return p;
+    p = planes_plan(M, d_out, d_in, sm_count, K, g, planes_chain(M, d_out, d_in, sm_count, g));
+    p.fits = p.fits && planes_pay(p, M, d_out, d_in, g, quant);
+    return p;
 }
 
 }  // namespace

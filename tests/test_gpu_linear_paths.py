@@ -38,7 +38,7 @@ def _run(x, C16, idx, d_out, d_in, bias, q4=False, off=0):
     from tests import gpu_util as u
     M, (K, g) = x.shape[0], C16.shape
     c = u.ctx()
-    c.ensure_workspace(len(idx), g, K, at_least=cc.cc_linear_workspace_bytes(c, M, d_out, d_in))
+    c.ensure_workspace(len(idx), g, K, at_least=cc.cc_linear_workspace_bytes_preferred(c, M, d_out, d_in, g, K))
     room = torch.full((off + K * g,), float("nan"), dtype=torch.float16, device="cuda")
     room[off:] = torch.from_numpy(C16.reshape(-1)).cuda()
     book, codes, y = room[off:], u.dev(idx.view(np.int16)).view(torch.uint16), torch.full((M, d_out), float("nan"), device="cuda")
