@@ -4,6 +4,7 @@ import pytest
 import torch
 
 from tests.test_gpu_linear_paths import _case, _run, _want
+from tests.test_planes_plan import LAYERS
 
 pytestmark = pytest.mark.gpu
 
@@ -25,6 +26,11 @@ def test_linear_planes(M, d_out, d_in, g, K, q4):
     assert np.all(np.abs(y - want) <= bound), float(np.max(np.abs(y - want) / bound))
     y2, _ = _run(x, C16, idx, d_out, d_in, bias, q4)
     assert np.array_equal(y.view(np.uint32), y2.view(np.uint32))
+
+
+@pytest.mark.parametrize("M,d_out,d_in,g,K,q4", [layer for layer, _ in LAYERS])
+def test_linear_planes_where_they_are_taken(M, d_out, d_in, g, K, q4):
+    test_linear_planes(M, d_out, d_in, g, K, q4)
 
 
 @pytest.mark.parametrize("M,d_out,d_in,g,K", [

@@ -1,7 +1,21 @@
 """The planes' layer forward (cc_linear_planes.cu): its launch plans, walked on the host.  No plan may ask for more shared memory or
-tensor memory than there is, longer chains than allowed, or blocks without work."""
+tensor memory than there is, longer chains than allowed, or blocks without work; the layers that the GPU tests give it are layers it takes."""
 import os
 import subprocess
+
+# M, d_out, d_in, g, K, 4-bit codebook: layers for the planes; coordinates a look-up and stages that their plans have on 148 SMs.
+LAYERS = [
+    ((65, 3134, 640, 1, 65536, False), (1, 2)), ((200, 4100, 2100, 4, 65536, False), (1, 2)), ((256, 8192, 1280, 4, 65536, False), (1, 2)),
+    ((33, 10000, 1300, 6, 65500, False), (1, 4)), ((48, 14000, 1100, 7, 65536, False), (1, 4)),
+    ((128, 208, 257, 8, 26294, False), (2, 2)), ((129, 793, 523, 2, 25467, False), (2, 2)), ((256, 2050, 1030, 8, 32768, False), (2, 2)),
+    ((70, 1030, 1200, 8, 32768, True), (2, 2)), ((192, 1030, 1200, 4, 16384, True), (2, 4)), ((12, 903, 1300, 9, 3000, False), (2, 4)),
+    ((129, 453, 895, 2, 968, False), (2, 4)), ((60, 1030, 1025, 2, 20000, False), (2, 4)),
+    # the last whole stage is the first of a block of the grid, in_features end behind it
+    ((26, 1085, 4491, 16, 19780, False), (4, 2)), ((91, 260, 2380, 16, 17185, False), (4, 2)),
+    ((200, 442, 1541, 3, 8220, False), (4, 2)), ((255, 446, 1345, 3, 7016, False), (4, 2)), ((192, 568, 1920, 4, 8753, True), (4, 2)),
+    ((16, 514, 1000, 4, 300, False), (4, 4)), ((128, 777, 900, 4, 3000, False), (4, 4)), ((129, 737, 1088, 4, 858, True), (4, 4)),
+    ((6, 207, 64, 16, 22, False), (4, 4)),
+]
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2503_13089_b200", "csrc")
 
@@ -44,6 +58,28 @@ int main() {
 def test_no_plan_of_the_planes_exceeds_its_limits(tmp_path):
     src, exe = tmp_path / "walk.cpp", tmp_path / "walk"
     src.write_text(WALK)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    out = subprocess.run([str(exe)], stdout=subprocess.PIPE, text=True)
+    assert out.returncode == 0, out.stdout
+
+
+def test_the_layers_of_the_gpu_tests_take_the_planes(tmp_path):
+    rows = "\n".join("    {%s}," % ", ".join(str(int(v)) for v in layer + plan) for layer, plan in LAYERS)
+    src, exe = tmp_path / "layers.cpp", tmp_path / "layers"
+    src.write_text("#include <cstdio>\n#include \"cc_linear_plan.h\"\nstatic const int L[][8] = {\n%s\n};\n" % rows + r"""
+int main() {
+    int bad = 0;
+    for (const auto& l : L)
+        for (int words = 0; words < 2; ++words) {
+            const PlanesPlan p = planes_for(l[0], l[1], l[2], 148, l[4], l[3], l[5]);
+            if (!p.fits || p.PP != l[6] || p.stages != l[7] || gemv_for(l[0], l[1], l[2], 148, l[4], l[3], l[5], words).fits) {
+                printf("M=%d %dx%d g=%d K=%d q4=%d: fits %d, PP %d, stages %d\n", l[0], l[1], l[2], l[3], l[4], l[5], p.fits, p.PP, p.stages);
+                ++bad;
+            }
+        }
+    return bad != 0;
+}
+""")
     subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
     out = subprocess.run([str(exe)], stdout=subprocess.PIPE, text=True)
     assert out.returncode == 0, out.stdout
