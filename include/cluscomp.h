@@ -196,16 +196,16 @@ cc_status cc_tensor_scores(cc_ctx* ctx, const uint16_t* X, int64_t N, int g, con
 cc_status cc_tensor_finish_only(cc_ctx* ctx, const uint16_t* X, int64_t N, int g, const float* C, int K,
                                 const void* scan, uint16_t* idx, float* dist, void* stream);
 
-/* Self-test of the bounded waits of the tensor-core E-step (no counterpart in the paper).  Every
- * wait of those kernels on a shared-memory barrier gives up after a clock limit, raises a flag that
+/* Self-test of the bounded waits of the tensor-core E-step and of the small fit (no counterpart in the paper).
+ * Every wait of the former's kernels on a shared-memory barrier gives up after a clock limit, raises a flag that
  * makes the CTA's other waits return, and the kernel then reports CC_ERR_DEVICE_TIMEOUT through
- * cc_poll_status instead of hanging.  This call runs one warp through that wait code with the
- * given limit (1e3 .. 4e9 clock cycles) and copies to the HOST arrays:
- *   results[0] = 1: a wait on a barrier whose phase completes succeeds;
- *   results[1] = 0: a wait on a barrier nobody arrives on gives up;
+ * cc_poll_status instead of hanging; the latter's blocks wait for counters in memory, with the same end.  This call runs
+ * one warp through that wait code with the given limit (1e3 .. 4e9 clock cycles) and copies to the HOST arrays:
+ *   results[0] = 1: a wait on a barrier whose phase completes, and one on a counter that has arrived, succeed;
+ *   results[1] = 0: a wait on a barrier nobody arrives on, and one on a counter nobody raises, give up after the limit;
  *   results[2] = 1: the abort flag is up afterwards;
- *   results[3] = 0: a further wait returns unsuccessfully;
- *   cycles[0], cycles[1]: how long the second and third wait took (the second a little more than
+ *   results[3] = 0: a further wait on the barrier returns unsuccessfully;
+ *   cycles[0], cycles[1]: how long the second (the longer of the two) and third wait took (the second a little more than
  *   the limit, the third far less).
  * Synchronous; allocates and frees 64 bytes of device memory. */
 cc_status cc_selftest_bounded_wait(cc_ctx* ctx, int64_t limit_cycles, int32_t* results, int64_t* cycles);
@@ -380,7 +380,8 @@ cc_status cc_linear_forward_q4(cc_ctx* ctx, const uint16_t* x, int64_t M, const 
                                int g, const uint16_t* idx, int64_t d_out, int64_t d_in, const float* bias, float* y,
                                void* stream);
 
-/* Waits for `stream`, reads the device status word and clears it.  Returns CC_OK,
+/* Waits for `stream`, reads the device status word and clears it (after a time-out also the counters that a kernel which gave
+ * up may have left behind, so that the next call starts as after cc_set_workspace).  Returns CC_OK,
  * CC_ERR_NONFINITE, CC_ERR_DEVICE_TIMEOUT or CC_ERR_CUDA. */
 cc_status cc_poll_status(cc_ctx* ctx, void* stream);
 

@@ -531,13 +531,17 @@ cc_status cc_selftest_bounded_wait(cc_ctx* ctx, int64_t limit_cycles, int32_t* r
     int* out_dev = static_cast<int*>(dev);
     long long* cyc_dev = reinterpret_cast<long long*>(static_cast<char*>(dev) + 16);
     cc_status st = CC_OK;
-    long long cyc[2] = {0, 0};
+    struct { int32_t out[4]; long long cyc[2], gate_cyc; int32_t gate_out[2]; unsigned gates[2]; } got = {};
+    static_assert(sizeof(got) <= 64, "fits the device buffer");
     if (cudaMemset(dev, 0, 64) != cudaSuccess || cc_launch_wait_selftest(limit_cycles, out_dev, cyc_dev, 0) != cudaSuccess ||
-        cudaMemcpy(results, out_dev, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost) != cudaSuccess ||
-        cudaMemcpy(cyc, cyc_dev, sizeof(cyc), cudaMemcpyDeviceToHost) != cudaSuccess)
+        cc_launch_gate_selftest(reinterpret_cast<unsigned*>(out_dev + 12), limit_cycles, out_dev + 10, cyc_dev + 2, 0) != cudaSuccess ||
+        cudaMemcpy(&got, dev, sizeof(got), cudaMemcpyDeviceToHost) != cudaSuccess)
         st = CC_ERR_CUDA;
-    cycles[0] = cyc[0];
-    cycles[1] = cyc[1];
+    for (int i = 0; i < 4; ++i) results[i] = got.out[i];
+    results[0] = got.out[0] && got.gate_out[0];
+    results[1] = got.out[1] || got.gate_out[1] || got.cyc[0] <= limit_cycles || got.gate_cyc <= limit_cycles;
+    cycles[0] = got.cyc[0] > got.gate_cyc ? got.cyc[0] : got.gate_cyc;
+    cycles[1] = got.cyc[1];
     cudaFree(dev);
     return st;
 }
@@ -779,6 +783,9 @@ cc_status cc_poll_status(cc_ctx* ctx, void* stream) {
     if (cudaMemcpyAsync(&word, ctx->ws, sizeof(word), cudaMemcpyDeviceToHost, st) != cudaSuccess) return CC_ERR_CUDA;
     if (cudaMemsetAsync(ctx->ws, 0, sizeof(word), st) != cudaSuccess) return CC_ERR_CUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return CC_ERR_CUDA;
+    // what gave up may have left counters behind that the next call takes to be zero
+    if ((word & CC_DEV_TIMEOUT) && (cudaMemsetAsync(ctx->ws, 0, CC_STATUS_BYTES, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess))
+        return CC_ERR_CUDA;
     return status_of(word);
 }
 

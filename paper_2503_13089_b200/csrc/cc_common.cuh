@@ -87,13 +87,14 @@ cudaError_t launch_after(dim3 grid, dim3 block, size_t smem, cudaStream_t st, vo
 
 // Status block at the start of every workspace: cleared by cc_set_workspace.
 constexpr size_t CC_STATUS_BYTES = 4096;
-constexpr int CC_ARRIVAL_WORD = 64, CC_ARRIVAL_COUNTERS = 960;
+constexpr int CC_ARRIVAL_WORD = 64, CC_ARRIVAL_COUNTERS = 960, CC_GATE_WORD = 56;
 
 // Carving of the workspace for a problem (N, g, K).  All offsets 256-byte aligned.
 struct WsLayout {
     size_t status;     // CC_STATUS_BYTES: 1024 x u32: [0] status bits, [2..3] flagged counter (u64), [8] last-block counter of the objective
                        // sum, [32..35] tensor-path parameters, [36] codebook quantiser's maximum, [40] largest distance, [41] a counter,
-                       // [48..53] exact objective sum (zero between calls), [64..1023] arrival
+                       // [48..53] exact objective sum, [56..57] the counters at which the blocks of a small
+                       // fit meet (both zero between calls), [64..1023] arrival
                        // counters of the layer forward's split reduction (zero between calls)
     size_t cprep;      // staged codebook for the FFMA E-step
     size_t flagged;    // u32 list of points sent to the exact stage
@@ -193,6 +194,7 @@ cudaError_t cc_launch_assign_tensor(cc_ctx*, const WsLayout&, const uint16_t* X,
                                     cudaStream_t);
 // Verification aid: every comparison score of the tensor-core scan, N x cc_tensor_score_ld(K) floats.
 int cc_tensor_score_ld(int K);
+cudaError_t cc_launch_gate_selftest(unsigned* gates_dev, long long limit_cycles, int* out_dev, long long* cycles_dev, cudaStream_t);
 cudaError_t cc_launch_wait_selftest(long long limit_cycles, int* out_dev, long long* cycles_dev, cudaStream_t);
 cudaError_t cc_launch_tensor_scores(cc_ctx*, const WsLayout&, const uint16_t* X, int64_t N, int g, const float* C,
                                     int K, float* scores, cudaStream_t);

@@ -50,33 +50,47 @@ __device__ __forceinline__ double exact_distance(const float (&x)[G], const ull*
     return d;
 }
 
-// mode: SMALL_E (E-step alone), SMALL_FIRST (and all points added to the sums, which are zero), SMALL_NEXT (and the points
-// whose code changed moved; idx holds the codes that the sums correspond to).
-// flagged: list of the points with more than one candidate, counted in status words 2..3 (or nullptr).
 // Thread 0's wait until a counter has reached `target`; false if that takes too long (about 2 s).
 constexpr long long SM_WAIT_LIMIT = 4000000000LL;
-__device__ __forceinline__ bool gate_reached(const unsigned* gate, unsigned target) {
+__device__ __forceinline__ bool gate_reached(const unsigned* gate, unsigned target, long long limit = SM_WAIT_LIMIT) {
     const long long t0 = clock64();
     for (;;) {
         unsigned v;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(gate) : "memory");
         if (v >= target) return true;
-        if (clock64() - t0 > SM_WAIT_LIMIT) return false;
+        if (clock64() - t0 > limit) return false;
     }
 }
 __device__ __forceinline__ void gate_arrive(unsigned* gate) { asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(gate) : "memory"); }
 
+// Self-test of that wait: on a counter that has arrived and on one that never will.  out: {result of the first, of the second};
+// cycles: duration of the second.
+__global__ void __launch_bounds__(32)
+gate_selftest_kernel(unsigned* gates, long long limit, int* __restrict__ out, long long* __restrict__ cycles) {
+    if (threadIdx.x != 0) return;
+    gate_arrive(gates);
+    out[0] = gate_reached(gates, 1u, limit);
+    const long long t0 = clock64();
+    out[1] = gate_reached(gates + 1, 1u, limit);
+    *cycles = clock64() - t0;
+}
+
+// mode: SMALL_E (E-step alone), SMALL_FIRST (and all points added to the sums, which are zero), SMALL_NEXT (and the points
+// whose code changed moved; idx holds the codes that the sums correspond to).
+// flagged: list of the points with more than one candidate, counted in status words 2..3 (or nullptr).
+// LOOP: gates are two counters, zero at the launch and left so: blocks through with their additions, and with reading the sums.  A launch that
+// gives up leaves them as they are, since other blocks may still arrive; whoever reads its time-out clears them (cc_poll_status).
 template <int G, bool LOOP>
 __global__ void __launch_bounds__(SM_THREADS)
 small_kernel(const uint16_t* __restrict__ X, int64_t N, float* C, int K, int mode, uint16_t* idx, float* __restrict__ dist,
              ull* __restrict__ sum_lo, ull* __restrict__ sum_hi, int* __restrict__ counts, int with_means,
              double* __restrict__ partials, double* __restrict__ objective, unsigned* __restrict__ status,
-             unsigned* __restrict__ flagged, int64_t* __restrict__ n_flagged, int iters) {
+             unsigned* __restrict__ flagged, int64_t* __restrict__ n_flagged, int iters, unsigned* __restrict__ gates) {
     constexpr int GP = (G + 1) / 2;
     extern __shared__ __align__(16) ull sm_c[];      // K rounded up to whole chunks, GP pairs of -c each
     __shared__ double sh[SM_THREADS / 32];
     __shared__ bool last;
-    unsigned* met = status + CC_ARRIVAL_WORD, *read_up = met + 1;    // LOOP: blocks through with their additions; with reading the sums
+    unsigned* met = gates, *read_up = gates + 1;
     const int tid = threadIdx.x, lane = tid & 31, k = tid & (SM_LPP - 1);
     const int n_chunks = (K + SM_CHUNK - 1) / SM_CHUNK;
     for (int e = tid; e < n_chunks * SM_CHUNK * GP; e += SM_THREADS) {
@@ -106,7 +120,7 @@ small_kernel(const uint16_t* __restrict__ X, int64_t N, float* C, int K, int mod
     int it = 0;
     bool gated = false;                                 // the gate before this iteration's additions has been passed
     auto give_up = [&]() {
-        if (tid == 0) { atomicOr(status, CC_DEV_TIMEOUT); *met = 0u; *read_up = 0u; }
+        if (tid == 0) atomicOr(status, CC_DEV_TIMEOUT);
     };
     for (;;) {                                          // LOOP: iterations
     for (int64_t base = ((int64_t)blockIdx.x * SM_GROUPS + tid / SM_LPP) * SM_P; base - (tid / SM_LPP) * SM_P < N; base += step) {
@@ -340,7 +354,7 @@ cudaError_t launch_small(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int6
     }
     char* ws = static_cast<char*>(ctx->ws);
     int64_t blocks = (N + SM_GROUPS * SM_P - 1) / (SM_GROUPS * SM_P);
-    const int64_t cap = ctx->sm_count;                  // at most CC_OBJ_BLOCKS partial sums
+    const int64_t cap = ctx->sm_count < CC_OBJ_BLOCKS ? ctx->sm_count : CC_OBJ_BLOCKS;      // a partial sum each
     if (blocks > cap) blocks = cap;
     if (n_flagged) {
         const cudaError_t e = cudaMemsetAsync(ws + L.status + 8, 0, 8, st);
@@ -364,10 +378,10 @@ cudaError_t launch_small(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int6
         cfg.attrs = &at;
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, small_kernel<G, true>, X, N, C, K, mode, idx, dist, sum_lo, sum_hi, (int*)counts, (int)means, partials, objective,
-                                  status, flagged, n_flagged, iters);
+                                  status, flagged, n_flagged, iters, status + CC_GATE_WORD);
     }
     small_kernel<G, false><<<(unsigned)blocks, SM_THREADS, small_smem<G>(K), st>>>(
-        X, N, C, K, mode, idx, dist, sum_lo, sum_hi, counts, means, partials, objective, status, flagged, n_flagged, 1);
+        X, N, C, K, mode, idx, dist, sum_lo, sum_hi, counts, means, partials, objective, status, flagged, n_flagged, 1, nullptr);
     return cudaGetLastError();
 }
 
@@ -426,4 +440,9 @@ cudaError_t cc_launch_small_loop(cc_ctx* ctx, const WsLayout& L, const uint16_t*
     }
 #undef CALL
     return e;
+}
+
+cudaError_t cc_launch_gate_selftest(unsigned* gates_dev, long long limit, int* out_dev, long long* cycles_dev, cudaStream_t st) {
+    gate_selftest_kernel<<<1, 32, 0, st>>>(gates_dev, limit, out_dev, cycles_dev);
+    return cudaGetLastError();
 }
