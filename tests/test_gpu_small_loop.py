@@ -71,3 +71,32 @@ def test_small_fit_whatever_the_workspace_holds_and_after_a_time_out():
     cc.cc_poll_status(c)
     assert _fit(c, X, C0, iters) == want
     c.close()
+
+
+def test_small_fit_where_the_cooperative_launch_is_refused():
+    """With more blocks than the device holds at once (a context that takes it to have 5000 SMs) the launch of all iterations is
+    refused; the fit then runs one launch an iteration.  Codes, centroids, counts and distances are the same bits; the objective is
+    summed over other blocks (float64, 3 10^5 positive terms: relative difference below 10^-10)."""
+    import ctypes as ct
+    from paper_2503_13089_b200 import binding as cc
+    from tests import gpu_util as u
+    N, g, K, iters = 300000, 4, 8, 4
+    rng = np.random.default_rng(23)
+    X = u.half_dev(rng.standard_t(3.0, (N, g)).astype(np.float16))
+    c = cc.Context(0)
+    c.ensure_workspace(N, g, K)
+    C0 = torch.empty((K, g), device="cuda")
+    cc.cc_init_codebook(c, X, N, g, K, 5, C0)
+    want = _fit(c, X, C0, iters)
+    n0 = cc.cc_launch_count(c)
+    _fit(c, X, C0, iters)
+    assert cc.cc_launch_count(c) - n0 == 1
+    fields = (ct.c_int * 2).from_address(c._h.value)     # cc_ctx begins with the device and its number of SMs
+    assert fields[0] == 0 and fields[1] == torch.cuda.get_device_properties(0).multi_processor_count
+    fields[1] = 5000
+    n0 = cc.cc_launch_count(c)
+    got = _fit(c, X, C0, iters)
+    assert cc.cc_launch_count(c) - n0 == iters
+    assert got[:4] == want[:4]
+    assert np.allclose(np.frombuffer(got[4]), np.frombuffer(want[4]), rtol=1e-10, atol=0.0)
+    c.close()
