@@ -295,7 +295,7 @@ cudaError_t fit_small(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t
     char* ws = static_cast<char*>(ctx->ws);
     cudaError_t e = cudaMemsetAsync(ws + L.sum_lo, 0, L.sum_hi - L.sum_lo + sizeof(int64_t) * (size_t)K * g, st);   // both sums
     if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, sizeof(int32_t) * (size_t)K, st);
-    if (e == cudaSuccess && iters > 1 && cc_small_loop_applies(ctx, g, K)) {
+    if (e == cudaSuccess && iters > 1 && cc_small_loop_applies(ctx, N, g, K)) {
         e = cc_launch_small_loop(ctx, L, X, N, g, C, K, iters, idx, dist, counts, objective_trace, st);
         // refused where this process may use fewer SMs than the device has: nothing has run, and a launch an iteration needs no SM in particular
         if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported) return e;

@@ -229,7 +229,7 @@ bool cc_small_applies(const cc_ctx*, int64_t N, int g, int K);
 bool cc_small_fit_applies(const cc_ctx*, int64_t N, int g, int K);   // whole iterations
 cudaError_t cc_launch_small(cc_ctx*, const WsLayout&, const uint16_t* X, int64_t N, int g, float* C, int K, int mode, uint16_t* idx,
                             float* dist, int32_t* counts, double* objective, int64_t* n_flagged, cudaStream_t);
-bool cc_small_loop_applies(const cc_ctx*, int g, int K);                                   // all iterations in one launch
+bool cc_small_loop_applies(const cc_ctx*, int64_t N, int g, int K);                        // all iterations in one launch
 cudaError_t cc_launch_small_loop(cc_ctx*, const WsLayout&, const uint16_t* X, int64_t N, int g, float* C, int K, int iters, uint16_t* idx,
                                  float* dist, int32_t* counts, double* objective_trace, cudaStream_t);
 

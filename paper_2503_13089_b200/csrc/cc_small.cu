@@ -425,7 +425,15 @@ cudaError_t cc_launch_small(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, i
 }
 
 // All iterations in one launch (the sums and counts are zero); cc_small_loop_applies says where.
-bool cc_small_loop_applies(const cc_ctx* ctx, int g, int K) { return K * g <= SM_MEANS && ctx->empty_rule == CC_EMPTY_KEEP; }
+// What it saves, about 2.5 us an iteration, is lost again where a block takes many steps of long sub-vectors (its registers keep the loop
+// over the iterations as well).  Ten iterations, launch an iteration / all in one, us: 32768 points, g = 4, K = 256 168 / 144; 30,000, K =
+// 1024 298 / 274; 300,000, K = 64 575 / 550; 4 M, K = 8 (five) 3965 / 3950; 12 M, K = 2 (five) 10048 / 10072; 800,000, g = 6, K = 8 2040 /
+// 2021; 200,000, g = 8, K = 128 501 / 480, 2 M, K = 4 (five) 3422 / 3504; 60,000, g = 16, K = 64 470 / 457, 100,000, K = 4 734 / 724, K = 64
+// 689 / 687, 200,000, K = 4 1123 / 1147, K = 64 1227 / 1296, 400,000, K = 16 1967 / 2079; g = 12, 50,000, K = 32 362 / 348, 200,000 969 / 998.
+constexpr int64_t SM_LOOP_VALUES = 2000000;
+bool cc_small_loop_applies(const cc_ctx* ctx, int64_t N, int g, int K) {
+    return K * g <= SM_MEANS && ctx->empty_rule == CC_EMPTY_KEEP && (g <= 6 || N * g <= SM_LOOP_VALUES);
+}
 
 cudaError_t cc_launch_small_loop(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, int g, float* C, int K, int iters, uint16_t* idx,
                                  float* dist, int32_t* counts, double* objective_trace, cudaStream_t st) {
