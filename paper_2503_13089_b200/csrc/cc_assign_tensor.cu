@@ -762,10 +762,16 @@ finish_tensor_kernel(const uint16_t* __restrict__ X, int64_t N, const float* __r
     }
 }
 
-// Winners chunk by chunk where 32 points meet few chunks.  E-step of 4.2 M points, a group of lanes per point / by chunk, in us:
-// g = 4, K = 256 640 / 614, K = 512 650 / 638, K = 1024 660 / 680; g = 6 821 / 759, 827 / 790, 860 / 850; g = 8 972 / 858, 1061 / 913, 1182 /
-// 1011; g = 16 1136 / 997, 1363 / 1166, 1490 / 1465, K = 2048 1740 / 1935.
-constexpr bool finish_by_chunk(int K, int g) { return K <= (g <= 4 ? 512 : 1024); }
+// Winners chunk by chunk where 32 points meet few chunks: up to so many centroids, by the length of the sub-vectors.  What a point reads
+// with a group of lanes for itself grows with that length, what it costs by chunk with the chunks that 32 points win in and with the registers
+// that two centroids take.  E-step of 4.2 M points (2.1 M from g = 9 on), a group of lanes per point / by chunk, in us:
+//   g = 1, K = 100 331 / 345; g = 2, K = 256 299 / 313; g = 3, K = 100 336 / 331, 256 340 / 342; g = 4, K = 256 384 / 361, 512 421 / 419, 768 468 / 485;
+//   g = 5, K = 512 470 / 455, 768 506 / 514; g = 6, K = 768 547 / 533, 1024 593 / 599; g = 7, K = 1024 644 / 640, 1536 740 / 774; g = 8, K = 1024
+//   724 / 714, 1536 832 / 868; g = 9, K = 768 364 / 348, 1024 388 / 388; g = 10, K = 1024 409 / 393, 1280 435 / 437; g = 11, K = 768 420 / 409, 1024
+//   436 / 448; g = 12, K = 1024 467 / 462, 1536 523 / 554; g = 13, K = 768 488 / 463, 1024 503 / 504; g = 14, K = 768 500 / 471, 1024 519 / 519;
+//   g = 15, K = 768 537 / 526, 1024 552 / 577; g = 16, K = 384 557 / 548, 512 562 / 572, 1024 626 / 697.
+constexpr int FINISH_CHUNK_MOST[17] = {0, 0, 0, 128, 512, 512, 768, 1024, 1024, 1024, 1024, 768, 1024, 768, 1024, 768, 384};
+constexpr bool finish_by_chunk(int K, int g) { return K <= FINISH_CHUNK_MOST[g]; }
 
 template <int G>
 cudaError_t launch_tensor(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int64_t N, const float* C, int K,
