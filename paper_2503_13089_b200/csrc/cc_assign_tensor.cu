@@ -850,10 +850,12 @@ cudaError_t launch_tensor(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, int
             int64_t fblocks = (N + 255) / 256;            // a warp takes 32 points per round
             const int64_t cap = (int64_t)ctx->sm_count * 32;
             if (fblocks > cap) fblocks = cap;
-            if (finish_by_chunk(K, G)) launch_after(dim3((unsigned)fblocks), dim3(256), 0, st, finish_tensor_kernel<G, true>,
-                     X, N, C, K, Kpad / TCHUNK, rescan, tstate, params, idx, dist, status, reinterpret_cast<unsigned*>(ws + L.flagged));
-            else launch_after(dim3((unsigned)fblocks), dim3(256), 0, st, finish_tensor_kernel<G, false>,
-                     X, N, C, K, Kpad / TCHUNK, rescan, tstate, params, idx, dist, status, reinterpret_cast<unsigned*>(ws + L.flagged));
+            unsigned* flagged = reinterpret_cast<unsigned*>(ws + L.flagged);
+            auto finish = finish_tensor_kernel<G, false>;
+            if constexpr (FINISH_CHUNK_MOST[G] > 0) {
+                if (finish_by_chunk(K, G)) finish = finish_tensor_kernel<G, true>;
+            }
+            launch_after(dim3((unsigned)fblocks), dim3(256), 0, st, finish, X, N, C, K, Kpad / TCHUNK, rescan, tstate, params, idx, dist, status, flagged);
         }
     }
     return cudaGetLastError();

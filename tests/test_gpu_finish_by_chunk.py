@@ -9,6 +9,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("N,g,K", [
     (1, 4, 1), (31, 4, 63), (33, 4, 64), (1000, 4, 65), (40000, 4, 512), (40000, 4, 513), (5003, 1, 200), (20000, 5, 1024), (20001, 8, 1000), (9999, 16, 257),
+    (5001, 3, 128), (5001, 3, 129), (5001, 2, 64), (7000, 13, 768), (7000, 15, 769), (9999, 16, 384), (9999, 16, 385),           # where the rule changes
 ])
 def test_finish_by_chunk(N, g, K):
     from paper_2503_13089_b200 import binding as cc
