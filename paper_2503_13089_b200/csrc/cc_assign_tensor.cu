@@ -109,57 +109,57 @@ __device__ __forceinline__ void load_halves(const uint16_t* __restrict__ row, un
 }
 
 // A operand rows [x repeated SPLIT times, 2^15, 2^6, 2^-3, 2^-12, 0..] of points base + e,
-// e = first, first + step, .. < count, into the tiles at sA (canonical layout, 16 bytes at a time).
-template <int G>
-__device__ __forceinline__ void build_a_rows(const uint16_t* __restrict__ X, int64_t N, int64_t base, int first,
-                                             int step, int count, unsigned char* sA, bool& nonfinite,
-                                             const TcParams* __restrict__ params) {
+// e = first, first + STEP, .. < count, into the tiles at sA (canonical layout, 16 bytes at a time).
+template <int G, int STEP>
+__device__ __forceinline__ void build_a_rows(const uint16_t* __restrict__ X, int64_t N, int64_t base, int first, int count,
+                                             unsigned char* sA, bool& nonfinite, const TcParams* __restrict__ params) {
     using Cfg = TcCfg<G>;
     constexpr int KD = Cfg::KD, SPLIT = Cfg::SPLIT, NQ = Cfg::NQ;
     int ne = 0;                                  // only the two-piece norm has call-dependent constants
     if constexpr (NQ == 2) ne = norm_exponent(scale_from_range(params->cmax_bits, params->qmax_bits), params->qmax_bits);
-    // Several loads under way per thread, unconditional so that none waits for another: in the persistent scan one warp builds
-    // the 1024 rows of a group, and with one point at a time the latencies of its loads (31,000 clocks a group) were the time of
+    // Where one warp builds the 1024 rows of a group (the persistent scan), several loads under way per thread, unconditional so that none waits for
+    // another: with one point at a time the latencies of its loads (31,000 clocks a group) were the time of
     // every scan over fewer than 3000 centroids: E-step of 4.2 M points, g = 4, K = 256 614 -> 374 us, K = 1024 680 -> 526; g = 8, K = 512
-    // 913 -> 577, K = 2048 1183 -> 952.
-    constexpr int W = (G + 1) / 2, BATCH = W > 4 ? 4 : 8;
-    for (int e0 = first; e0 < count; e0 += BATCH * step) {
+    // 913 -> 577, K = 2048 1183 -> 952.  Where a whole block does, a thread has two rows at the most (18,000 points, g = 4,
+    // K = 18000 65.9 us with eight loads a thread, six of them for nothing, 65.1 so; 75,000, K = 4096 51.4 and 50.9).
+    constexpr int W = (G + 1) / 2, BATCH = STEP > 32 ? 2 : W > 4 ? 4 : 8;
+    for (int e0 = first; e0 < count; e0 += BATCH * STEP) {
         unsigned xw[BATCH][W];
 #pragma unroll
         for (int b = 0; b < BATCH; ++b) {
-            const int64_t i = base + e0 + (int64_t)b * step;
+            const int64_t i = base + e0 + b * STEP;
             load_halves<G>(X + (i < N ? i : N - 1) * G, xw[b]);
         }
 #pragma unroll
         for (int b = 0; b < BATCH; ++b) {
-        const int e = e0 + b * step;
-        if (e >= count) break;
-        const bool live = base + e < N;
-        unsigned short h[KD];
+            const int e = e0 + b * STEP;
+            if (e >= count) break;
+            const bool live = base + e < N;
+            unsigned short h[KD];
 #pragma unroll
-        for (int t = 0; t < G; ++t) {
-            unsigned v = (t & 1) ? xw[b][t / 2] >> 16 : xw[b][t / 2] & 0xffffu;
-            if (!live) v = 0u;
-            if ((v & 0x7c00u) == 0x7c00u) nonfinite = true;
-            h[t] = (unsigned short)v;
-        }
+            for (int t = 0; t < G; ++t) {
+                unsigned v = (t & 1) ? xw[b][t / 2] >> 16 : xw[b][t / 2] & 0xffffu;
+                if (!live) v = 0u;
+                if ((v & 0x7c00u) == 0x7c00u) nonfinite = true;
+                h[t] = (unsigned short)v;
+            }
 #pragma unroll
-        for (int k = G; k < KD; ++k) {
-            h[k] = (k < SPLIT * G) ? h[k % G]
-                 : (k < SPLIT * G + NQ) ? __half_as_ushort(__float2half_rn(qconst<NQ>(k - SPLIT * G, ne)))
-                 : (unsigned short)0;
-        }
-        unsigned char* tile = sA + (e / TM) * Cfg::A_TILE;
-        const int r = e % TM;
+            for (int k = G; k < KD; ++k) {
+                h[k] = (k < SPLIT * G) ? h[k % G]
+                     : (k < SPLIT * G + NQ) ? __half_as_ushort(__float2half_rn(qconst<NQ>(k - SPLIT * G, ne)))
+                     : (unsigned short)0;
+            }
+            unsigned char* tile = sA + (e / TM) * Cfg::A_TILE;
+            const int r = e % TM;
 #pragma unroll
-        for (int kc = 0; kc < KD / 8; ++kc) {
-            uint4 w;
-            w.x = (unsigned)h[kc * 8 + 0] | ((unsigned)h[kc * 8 + 1] << 16);
-            w.y = (unsigned)h[kc * 8 + 2] | ((unsigned)h[kc * 8 + 3] << 16);
-            w.z = (unsigned)h[kc * 8 + 4] | ((unsigned)h[kc * 8 + 5] << 16);
-            w.w = (unsigned)h[kc * 8 + 6] | ((unsigned)h[kc * 8 + 7] << 16);
-            *reinterpret_cast<uint4*>(tile + canon_bytes(r, kc * 8, TM)) = w;
-        }
+            for (int kc = 0; kc < KD / 8; ++kc) {
+                uint4 w;
+                w.x = (unsigned)h[kc * 8 + 0] | ((unsigned)h[kc * 8 + 1] << 16);
+                w.y = (unsigned)h[kc * 8 + 2] | ((unsigned)h[kc * 8 + 3] << 16);
+                w.z = (unsigned)h[kc * 8 + 4] | ((unsigned)h[kc * 8 + 5] << 16);
+                w.w = (unsigned)h[kc * 8 + 6] | ((unsigned)h[kc * 8 + 7] << 16);
+                *reinterpret_cast<uint4*>(tile + canon_bytes(r, kc * 8, TM)) = w;
+            }
         }
     }
 }
@@ -207,7 +207,7 @@ assign_tensor_kernel(const uint16_t* __restrict__ X, int64_t N, const uint16_t* 
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     bool nonfinite = false;
-    build_a_rows<G>(X, N, base, tid, TC_THREADS, na * TM, sA, nonfinite, params);
+    build_a_rows<G, TC_THREADS>(X, N, base, tid, na * TM, sA, nonfinite, params);
     if (nonfinite) atomicOr(status, CC_DEV_NONFINITE);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> async proxy (MMA)
     if (warp == 0) {
@@ -434,7 +434,7 @@ assign_tensor_persistent_kernel(const uint16_t* __restrict__ X, int64_t N, const
     }
     // first group's A operand: built by everybody
     bool nonfinite = false;
-    build_a_rows<G>(X, N, (int64_t)blockIdx.x * (NA * TM), tid, PERSIST_THREADS, NA * TM, sA, nonfinite, params);
+    build_a_rows<G, PERSIST_THREADS>(X, N, (int64_t)blockIdx.x * (NA * TM), tid, NA * TM, sA, nonfinite, params);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes -> async proxy (MMA)
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -539,7 +539,7 @@ assign_tensor_persistent_kernel(const uint16_t* __restrict__ X, int64_t N, const
                 if (!ok) break;
             }
             const int64_t group = (int64_t)blockIdx.x + (int64_t)it * gridDim.x;
-            build_a_rows<G>(X, N, group * (NA * TM), lane, 32, NA * TM, sA + buf * A_SET, nonfinite, params);
+            build_a_rows<G, 32>(X, N, group * (NA * TM), lane, NA * TM, sA + buf * A_SET, nonfinite, params);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0)
