@@ -31,12 +31,6 @@ __device__ __forceinline__ ull pack2(float lo, float hi) {
 __device__ __forceinline__ void unpack2(ull v, float& lo, float& hi) {
     asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
 }
-// Two FP32 FMAs in one instruction (sm_100 packed form); each lane rounds like fma.rn.f32.
-__device__ __forceinline__ ull fma2(ull a, ull b, ull c) {
-    ull d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
 __device__ __forceinline__ float min3(float a, float b, float c) {
     float d;
     asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));

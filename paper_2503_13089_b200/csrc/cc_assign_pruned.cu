@@ -407,8 +407,8 @@ pruned_list_kernel(const ListArgs a) {
 // A pair costs nothing to a warp that needs neither of it: the MMA thread releases the accumulator in its stead.
 // Pairs are announced on a ring of barriers, and every warp looks at (waits for and releases) one pair in half a ring
 // at the least, which keeps it within one phase of every barrier, and a tile's last pair, after which the tile's
-// A rows are free.  A look that a warp does not need holds the accumulator up: one in sixteen instead of one in four (5.6 M
-// points, g = 8, K = 65536, twenty iterations 346 -> 341 ms).
+// A rows are free.  A look that a warp does not need holds the accumulator up: one in sixteen instead of one in four is 0.5 % of a fit (twenty
+// iterations, 2.8 M points, g = 6, K = 65500 92.4 -> 91.9 ms; 5.6 M, g = 8, K = 65536 345.2 -> 342.9, where runs differ by 0.9 %).
 // Measured on the way here: a successful wait on an mbarrier costs an issuing thread about 110 cycles right behind
 // an MMA, a further one 45, the MMA and its commit together 48 (N = 64); a waiting warp is back at work about 90
 // cycles after the arrival.  What counts is therefore the chain of a pair: announcement, load of the accumulator, its
@@ -465,33 +465,12 @@ __device__ __forceinline__ void write_a_row(const unsigned* xw, int ne, unsigned
     }
 }
 
-// A point's halves as they are, two to a word (rows beyond N: zeros).
+// A point's halves as they are, two to a word (rows beyond N: zeros; nothing beside an odd one's last half).
 template <int G>
-__device__ __forceinline__ void load_words(const uint16_t* __restrict__ Xs, int64_t i, int64_t N, unsigned* w) {
-    constexpr int W = (G + 1) / 2;
+__device__ __forceinline__ void load_words(const uint16_t* __restrict__ Xs, int64_t i, int64_t N, unsigned (&w)[(G + 1) / 2]) {
 #pragma unroll
-    for (int v = 0; v < W; ++v) w[v] = 0u;
-    if (i >= N) return;
-    const uint16_t* row = Xs + i * G;
-    if constexpr (G % 8 == 0) {
-#pragma unroll
-        for (int v = 0; v < G / 8; ++v) {
-            const uint4 u = __ldg(reinterpret_cast<const uint4*>(row) + v);
-            w[4 * v] = u.x; w[4 * v + 1] = u.y; w[4 * v + 2] = u.z; w[4 * v + 3] = u.w;
-        }
-    } else if constexpr (G % 4 == 0) {
-#pragma unroll
-        for (int v = 0; v < G / 4; ++v) {
-            const uint2 u = __ldg(reinterpret_cast<const uint2*>(row) + v);
-            w[2 * v] = u.x; w[2 * v + 1] = u.y;
-        }
-    } else if constexpr (G % 2 == 0) {
-#pragma unroll
-        for (int v = 0; v < G / 2; ++v) w[v] = __ldg(reinterpret_cast<const unsigned*>(row) + v);
-    } else {
-#pragma unroll
-        for (int t = 0; t < G; ++t) w[t / 2] |= (unsigned)__ldg(row + t) << (16 * (t & 1));
-    }
+    for (int v = 0; v < (G + 1) / 2; ++v) w[v] = 0u;
+    if (i < N) load_halves<G>(Xs + i * G, w);
 }
 
 template <int G>

@@ -10,6 +10,38 @@ typedef unsigned long long ull;
 
 constexpr float kBig = 3.0e38f;   // score of the padding centroids; above any real score
 
+// Two FP32 FMAs in one instruction (sm_100 packed form); each lane rounds like fma.rn.f32.
+__device__ __forceinline__ ull fma2(ull a, ull b, ull c) {
+    ull d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// G halves as they are, two to a word (the high half of the last one zero with odd G).
+template <int G>
+__device__ __forceinline__ void load_halves(const uint16_t* __restrict__ row, unsigned (&w)[(G + 1) / 2]) {
+    if constexpr (G % 8 == 0) {
+#pragma unroll
+        for (int v = 0; v < G / 8; ++v) {
+            const uint4 u = __ldg(reinterpret_cast<const uint4*>(row) + v);
+            w[4 * v] = u.x; w[4 * v + 1] = u.y; w[4 * v + 2] = u.z; w[4 * v + 3] = u.w;
+        }
+    } else if constexpr (G % 4 == 0) {
+#pragma unroll
+        for (int v = 0; v < G / 4; ++v) {
+            const uint2 u = __ldg(reinterpret_cast<const uint2*>(row) + v);
+            w[2 * v] = u.x; w[2 * v + 1] = u.y;
+        }
+    } else if constexpr (G % 2 == 0) {
+#pragma unroll
+        for (int v = 0; v < G / 2; ++v) w[v] = __ldg(reinterpret_cast<const unsigned*>(row) + v);
+    } else {
+#pragma unroll
+        for (int v = 0; v < G / 2; ++v) w[v] = (unsigned)__ldg(row + 2 * v) | (unsigned)__ldg(row + 2 * v + 1) << 16;
+        w[G / 2] = __ldg(row + G - 1);
+    }
+}
+
 // Load one point (G halves) as floats; rows beyond N read as zeros.
 template <int G>
 __device__ __forceinline__ void load_point(const uint16_t* __restrict__ X, int64_t i, int64_t N, float* x,

@@ -83,31 +83,6 @@ prep_tensor_kernel(const float* __restrict__ C, int K, int Kpad, TcParams* __res
     *reinterpret_cast<uint4*>(dst) = w;
 }
 
-// G halves as they are, two to a word (the high half of the last one is arbitrary with odd G).
-template <int G>
-__device__ __forceinline__ void load_halves(const uint16_t* __restrict__ row, unsigned (&w)[(G + 1) / 2]) {
-    if constexpr (G % 8 == 0) {
-#pragma unroll
-        for (int v = 0; v < G / 8; ++v) {
-            const uint4 u = __ldg(reinterpret_cast<const uint4*>(row) + v);
-            w[4 * v] = u.x; w[4 * v + 1] = u.y; w[4 * v + 2] = u.z; w[4 * v + 3] = u.w;
-        }
-    } else if constexpr (G % 4 == 0) {
-#pragma unroll
-        for (int v = 0; v < G / 4; ++v) {
-            const uint2 u = __ldg(reinterpret_cast<const uint2*>(row) + v);
-            w[2 * v] = u.x; w[2 * v + 1] = u.y;
-        }
-    } else if constexpr (G % 2 == 0) {
-#pragma unroll
-        for (int v = 0; v < G / 2; ++v) w[v] = __ldg(reinterpret_cast<const unsigned*>(row) + v);
-    } else {
-#pragma unroll
-        for (int v = 0; v < G / 2; ++v) w[v] = (unsigned)__ldg(row + 2 * v) | (unsigned)__ldg(row + 2 * v + 1) << 16;
-        w[G / 2] = __ldg(row + G - 1);
-    }
-}
-
 // A operand rows [x repeated SPLIT times, 2^15, 2^6, 2^-3, 2^-12, 0..] of points base + e,
 // e = first, first + STEP, .. < count, into the tiles at sA (canonical layout, 16 bytes at a time).
 template <int G, int STEP>

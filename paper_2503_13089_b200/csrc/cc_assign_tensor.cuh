@@ -198,7 +198,6 @@ __device__ __forceinline__ float chunk_min64(const uint32_t* v0, const uint32_t*
     return fminf(min3(w0, w1, u[6]), val(63));
 }
 
-__device__ __forceinline__ ull fma2(ull a, ull b, ull c) { ull r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 __device__ __forceinline__ float redux_min(float v) {
     float r;
     asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));

@@ -6,7 +6,10 @@
 // them into 16-byte pieces of matrix rows in a staging tile of its warp, and the warp writes whole 64-byte row segments.  The warps
 // of a CTA stand side by side along the in_features; no warp waits for another.  All plane groups walk in step, so that the
 // codes come from DRAM once.
-// Bound: shared-memory wavefronts (look-ups 3, operand pieces and the way out of the staging tile 2 for 32 codes).
+// Bound: not found.  Neither the shared-memory wavefronts (look-ups 3, operand pieces and the way out of the staging tile 2 for 32
+// codes) nor the bytes account for its time: 8192 x 8192, g = 5, K = 30000 22 and 25 us of 65; nor do conflicts of the look-ups (K = 100
+// 51 us) or filling the table (8192 x 376 8.3 us with K = 100 and with 30000).  A warp does codes, look-ups, staging and stores one after
+// the other, and there are 16 of them on an SM.
 // Not for rows of 4, 8 or 16 values, each of which is one load: 8192 x 28672, g = 4, K = 65536 187 us gathered, 245 so (one coordinate
 // a look-up), K = 4096 138 and 173; g = 8, 8192 x 8192, K = 20000 44.6 and 45.3.  Nor with one coordinate a look-up, where the table
 // of two does not fit: g = 9, K = 65536 75.0 and 72.6, g = 7, 20000 x 11008 261 and 267.
@@ -115,7 +118,7 @@ cudaError_t launch(cc_ctx* ctx, const uint16_t* C16, int K, int g, const uint16_
     const int groups = (g + PP - 1) / PP;
     const dim3 grid((unsigned)(ctx->sm_count / groups < 1 ? 1 : ctx->sm_count / groups), (unsigned)groups);
     ProfScope ps(ctx, CC_K_DECODE, st);
-    launch_after(dim3(grid), dim3(DP_THREADS), (size_t)plane_table_bytes(K, PP) + DP_WARPS * DP_STAGE, st, decode_planes_kernel<MODE>,
+    launch_after(grid, dim3(DP_THREADS), (size_t)plane_table_bytes(K, PP) + DP_WARPS * DP_STAGE, st, decode_planes_kernel<MODE>,
                     C16, K, g, idx, out_groups, d_out, d_in, W_hat);
     return cudaGetLastError();
 }

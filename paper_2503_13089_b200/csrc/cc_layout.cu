@@ -629,10 +629,10 @@ cudaError_t cc_launch_reshape(cc_ctx* ctx, const uint16_t* W, int64_t d_out, int
         const int64_t out_pad = pad_to(d_out, g);
         dim3 grid((unsigned)((d_in + TD - 1) / TD), (unsigned)((out_pad + TD - 1) / TD));
         if (d_in % 8 == 0 && out_pad % 8 == 0)
-            launch_after(dim3(grid), dim3(256), 0, st, reshape_transpose_vec_kernel,
+            launch_after(grid, dim3(256), 0, st, reshape_transpose_vec_kernel,
                     W, d_out, d_in, out_pad, X);
         else
-            launch_after(dim3(grid), dim3(256), 0, st, reshape_transpose_any_kernel,
+            launch_after(grid, dim3(256), 0, st, reshape_transpose_any_kernel,
                     W, d_out, d_in, out_pad, X);
     } else {
         const int64_t in_pad = pad_to(d_in, g);
@@ -668,15 +668,15 @@ cudaError_t cc_launch_decode(cc_ctx* ctx, const uint16_t* C16, int K, int g, con
             if (g == 8) return launch_decode_pipe<8>(ctx->sm_count, C16, idx, K, d_out, d_in, out_pad, W_hat, (int)grid.x, (int)grid.y, st);
             return launch_decode_pipe<16>(ctx->sm_count, C16, idx, K, d_out, d_in, out_pad, W_hat, (int)grid.x, (int)grid.y, st);
         }
-        if (vec && g == 4) launch_after(dim3(grid), dim3(256), 0, st, decode_transpose_vec_kernel<4>,
+        if (vec && g == 4) launch_after(grid, dim3(256), 0, st, decode_transpose_vec_kernel<4>,
                     C16, idx, d_out, d_in, out_pad, W_hat);
-        else if (vec && g == 8) launch_after(dim3(grid), dim3(256), 0, st, decode_transpose_vec_kernel<8>,
+        else if (vec && g == 8) launch_after(grid, dim3(256), 0, st, decode_transpose_vec_kernel<8>,
                     C16, idx, d_out, d_in, out_pad, W_hat);
-        else if (vec && g == 16) launch_after(dim3(grid), dim3(256), 0, st, decode_transpose_vec_kernel<16>,
+        else if (vec && g == 16) launch_after(grid, dim3(256), 0, st, decode_transpose_vec_kernel<16>,
                     C16, idx, d_out, d_in, out_pad, W_hat);
-        else if (g % 2 == 0) launch_after(dim3(grid), dim3(256), 0, st, decode_transpose_any_kernel<true>,
+        else if (g % 2 == 0) launch_after(grid, dim3(256), 0, st, decode_transpose_any_kernel<true>,
                     C16, K, g, idx, d_out, d_in, out_pad, W_hat);
-        else launch_after(dim3(grid), dim3(256), 0, st, decode_transpose_any_kernel<false>,
+        else launch_after(grid, dim3(256), 0, st, decode_transpose_any_kernel<false>,
                     C16, K, g, idx, d_out, d_in, out_pad, W_hat);
     } else {
         const int64_t in_pad = pad_to(d_in, g);

@@ -738,7 +738,9 @@ cudaError_t launch_linear_s(cc_ctx* ctx, const LinearPlan& p, const uint16_t* x,
         have = true;
     }
     const dim3 grid(p.o_tiles, p.tok_blocks, p.splits);
-    return launch_after(grid, dim3(LTHREADS), p.smem, st, linear_forward_kernel<G, QUANT, PADDED, STAGES>, x, M, C16, qtab, qscale, K, idx, d_out, d_in, out_groups, p.NT, p.a_pad, p.tmem_cols, p.chunks_per_split, out, split_stride, bias, status, arrived, bias_final, y_final);
+    return launch_after(grid, dim3(LTHREADS), p.smem, st, linear_forward_kernel<G, QUANT, PADDED, STAGES>,
+                        x, M, C16, qtab, qscale, K, idx, d_out, d_in, out_groups, p.NT, p.a_pad, p.tmem_cols, p.chunks_per_split, out,
+                        split_stride, bias, status, arrived, bias_final, y_final);
 }
 
 // Two stages exist where the plan can ask for them: beside the 4-bit table, and for rows of at most 8 bytes.
@@ -774,7 +776,9 @@ cudaError_t launch_gemv_w(cc_ctx* ctx, const GemvPlan& p, const uint16_t* x, int
         have = true;
     }
     const dim3 grid(p.o_blocks, p.splits, p.slices);
-    return launch_after(grid, dim3(LG_THREADS), p.smem, st, linear_gemv_kernel<G, MT, QUANT, PW>, x, M, static_cast<const unsigned char*>(book), qscale, K, p.slice_rows, idx, d_out, d_in, out_groups, p.rows_per_split, out, split_stride, status, arrived, bias, y, p.splits * p.slices == 1);
+    return launch_after(grid, dim3(LG_THREADS), p.smem, st, linear_gemv_kernel<G, MT, QUANT, PW>,
+                        x, M, static_cast<const unsigned char*>(book), qscale, K, p.slice_rows, idx, d_out, d_in, out_groups, p.rows_per_split,
+                        out, split_stride, status, arrived, bias, y, p.splits * p.slices == 1);
 }
 
 template <int G, int MT, bool QUANT>

@@ -2,8 +2,8 @@
 //
 // Gathering whole rows of a large codebook from L2 costs a request per code, of which an SM gets about 0.73 a clock
 // through.  A plane of the largest codebook (65536 FP16 values) is 128 KB: an SM that holds one looks its coordinate of
-// every code up in shared memory, 32 codes in about 3.5 clocks (the most that share a bank among 32 random ones), and so
-// 16 codes of g = 4 take as long as 10 gathers did.  Codes are read once per plane, coalesced and from L2.
+// every code up in shared memory, 32 codes in about 3.5 clocks (the most that share a bank among 32 random ones): 16 codes of
+// g = 4 are 64 look-ups, 7 clocks or those of 5 gathers.  Codes are read once per plane, coalesced and from L2.
 // Smaller codebooks put 2 or 4 planes side by side (PP values to a table row): one look-up brings as many values, at 3.5
 // and 6.2 clocks for 32 lanes.
 #pragma once
@@ -40,8 +40,12 @@ template <int MODE> struct PlaneCodes {
     static constexpr int HI = MODE == PC_EVEN ? 1 : (MODE == PC_ODD ? 4 : 8);
     unsigned lo[8], hi[HI];
 
-    static __device__ __forceinline__ unsigned word_at(const unsigned char* __restrict__ idx, unsigned off) { return __ldg(reinterpret_cast<const unsigned*>(idx + off)); }
-    static __device__ __forceinline__ unsigned code_at(const unsigned char* __restrict__ idx, unsigned off) { return __ldg(reinterpret_cast<const uint16_t*>(idx + off)); }
+    static __device__ __forceinline__ unsigned word_at(const unsigned char* __restrict__ idx, unsigned off) {
+        return __ldg(reinterpret_cast<const unsigned*>(idx + off));
+    }
+    static __device__ __forceinline__ unsigned code_at(const unsigned char* __restrict__ idx, unsigned off) {
+        return __ldg(reinterpret_cast<const uint16_t*>(idx + off));
+    }
 
     // off: byte offset of the first; row: bytes of a row of codes; second: 2 if the other group exists, else 0 (PC_EVEN: it does)
     __device__ __forceinline__ void request(const unsigned char* __restrict__ idx, unsigned off, unsigned row, unsigned second) {

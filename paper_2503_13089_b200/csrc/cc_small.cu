@@ -33,7 +33,6 @@ constexpr int SM_CHUNK = 4 * SM_LPP;                 // centroids a group takes 
 constexpr int SM_MEANS = 4096;                       // K g up to which the last block forms the means
 
 __device__ __forceinline__ ull f2_add(ull a, ull b) { ull r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ ull f2_fma(ull a, ull b, ull c) { ull r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 __device__ __forceinline__ ull f2_pack(float lo, float hi) { ull r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r; }
 __device__ __forceinline__ float f2_sum(ull a) { float lo, hi; asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a)); return lo + hi; }
 
@@ -156,7 +155,7 @@ small_kernel(const uint16_t* __restrict__ X, int64_t N, float* C, int K, int mod
                 for (int p = 0; p < SM_P; ++p) {
                     ull d2 = 0ull;
 #pragma unroll
-                    for (int t = 0; t < GP; ++t) { const ull df = f2_add(x2[p][t], cv[t]); d2 = f2_fma(df, df, d2); }
+                    for (int t = 0; t < GP; ++t) { const ull df = f2_add(x2[p][t], cv[t]); d2 = fma2(df, df, d2); }
                     const float d = f2_sum(d2);
                     m[p] = e == 0 ? d : fminf(m[p], d);
                 }
@@ -225,7 +224,7 @@ small_kernel(const uint16_t* __restrict__ X, int64_t N, float* C, int K, int mod
                         const ull* row = sm_c + jj * GP;
                         ull d2 = 0ull;
 #pragma unroll
-                        for (int t = 0; t < GP; ++t) { const ull df = f2_add(x2[p][t], row[t]); d2 = f2_fma(df, df, d2); }
+                        for (int t = 0; t < GP; ++t) { const ull df = f2_add(x2[p][t], row[t]); d2 = fma2(df, df, d2); }
                         if (f2_sum(d2) <= b1[p]) {
                             const double d = exact_distance<G>(xv[p], row);
                             if (d < D || (d == D && jj < jm)) { D = d; jm = jj; }

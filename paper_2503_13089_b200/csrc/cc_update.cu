@@ -318,7 +318,8 @@ cudaError_t cc_launch_update(cc_ctx* ctx, const WsLayout& L, const uint16_t* X, 
     if (e != cudaSuccess) return e;
     {
         ProfScope ps(ctx, CC_K_UPDATE_FINISH, st);
-        launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, update_finish_kernel, reinterpret_cast<long long*>(ws + L.sum_lo), reinterpret_cast<long long*>(ws + L.sum_hi), count_copies, counts, K, g, R, C);
+        launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, update_finish_kernel,
+                     reinterpret_cast<long long*>(ws + L.sum_lo), reinterpret_cast<long long*>(ws + L.sum_hi), count_copies, counts, K, g, R, C);
     }
     if (ctx->empty_rule == CC_EMPTY_SPLIT_LARGEST) return cc_launch_split_empty(ctx, L, C, K, g, counts, st);
     return cudaGetLastError();
@@ -335,7 +336,8 @@ cudaError_t cc_launch_codebook_grad(cc_ctx* ctx, const WsLayout& L, const uint16
     const cudaError_t e = accumulate_all(ctx, L, dX, N, g, idx, K, counts, R, &count_copies, false, st);
     if (e != cudaSuccess) return e;
     ProfScope ps(ctx, CC_K_UPDATE_FINISH, st);
-    launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, grad_finish_kernel, reinterpret_cast<long long*>(ws + L.sum_lo), reinterpret_cast<long long*>(ws + L.sum_hi), K * g, R, dC);
+    launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, grad_finish_kernel,
+                 reinterpret_cast<long long*>(ws + L.sum_lo), reinterpret_cast<long long*>(ws + L.sum_hi), K * g, R, dC);
     return cudaGetLastError();
 }
 
@@ -344,7 +346,8 @@ cudaError_t cc_launch_update_means(cc_ctx* ctx, const WsLayout& L, int g, int K,
     char* ws = static_cast<char*>(ctx->ws);
     {
         ProfScope ps(ctx, CC_K_UPDATE_FINISH, st);
-        launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, update_finish_kernel, reinterpret_cast<long long*>(ws + L.sum_lo), reinterpret_cast<long long*>(ws + L.sum_hi), counts, counts, K, g, 1, C);
+        launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, update_finish_kernel,
+                     reinterpret_cast<long long*>(ws + L.sum_lo), reinterpret_cast<long long*>(ws + L.sum_hi), counts, counts, K, g, 1, C);
     }
     if (ctx->empty_rule == CC_EMPTY_SPLIT_LARGEST) return cc_launch_split_empty(ctx, L, C, K, g, counts, st);
     return cudaGetLastError();
@@ -433,6 +436,7 @@ extern "C" cc_status cc_update_static(int device, const uint16_t* X, int64_t N, 
 #undef CALL
         if (e != cudaSuccess) return CC_ERR_CUDA;
     }
-    launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, update_finish_kernel, reinterpret_cast<long long*>(sum_lo), reinterpret_cast<long long*>(sum_hi), counts, counts, K, g, 1, C);
+    launch_after(dim3((K * g + 255) / 256), dim3(256), 0, st, update_finish_kernel,
+                 reinterpret_cast<long long*>(sum_lo), reinterpret_cast<long long*>(sum_hi), counts, counts, K, g, 1, C);
     return cudaGetLastError() == cudaSuccess ? CC_OK : CC_ERR_CUDA;
 }
