@@ -22,7 +22,8 @@
  *  - N = number of sub-vectors, g = sub-vector dimension (1..16),
  *    K = number of centroids (1..65536, the paper keeps n <= 2^16 so that a
  *    code fits 16 bits; codes are 0-based).  N < 2^31.
- *  - The same inputs give bit-identical outputs on every call.
+ *  - The same inputs give bit-identical outputs on every call (those of the layer forward with a workspace of the
+ *    same size: see cc_linear_workspace_bytes_preferred).
  *  - Scratch memory is one caller-owned workspace (cc_workspace_bytes /
  *    cc_set_workspace); the library itself allocates no device memory except
  *    in cc_compress_host (a buffer kept in the context).

@@ -657,21 +657,6 @@ int64_t linear_pad_from(int g, int K) {
     return g % 2 ? LINEAR_PAD_ODD : LINEAR_PAD_EVEN;
 }
 
-// Tokens from which decoding the weight once and multiplying it afterwards (cc_linear_wide.cu) is the faster way, gathering /
-// decoding in us: 4096 x 4096, g = 4, K = 65536, 128 tokens 42 / 46, 192 tokens 52 / 46, 512 tokens 85 / 52.  Earlier where
-// the tiles of this kernel fill the SMs by themselves, so that its waves are the coarser (11008 x 4096, g = 8, 128 tokens
-// 95 / 67; g = 6, 33 tokens 83 / about 80).  Later where it splits the in_features and so keeps the SMs busier than the few whole
-// tiles of the product do: from 224 tokens on for long in_features and short rows (4096 x 11008, g = 4: K = 256, 192 tokens 58 / 67,
-// K = 8000 65 / 71, at 224 tokens 82 / 71; g = 8, K = 16000, 192 tokens 82 / 75), from 256 on for the 4-bit codebook in shared
-// memory with four splits or more (1024 x 4096, g = 6, 192 tokens 19 / 26, 224 tokens 23 / 26; FP16, 2048 x 2048, eight splits, g = 8,
-// 224 tokens 19 / 16).
-constexpr int LINEAR_WIDE_FEWEST = 96, LINEAR_WIDE_FROM = 192, LINEAR_WIDE_LONG = 224, LINEAR_WIDE_Q4 = 256;
-int linear_wide_from(int fill, int64_t d_in, int g, bool quant) {
-    if (fill == 1) return LINEAR_WIDE_FEWEST;
-    if (quant && fill >= 4) return LINEAR_WIDE_Q4;
-    return !quant && fill > 2 && g <= 6 && d_in > 8192 ? LINEAR_WIDE_LONG : LINEAR_WIDE_FROM;
-}
-
 }  // namespace
 
 size_t cc_linear_scratch_bytes(int64_t M, int64_t d_out, int64_t d_in, int sm_count) {
@@ -699,8 +684,12 @@ size_t cc_linear_scratch_bytes_preferred(int64_t M, int64_t d_out, int64_t d_in,
     bool few = true;
     for (int words = 0; words < 2; ++words)
         few = few && gemv_for(M, d_out, d_in, sm_count, K, g, false, words).fits && (!q4 || gemv_for(M, d_out, d_in, sm_count, K, g, true, words).fits);
-    const PlanesPlan p = planes_for(M, d_out, d_in, sm_count, K, g, false);      // the 4-bit codebook's plan is the same, or there is none
-    return !few && p.fits && CC_LINEAR_SCRATCH_FROM + p.bytes > need ? CC_LINEAR_SCRATCH_FROM + p.bytes : need;
+    size_t most = need;
+    for (int quant = 0; quant <= (q4 ? 1 : 0) && !few; ++quant) {
+        const PlanesPlan p = planes_for(M, d_out, d_in, sm_count, K, g, quant);
+        if (p.fits && CC_LINEAR_SCRATCH_FROM + p.bytes > most) most = CC_LINEAR_SCRATCH_FROM + p.bytes;
+    }
+    return most;
 }
 
 int cc_linear_q_table_max(void) { return LQ_TABLE_MAX; }

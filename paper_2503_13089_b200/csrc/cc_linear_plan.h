@@ -215,6 +215,21 @@ inline LinearPlan linear_plan(int64_t M, int64_t d_out, int64_t d_in, int sm_cou
     return p;
 }
 
+// Tokens from which decoding the weight once and multiplying it afterwards (cc_linear_wide.cu) is the faster way, gathering /
+// decoding in us: 4096 x 4096, g = 4, K = 65536, 128 tokens 42 / 46, 192 tokens 52 / 46, 512 tokens 85 / 52.  Earlier where
+// the tiles of this kernel fill the SMs by themselves, so that its waves are the coarser (11008 x 4096, g = 8, 128 tokens
+// 95 / 67; g = 6, 33 tokens 83 / about 80).  Later where it splits the in_features and so keeps the SMs busier than the few whole
+// tiles of the product do: from 224 tokens on for long in_features and short rows (4096 x 11008, g = 4: K = 256, 192 tokens 58 / 67,
+// K = 8000 65 / 71, at 224 tokens 82 / 71; g = 8, K = 16000, 192 tokens 82 / 75), from 256 on for the 4-bit codebook in shared
+// memory with four splits or more (1024 x 4096, g = 6, 192 tokens 19 / 26, 224 tokens 23 / 26; FP16, 2048 x 2048, eight splits, g = 8,
+// 224 tokens 19 / 16).
+constexpr int LINEAR_WIDE_FEWEST = 96, LINEAR_WIDE_FROM = 192, LINEAR_WIDE_LONG = 224, LINEAR_WIDE_Q4 = 256;
+inline int linear_wide_from(int fill, int64_t d_in, int g, bool quant) {
+    if (fill == 1) return LINEAR_WIDE_FEWEST;
+    if (quant && fill >= 4) return LINEAR_WIDE_Q4;
+    return !quant && fill > 2 && g <= 6 && d_in > 8192 ? LINEAR_WIDE_LONG : LINEAR_WIDE_FROM;
+}
+
 // ---- Layer forward plane by plane.
 constexpr int PL_ROWS = 128, PL_KB = 64, PL_NT_MAX = 256, PL_SPLITS_MAX = 64;
 constexpr size_t PL_SMEM = 226 * 1024, PL_HEAD = 256;
@@ -295,7 +310,10 @@ inline PlanesPlan planes_plan(int64_t M, int64_t d_out, int64_t d_in, int sm_cou
 //   few in_features for many out_features, whose tiles keep the SMs busy without parts: 101 tokens, 6848 x 1011, g = 8, K = 2499, 4 bits 16.4 /
 //     18.0, 5 tokens, 10624 x 686, g = 4, K = 39870 13.9 / 15.2 (odd g: 66 tokens, 8000 x 896, g = 5 22 / 18);
 //   many tokens on few codes: 224 tokens, 768 x 512, g = 4, K = 17749 12.9 / 14.3.
-// Over 162 drawn layers of 5 to 256 tokens the planes alone are 1.22 times as fast in the mean, with these bounds 1.24.
+// Over 260 drawn layers of 3 to 256 tokens, in device time (replayed from a graph), these bounds and PLANES_WIDE_IN make the layer 1.16 times as fast
+// in the mean, the 138 that take the planes 1.32; 14 of those are slower by more than 5 %, at worst 1.32 times (8 tokens, 384 x 12480, g = 16).
+// Called one by one from Python the three launches take the host 13.7 us, where one takes 9 and two 11.4: layers of less than half a million
+// weights are up to 1.5 times as slow then, though the device is done in 0.7 of the time.
 // Up to 64 tokens the answer may not depend on the form of the codebook (both give the same bits there).
 inline bool planes_pay(const PlanesPlan& p, int64_t M, int64_t d_out, int64_t d_in, int g, bool quant) {
     const int64_t codes = (d_out + g - 1) / g * d_in;
@@ -314,10 +332,22 @@ inline int planes_chain(int64_t M, int64_t d_out, int64_t d_in, int sm_count, in
     return p.chunks_per_split < PLANES_CHAIN_MOST ? p.chunks_per_split : PLANES_CHAIN_MOST;
 }
 
+// In_features from which the planes take a layer that would otherwise be decoded once and multiplied.  That way costs little beside a gather a
+// code, while the planes write and read partial sums of all out_features however few the in_features are.  Decoded once / planes, device
+// time in us: 158 tokens, 12544 x 256, g = 3, K = 1110 13.8 / 35.5; 199, 1472 x 384, g = 2 6.8 / 13.4; 203, 6976 x 350, g = 7 15 / 23; 249, 2688 x
+// 1032, g = 9 12 / 18; 102, 8384 x 1239, g = 4, 4 bits 15 / 23; 123, 8832 x 1216, g = 4, K = 44770, 4 bits 17 / 24; 154, 11392 x 2358, g = 4, 4 bits 31 / 46;
+// 186, 6464 x 2624, g = 4, 4 bits 22 / 35; but 254, 1514 x 2816, g = 12 22 / 19; 193, 1728 x 3392, g = 7 25 / 17; 195, 832 x 4224, g = 2 21 / 18; 183,
+// 10240 x 4480, g = 8, 4 bits 61 / 56; 122, 11494 x 7104, g = 4, K = 65536 144 / 94; 162, 11133 x 14528, g = 6 306 / 139 (three of 21 longer layers, all
+// g = 4 with 160 tokens or more, 10 to 13 % slower: 185, 12416 x 5184 77 / 87).
+constexpr int PLANES_WIDE_IN = 2700;
+
 // The plan with which the planes take a call that the look-up kernel does not; .fits is false where they do not.
 inline PlanesPlan planes_for(int64_t M, int64_t d_out, int64_t d_in, int sm_count, int K, int g, bool quant) {
     PlanesPlan p = {};
     if (M > PL_NT_MAX) return p;
+    const LinearPlan l = quant ? linear_plan(M, d_out, d_in, sm_count, M >= LQ_WIDE_FROM ? LNT_MAX : LQ_NT_MAX, (size_t)K * (g / 2), g)
+                               : linear_plan(M, d_out, d_in, sm_count, LNT_MAX, 0, g);
+    if (d_in <= PLANES_WIDE_IN && M >= linear_wide_from(l.fill, d_in, g, quant)) return p;
     p = planes_plan(M, d_out, d_in, sm_count, K, g, planes_chain(M, d_out, d_in, sm_count, g));
     p.fits = p.fits && planes_pay(p, M, d_out, d_in, g, quant);
     return p;

@@ -34,7 +34,7 @@ def test_linear_planes_where_they_are_taken(M, d_out, d_in, g, K, q4):
 
 
 @pytest.mark.parametrize("M,d_out,d_in,g,K", [
-    (33, 10000, 1300, 6, 65500), (200, 4100, 2100, 4, 65536),                # one coordinate a look-up; four and two stages
+    (33, 10000, 1300, 6, 65500), (200, 3000, 2760, 4, 65536),                # one coordinate a look-up; four and two stages
     (129, 793, 523, 2, 25467), (12, 903, 1300, 9, 3000),                     # two
     (26, 1085, 4491, 16, 19780), (91, 260, 2380, 16, 17185), (128, 777, 900, 4, 3000),  # four
 ])

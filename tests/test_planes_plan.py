@@ -5,14 +5,14 @@ import subprocess
 
 # M, d_out, d_in, g, K, 4-bit codebook: layers for the planes; coordinates a look-up and stages that their plans have on 148 SMs.
 LAYERS = [
-    ((65, 3134, 640, 1, 65536, False), (1, 2)), ((200, 4100, 2100, 4, 65536, False), (1, 2)), ((256, 8192, 1280, 4, 65536, False), (1, 2)),
+    ((65, 3134, 640, 1, 65536, False), (1, 2)), ((200, 3000, 2760, 4, 65536, False), (1, 2)), ((256, 2050, 4160, 4, 65536, False), (1, 2)),
     ((33, 10000, 1300, 6, 65500, False), (1, 4)), ((48, 14000, 1100, 7, 65536, False), (1, 4)),
-    ((128, 208, 257, 8, 26294, False), (2, 2)), ((129, 793, 523, 2, 25467, False), (2, 2)), ((256, 2050, 1030, 8, 32768, False), (2, 2)),
+    ((91, 244, 453, 9, 30917, False), (2, 2)), ((129, 793, 523, 2, 25467, False), (2, 2)), ((256, 1030, 2800, 8, 32768, False), (2, 2)),
     ((70, 1030, 1200, 8, 32768, True), (2, 2)), ((192, 1030, 1200, 4, 16384, True), (2, 4)), ((12, 903, 1300, 9, 3000, False), (2, 4)),
     ((129, 453, 895, 2, 968, False), (2, 4)), ((60, 1030, 1025, 2, 20000, False), (2, 4)),
     # the last whole stage is the first of a block of the grid, in_features end behind it
     ((26, 1085, 4491, 16, 19780, False), (4, 2)), ((91, 260, 2380, 16, 17185, False), (4, 2)),
-    ((200, 442, 1541, 3, 8220, False), (4, 2)), ((255, 446, 1345, 3, 7016, False), (4, 2)), ((192, 568, 1920, 4, 8753, True), (4, 2)),
+    ((192, 202, 3008, 3, 8722, False), (4, 2)), ((255, 212, 2827, 3, 7899, False), (4, 2)), ((192, 568, 1920, 4, 8753, True), (4, 2)),
     ((16, 514, 1000, 4, 300, False), (4, 4)), ((128, 777, 900, 4, 3000, False), (4, 4)), ((129, 737, 1088, 4, 858, True), (4, 4)),
     ((6, 207, 64, 16, 22, False), (4, 4)),
 ]
