@@ -125,13 +125,17 @@ cudaError_t launch(cc_ctx* ctx, const uint16_t* C16, int K, int g, const uint16_
 
 }  // namespace
 
-// Where it is the faster one.  Gathering / so, in us: 8192 x 8192, g = 5, K = 30000 91.6 / 65.4, g = 7, K = 5000 73.8 / 52.3; 13952 x
-// 9472, g = 9, K = 9371 141 / 101; 11520 x 768, g = 9, K = 13095 12.2 / 11.1; 2000 x 2000, g = 5, K = 3000 7.4 / 6.7; but 768 x 448, g = 9,
-// K = 14017 3.0 / 5.3 (every CTA reads the whole codebook for its table).
+// Where it is the faster one: every CTA fills its table from the whole codebook, some 0.02 us for 1000 values of it, which the matrix has to be
+// large enough to make up for; rows of five values gain most.  Gathering / so, in us: 8192 x 8192, g = 5, K = 30000 91.6 / 65.4, g = 7, K = 5000
+// 73.8 / 52.3; 13952 x 9472, g = 9, K = 9371 141 / 101; but 768 x 448, g = 9, K = 14017 3.0 / 5.3.  Around the bound on values a row of the codebook
+// (dp_per_row): g = 5, 3 M values, K = 30000 8.8 / 11.4, 4 M, K = 30000 10.3 / 9.2; 9 M values: g = 7, K = 30000 12.5 / 14.6, 16000 12.5 / 11.2, g = 9, K =
+// 24000 11.6 / 12.7, 16000 11.5 / 11.4, 8000 11.5 / 10.3, g = 11, K = 16000 11.1 / 12.6, g = 15, K = 24000 11.1 / 13.7, 8000 11.1 / 10.2; 6 M: g = 9, K = 24000
+// 8.9 / 11.3, 16000 8.9 / 8.4, g = 13, K = 8000 8.5 / 11.3; 4.4 M, g = 15, K = 30952 8.9 / 15.3.
 constexpr int64_t DP_FROM = 3000000;                 // values
+constexpr int64_t dp_per_row(int g) { return g <= 5 ? 110 : g <= 7 ? 340 : g <= 9 ? 500 : 800; }
 bool cc_decode_planes_applies(int K, int g, int64_t d_out, int64_t d_in, const void* W_hat) {
     return g % 2 && g >= 5 && d_in % 8 == 0 && (reinterpret_cast<uintptr_t>(W_hat) & 15u) == 0 && d_out * d_in >= DP_FROM &&
-           plane_table_bytes(K, PP) + DP_WARPS * DP_STAGE <= DP_SMEM;
+           d_out * d_in >= dp_per_row(g) * K && plane_table_bytes(K, PP) + DP_WARPS * DP_STAGE <= DP_SMEM;
 }
 
 cudaError_t cc_launch_decode_planes(cc_ctx* ctx, const uint16_t* C16, int K, int g, const uint16_t* idx, int64_t d_out, int64_t d_in,

@@ -9,6 +9,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("d_out,d_in,g,K,off", [
     (1733, 1736, 5, 3000, 0), (1735, 1736, 5, 37376, 0), (2304, 1320, 9, 1, 0), (3001, 1000, 7, 16001, 0), (1750, 2008, 7, 999, 1), (1760, 1800, 15, 65, 1),
     (37000, 88, 11, 2000, 0), (12, 260000, 13, 300, 0),
+    (2401, 1736, 5, 37376, 0), (3001, 1880, 7, 16001, 0), (3001, 1808, 7, 16001, 0), (2000, 1600, 11, 4000, 1), (2000, 1592, 11, 4000, 1),   # on both sides of the bound
 ])
 def test_decode_planes(d_out, d_in, g, K, off):
     """off: codes that start on an odd address of 16-bit words."""
